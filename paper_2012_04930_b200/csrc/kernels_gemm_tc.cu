@@ -76,6 +76,21 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+// One lane of the (converged) warp, chosen by the hardware.  The compiler then knows that a single thread runs the
+// branch and keeps descriptors and tensor-memory addresses in uniform registers; behind `lane == 0` every
+// tcgen05.mma first moves its operands there one at a time, about 46 clocks per instruction at best (kind::f16,
+// unrolled loop, operands ready) against 9 clocks behind elect.sync, where the tensor pipe sets the pace.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n"
+      " .reg .pred p;\n"
+      " elect.sync _|p, 0xffffffff;\n"
+      " selp.u32 %0, 1, 0, p;\n"
+      "}\n"
+      : "=r"(p));
+  return p != 0;
+}
 __device__ __forceinline__ int tc_error_now() { return *reinterpret_cast<volatile int*>(&g_tc_error); }
 
 // Bounded wait: false when the phase did not complete within kSpinCycles, or when the error word has been set in
@@ -217,9 +232,9 @@ __device__ __forceinline__ void split_buffer(const uint8_t* hi_buf, uint8_t* lo_
 // accumulator buffer fit (64-column tiles; 128-column tiles when every CTA has a single item, so one buffer),
 // A_hi [B_hi | B_lo] is ONE instruction of 2 BN columns into two accumulators that the epilogue adds, and with
 // A_lo B_hi that makes two instructions per 8 k; otherwise the three products are three instructions into one
-// accumulator.  Measured with clock64 around the issue loop: a 128 x 128 x 32 k-block takes the issuing thread about
-// 800 clocks with two instructions per 8 k, the TF32 rate of the tensor pipe for its 3 x 128 x 128 x 32 products
-// (about 2000 multiply-adds per clock and SM), and 1000 with three.
+// accumulator.  With the issuing thread behind elect.sync the tensor pipe sets the pace (see elect_one); behind
+// `lane == 0` an instruction cost it 97 clocks whether 128 or 256 columns wide.  51 249 x 128 x 602: 57 -> 47 us,
+// 269 498 x 256 x 256: 201 -> 151 us, 256 x 256 x 269 498: 169 -> 151 us (L2 flushed).
 template <int BN_, bool A_MN_, bool B_MN_, bool DB_>
 struct Shape {
   static constexpr int BN = BN_;
@@ -320,7 +335,7 @@ gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
 
   if (warp == 0 || warp == 2) {
     // ---------------- TMA producers: warp 0 streams A, warp 2 streams B ----------------
-    if (lane == 0) {
+    if (elect_one()) {
       const bool is_a = warp == 0;
       const uint32_t ring = is_a ? NA : NS;
       uint64_t* full = is_a ? full_a : full_b;
@@ -367,7 +382,7 @@ gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    if (elect_one()) {
       // instruction descriptor: D fp32, A (tensor memory) and B tf32, B K-major or MN-major, N x 128
       const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((B_MN ? 1u : 0u) << 16) | ((uint32_t)(BN >> 3) << 17) |
                              ((uint32_t)(BM >> 4) << 24);

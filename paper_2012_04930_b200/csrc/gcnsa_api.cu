@@ -63,6 +63,16 @@ using namespace gcnsa;
 
 extern "C" int64_t gcnsa_launch_count(void);
 
+// Activations, work buffers and reduction scratch of one pass over a partition.  Lane 0 serves the calls that go
+// partition by partition; a recorded epoch runs several partitions at once, one per lane (epoch_lanes).
+struct Lane {
+  float* H[GCNSA_MAX_LAYERS + 1] = {nullptr};  // H[l], l >= 1
+  float* S[GCNSA_MAX_LAYERS] = {nullptr};      // A_hat H^{l-1} of layers that aggregate first
+  float *tmp_a = nullptr, *tmp_b = nullptr, *dlogits = nullptr;
+  void *ws = nullptr, *sc = nullptr;
+  const float* s0_used = nullptr;  // A_hat H^0 the latest forward used (the cached one or S[0])
+};
+
 struct gcnsa_model {
   Env env;
   gcnsa_model_opts o{};
@@ -86,14 +96,12 @@ struct gcnsa_model {
   std::vector<float*> ax;
   std::vector<int64_t> ax_version;  // x_version of the partition the product was computed from (0 = none yet)
   uint64_t ax_uid = 0;
-  const float* s0_used = nullptr;   // A_hat H^0 the latest forward used (the cached one or S[0])
-  float* H[GCNSA_MAX_LAYERS + 1] = {nullptr};  // H[l], l >= 1
-  float* S[GCNSA_MAX_LAYERS] = {nullptr};      // A_hat H^{l-1} of layers that aggregate first
-  float *tmp_a = nullptr, *tmp_b = nullptr, *dlogits = nullptr, *loss_parts = nullptr;
+  std::vector<Lane> lanes;        // at least one
+  float* gparts = nullptr;        // [m x count]: the gradient of every partition of an epoch
+  float* loss_parts = nullptr;
   // evaluation buffers (allocated on first gcnsa_evaluate)
   int32_t *ev_pred = nullptr, *ev_hits = nullptr;
   uint8_t* ev_mask = nullptr;
-  void *ws = nullptr, *sc = nullptr;
   size_t ws_bytes = 0, sc_bytes = 0;
   int64_t ld_max = 0;
   int32_t last_forward = -1, accumulated = 0;
@@ -442,6 +450,40 @@ static int copy_param(const gcnsa_model* M, float* base, int32_t layer, bool is_
   return GCNSA_OK;
 }
 
+// How many partitions a recorded epoch works on at once: up to kMaxLanes while a partition has at most kLaneNnz stored
+// entries.  The kernels of such a partition are microseconds long and leave most of the chip idle, so the epoch is a
+// chain of launch latencies that the branches overlap (2 000 vertices, 2 partitions: 145 -> 83 us per epoch; 20 000
+// vertices, 4 partitions: 403 -> 224 us; 58 241 vertices, 1.9 M entries in each of 3 partitions: 835 -> 684 us).  At
+// 20.8 M entries per partition every sparse product fills the chip by itself and two of them at once evict each
+// other's source rows from L1 and L2 (233 K vertices, 5 partitions: 7.1 ms with one lane, 8.1 with two, 9.0 with
+// five); at 10 M entries two lanes gain 1 % and four lose 3 % (2.45 M vertices), which does not pay for the memory.
+constexpr int64_t kMaxLanes = 8, kLaneNnz = 4 << 20;
+static int epoch_lanes(const gcnsa_model_opts& o, const gcnsa_parts* parts) {
+  int64_t nnz_max = 0;
+  for (const DevPart& d : parts->parts) nnz_max = std::max<int64_t>(nnz_max, d.info.nnz);
+  if (!o.epoch_graph || nnz_max > kLaneNnz) return 1;
+  return (int)std::max<int64_t>(1, std::min<int64_t>(parts->m, kMaxLanes));
+}
+
+static bool alloc_lane(gcnsa_model* M, Lane& W, size_t act) {
+  auto get = [&](size_t bytes) { return (float*)M->dalloc(bytes); };
+  W.tmp_a = get(act);
+  W.tmp_b = get(act);
+  W.dlogits = get((size_t)M->n_max * GCNSA_LD(M->o.dims[M->L]) * sizeof(float));
+  W.ws = get(std::max<size_t>(M->ws_bytes, 256));
+  W.sc = get(std::max<size_t>(M->sc_bytes, 256));
+  bool ok = W.tmp_a && W.tmp_b && W.dlogits && W.ws && W.sc;
+  for (int l = 0; l < M->L && ok; ++l) {
+    W.H[l + 1] = get((size_t)M->n_max * GCNSA_LD(M->o.dims[l + 1]) * sizeof(float));
+    ok = W.H[l + 1] != nullptr;
+    if (ok && !M->transform_first[l]) {
+      W.S[l] = get((size_t)M->n_max * GCNSA_LD(M->o.dims[l]) * sizeof(float));
+      ok = W.S[l] != nullptr;
+    }
+  }
+  return ok;
+}
+
 int gcnsa_model_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcnsa_model_opts* opts,
                        const float* const* w0, const float* const* b0, gcnsa_model** out) {
   if (!out) return fail(GCNSA_ERR_ARG, "out is NULL");
@@ -490,25 +532,33 @@ int gcnsa_model_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcn
   M->theta = (float*)M->dalloc(pbytes); M->gsum = (float*)M->dalloc(pbytes);
   M->am = (float*)M->dalloc(pbytes);    M->av = (float*)M->dalloc(pbytes);
   const size_t act = (size_t)M->n_max * (size_t)M->ld_max * sizeof(float);
-  M->tmp_a = (float*)M->dalloc(act); M->tmp_b = (float*)M->dalloc(act);
-  M->dlogits = (float*)M->dalloc((size_t)M->n_max * GCNSA_LD(parts->c) * sizeof(float));
+  M->gparts = (float*)M->dalloc(pbytes * (size_t)M->m);
   M->loss_parts = (float*)M->dalloc((size_t)(M->m + 1) * sizeof(float));
   M->adam_state = (double*)M->dalloc(4 * sizeof(double));
-  bool ok = M->theta && M->gsum && M->am && M->av && M->tmp_a && M->tmp_b && M->dlogits && M->loss_parts && M->adam_state;
+  bool ok = M->theta && M->gsum && M->am && M->av && M->gparts && M->loss_parts && M->adam_state;
   size_t ws = 0, sc = softmax_ce_scratch(M->n_max);
-  for (int l = 0; l < M->L && ok; ++l) {
+  for (int l = 0; l < M->L; ++l) {
     const int64_t din = opts->dims[l], dout = opts->dims[l + 1];
-    M->H[l + 1] = (float*)M->dalloc((size_t)M->n_max * GCNSA_LD(dout) * sizeof(float));
-    ok = ok && M->H[l + 1];
-    if (!M->transform_first[l]) {
-      M->S[l] = (float*)M->dalloc((size_t)M->n_max * GCNSA_LD(din) * sizeof(float));
-      ok = ok && M->S[l];
-    }
     ws = std::max(ws, gemm_workspace(opts->gemm_mode, 1, 0, din, dout, M->n_max));
     ws = std::max(ws, gemm_workspace(opts->gemm_mode, 0, 0, M->n_max, dout, din));
     ws = std::max(ws, gemm_workspace(opts->gemm_mode, 0, 1, M->n_max, din, dout));
     sc = std::max(sc, colsum_scratch(M->n_max, (int32_t)dout));
     sc = std::max(sc, gemm_colsum_scratch(M->n_max, (int32_t)din));  // the fused bias gradient of the layer below
+  }
+  M->ws_bytes = ws; M->sc_bytes = sc;
+  M->lanes.resize((size_t)epoch_lanes(*opts, parts));
+  for (size_t i = 0; i < M->lanes.size() && ok; ++i) {
+    const size_t mark = M->owned.size();
+    ok = alloc_lane(M, M->lanes[i], act);
+    if (!ok && i > 0) {  // lanes after the first only make a recorded epoch faster
+      while (M->owned.size() > mark) {
+        M->env.release(M->owned.back());
+        M->owned.pop_back();
+      }
+      M->lanes.resize(i);
+      ok = true;
+      break;
+    }
   }
   if (ok && opts->cache_ax) {
     M->ax.assign((size_t)parts->m, nullptr);
@@ -533,26 +583,24 @@ int gcnsa_model_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcn
       cudaMemsetAsync(M->theta_acc, 0, pb, M->env.stream());
     }
   }
-  if (ok) {
-    M->ws_bytes = ws; M->sc_bytes = sc;
-    M->ws = M->dalloc(std::max<size_t>(ws, 256)); M->sc = M->dalloc(std::max<size_t>(sc, 256));
-    ok = M->ws && M->sc;
-  }
   if (!ok) return fail_free(fail(GCNSA_ERR_OOM, "device allocation failed"));
   cudaStream_t s = M->env.stream();
   cudaError_t e = cudaMemsetAsync(M->theta, 0, pbytes, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(M->gsum, 0, pbytes, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(M->am, 0, pbytes, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(M->av, 0, pbytes, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(M->tmp_a, 0, act, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(M->tmp_b, 0, act, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(M->dlogits, 0, (size_t)M->n_max * GCNSA_LD(parts->c) * sizeof(float), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(M->gparts, 0, pbytes * (size_t)M->m, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(M->loss_parts, 0, (size_t)(M->m + 1) * sizeof(float), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(M->adam_state, 0, 4 * sizeof(double), s);
-  for (int l = 0; l < M->L && e == cudaSuccess; ++l) {
-    e = cudaMemsetAsync(M->H[l + 1], 0, (size_t)M->n_max * GCNSA_LD(opts->dims[l + 1]) * sizeof(float), s);
-    if (e == cudaSuccess && M->S[l])
-      e = cudaMemsetAsync(M->S[l], 0, (size_t)M->n_max * GCNSA_LD(opts->dims[l]) * sizeof(float), s);
+  for (Lane& W : M->lanes) {
+    if (e == cudaSuccess) e = cudaMemsetAsync(W.tmp_a, 0, act, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(W.tmp_b, 0, act, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(W.dlogits, 0, (size_t)M->n_max * GCNSA_LD(parts->c) * sizeof(float), s);
+    for (int l = 0; l < M->L && e == cudaSuccess; ++l) {
+      e = cudaMemsetAsync(W.H[l + 1], 0, (size_t)M->n_max * GCNSA_LD(opts->dims[l + 1]) * sizeof(float), s);
+      if (e == cudaSuccess && W.S[l])
+        e = cudaMemsetAsync(W.S[l], 0, (size_t)M->n_max * GCNSA_LD(opts->dims[l]) * sizeof(float), s);
+    }
   }
   if (e != cudaSuccess) return fail_free(cuda_fail(e, "cudaMemsetAsync"));
   for (int l = 0; l < M->L; ++l) {
@@ -578,12 +626,15 @@ static int ensure_ax(gcnsa_model* M, const gcnsa_parts* P, int32_t p) {
   return GCNSA_OK;
 }
 
-int gcnsa_forward(gcnsa_model* M, const gcnsa_parts* P, int32_t p, float* loss_dev) {
-  if (!M || !P || p < 0 || p >= P->m) return fail(GCNSA_ERR_ARG, "bad partition index or NULL");
+static int check_model(const gcnsa_model* M, const gcnsa_parts* P) {
   if (P->m != M->m || P->f != M->o.dims[0] || P->c != M->o.dims[M->L] || P->n_max > M->n_max)
     return fail(GCNSA_ERR_ARG, "model was created for other partitions");
+  return GCNSA_OK;
+}
+
+// forward pass of partition p in the buffers of lane W on stream s; the partition's loss goes to loss_parts[p]
+static int forward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& W, void* s) {
   const DevPart& d = P->parts[p];
-  void* s = M->env.e.stream;
   const int64_t n = d.info.n, nnz = d.info.nnz;
   const float* h = d.x;
   int64_t ldh = P->ldx;
@@ -600,20 +651,20 @@ int gcnsa_forward(gcnsa_model* M, const gcnsa_parts* P, int32_t p, float* loss_d
       // factored_norm: A_hat T = diag(dinv) (A + I) (diag(dinv) T): the GEMM's epilogue scales the rows of T and
       // the product reads no values
       PROF(M, 1, gemm_bytes(n, dout, din), 2.0 * n * dout * din,
-           launch_gemm(s, M->o.gemm_mode, 0, 0, n, dout, din, h, ldh, w, M->w_ld[l], M->tmp_a, ldo, 0,
-                       fact ? GCNSA_EPI_ROWSCALE : GCNSA_EPI_NONE, fact ? d.dinv : nullptr, 0, M->ws, M->ws_bytes));
+           launch_gemm(s, M->o.gemm_mode, 0, 0, n, dout, din, h, ldh, w, M->w_ld[l], W.tmp_a, ldo, 0,
+                       fact ? GCNSA_EPI_ROWSCALE : GCNSA_EPI_NONE, fact ? d.dinv : nullptr, 0, W.ws, M->ws_bytes));
       const float* val = fact ? nullptr : d.val;
       if (last && M->o.loss_rows_only && !M->all_rows_once) {
         // training reads the logits of the rows that carry loss only: the other rows are not computed
         PROF_SPMM(M, spmm_cost(d.info.n_train, n, d.m_nnz, dout, !fact),
-             launch_spmm(s, d.info.n_train, d.rowptr, d.col, val, rs, d.m_order, d.m_n_long, M->tmp_a, ldo, dout, epi, bias, 0,
-                         M->H[l + 1], ldo, SpmmBounds{n, n, nnz}));
+             launch_spmm(s, d.info.n_train, d.rowptr, d.col, val, rs, d.m_order, d.m_n_long, W.tmp_a, ldo, dout, epi, bias, 0,
+                         W.H[l + 1], ldo, SpmmBounds{n, n, nnz}));
       } else {
         PROF_SPMM(M, spmm_cost(n, n, nnz, dout, !fact),
-             launch_spmm(s, n, d.rowptr, d.col, val, rs, d.order, d.n_long, M->tmp_a, ldo, dout, epi, bias, 0, M->H[l + 1], ldo, SpmmBounds{n, n, nnz}));
+             launch_spmm(s, n, d.rowptr, d.col, val, rs, d.order, d.n_long, W.tmp_a, ldo, dout, epi, bias, 0, W.H[l + 1], ldo, SpmmBounds{n, n, nnz}));
       }
     } else {
-      const float* agg = M->S[l];
+      const float* agg = W.S[l];
       if (l == 0 && M->o.cache_ax && P->uid == M->ax_uid) {
         // A_hat X does not change between epochs: computed when the feature rows were (re)written, reused otherwise
         int rc = ensure_ax(M, P, p);
@@ -621,43 +672,37 @@ int gcnsa_forward(gcnsa_model* M, const gcnsa_parts* P, int32_t p, float* loss_d
         agg = M->ax[p];
       } else {
         PROF_SPMM(M, spmm_cost(n, n, nnz, din, true),
-             launch_spmm(s, n, d.rowptr, d.col, d.val, nullptr, d.order, d.n_long, h, ldh, din, GCNSA_EPI_NONE, nullptr, 0, M->S[l], ldh, SpmmBounds{n, n, nnz}));
+             launch_spmm(s, n, d.rowptr, d.col, d.val, nullptr, d.order, d.n_long, h, ldh, din, GCNSA_EPI_NONE, nullptr, 0, W.S[l], ldh, SpmmBounds{n, n, nnz}));
       }
-      if (l == 0) M->s0_used = agg;
+      if (l == 0) W.s0_used = agg;
       PROF(M, 1, gemm_bytes(n, dout, din), 2.0 * n * dout * din,
-           launch_gemm(s, M->o.gemm_mode, 0, 0, n, dout, din, agg, ldh, w, M->w_ld[l], M->H[l + 1], ldo, 0, epi, bias,
-                       0, M->ws, M->ws_bytes));
+           launch_gemm(s, M->o.gemm_mode, 0, 0, n, dout, din, agg, ldh, w, M->w_ld[l], W.H[l + 1], ldo, 0, epi, bias,
+                       0, W.ws, M->ws_bytes));
     }
-    h = M->H[l + 1];
+    h = W.H[l + 1];
     ldh = ldo;
   }
   const int64_t ldc = GCNSA_LD(P->c);
   PROF(M, 2, 8.0 * n * P->c + 5.0 * n, 0.0,
-       launch_softmax_ce(s, n, P->c, h, ldc, d.y, d.mask, d.info.n_train, M->loss_parts + p, M->dlogits, ldc, M->sc));
-  if (loss_dev)
-    CK(cudaMemcpyAsync(loss_dev, M->loss_parts + p, sizeof(float), cudaMemcpyDeviceToDevice, (cudaStream_t)s));
-  M->last_forward = p;
-  M->last_n = n;
+       launch_softmax_ce(s, n, P->c, h, ldc, d.y, d.mask, d.info.n_train, M->loss_parts + p, W.dlogits, ldc, W.sc));
   return GCNSA_OK;
 }
 
-int gcnsa_backward(gcnsa_model* M, const gcnsa_parts* P, int32_t p) {
-  if (!M || !P || p < 0 || p >= P->m) return fail(GCNSA_ERR_ARG, "bad partition index or NULL");
-  if (M->last_forward != p) return fail(GCNSA_ERR_ORDER, "gcnsa_backward needs gcnsa_forward on the same partition first");
-  if (M->accumulated >= M->m) return fail(GCNSA_ERR_ORDER, "all M partitions are accumulated already: call gcnsa_step");
+// backward pass of partition p after forward_lane in the same lane; dW, db go to grad (flat parameter layout), added
+// to what is there when acc is 1
+static int backward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& W, void* s, float* grad, int acc) {
   const DevPart& d = P->parts[p];
-  void* s = M->env.e.stream;
   const int64_t n = d.info.n, nnz = d.info.nnz;
-  const float* g = M->dlogits;  // gradient w.r.t. Z^l, [n x LD(dims[l+1])]
+  const float* g = W.dlogits;  // gradient w.r.t. Z^l, [n x LD(dims[l+1])]
   const bool fact = M->o.factored_norm != 0;
   const float* rs = fact ? d.dinv : nullptr;
   bool bias_done = false, g_scaled = false;  // what the producer of g has done for this layer already
   for (int l = M->L - 1; l >= 0; --l) {
     const int32_t din = M->o.dims[l], dout = M->o.dims[l + 1];
     const int64_t ldo = GCNSA_LD(dout), ldi = GCNSA_LD(din);
-    const float* hprev = l == 0 ? d.x : M->H[l];
+    const float* hprev = l == 0 ? d.x : W.H[l];
     const float* w = M->theta + M->w_off[l];
-    float* gw = M->gsum + M->w_off[l];
+    float* gw = grad + M->w_off[l];
     // with factored_norm the products of the layers that multiply by W first read diag(dinv) G: the column-sum
     // kernel, which reads every element of G anyway, writes that copy to tmp_a (G itself below the last layer)
     bool scaled = false;
@@ -666,10 +711,10 @@ int gcnsa_backward(gcnsa_model* M, const gcnsa_parts* P, int32_t p) {
     } else if (M->o.use_bias) {
       if (fact && M->transform_first[l]) {
         PROF(M, 2, 12.0 * n * dout, 0.0,
-             launch_colsum_scaled(s, n, dout, g, ldo, M->gsum + M->b_off[l], 1, M->sc, d.dinv, M->tmp_a, ldo));
+             launch_colsum_scaled(s, n, dout, g, ldo, grad + M->b_off[l], acc, W.sc, d.dinv, W.tmp_a, ldo));
         scaled = true;
       } else {
-        PROF(M, 2, 4.0 * n * dout, 0.0, launch_colsum(s, n, dout, g, ldo, M->gsum + M->b_off[l], 1, M->sc));
+        PROF(M, 2, 4.0 * n * dout, 0.0, launch_colsum(s, n, dout, g, ldo, grad + M->b_off[l], acc, W.sc));
       }
     }
     if (M->transform_first[l]) {
@@ -677,63 +722,86 @@ int gcnsa_backward(gcnsa_model* M, const gcnsa_parts* P, int32_t p) {
       if (fact) {
         // A_hat^T G = diag(dinv) (A + I)^T (diag(dinv) G): the scaled copy is in tmp_a (free at this point; for
         // the layers below the last, G is tmp_a itself and was scaled in place after its column sums were taken)
-        if (!scaled) PROF(M, 2, 8.0 * n * dout, 0.0, launch_scale_rows(s, n, dout, d.dinv, g, ldo, M->tmp_a, ldo));
-        g = M->tmp_a;
+        if (!scaled) PROF(M, 2, 8.0 * n * dout, 0.0, launch_scale_rows(s, n, dout, d.dinv, g, ldo, W.tmp_a, ldo));
+        g = W.tmp_a;
       }
       if (l == M->L - 1) {
         // the logit gradient has zero rows outside T_p: only the non-zeros whose column carries loss contribute
         PROF_SPMM(M, spmm_cost(n, d.info.n_train, d.tm_nnz, dout, !fact),
              launch_spmm(s, n, d.tm_rowptr, d.tm_col, fact ? nullptr : d.tm_val, rs, d.tm_order, d.tm_n_long, g, ldo, dout,
-                         GCNSA_EPI_NONE, nullptr, 0, M->tmp_b, ldo, SpmmBounds{n, n, d.tm_nnz}));
+                         GCNSA_EPI_NONE, nullptr, 0, W.tmp_b, ldo, SpmmBounds{n, n, d.tm_nnz}));
       } else {
         PROF_SPMM(M, spmm_cost(n, n, nnz, dout, !fact),
              launch_spmm(s, n, d.t_rowptr, d.t_col, fact ? nullptr : d.t_val, rs, d.t_order, d.t_n_long, g, ldo, dout,
-                         GCNSA_EPI_NONE, nullptr, 0, M->tmp_b, ldo, SpmmBounds{n, n, nnz}));
+                         GCNSA_EPI_NONE, nullptr, 0, W.tmp_b, ldo, SpmmBounds{n, n, nnz}));
       }
       PROF(M, 1, gemm_bytes(din, dout, n), 2.0 * n * dout * din,
-           launch_gemm(s, M->o.gemm_mode, 1, 0, din, dout, n, hprev, ldi, M->tmp_b, ldo, gw, M->w_ld[l], 1, GCNSA_EPI_NONE,
-                       nullptr, 0, M->ws, M->ws_bytes));
+           launch_gemm(s, M->o.gemm_mode, 1, 0, din, dout, n, hprev, ldi, W.tmp_b, ldo, gw, M->w_ld[l], acc, GCNSA_EPI_NONE,
+                       nullptr, 0, W.ws, M->ws_bytes));
       bias_done = g_scaled = false;
       if (l > 0 && M->o.use_bias) {
         // G^{l-1}, its column sums (the bias gradient of layer l - 1) and, where the next transposed product wants
         // it, diag(dinv) G^{l-1} in place: one pass in the product's epilogue
         const bool want_scaled = fact && M->transform_first[l - 1];
         PROF(M, 1, gemm_bytes(n, din, dout) + 4.0 * n * din, 2.0 * n * dout * din,
-             launch_gemm_mask_colsum(s, M->o.gemm_mode, 0, 1, n, din, dout, M->tmp_b, ldo, w, M->w_ld[l], M->tmp_a, ldi, hprev,
-                                     ldi, want_scaled ? d.dinv : nullptr, M->gsum + M->b_off[l - 1], 1, M->sc, M->ws,
+             launch_gemm_mask_colsum(s, M->o.gemm_mode, 0, 1, n, din, dout, W.tmp_b, ldo, w, M->w_ld[l], W.tmp_a, ldi, hprev,
+                                     ldi, want_scaled ? d.dinv : nullptr, grad + M->b_off[l - 1], acc, W.sc, W.ws,
                                      M->ws_bytes));
         bias_done = true;
         g_scaled = want_scaled;
-        g = M->tmp_a;
+        g = W.tmp_a;
       } else if (l > 0) {
         PROF(M, 1, gemm_bytes(n, din, dout) + 4.0 * n * din, 2.0 * n * dout * din,
-             launch_gemm(s, M->o.gemm_mode, 0, 1, n, din, dout, M->tmp_b, ldo, w, M->w_ld[l], M->tmp_a, ldi, 0, GCNSA_EPI_MASK,
-                         hprev, ldi, M->ws, M->ws_bytes));
-        g = M->tmp_a;
+             launch_gemm(s, M->o.gemm_mode, 0, 1, n, din, dout, W.tmp_b, ldo, w, M->w_ld[l], W.tmp_a, ldi, 0, GCNSA_EPI_MASK,
+                         hprev, ldi, W.ws, M->ws_bytes));
+        g = W.tmp_a;
       }
     } else {
       bias_done = g_scaled = false;
       // dW += S^T G;  R = G W^T;  G^{l-1} = (A_hat^T R) .* [H^{l-1} > 0]
       PROF(M, 1, gemm_bytes(din, dout, n), 2.0 * n * dout * din,
-           launch_gemm(s, M->o.gemm_mode, 1, 0, din, dout, n, l == 0 ? M->s0_used : M->S[l], ldi, g, ldo, gw, M->w_ld[l], 1,
-                       GCNSA_EPI_NONE, nullptr, 0, M->ws, M->ws_bytes));
+           launch_gemm(s, M->o.gemm_mode, 1, 0, din, dout, n, l == 0 ? W.s0_used : W.S[l], ldi, g, ldo, gw, M->w_ld[l], acc,
+                       GCNSA_EPI_NONE, nullptr, 0, W.ws, M->ws_bytes));
       if (l > 0) {
         PROF(M, 1, gemm_bytes(n, din, dout), 2.0 * n * dout * din,
-             launch_gemm(s, M->o.gemm_mode, 0, 1, n, din, dout, g, ldo, w, M->w_ld[l], M->tmp_b, ldi, 0,
-                         fact ? GCNSA_EPI_ROWSCALE : GCNSA_EPI_NONE, fact ? d.dinv : nullptr, 0, M->ws, M->ws_bytes));
+             launch_gemm(s, M->o.gemm_mode, 0, 1, n, din, dout, g, ldo, w, M->w_ld[l], W.tmp_b, ldi, 0,
+                         fact ? GCNSA_EPI_ROWSCALE : GCNSA_EPI_NONE, fact ? d.dinv : nullptr, 0, W.ws, M->ws_bytes));
         if (l == M->L - 1) {  // R = G W^T has the zero rows of G
           PROF_SPMM(M, spmm_cost(n, d.info.n_train, d.tm_nnz, din, !fact, true),
-               launch_spmm(s, n, d.tm_rowptr, d.tm_col, fact ? nullptr : d.tm_val, rs, d.tm_order, d.tm_n_long, M->tmp_b, ldi, din,
-                           GCNSA_EPI_MASK, hprev, ldi, M->tmp_a, ldi, SpmmBounds{n, n, d.tm_nnz}));
+               launch_spmm(s, n, d.tm_rowptr, d.tm_col, fact ? nullptr : d.tm_val, rs, d.tm_order, d.tm_n_long, W.tmp_b, ldi, din,
+                           GCNSA_EPI_MASK, hprev, ldi, W.tmp_a, ldi, SpmmBounds{n, n, d.tm_nnz}));
         } else {
           PROF_SPMM(M, spmm_cost(n, n, nnz, din, !fact, true),
-               launch_spmm(s, n, d.t_rowptr, d.t_col, fact ? nullptr : d.t_val, rs, d.t_order, d.t_n_long, M->tmp_b, ldi, din,
-                           GCNSA_EPI_MASK, hprev, ldi, M->tmp_a, ldi, SpmmBounds{n, n, nnz}));
+               launch_spmm(s, n, d.t_rowptr, d.t_col, fact ? nullptr : d.t_val, rs, d.t_order, d.t_n_long, W.tmp_b, ldi, din,
+                           GCNSA_EPI_MASK, hprev, ldi, W.tmp_a, ldi, SpmmBounds{n, n, nnz}));
         }
-        g = M->tmp_a;
+        g = W.tmp_a;
       }
     }
   }
+  return GCNSA_OK;
+}
+
+int gcnsa_forward(gcnsa_model* M, const gcnsa_parts* P, int32_t p, float* loss_dev) {
+  if (!M || !P || p < 0 || p >= P->m) return fail(GCNSA_ERR_ARG, "bad partition index or NULL");
+  int rc = check_model(M, P);
+  if (rc) return rc;
+  rc = forward_lane(M, P, p, M->lanes[0], M->env.e.stream);
+  if (rc) return rc;
+  if (loss_dev)
+    CK(cudaMemcpyAsync(loss_dev, M->loss_parts + p, sizeof(float), cudaMemcpyDeviceToDevice, M->env.stream()));
+  M->last_forward = p;
+  M->last_n = P->parts[p].info.n;
+  return GCNSA_OK;
+}
+
+int gcnsa_backward(gcnsa_model* M, const gcnsa_parts* P, int32_t p) {
+  if (!M || !P || p < 0 || p >= P->m) return fail(GCNSA_ERR_ARG, "bad partition index or NULL");
+  if (M->last_forward != p) return fail(GCNSA_ERR_ORDER, "gcnsa_backward needs gcnsa_forward on the same partition first");
+  if (M->accumulated >= M->m) return fail(GCNSA_ERR_ORDER, "all M partitions are accumulated already: call gcnsa_step");
+  void* s = M->env.e.stream;
+  const int rc = backward_lane(M, P, p, M->lanes[0], s, M->gsum, 1);
+  if (rc) return rc;
   if (M->o.agg_mode == GCNSA_AGG_PARAM_AVG) {
     // this partition's own optimizer step from the aggregated parameters (Section 3.2), folded into the mean
     if (M->accumulated == 0)  // t -> t + 1 once per epoch
@@ -765,15 +833,85 @@ int gcnsa_step(gcnsa_model* M) {
   return GCNSA_OK;
 }
 
-static int epoch_body(gcnsa_model* M, const gcnsa_parts* P, float* loss_dev) {
+// The streams a recorded epoch forks into (only while it is being recorded: a replay has the branches in its graph).
+struct Fork {
+  std::vector<cudaStream_t> side;
+  std::vector<cudaEvent_t> ev;
+  size_t used = 0;
+  bool make(int n) {
+    for (int i = 0; i < n; ++i) {
+      cudaStream_t st;
+      if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) return false;
+      side.push_back(st);
+    }
+    return true;
+  }
+  // `to` waits for what `from` has been given so far
+  cudaError_t edge(cudaStream_t from, cudaStream_t to) {
+    if (used == ev.size()) {
+      cudaEvent_t e;
+      cudaError_t rc = cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
+      if (rc != cudaSuccess) return rc;
+      ev.push_back(e);
+    }
+    cudaEvent_t e = ev[used++];
+    cudaError_t rc = cudaEventRecord(e, from);
+    return rc == cudaSuccess ? cudaStreamWaitEvent(to, e, 0) : rc;
+  }
+  ~Fork() {
+    for (cudaStream_t st : side) cudaStreamDestroy(st);
+    for (cudaEvent_t e : ev) cudaEventDestroy(e);
+  }
+};
+
+// the step from the gradients of all partitions in gparts
+static int optimizer_step(gcnsa_model* M, cudaStream_t s) {
+  const float inv_m = 1.0f / (float)M->m;
+  if (M->o.agg_mode == GCNSA_AGG_PARAM_AVG)
+    PROF(M, 2, 32.0 * M->count * M->m, 0.0,
+         launch_adam_local_parts(s, M->count, M->m, M->theta, M->gparts, M->am_parts, M->av_parts, inv_m, M->o.lr,
+                                 M->o.beta1, M->o.beta2, M->o.eps, M->adam_state));
+  else
+    PROF(M, 2, (24.0 + 4.0 * M->m) * M->count, 0.0,
+         launch_adam_parts(s, M->count, M->m, M->theta, M->gparts, M->am, M->av, inv_m, M->o.lr, M->o.beta1, M->o.beta2,
+                           M->o.eps, M->adam_state));
+  return GCNSA_OK;
+}
+
+// One epoch: forward and backward of every partition, each with a gradient buffer of its own, then the optimizer over
+// all of them.  fork == NULL: everything on the model's stream, partition after partition.  Otherwise lane i takes
+// partitions ..., i counted from the last one backwards in steps of the number of lanes (so lane 0 ends with the
+// activations of the last partition, as without lanes) on a branch of its own; the sums are added in partition order
+// in both cases, so the results are the same bit for bit.
+static int epoch_body(gcnsa_model* M, const gcnsa_parts* P, float* loss_dev, Fork* fork) {
+  int rc = check_model(M, P);
+  if (rc) return rc;
+  cudaStream_t s = M->env.stream();
+  const int lanes = fork ? (int)M->lanes.size() : 1;
+  auto stream_of = [&](int lane) { return lane == 0 || !fork ? s : fork->side[lane - 1]; };
+  cudaStream_t aux = fork ? fork->side[lanes - 1] : s;
+  if (fork)
+    for (cudaStream_t st : fork->side) CK(fork->edge(s, st));
+  PROF(M, 2, 0.0, 0.0, launch_adam_advance(aux, M->adam_state, M->o.beta1, M->o.beta2));  // t -> t + 1
   for (int32_t p = 0; p < P->m; ++p) {
-    int rc = gcnsa_forward(M, P, p, nullptr);
-    if (rc == GCNSA_OK) rc = gcnsa_backward(M, P, p);
+    const int lane = (P->m - 1 - p) % lanes;
+    rc = forward_lane(M, P, p, M->lanes[lane], stream_of(lane));
+    if (rc == GCNSA_OK)
+      rc = backward_lane(M, P, p, M->lanes[lane], stream_of(lane), M->gparts + (size_t)p * M->count, 0);
     if (rc) return rc;
   }
-  int rc = gcnsa_step(M);
+  if (fork)
+    for (cudaStream_t st : fork->side) CK(fork->edge(st, s));
+  if (loss_dev) {
+    if (fork) CK(fork->edge(s, aux));
+    CKL(launch_mean(aux, M->loss_parts, M->m, loss_dev));
+  }
+  rc = optimizer_step(M, s);
   if (rc) return rc;
-  if (loss_dev) CKL(launch_mean(M->env.e.stream, M->loss_parts, M->m, loss_dev));
+  if (loss_dev && fork) CK(fork->edge(aux, s));
+  M->last_forward = -1;
+  M->last_n = P->parts[P->m - 1].info.n;
+  M->t += 1;
   return GCNSA_OK;
 }
 
@@ -782,7 +920,7 @@ int gcnsa_epoch(gcnsa_model* M, const gcnsa_parts* P, float* loss_dev) {
   if (M->accumulated != 0) return fail(GCNSA_ERR_ORDER, "gcnsa_epoch needs an empty gradient sum");
   cudaStream_t s = M->env.stream();
   const bool want_graph = M->o.epoch_graph && !M->graph_off && !M->prof_on && s != nullptr;
-  if (!want_graph) return epoch_body(M, P, loss_dev);
+  if (!want_graph) return epoch_body(M, P, loss_dev, nullptr);
   if (M->o.cache_ax && P->uid == M->ax_uid && P->m == M->m)  // outside the recording: a replay only reads the cached products
     for (int32_t p = 0; p < P->m; ++p) {
       int rc = ensure_ax(M, P, p);
@@ -798,12 +936,13 @@ int gcnsa_epoch(gcnsa_model* M, const gcnsa_parts* P, float* loss_dev) {
     const int64_t launches0 = gcnsa_launch_count();
     cudaGraph_t graph = nullptr;
     int rc = GCNSA_OK;
-    if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+    Fork fork;
+    if (!fork.make((int)M->lanes.size()) || cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
       cudaGetLastError();
       M->graph_off = true;
-      return epoch_body(M, P, loss_dev);
+      return epoch_body(M, P, loss_dev, nullptr);
     }
-    rc = epoch_body(M, P, loss_dev);
+    rc = epoch_body(M, P, loss_dev, &fork);
     cudaError_t e = cudaStreamEndCapture(s, &graph);
     M->t = t0;  // the host's copy of the step count advances when the graph runs
     M->accumulated = 0;
@@ -816,7 +955,7 @@ int gcnsa_epoch(gcnsa_model* M, const gcnsa_parts* P, float* loss_dev) {
       cudaGetLastError();
       M->graph_exec = nullptr;
       M->graph_off = true;  // this stream or driver cannot record the epoch: plain launches from now on
-      return epoch_body(M, P, loss_dev);
+      return epoch_body(M, P, loss_dev, nullptr);
     }
     cudaGraphDestroy(graph);
     M->graph_parts_uid = P->uid;
@@ -835,6 +974,8 @@ int gcnsa_epoch_host(gcnsa_model* M, gcnsa_parts* P, const float* const* x_host,
   if (M->accumulated != 0) return fail(GCNSA_ERR_ORDER, "gcnsa_epoch_host needs an empty gradient sum");
   for (int32_t p = 0; p < P->m; ++p)
     if (!x_host[p]) return fail(GCNSA_ERR_ARG, "x_host[p] is NULL");
+  int rc = check_model(M, P);
+  if (rc) return rc;
   cudaStream_t s = M->env.stream();
   if (!P->copy_stream) {  // first use: copy stream, events, two staging buffers
     CK(cudaStreamCreateWithFlags(&P->copy_stream, cudaStreamNonBlocking));
@@ -865,13 +1006,17 @@ int gcnsa_epoch_host(gcnsa_model* M, gcnsa_parts* P, const float* const* x_host,
   }
   for (int32_t p = 0; p < P->m; ++p) {
     CK(cudaStreamWaitEvent(s, P->ready[p], 0));
-    int rc = gcnsa_forward(M, P, p, nullptr);
-    if (rc == GCNSA_OK) rc = gcnsa_backward(M, P, p);
+    rc = forward_lane(M, P, p, M->lanes[0], s);
+    if (rc == GCNSA_OK) rc = backward_lane(M, P, p, M->lanes[0], s, M->gparts + (size_t)p * M->count, 0);
     if (rc) return rc;
     CK(cudaEventRecord(P->consumed[p], s));
   }
-  int rc = gcnsa_step(M);
+  PROF(M, 2, 0.0, 0.0, launch_adam_advance(s, M->adam_state, M->o.beta1, M->o.beta2));  // t -> t + 1
+  rc = optimizer_step(M, s);
   if (rc) return rc;
+  M->last_forward = -1;
+  M->last_n = P->parts[P->m - 1].info.n;
+  M->t += 1;
   float* mean_dev = M->loss_parts + M->m;  // slot after the M partition losses
   CKL(launch_mean(M->env.e.stream, M->loss_parts, M->m, mean_dev));
   CK(cudaMemcpyAsync(loss_host, mean_dev, sizeof(float), cudaMemcpyDeviceToHost, M->env.stream()));
@@ -909,10 +1054,10 @@ int gcnsa_model_get(const gcnsa_model* M, int32_t what, int32_t layer, void* hos
   int64_t cols = 0;
   if (what == GCNSA_GET_ACT) {
     if (layer < 1 || layer > M->L) return fail(GCNSA_ERR_ARG, "layer out of range");
-    src = M->H[layer];
+    src = M->lanes[0].H[layer];
     cols = M->o.dims[layer];
   } else if (what == GCNSA_GET_DLOGITS) {
-    src = M->dlogits;
+    src = M->lanes[0].dlogits;
     cols = M->o.dims[M->L];
   } else {
     return fail(GCNSA_ERR_ARG, "unknown tensor id");
@@ -981,7 +1126,7 @@ int gcnsa_evaluate(gcnsa_model* M, const gcnsa_parts* P, int32_t p, const uint8_
   cudaStream_t s = M->env.stream();
   if (mask_host && n > 0) CK(cudaMemcpyAsync(M->ev_mask, mask_host, (size_t)n, cudaMemcpyHostToDevice, s));
   int blocks = 0;
-  CKL(launch_argmax_hits(s, n, P->c, M->H[M->L], GCNSA_LD(P->c), d.y, mask_host ? M->ev_mask : nullptr, M->ev_pred,
+  CKL(launch_argmax_hits(s, n, P->c, M->lanes[0].H[M->L], GCNSA_LD(P->c), d.y, mask_host ? M->ev_mask : nullptr, M->ev_pred,
                          M->ev_hits, &blocks));
   std::vector<int32_t> hits((size_t)std::max(blocks, 1), 0);
   if (n > 0) CK(cudaMemcpyAsync(hits.data(), M->ev_hits, (size_t)blocks * sizeof(int32_t), cudaMemcpyDeviceToHost, s));

@@ -214,6 +214,17 @@ __global__ void adam_advance(double* __restrict__ state, double b1, double b2) {
   state[2] = 1.0 / (1.0 - pow(b2, t));
 }
 
+// One Adam update of an entry with gradient g: the moments are written back, the step is returned (to be subtracted).
+// Roundings are spelled out, so that every kernel that takes the step takes the same one bit for bit.
+__device__ __forceinline__ float adam_delta(float g, float* __restrict__ m, float* __restrict__ v, float lr, float b1,
+                                            float b2, float eps, float c1, float c2) {
+  const float mi = fmaf(1.f - b1, g, __fmul_rn(b1, *m));
+  const float vi = fmaf(__fmul_rn(1.f - b2, g), g, __fmul_rn(b2, *v));
+  *m = mi;
+  *v = vi;
+  return __fdiv_rn(__fmul_rn(lr, __fmul_rn(mi, c1)), __fadd_rn(sqrtf(__fmul_rn(vi, c2)), eps));
+}
+
 __global__ void adam_kernel_dev(int64_t count, float* __restrict__ theta, float* __restrict__ gsum, float* __restrict__ m,
                                 float* __restrict__ v, float inv_m, float lr, float b1, float b2, float eps,
                                 const double* __restrict__ state) {
@@ -221,11 +232,7 @@ __global__ void adam_kernel_dev(int64_t count, float* __restrict__ theta, float*
   if (i >= count) return;
   const float c1 = (float)state[1], c2 = (float)state[2];
   const float g = gsum[i] * inv_m;
-  const float mi = b1 * m[i] + (1.f - b1) * g;
-  const float vi = b2 * v[i] + (1.f - b2) * g * g;
-  m[i] = mi;
-  v[i] = vi;
-  theta[i] -= lr * (mi * c1) / (sqrtf(vi * c2) + eps);
+  theta[i] -= adam_delta(g, m + i, v + i, lr, b1, b2, eps, c1, c2);
   gsum[i] = 0.f;
 }
 
@@ -237,13 +244,43 @@ __global__ void adam_local_kernel_dev(int64_t count, const float* __restrict__ t
   if (i >= count) return;
   const float c1 = (float)state[1], c2 = (float)state[2];
   const float g = gsum[i];
-  const float mi = b1 * m[i] + (1.f - b1) * g;
-  const float vi = b2 * v[i] + (1.f - b2) * g * g;
-  m[i] = mi;
-  v[i] = vi;
-  const float th = (theta[i] - lr * (mi * c1) / (sqrtf(vi * c2) + eps)) * inv_m;
-  acc[i] = first ? th : acc[i] + th;
+  const float th = __fmul_rn(theta[i] - adam_delta(g, m + i, v + i, lr, b1, b2, eps, c1, c2), inv_m);
+  acc[i] = first ? th : __fadd_rn(acc[i], th);
   gsum[i] = 0.f;
+}
+
+// The optimizer over the gradients of all partitions of an epoch, parts[p * count + i], added in partition order: the
+// sums adam_kernel_dev finds in gsum when the backward passes add into one buffer, so the same result bit for bit.
+__global__ void adam_parts_kernel(int64_t count, int n_parts, float* __restrict__ theta, const float* __restrict__ parts,
+                                  float* __restrict__ m, float* __restrict__ v, float inv_m, float lr, float b1, float b2,
+                                  float eps, const double* __restrict__ state) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= count) return;
+  const float c1 = (float)state[1], c2 = (float)state[2];
+  float sum = 0.f;
+  for (int p = 0; p < n_parts; ++p) sum += parts[(int64_t)p * count + i];
+  const float g = sum * inv_m;
+  theta[i] -= adam_delta(g, m + i, v + i, lr, b1, b2, eps, c1, c2);
+}
+
+// Parameter averaging (Section 3.2): every partition's own Adam step from theta with its own moments, theta becomes
+// the mean of the results, added in partition order.
+__global__ void adam_local_parts_kernel(int64_t count, int n_parts, float* __restrict__ theta,
+                                        const float* __restrict__ parts, float* __restrict__ m, float* __restrict__ v,
+                                        float inv_m, float lr, float b1, float b2, float eps,
+                                        const double* __restrict__ state) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= count) return;
+  const float c1 = (float)state[1], c2 = (float)state[2];
+  const float th0 = theta[i];
+  float acc = 0.f;
+  for (int p = 0; p < n_parts; ++p) {
+    const int64_t k = (int64_t)p * count + i;
+    const float g = parts[k];
+    const float th = __fmul_rn(th0 - adam_delta(g, m + k, v + k, lr, b1, b2, eps, c1, c2), inv_m);
+    acc = p == 0 ? th : __fadd_rn(acc, th);
+  }
+  theta[i] = acc;
 }
 
 __global__ void adam_kernel(int64_t count, float* __restrict__ theta, float* __restrict__ gsum, float* __restrict__ m,
@@ -252,12 +289,8 @@ __global__ void adam_kernel(int64_t count, float* __restrict__ theta, float* __r
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const float g = gsum[i] * inv_m;
-  const float mi = b1 * m[i] + (1.f - b1) * g;
-  const float vi = b2 * v[i] + (1.f - b2) * g * g;
-  m[i] = mi;
-  v[i] = vi;
   // c1 = 1 / (1 - beta1^t), c2 = 1 / (1 - beta2^t)
-  theta[i] -= lr * (mi * c1) / (sqrtf(vi * c2) + eps);
+  theta[i] -= adam_delta(g, m + i, v + i, lr, b1, b2, eps, c1, c2);
   gsum[i] = 0.f;
 }
 
@@ -392,6 +425,24 @@ int launch_adam_local_dev(void* stream, int64_t count, const float* theta, float
   if (count == 0) return 0;
   adam_local_kernel_dev<<<(unsigned)((count + 255) / 256), 256, 0, (cudaStream_t)stream>>>(
       count, theta, gsum, m, v, acc, first, inv_m, lr, beta1, beta2, eps, state);
+  note_launch();
+  return (int)cudaGetLastError();
+}
+
+int launch_adam_parts(void* stream, int64_t count, int n_parts, float* theta, const float* parts, float* m, float* v,
+                      float inv_m, float lr, float beta1, float beta2, float eps, const double* state) {
+  if (count == 0) return 0;
+  adam_parts_kernel<<<(unsigned)((count + 255) / 256), 256, 0, (cudaStream_t)stream>>>(count, n_parts, theta, parts, m, v,
+                                                                                      inv_m, lr, beta1, beta2, eps, state);
+  note_launch();
+  return (int)cudaGetLastError();
+}
+
+int launch_adam_local_parts(void* stream, int64_t count, int n_parts, float* theta, const float* parts, float* m, float* v,
+                            float inv_m, float lr, float beta1, float beta2, float eps, const double* state) {
+  if (count == 0) return 0;
+  adam_local_parts_kernel<<<(unsigned)((count + 255) / 256), 256, 0, (cudaStream_t)stream>>>(
+      count, n_parts, theta, parts, m, v, inv_m, lr, beta1, beta2, eps, state);
   note_launch();
   return (int)cudaGetLastError();
 }

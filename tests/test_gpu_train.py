@@ -404,6 +404,29 @@ def test_recorded_epoch_equals_plain_launches(small_wl, agg_mode):
         parts.close()
 
 
+@pytest.mark.parametrize("m", [1, 2, 8, 11])
+def test_partitions_of_a_recorded_epoch_run_side_by_side(tiny_wl, m):
+    """A recorded epoch works on up to eight partitions at once (fewer, as many and more partitions than that): bit for
+    bit the plain launches, and the activations left behind are those of the last partition."""
+    w = tiny_wl
+    with torch.cuda.stream(torch.cuda.Stream()):
+        env = gcnsa.make_env(0)
+        parts = gcnsa.Parts(env, w.rowptr, w.col, w.x, w.y, w.train_mask, w.dims[-1], m, w.overlap_ppm, w.seed)
+        models = [gcnsa.Model(env, parts, w.dims, w.w0, w.b0, lr=w.lr, epoch_graph=k) for k in (0, 1)]
+        loss = torch.zeros(2, device="cuda")
+        for _ in range(3):
+            for k, m_ in enumerate(models):
+                m_.epoch(loss[k:].data_ptr())
+        rows = parts.info(m - 1).n
+        for what, l in [(gcnsa.GET_W, 0), (gcnsa.GET_W, 1), (gcnsa.GET_B, 0), (gcnsa.GET_B, 1), (gcnsa.GET_ADAM_V_W, 0)]:
+            assert np.array_equal(models[0].get(what, l), models[1].get(what, l))
+        assert np.array_equal(models[0].get(gcnsa.GET_ACT, 1, rows), models[1].get(gcnsa.GET_ACT, 1, rows))
+        assert loss[0].item() == loss[1].item()
+        for m_ in models:
+            m_.close()
+        parts.close()
+
+
 def test_recorded_epoch_on_the_default_stream_falls_back(tiny_wl):
     """The legacy default stream cannot be recorded: epoch_graph then runs
     plain launches with the same results."""

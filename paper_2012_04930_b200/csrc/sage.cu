@@ -284,23 +284,54 @@ __global__ void sage_begin_batch(int64_t* state, const int32_t* __restrict__ ord
 __global__ void sage_loss_add(float* acc, const float* loss, float weight) {
   if (threadIdx.x == 0 && blockIdx.x == 0) acc[0] += loss[0] * weight;
 }
-// epoch[0] += part[0] * scale; part[0] = 0
-__global__ void sage_loss_fold(float* epoch, float* part, float scale) {
+// dst[0] = part[0] * scale; part[0] = 0: a worker's epoch is over
+__global__ void sage_loss_fold(float* dst, float* part, float scale) {
   if (threadIdx.x == 0 && blockIdx.x == 0) {
-    epoch[0] += part[0] * scale;
+    dst[0] = part[0] * scale;
     part[0] = 0.f;
   }
 }
-// acc = (first ? 0 : acc) + w * scale
-__global__ void sage_param_mean(int64_t count, const float* __restrict__ w, float* __restrict__ acc, int first, float scale) {
+// The end of an epoch (Section 3.2): theta = mean of the workers' copies [m x count], added in worker order; the
+// working copy of the last worker becomes theta as well; loss[0] = sum of the workers' losses.
+__global__ void sage_param_mean(int64_t count, int m, const float* copies, float* __restrict__ theta, float* work,
+                                float scale, const float* __restrict__ loss_parts,
+                                float* __restrict__ loss) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < count) acc[i] = (first ? 0.f : acc[i]) + w[i] * scale;
+  if (i < count) {
+    float acc = 0.f;
+    for (int p = 0; p < m; ++p) acc = fmaf(copies[(int64_t)p * count + i], scale, acc);
+    theta[i] = acc;
+    work[i] = acc;
+  }
+  if (i == 0) {
+    float sum = 0.f;
+    for (int p = 0; p < m; ++p) sum += loss_parts[p];
+    loss[0] = sum;
+  }
 }
 
 }  // namespace
 }  // namespace gcnsa
 
 using namespace gcnsa;
+
+// Everything one worker's batches need: order, samples, activations, gradient, scratch.  An epoch runs several
+// workers at once, one per lane.
+struct SageLane {
+  float* grad = nullptr;
+  // batch order of one (partition, epoch)
+  u64* keys = nullptr;
+  int32_t* order = nullptr;
+  int32_t order_p = -1;
+  int64_t order_epoch = -1;
+  uint64_t order_uid = 0;
+  // the batch
+  int32_t *b1 = nullptr, *cnt2 = nullptr, *s1 = nullptr, *cnt1 = nullptr, *yb = nullptr;
+  float *cat1 = nullptr, *h1 = nullptr, *cat2 = nullptr, *logits = nullptr, *g = nullptr, *dcat2 = nullptr, *dz1 = nullptr;
+  float* loss = nullptr;  // [0] batch loss, [1] sum over the worker's batches
+  int64_t* batch_state = nullptr;
+  void *ws = nullptr, *sc = nullptr;
+};
 
 struct gcnsa_sage {
   Env env;
@@ -310,25 +341,20 @@ struct gcnsa_sage {
   int64_t count = 0, w1_off = 0, b1_off = 0, w2_off = 0, b2_off = 0;  // flat parameter layout
   int64_t max_rows1 = 0;  // batch (1 + r2): rows of the hidden layer per batch
   int64_t epoch = 0;
-  // parameters: aggregated, the worker's working copy, the running mean, the batch gradient, moments per worker
-  float *theta = nullptr, *work = nullptr, *acc = nullptr, *grad = nullptr, *am = nullptr, *av = nullptr;
+  // parameters: aggregated; per worker its copy and its moments ([m x count] each)
+  float *theta = nullptr, *copies = nullptr, *am = nullptr, *av = nullptr;
   double* adam_state = nullptr;  // [m x 4]
-  // batch order of one (partition, epoch)
-  u64* keys = nullptr;
-  int32_t* order = nullptr;
-  int32_t order_p = -1;
-  int64_t order_epoch = -1;
-  uint64_t order_uid = 0;
-  // the batch
-  int32_t *b1 = nullptr, *cnt2 = nullptr, *s1 = nullptr, *cnt1 = nullptr, *yb = nullptr;
+  float* loss_parts = nullptr;   // [m] a worker's share of the epoch loss
+  float* loss = nullptr;         // epoch loss
   uint8_t* ones = nullptr;
-  float *cat1 = nullptr, *h1 = nullptr, *cat2 = nullptr, *logits = nullptr, *g = nullptr, *dcat2 = nullptr, *dz1 = nullptr;
-  float* loss = nullptr;  // [0] batch loss, [1] partition sum, [2] epoch loss
-  void *ws = nullptr, *sc = nullptr;
   size_t ws_bytes = 0;
+  std::vector<SageLane> lanes;   // lane 0 also serves the calls that go batch by batch
+  std::vector<cudaStream_t> side;  // streams of lanes 1, 2, ...
+  cudaEvent_t fork_ev = nullptr;
+  std::vector<cudaEvent_t> join_ev;
+  int work_p = 0;                // whose copy GCNSA_SAGE_WORK_* and the step-by-step calls address
   int64_t last_nb = 0, last_rows1 = 0;
   // recorded full-size batch of every worker (batch_graph): keyed by the partitions object
-  int64_t* batch_state = nullptr;
   std::vector<cudaGraphExec_t> batch_exec;
   std::vector<int> batch_kernels;
   uint64_t batch_uid = 0;
@@ -391,19 +417,18 @@ int check_model(const gcnsa_sage* S, const gcnsa_parts* P) {
 }
 
 // the batch order of (p, epoch): the loss-carrying vertices of the partition in ascending key order
-int ensure_order(gcnsa_sage* S, const gcnsa_parts* P, int32_t p, int64_t epoch) {
-  if (S->order_p == p && S->order_epoch == epoch && S->order_uid == P->uid) return GCNSA_OK;
+int ensure_order(gcnsa_sage* S, const gcnsa_parts* P, int32_t p, int64_t epoch, SageLane& W, cudaStream_t s) {
+  if (W.order_p == p && W.order_epoch == epoch && W.order_uid == P->uid) return GCNSA_OK;
   const DevPart& d = P->parts[p];
   const int64_t nt = d.info.n_train;
-  cudaStream_t s = S->env.stream();
   if (nt > 0) {
     const u64 prefix = key_prefix(S->o.seed, kTagBatch, (u64)p, (u64)epoch, 0);
-    sage_keys<<<blocks_for(nt, 256), 256, 0, s>>>(d.m_order, nt, prefix, S->keys);
+    sage_keys<<<blocks_for(nt, 256), 256, 0, s>>>(d.m_order, nt, prefix, W.keys);
     SLAUNCHED("sage_keys");
-    sage_rank<<<blocks_for(nt, 256), 256, 0, s>>>(d.m_order, S->keys, nt, S->order);
+    sage_rank<<<blocks_for(nt, 256), 256, 0, s>>>(d.m_order, W.keys, nt, W.order);
     SLAUNCHED("sage_rank");
   }
-  S->order_p = p; S->order_epoch = epoch; S->order_uid = P->uid;
+  W.order_p = p; W.order_epoch = epoch; W.order_uid = P->uid;
   return GCNSA_OK;
 }
 
@@ -412,106 +437,106 @@ int64_t n_batches(const gcnsa_sage* S, const gcnsa_parts* P, int32_t p) {
 }
 
 // recorded = true: the launches are being captured for replay; the batch index and the epoch then come from
-// S->batch_state on the device (a full-size batch), b and epoch are not used
-int run_batch(gcnsa_sage* S, const gcnsa_parts* P, int32_t p, int64_t epoch, int64_t b, bool apply, bool recorded = false) {
-  int rc = recorded ? GCNSA_OK : ensure_order(S, P, p, epoch);
+// W.batch_state on the device (a full-size batch), b and epoch are not used
+int run_batch(gcnsa_sage* S, const gcnsa_parts* P, int32_t p, int64_t epoch, int64_t b, bool apply, SageLane& W, cudaStream_t s,
+              bool recorded = false) {
+  int rc = recorded ? GCNSA_OK : ensure_order(S, P, p, epoch, W, s);
   if (rc) return rc;
   const DevPart& d = P->parts[p];
-  cudaStream_t s = S->env.stream();
-  void* sv = S->env.e.stream;
+  void* sv = s;
   const int64_t nt = d.info.n_train, B = S->o.batch;
   const int64_t nb = recorded ? B : std::min<int64_t>(B, nt - b * B);
   const int r1 = S->o.fanout[0], r2 = S->o.fanout[1];
   const int64_t rows1 = nb * (1 + r2);
-  const int32_t* targets = S->order + b * B;
+  const int32_t* targets = W.order + b * B;
   const int mode = S->o.gemm_mode;
 
   // ---- the batch's vertices and their samples
   S->prof_begin();
-  const int64_t* state = recorded ? S->batch_state : nullptr;
+  const int64_t* state = recorded ? W.batch_state : nullptr;
   const u64 ep = recorded ? 0 : (u64)epoch * 256;
   if (recorded) {
-    sage_begin_batch<<<1, 256, 0, s>>>(S->batch_state, S->order, (int)B, S->b1);
+    sage_begin_batch<<<1, 256, 0, s>>>(W.batch_state, W.order, (int)B, W.b1);
     SLAUNCHED("sage_begin_batch");
   } else {
-    SCK(cudaMemcpyAsync(S->b1, targets, (size_t)nb * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
+    SCK(cudaMemcpyAsync(W.b1, targets, (size_t)nb * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
   }
   if (r2 > 0) {
-    sage_sample<<<blocks_for(nb * 32, kSampleWarps * 32), kSampleWarps * 32, 0, s>>>(d.rowptr, d.col, S->b1, nb, r2, S->o.seed, (u64)p,
-                                                        ep + 2, state, S->b1 + nb, S->cnt2);
+    sage_sample<<<blocks_for(nb * 32, kSampleWarps * 32), kSampleWarps * 32, 0, s>>>(d.rowptr, d.col, W.b1, nb, r2, S->o.seed, (u64)p,
+                                                        ep + 2, state, W.b1 + nb, W.cnt2);
     SLAUNCHED("sage_sample");
   } else {
-    SCK(cudaMemsetAsync(S->cnt2, 0, (size_t)nb * sizeof(int32_t), s));
+    SCK(cudaMemsetAsync(W.cnt2, 0, (size_t)nb * sizeof(int32_t), s));
   }
   if (r1 > 0) {
-    sage_sample<<<blocks_for(rows1 * 32, kSampleWarps * 32), kSampleWarps * 32, 0, s>>>(d.rowptr, d.col, S->b1, rows1, r1, S->o.seed, (u64)p,
-                                                           ep + 1, state, S->s1, S->cnt1);
+    sage_sample<<<blocks_for(rows1 * 32, kSampleWarps * 32), kSampleWarps * 32, 0, s>>>(d.rowptr, d.col, W.b1, rows1, r1, S->o.seed, (u64)p,
+                                                           ep + 1, state, W.s1, W.cnt1);
     SLAUNCHED("sage_sample");
   } else {
-    SCK(cudaMemsetAsync(S->cnt1, 0, (size_t)rows1 * sizeof(int32_t), s));
+    SCK(cudaMemsetAsync(W.cnt1, 0, (size_t)rows1 * sizeof(int32_t), s));
   }
   if (S->prof_on) {
-    sage_count_reads<<<blocks_for(rows1, 256), 256, 0, s>>>(S->b1, S->cnt1, rows1, S->read_rows);
+    sage_count_reads<<<blocks_for(rows1, 256), 256, 0, s>>>(W.b1, W.cnt1, rows1, S->read_rows);
     SLAUNCHED("sage_count_reads");
-    sage_count_reads<<<blocks_for(nb, 256), 256, 0, s>>>(nullptr, S->cnt2, nb, S->read_rows + 1);
+    sage_count_reads<<<blocks_for(nb, 256), 256, 0, s>>>(nullptr, W.cnt2, nb, S->read_rows + 1);
     SLAUNCHED("sage_count_reads");
   }
   S->prof_end(2, 0.0, 0.0);
   // ---- hidden layer: H1 = relu([x_v | mean x_u] [W_self ; W_neigh] + b)
   S->prof_begin();
-  sage_concat_mean<<<blocks_for(rows1 * 32, 256), 256, 0, s>>>(d.x, P->ldx, (int)S->f, S->b1, S->s1, S->cnt1, r1, 0, rows1,
-                                                              S->cat1, S->ldf);
+  sage_concat_mean<<<blocks_for(rows1 * 32, 256), 256, 0, s>>>(d.x, P->ldx, (int)S->f, W.b1, W.s1, W.cnt1, r1, 0, rows1,
+                                                              W.cat1, S->ldf);
   SLAUNCHED("sage_concat_mean");
   S->prof_end(0, 8.0 * (double)rows1 * (double)S->ldf, 0.0);  // the rows written; the rows read are counted on the device
-  float* w = S->work;
+  float* w = S->copies + (size_t)p * S->count;
   const double fl1 = 2.0 * (double)rows1 * (double)S->h * 2.0 * (double)S->f, fl2 = 2.0 * (double)nb * (double)S->c * 2.0 * (double)S->h;
   S->prof_begin();
-  SCKL(launch_gemm(sv, mode, 0, 0, rows1, S->h, 2 * S->ldf, S->cat1, 2 * S->ldf, w + S->w1_off, S->ldh, S->h1, S->ldh, 0,
-                   GCNSA_EPI_BIAS_RELU, w + S->b1_off, 0, S->ws, S->ws_bytes));
+  SCKL(launch_gemm(sv, mode, 0, 0, rows1, S->h, 2 * S->ldf, W.cat1, 2 * S->ldf, w + S->w1_off, S->ldh, W.h1, S->ldh, 0,
+                   GCNSA_EPI_BIAS_RELU, w + S->b1_off, 0, W.ws, S->ws_bytes));
   S->prof_end(1, 0.0, fl1);
   // ---- output layer: logits = [h_v | mean h_u] [W_self ; W_neigh] + b, the samples of vertex i in slots nb + i r2 + s
   S->prof_begin();
-  sage_concat_mean<<<blocks_for(nb * 32, 256), 256, 0, s>>>(S->h1, S->ldh, (int)S->h, nullptr, nullptr, S->cnt2, r2, nb, nb,
-                                                           S->cat2, S->ldh);
+  sage_concat_mean<<<blocks_for(nb * 32, 256), 256, 0, s>>>(W.h1, S->ldh, (int)S->h, nullptr, nullptr, W.cnt2, r2, nb, nb,
+                                                           W.cat2, S->ldh);
   SLAUNCHED("sage_concat_mean");
   S->prof_end(0, 8.0 * (double)nb * (double)S->ldh, 0.0);
   S->prof_begin();
-  SCKL(launch_gemm(sv, mode, 0, 0, nb, S->c, 2 * S->ldh, S->cat2, 2 * S->ldh, w + S->w2_off, S->ldc, S->logits, S->ldc, 0,
-                   GCNSA_EPI_BIAS, w + S->b2_off, 0, S->ws, S->ws_bytes));
+  SCKL(launch_gemm(sv, mode, 0, 0, nb, S->c, 2 * S->ldh, W.cat2, 2 * S->ldh, w + S->w2_off, S->ldc, W.logits, S->ldc, 0,
+                   GCNSA_EPI_BIAS, w + S->b2_off, 0, W.ws, S->ws_bytes));
   S->prof_end(1, 0.0, fl2);
   // ---- loss over the batch and its gradient
   S->prof_begin();
-  sage_gather_labels<<<blocks_for(nb, 256), 256, 0, s>>>(d.y, S->b1, nb, S->yb);
+  sage_gather_labels<<<blocks_for(nb, 256), 256, 0, s>>>(d.y, W.b1, nb, W.yb);
   SLAUNCHED("sage_gather_labels");
-  SCKL(launch_softmax_ce(sv, nb, (int32_t)S->c, S->logits, S->ldc, S->yb, S->ones, nb, S->loss, S->g, S->ldc, S->sc));
-  sage_loss_add<<<1, 32, 0, s>>>(S->loss + 1, S->loss, (float)nb);
+  SCKL(launch_softmax_ce(sv, nb, (int32_t)S->c, W.logits, S->ldc, W.yb, S->ones, nb, W.loss, W.g, S->ldc, W.sc));
+  sage_loss_add<<<1, 32, 0, s>>>(W.loss + 1, W.loss, (float)nb);
   SLAUNCHED("sage_loss_add");
   S->prof_end(2, 0.0, 0.0);
   // ---- backward
-  float* gr = S->grad;
+  float* gr = W.grad;
   S->prof_begin();
-  SCKL(launch_gemm(sv, mode, 1, 0, 2 * S->ldh, S->c, nb, S->cat2, 2 * S->ldh, S->g, S->ldc, gr + S->w2_off, S->ldc, 0,
-                   GCNSA_EPI_NONE, nullptr, 0, S->ws, S->ws_bytes));
-  SCKL(launch_gemm(sv, mode, 0, 1, nb, 2 * S->ldh, S->c, S->g, S->ldc, w + S->w2_off, S->ldc, S->dcat2, 2 * S->ldh, 0,
-                   GCNSA_EPI_NONE, nullptr, 0, S->ws, S->ws_bytes));
+  SCKL(launch_gemm(sv, mode, 1, 0, 2 * S->ldh, S->c, nb, W.cat2, 2 * S->ldh, W.g, S->ldc, gr + S->w2_off, S->ldc, 0,
+                   GCNSA_EPI_NONE, nullptr, 0, W.ws, S->ws_bytes));
+  SCKL(launch_gemm(sv, mode, 0, 1, nb, 2 * S->ldh, S->c, W.g, S->ldc, w + S->w2_off, S->ldc, W.dcat2, 2 * S->ldh, 0,
+                   GCNSA_EPI_NONE, nullptr, 0, W.ws, S->ws_bytes));
   S->prof_end(1, 0.0, 2.0 * fl2);
   S->prof_begin();
-  SCKL(launch_colsum(sv, nb, (int32_t)S->c, S->g, S->ldc, gr + S->b2_off, 0, S->sc));
-  sage_hidden_grad<<<blocks_for(rows1 * S->ldh, 256), 256, 0, s>>>(S->dcat2, S->h1, S->cnt2, nb, std::max(r2, 1), S->ldh, rows1,
-                                                                  S->dz1);
+  SCKL(launch_colsum(sv, nb, (int32_t)S->c, W.g, S->ldc, gr + S->b2_off, 0, W.sc));
+  sage_hidden_grad<<<blocks_for(rows1 * S->ldh, 256), 256, 0, s>>>(W.dcat2, W.h1, W.cnt2, nb, std::max(r2, 1), S->ldh, rows1,
+                                                                  W.dz1);
   SLAUNCHED("sage_hidden_grad");
   S->prof_end(2, 0.0, 0.0);
   S->prof_begin();
-  SCKL(launch_gemm(sv, mode, 1, 0, 2 * S->ldf, S->h, rows1, S->cat1, 2 * S->ldf, S->dz1, S->ldh, gr + S->w1_off, S->ldh, 0,
-                   GCNSA_EPI_NONE, nullptr, 0, S->ws, S->ws_bytes));
+  SCKL(launch_gemm(sv, mode, 1, 0, 2 * S->ldf, S->h, rows1, W.cat1, 2 * S->ldf, W.dz1, S->ldh, gr + S->w1_off, S->ldh, 0,
+                   GCNSA_EPI_NONE, nullptr, 0, W.ws, S->ws_bytes));
   S->prof_end(1, 0.0, fl1);
   S->prof_begin();
-  SCKL(launch_colsum(sv, rows1, (int32_t)S->h, S->dz1, S->ldh, gr + S->b1_off, 0, S->sc));
+  SCKL(launch_colsum(sv, rows1, (int32_t)S->h, W.dz1, S->ldh, gr + S->b1_off, 0, W.sc));
   // ---- the worker's Adam step (its own moments and step count)
   if (apply) {
     double* st = S->adam_state + 4 * (size_t)p;
     SCKL(launch_adam_advance(sv, st, S->o.beta1, S->o.beta2));
-    SCKL(launch_adam_dev(sv, S->count, S->work, S->grad, S->am + (size_t)p * S->count, S->av + (size_t)p * S->count, 1.0f,
+    SCKL(launch_adam_dev(sv, S->count, w, W.grad, S->am + (size_t)p * S->count, S->av + (size_t)p * S->count, 1.0f,
                          S->o.lr, S->o.beta1, S->o.beta2, S->o.eps, st));
   }
   S->prof_end(2, 0.0, 0.0);
@@ -527,12 +552,26 @@ extern "C" {
 int gcnsa_sage_destroy(gcnsa_sage* S) {
   if (!S) return GCNSA_OK;
   cudaStreamSynchronize(S->env.stream());
+  for (cudaStream_t st : S->side) cudaStreamSynchronize(st);
   for (void* p : S->owned) S->env.release(p);
   for (cudaEvent_t e : S->ev) cudaEventDestroy(e);
   for (cudaGraphExec_t g : S->batch_exec)
     if (g) cudaGraphExecDestroy(g);
+  for (cudaStream_t st : S->side) cudaStreamDestroy(st);
+  for (cudaEvent_t e : S->join_ev) cudaEventDestroy(e);
+  if (S->fork_ev) cudaEventDestroy(S->fork_ev);
   delete S;
   return GCNSA_OK;
+}
+
+// How many workers an epoch runs at once: up to eight while a batch has at most kLaneRows rows in the hidden layer.  The
+// two dozen kernels of a batch are a chain of microseconds on a fraction of the SMs, so workers side by side overlap
+// (116 K vertices, 5 workers, batches of 256: 63.2 ms per epoch with one lane, 47.7 with two, 38.4 with four, 29.9
+// with five; 20 000 vertices, 4 workers: 7.7 -> 4.2 ms).  Larger batches fill the chip by themselves and their lanes
+// would cost gigabytes.
+static int sage_lanes(int32_t m, int64_t max_rows1) {
+  constexpr int64_t kLaneRows = 32768;
+  return max_rows1 > kLaneRows ? 1 : std::max(1, std::min<int>(m, 8));
 }
 
 int gcnsa_sage_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcnsa_sage_opts* opts,
@@ -599,38 +638,62 @@ int gcnsa_sage_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcns
   S->ws_bytes = ws;
   const size_t sc = std::max(std::max(softmax_ce_scratch(B), colsum_scratch(S->max_rows1, (int32_t)S->h)),
                              colsum_scratch(B, (int32_t)S->c));
-  const Want wants[] = {
-      {(void**)&S->theta, pb}, {(void**)&S->work, pb}, {(void**)&S->acc, pb}, {(void**)&S->grad, pb},
-      {(void**)&S->am, pb * (size_t)S->m}, {(void**)&S->av, pb * (size_t)S->m},
-      {(void**)&S->adam_state, sizeof(double) * 4 * (size_t)S->m},
-      {(void**)&S->keys, sizeof(u64) * (size_t)nt_max}, {(void**)&S->order, sizeof(int32_t) * (size_t)nt_max},
-      {(void**)&S->b1, sizeof(int32_t) * (size_t)S->max_rows1}, {(void**)&S->cnt2, sizeof(int32_t) * (size_t)B},
-      {(void**)&S->s1, sizeof(int32_t) * (size_t)(S->max_rows1 * std::max<int64_t>(r1, 1))},
-      {(void**)&S->cnt1, sizeof(int32_t) * (size_t)S->max_rows1}, {(void**)&S->yb, sizeof(int32_t) * (size_t)B},
-      {(void**)&S->ones, (size_t)B},
-      {(void**)&S->cat1, sizeof(float) * (size_t)(S->max_rows1 * 2 * S->ldf)},
-      {(void**)&S->h1, sizeof(float) * (size_t)(S->max_rows1 * S->ldh)},
-      {(void**)&S->cat2, sizeof(float) * (size_t)(B * 2 * S->ldh)},
-      {(void**)&S->logits, sizeof(float) * (size_t)(B * S->ldc)}, {(void**)&S->g, sizeof(float) * (size_t)(B * S->ldc)},
-      {(void**)&S->dcat2, sizeof(float) * (size_t)(B * 2 * S->ldh)},
-      {(void**)&S->dz1, sizeof(float) * (size_t)(S->max_rows1 * S->ldh)},
-      {(void**)&S->loss, sizeof(float) * 4}, {(void**)&S->read_rows, sizeof(u64) * 2}, {(void**)&S->batch_state, sizeof(int64_t) * 2}, {&S->ws, ws}, {&S->sc, std::max<size_t>(sc, 256)}};
+  const size_t f4 = sizeof(float), i4 = sizeof(int32_t);
+  std::vector<Want> wants = {{(void**)&S->theta, pb}, {(void**)&S->copies, pb * (size_t)S->m},
+                             {(void**)&S->am, pb * (size_t)S->m}, {(void**)&S->av, pb * (size_t)S->m},
+                             {(void**)&S->adam_state, sizeof(double) * 4 * (size_t)S->m},
+                             {(void**)&S->loss_parts, f4 * (size_t)S->m}, {(void**)&S->loss, f4},
+                             {(void**)&S->ones, (size_t)B}, {(void**)&S->read_rows, sizeof(u64) * 2}};
+  auto lane_wants = [&](SageLane& W) {
+    return std::vector<Want>{
+        {(void**)&W.grad, pb}, {(void**)&W.keys, sizeof(u64) * (size_t)nt_max}, {(void**)&W.order, i4 * (size_t)nt_max},
+        {(void**)&W.b1, i4 * (size_t)S->max_rows1}, {(void**)&W.cnt2, i4 * (size_t)B},
+        {(void**)&W.s1, i4 * (size_t)(S->max_rows1 * std::max<int64_t>(r1, 1))},
+        {(void**)&W.cnt1, i4 * (size_t)S->max_rows1}, {(void**)&W.yb, i4 * (size_t)B},
+        {(void**)&W.cat1, f4 * (size_t)(S->max_rows1 * 2 * S->ldf)}, {(void**)&W.h1, f4 * (size_t)(S->max_rows1 * S->ldh)},
+        {(void**)&W.cat2, f4 * (size_t)(B * 2 * S->ldh)}, {(void**)&W.logits, f4 * (size_t)(B * S->ldc)},
+        {(void**)&W.g, f4 * (size_t)(B * S->ldc)}, {(void**)&W.dcat2, f4 * (size_t)(B * 2 * S->ldh)},
+        {(void**)&W.dz1, f4 * (size_t)(S->max_rows1 * S->ldh)}, {(void**)&W.loss, f4 * 2},
+        {(void**)&W.batch_state, sizeof(int64_t) * 2}, {&W.ws, ws}, {&W.sc, std::max<size_t>(sc, 256)}};
+  };
   cudaStream_t s = S->env.stream();
-  for (const Want& wnt : wants) {
-    *wnt.slot = S->dalloc(std::max<size_t>(wnt.bytes, 256));
-    if (!*wnt.slot) {
-      fail(GCNSA_ERR_OOM, "device allocation failed");
-      return fail_free(GCNSA_ERR_OOM);
+  auto obtain = [&](const std::vector<Want>& list) {
+    for (const Want& w : list) {
+      *w.slot = S->dalloc(std::max<size_t>(w.bytes, 256));
+      if (!*w.slot) return fail(GCNSA_ERR_OOM, "device allocation failed");
+      const cudaError_t e = cudaMemsetAsync(*w.slot, 0, std::max<size_t>(w.bytes, 256), s);
+      if (e != cudaSuccess) return cuda_err(e, "cudaMemsetAsync");
     }
-    if (wnt.slot != &S->ws) {
-      cudaError_t e = cudaMemsetAsync(*wnt.slot, 0, std::max<size_t>(wnt.bytes, 256), s);
-      if (e != cudaSuccess) {
-        cuda_err(e, "cudaMemsetAsync");
-        return fail_free(GCNSA_ERR_CUDA);
+    return (int)GCNSA_OK;
+  };
+  int rc = obtain(wants);
+  S->lanes.resize((size_t)sage_lanes(S->m, S->max_rows1));
+  for (size_t i = 0; i < S->lanes.size() && rc == GCNSA_OK; ++i) {
+    const size_t mark = S->owned.size();
+    rc = obtain(lane_wants(S->lanes[i]));
+    if (rc == GCNSA_ERR_OOM && i > 0) {  // lanes after the first only make the epoch faster
+      while (S->owned.size() > mark) {
+        S->env.release(S->owned.back());
+        S->owned.pop_back();
       }
+      S->lanes.resize(i);
+      rc = GCNSA_OK;
+      break;
     }
   }
-  cudaError_t e = cudaMemsetAsync(S->ones, 1, (size_t)B, s);
+  if (rc != GCNSA_OK) return fail_free(rc);
+  cudaError_t e = cudaEventCreateWithFlags(&S->fork_ev, cudaEventDisableTiming);
+  for (size_t i = 1; i < S->lanes.size() && e == cudaSuccess; ++i) {
+    cudaStream_t st;
+    cudaEvent_t ev;
+    e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+    if (e == cudaSuccess) {
+      S->side.push_back(st);
+      e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+      if (e == cudaSuccess) S->join_ev.push_back(ev);
+    }
+  }
+  if (e == cudaSuccess) e = cudaMemsetAsync(S->ones, 1, (size_t)B, s);
   // initial parameters: W_self in rows [0, f) of the stacked matrix, W_neigh in rows [ld, ld + f)
   const int64_t din[2] = {S->f, S->h}, dout[2] = {S->h, S->c}, ldin[2] = {S->ldf, S->ldh}, ldo[2] = {S->ldh, S->ldc};
   const int64_t w_off[2] = {S->w1_off, S->w2_off}, b_off[2] = {S->b1_off, S->b2_off};
@@ -643,7 +706,8 @@ int gcnsa_sage_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcns
     if (e == cudaSuccess && b0 && b0[l])
       e = cudaMemcpyAsync(S->theta + b_off[l], b0[l], hp, cudaMemcpyHostToDevice, s);
   }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(S->work, S->theta, pb, cudaMemcpyDeviceToDevice, s);
+  for (int32_t p = 0; p < S->m && e == cudaSuccess; ++p)
+    e = cudaMemcpyAsync(S->copies + (size_t)p * S->count, S->theta, pb, cudaMemcpyDeviceToDevice, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {
     cuda_err(e, "upload of the initial parameters");
@@ -667,9 +731,47 @@ int gcnsa_sage_batch(gcnsa_sage* S, const gcnsa_parts* P, int32_t p, int64_t epo
   if (rc) return rc;
   if (p < 0 || p >= P->m || epoch < 0 || epoch >= (1LL << 40)) return fail(GCNSA_ERR_ARG, "partition index or epoch out of range");
   if (b < 0 || b >= n_batches(S, P, p)) return fail(GCNSA_ERR_ARG, "batch index out of range");
-  rc = run_batch(S, P, p, epoch, b, apply != 0);
+  // the working copy as it stands: the one of the worker that ran last
+  cudaStream_t s = S->env.stream();
+  if (S->work_p != p)
+    SCK(cudaMemcpyAsync(S->copies + (size_t)p * S->count, S->copies + (size_t)S->work_p * S->count,
+                        (size_t)S->count * sizeof(float), cudaMemcpyDeviceToDevice, s));
+  S->work_p = p;
+  SageLane& W = S->lanes[0];
+  rc = run_batch(S, P, p, epoch, b, apply != 0, W, s);
   if (rc) return rc;
-  if (loss_dev) SCK(cudaMemcpyAsync(loss_dev, S->loss, sizeof(float), cudaMemcpyDeviceToDevice, S->env.stream()));
+  if (loss_dev) SCK(cudaMemcpyAsync(loss_dev, W.loss, sizeof(float), cudaMemcpyDeviceToDevice, s));
+  return GCNSA_OK;
+}
+
+// the graph of worker p's full-size batch in lane W, recorded on stream s unless it is there already
+static int ensure_batch_graph(gcnsa_sage* S, const gcnsa_parts* P, int32_t p, SageLane& W, cudaStream_t s) {
+  if (S->batch_uid != P->uid || (int32_t)S->batch_exec.size() != P->m) {
+    for (cudaGraphExec_t g : S->batch_exec)
+      if (g) cudaGraphExecDestroy(g);
+    S->batch_exec.assign((size_t)P->m, nullptr);
+    S->batch_kernels.assign((size_t)P->m, 0);
+    S->batch_uid = P->uid;
+  }
+  if (S->batch_exec[p]) return GCNSA_OK;
+  const int64_t launches0 = gcnsa_launch_count();
+  cudaGraph_t graph = nullptr;
+  if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+    const int rc = run_batch(S, P, p, S->epoch, 0, true, W, s, true);
+    const cudaError_t e = cudaStreamEndCapture(s, &graph);
+    const int recorded = (int)(gcnsa_launch_count() - launches0);
+    note_launch(-recorded);  // recorded, not launched
+    if (rc != GCNSA_OK || e != cudaSuccess || !graph || cudaGraphInstantiate(&S->batch_exec[p], graph, 0) != cudaSuccess) {
+      S->batch_exec[p] = nullptr;
+      S->graph_off = true;  // this stream or driver cannot record a batch: plain launches from now on
+    }
+    S->batch_kernels[p] = recorded;
+    if (graph) cudaGraphDestroy(graph);
+    cudaGetLastError();
+  } else {
+    cudaGetLastError();
+    S->graph_off = true;
+  }
   return GCNSA_OK;
 }
 
@@ -678,70 +780,100 @@ int gcnsa_sage_epoch(gcnsa_sage* S, const gcnsa_parts* P, float* loss_dev) {
   if (rc) return rc;
   cudaStream_t s = S->env.stream();
   const size_t pb = (size_t)S->count * sizeof(float);
-  SCK(cudaMemsetAsync(S->loss, 0, 4 * sizeof(float), s));
-  for (int32_t p = 0; p < P->m; ++p) {
+  // Workers are independent within an epoch: lane i takes workers ..., counted from the last one backwards in steps of
+  // the number of lanes (lane 0 ends with the last worker), each lane on a stream of its own.
+  const int lanes = S->prof_on || s == nullptr ? 1 : (int)S->lanes.size();
+  auto stream_of = [&](int lane) { return lane == 0 ? s : S->side[lane - 1]; };
+  if (lanes > 1) {
+    SCK(cudaEventRecord(S->fork_ev, s));
+    for (int i = 1; i < lanes; ++i) SCK(cudaStreamWaitEvent(stream_of(i), S->fork_ev, 0));
+  }
+  // where a lane stands: worker p, its next batch, its batches and how many of them are replayed
+  struct At { int32_t p; int64_t b, nbatch, nreplay; };
+  std::vector<At> at((size_t)lanes);
+  auto begin = [&](int lane, int32_t p) -> int {
+    SageLane& W = S->lanes[lane];
+    cudaStream_t st = stream_of(lane);
+    At& a = at[lane];
+    a.p = p; a.b = 0; a.nbatch = n_batches(S, P, p); a.nreplay = 0;
     // the worker starts the epoch from the aggregated parameters (Section 3.2)
-    SCK(cudaMemcpyAsync(S->work, S->theta, pb, cudaMemcpyDeviceToDevice, s));
-    const int64_t nbatch = n_batches(S, P, p);
-    int64_t b = 0;
+    SCK(cudaMemcpyAsync(S->copies + (size_t)p * S->count, S->theta, pb, cudaMemcpyDeviceToDevice, st));
+    SCK(cudaMemsetAsync(W.loss, 0, 2 * sizeof(float), st));
     // the worker's full-size batches are one kernel sequence with the same shapes: recorded once per worker and
     // replayed, the batch index advancing on the device; the ragged last batch runs as plain launches
     const int64_t nfull = P->parts[p].info.n_train / S->o.batch;
     if (S->o.batch_graph && !S->graph_off && !S->prof_on && s != nullptr && nfull > 1) {
-      rc = ensure_order(S, P, p, S->epoch);
-      if (rc) return rc;
-      if (S->batch_uid != P->uid || (int32_t)S->batch_exec.size() != P->m) {
-        for (cudaGraphExec_t g : S->batch_exec)
-          if (g) cudaGraphExecDestroy(g);
-        S->batch_exec.assign((size_t)P->m, nullptr);
-        S->batch_kernels.assign((size_t)P->m, 0);
-        S->batch_uid = P->uid;
-      }
-      if (!S->batch_exec[p]) {
-        const int64_t launches0 = gcnsa_launch_count();
-        cudaGraph_t graph = nullptr;
-        if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-          rc = run_batch(S, P, p, S->epoch, 0, true, true);
-          const cudaError_t e = cudaStreamEndCapture(s, &graph);
-          const int recorded = (int)(gcnsa_launch_count() - launches0);
-          note_launch(-recorded);  // recorded, not launched
-          if (rc != GCNSA_OK || e != cudaSuccess || !graph ||
-              cudaGraphInstantiate(&S->batch_exec[p], graph, 0) != cudaSuccess) {
-            S->batch_exec[p] = nullptr;
-            S->graph_off = true;  // this stream or driver cannot record a batch: plain launches from now on
-          }
-          S->batch_kernels[p] = recorded;
-          if (graph) cudaGraphDestroy(graph);
-          cudaGetLastError();
-        } else {
-          cudaGetLastError();
-          S->graph_off = true;
-        }
-      }
+      int r = ensure_order(S, P, p, S->epoch, W, st);
+      if (r == GCNSA_OK) r = ensure_batch_graph(S, P, p, W, st);
+      if (r) return r;
       if (S->batch_exec[p]) {
-        sage_set_state<<<1, 1, 0, s>>>(S->batch_state, -1, S->epoch);
+        sage_set_state<<<1, 1, 0, st>>>(W.batch_state, -1, S->epoch);
         SLAUNCHED("sage_set_state");
-        for (; b < nfull; ++b) {
-          SCK(cudaGraphLaunch(S->batch_exec[p], s));
-          note_launch(S->batch_kernels[p]);
-        }
+        a.nreplay = nfull;
+      }
+    }
+    return GCNSA_OK;
+  };
+  auto finish = [&](int lane) -> int {
+    const int32_t p = at[lane].p;
+    const int64_t nt = P->parts[p].info.n_train;
+    sage_loss_fold<<<1, 32, 0, stream_of(lane)>>>(S->loss_parts + p, S->lanes[lane].loss + 1,
+                                                  nt > 0 ? 1.0f / ((float)nt * (float)P->m) : 0.f);
+    SLAUNCHED("sage_loss_fold");
+    return GCNSA_OK;
+  };
+  int open = 0;
+  for (int i = 0; i < lanes; ++i) {
+    const int32_t first = (P->m - 1 - i) % lanes;  // the smallest p with (m - 1 - p) % lanes == i
+    rc = begin(i, first);
+    if (rc) return rc;
+    ++open;
+  }
+  while (open > 0) {  // one batch of every lane in turn, so that all streams are fed
+    for (int i = 0; i < lanes; ++i) {
+      At& a = at[i];
+      if (a.p < 0) continue;
+      if (a.b < a.nreplay) {
+        SCK(cudaGraphLaunch(S->batch_exec[a.p], stream_of(i)));
+        note_launch(S->batch_kernels[a.p]);
         S->last_nb = S->o.batch;
         S->last_rows1 = (int64_t)S->o.batch * (1 + S->o.fanout[1]);
+        ++a.b;
+      } else if (a.b < a.nbatch) {
+        rc = run_batch(S, P, a.p, S->epoch, a.b, true, S->lanes[i], stream_of(i));
+        if (rc) return rc;
+        ++a.b;
+      }
+      if (a.b < a.nbatch) continue;
+      rc = finish(i);
+      if (rc) return rc;
+      const int32_t next = a.p + lanes;
+      if (next < P->m) {
+        rc = begin(i, next);
+        if (rc) return rc;
+      } else {
+        a.p = -1;
+        --open;
       }
     }
-    for (; b < nbatch; ++b) {
-      rc = run_batch(S, P, p, S->epoch, b, true);
-      if (rc) return rc;
-    }
-    const int64_t nt = P->parts[p].info.n_train;
-    sage_loss_fold<<<1, 32, 0, s>>>(S->loss + 2, S->loss + 1, nt > 0 ? 1.0f / ((float)nt * (float)P->m) : 0.f);
-    SLAUNCHED("sage_loss_fold");
-    sage_param_mean<<<blocks_for(S->count, 256), 256, 0, s>>>(S->count, S->work, S->acc, p == 0, 1.0f / (float)P->m);
-    SLAUNCHED("sage_param_mean");
   }
-  SCK(cudaMemcpyAsync(S->theta, S->acc, pb, cudaMemcpyDeviceToDevice, s));
-  SCK(cudaMemcpyAsync(S->work, S->acc, pb, cudaMemcpyDeviceToDevice, s));
-  if (loss_dev) SCK(cudaMemcpyAsync(loss_dev, S->loss + 2, sizeof(float), cudaMemcpyDeviceToDevice, s));
+  {  // the shape of the last worker's last batch is what gcnsa_sage_batch_export describes
+    const int64_t nt = P->parts[P->m - 1].info.n_train;
+    if (nt > 0) {
+      S->last_nb = nt - (n_batches(S, P, P->m - 1) - 1) * S->o.batch;
+      S->last_rows1 = S->last_nb * (1 + S->o.fanout[1]);
+    }
+  }
+  for (int i = 1; i < lanes; ++i) {
+    SCK(cudaEventRecord(S->join_ev[i - 1], stream_of(i)));
+    SCK(cudaStreamWaitEvent(s, S->join_ev[i - 1], 0));
+  }
+  S->work_p = P->m - 1;
+  sage_param_mean<<<blocks_for(S->count, 256), 256, 0, s>>>(S->count, P->m, S->copies, S->theta,
+                                                            S->copies + (size_t)S->work_p * S->count, 1.0f / (float)P->m,
+                                                            S->loss_parts, S->loss);
+  SLAUNCHED("sage_param_mean");
+  if (loss_dev) SCK(cudaMemcpyAsync(loss_dev, S->loss, sizeof(float), cudaMemcpyDeviceToDevice, s));
   S->epoch += 1;
   return GCNSA_OK;
 }
@@ -795,21 +927,22 @@ int gcnsa_sage_batch_export(const gcnsa_sage* S, const gcnsa_sage_batch_host* ds
   cudaStream_t s = S->env.stream();
   const size_t nb = (size_t)S->last_nb, rows1 = (size_t)S->last_rows1;
   const size_t r1 = (size_t)S->o.fanout[0];
-  if (dst->vertices && rows1) SCK(cudaMemcpyAsync(dst->vertices, S->b1, rows1 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  if (dst->count2 && nb) SCK(cudaMemcpyAsync(dst->count2, S->cnt2, nb * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+  const SageLane& W = S->lanes[0];
+  if (dst->vertices && rows1) SCK(cudaMemcpyAsync(dst->vertices, W.b1, rows1 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+  if (dst->count2 && nb) SCK(cudaMemcpyAsync(dst->count2, W.cnt2, nb * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   if (dst->samples1 && rows1 && r1)
-    SCK(cudaMemcpyAsync(dst->samples1, S->s1, rows1 * r1 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  if (dst->count1 && rows1) SCK(cudaMemcpyAsync(dst->count1, S->cnt1, rows1 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    SCK(cudaMemcpyAsync(dst->samples1, W.s1, rows1 * r1 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+  if (dst->count1 && rows1) SCK(cudaMemcpyAsync(dst->count1, W.cnt1, rows1 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   if (dst->hidden && rows1)
-    SCK(cudaMemcpy2DAsync(dst->hidden, (size_t)S->h * sizeof(float), S->h1, (size_t)S->ldh * sizeof(float),
+    SCK(cudaMemcpy2DAsync(dst->hidden, (size_t)S->h * sizeof(float), W.h1, (size_t)S->ldh * sizeof(float),
                           (size_t)S->h * sizeof(float), rows1, cudaMemcpyDeviceToHost, s));
   if (dst->logits && nb)
-    SCK(cudaMemcpy2DAsync(dst->logits, (size_t)S->c * sizeof(float), S->logits, (size_t)S->ldc * sizeof(float),
+    SCK(cudaMemcpy2DAsync(dst->logits, (size_t)S->c * sizeof(float), W.logits, (size_t)S->ldc * sizeof(float),
                           (size_t)S->c * sizeof(float), nb, cudaMemcpyDeviceToHost, s));
   if (dst->dlogits && nb)
-    SCK(cudaMemcpy2DAsync(dst->dlogits, (size_t)S->c * sizeof(float), S->g, (size_t)S->ldc * sizeof(float),
+    SCK(cudaMemcpy2DAsync(dst->dlogits, (size_t)S->c * sizeof(float), W.g, (size_t)S->ldc * sizeof(float),
                           (size_t)S->c * sizeof(float), nb, cudaMemcpyDeviceToHost, s));
-  if (dst->loss) SCK(cudaMemcpyAsync(dst->loss, S->loss, sizeof(float), cudaMemcpyDeviceToHost, s));
+  if (dst->loss) SCK(cudaMemcpyAsync(dst->loss, W.loss, sizeof(float), cudaMemcpyDeviceToHost, s));
   SCK(cudaStreamSynchronize(s));
   return GCNSA_OK;
 }
@@ -819,7 +952,8 @@ static int sage_param(const gcnsa_sage* S, int32_t what, int32_t layer, float** 
   if (!S) return fail(GCNSA_ERR_ARG, "model is NULL");
   if (layer < 0 || layer > 1) return fail(GCNSA_ERR_ARG, "layer out of range");
   const int kind = what % 3, which = what / 3;  // kind: self, neighbour, bias; which: aggregated, working copy, gradient
-  float* buf = which == 0 ? S->theta : which == 1 ? S->work : which == 2 ? S->grad : nullptr;
+  float* buf = which == 0 ? S->theta : which == 1 ? S->copies + (size_t)S->work_p * S->count
+                          : which == 2 ? S->lanes[0].grad : nullptr;
   if (!buf || what < 0) return fail(GCNSA_ERR_ARG, "unknown tensor id");
   const int64_t din = layer == 0 ? S->f : S->h, dout = layer == 0 ? S->h : S->c;
   const int64_t ldin = layer == 0 ? S->ldf : S->ldh, ldo = layer == 0 ? S->ldh : S->ldc;

@@ -204,6 +204,35 @@ def test_recorded_batches_equal_plain_launches(small_wl):
     assert n1 > n0
 
 
+@pytest.mark.parametrize("m", [1, 8, 11])
+def test_workers_side_by_side_equal_workers_one_after_another(tiny_wl, m):
+    """An epoch runs up to eight workers at once; while profiling it runs them one after another.  Losses, parameters
+    and the last worker's last batch are the same bit for bit (fewer, as many and more workers than lanes)."""
+    w = tiny_wl
+    dims = [w.dims[0], 16, w.dims[-1]]
+    ws, wn, bs = configs.sage_weights(dims, w.seed + 77)
+    results = []
+    with torch.cuda.stream(torch.cuda.Stream()):
+        for serial in (False, True):
+            env = gcnsa.make_env(0)
+            parts = gcnsa.Parts(env, w.rowptr, w.col, w.x, w.y, w.train_mask, w.dims[-1], m, w.overlap_ppm, w.seed)
+            model = gcnsa.Sage(env, parts, dims, ws, wn, bs, fanout=(5, 4), batch=32, lr=5e-4, seed=w.seed)
+            model.profile(serial)
+            loss = torch.zeros(1, device="cuda")
+            losses = []
+            for _ in range(2):
+                model.epoch(loss.data_ptr())
+                losses.append(loss.item())
+            results.append((losses, _gpu_params(model, gcnsa.SAGE_W_SELF), model.batch_export()))
+            model.close(); parts.close()
+    (l0, p0, b0), (l1, p1, b1) = results
+    assert l0 == l1
+    for a, b in zip(p0, p1):
+        assert np.array_equal(a, b)
+    for key in ("vertices", "samples1", "hidden", "logits", "nb"):
+        assert np.array_equal(b0[key], b1[key]), key
+
+
 def test_runs_are_bitwise_reproducible_and_arguments_are_checked(tiny_wl):
     w = tiny_wl
     outs = []

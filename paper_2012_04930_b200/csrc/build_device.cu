@@ -591,6 +591,181 @@ __global__ void __launch_bounds__(kSortWarps * 32) sort_scatter(const uint32_t* 
   }
 }
 
+// ------------------------------------------- plan of the tensor-core products ---
+// (DensePlan in internal.h.)  Where rows and columns that carry loss are concerned, `mask` is the rows' mask: rows and
+// columns of A + I are the same vertices.
+
+// positions: loss rows in index order from 0, the others in index order from `rest0` (a multiple of kDenseRows)
+__global__ void plan_positions(const uint8_t* __restrict__ mask, const int32_t* __restrict__ before, int64_t np,
+                               int64_t rest0, int32_t* pos, int32_t* row_at) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= np) return;
+  const int64_t at = mask[i] ? before[i] : rest0 + (i - before[i]);  // before = exclusive scan of the mask
+  pos[i] = (int32_t)at;
+  row_at[at] = (int32_t)i;
+}
+__global__ void plan_mask_flags(const uint8_t* __restrict__ mask, int64_t np, int32_t* flag) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < np) flag[i] = mask[i] ? 1 : 0;
+}
+// word w of lossbits: which of the columns 32 w .. 32 w + 31 carry loss
+__global__ void plan_loss_bits(const uint8_t* __restrict__ mask, int64_t np, int64_t words, uint32_t* lossbits) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= words * 32) return;  // whole warps
+  const unsigned b = __ballot_sync(kFull, i < np && mask[i] != 0);
+  if ((threadIdx.x & 31) == 0) lossbits[i >> 5] = b;
+}
+
+__device__ __forceinline__ int lower_bound(const int32_t* __restrict__ a, int lo, int hi, int32_t v) {
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (__ldg(a + mid) < v) lo = mid + 1;
+    else hi = mid;
+  }
+  return lo;
+}
+
+// Block (tile, column window): how many of the tile's rows have an entry in each column of the window, two 16-bit
+// counters to a word of shared memory (a count is at most kDenseRows).  Columns with kDenseMin or more get their bit in
+// sel[tile]; n_sel counts them by loss (even words) and not (odd words), covered adds up their entries.
+constexpr int kPlanWindow = 49152;  // columns per window: 96 KiB of counters, two blocks per SM
+constexpr int kPlanThreads = 512;
+__global__ void __launch_bounds__(kPlanThreads)
+plan_select(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col, int64_t np, const int32_t* __restrict__ row_at,
+            const uint32_t* __restrict__ lossbits, int64_t words, uint32_t* sel, int32_t* n_sel, u64* covered) {
+  extern __shared__ uint32_t cnt[];
+  const int tile = blockIdx.x, c0 = blockIdx.y * kPlanWindow;
+  const int c1 = (int)min((int64_t)c0 + kPlanWindow, np);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = kPlanThreads / 32;
+  for (int i = threadIdx.x; i < (c1 - c0 + 1) / 2; i += kPlanThreads) cnt[i] = 0u;
+  __syncthreads();
+  for (int r = warp; r < kDenseRows; r += nw) {
+    const int row = row_at[tile * kDenseRows + r];
+    if (row < 0) continue;
+    int beg = rowptr[row], end = rowptr[row + 1];
+    if (gridDim.y > 1) {
+      beg = lower_bound(col, beg, end, c0);
+      end = lower_bound(col, beg, end, c1);
+    }
+    for (int e = beg + lane; e < end; e += 32) {
+      const int c = __ldg(col + e) - c0;
+      atomicAdd(&cnt[c >> 1], 1u << (16 * (c & 1)));
+    }
+  }
+  __syncthreads();
+  int n_loss = 0, n_rest = 0;
+  unsigned sum = 0;
+  for (int b = 32 * warp; b < c1 - c0; b += 32 * nw) {  // a window starts on a word of sel: kPlanWindow is a multiple of 32
+    const int c = b + lane;
+    const unsigned k = c < c1 - c0 ? (cnt[c >> 1] >> (16 * (c & 1))) & 0xFFFFu : 0u;
+    const bool take = k >= (unsigned)kDenseMin;
+    const unsigned m = __ballot_sync(kFull, take);
+    if (take) sum += k;
+    if (lane == 0) {
+      const int64_t w = (c0 + b) >> 5;
+      sel[(int64_t)tile * words + w] = m;
+      const unsigned l = lossbits[w];
+      n_loss += __popc(m & l);
+      n_rest += __popc(m & ~l);
+    }
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(kFull, sum, off);
+  if (lane == 0) {
+    if (n_loss) atomicAdd(&n_sel[2 * tile], n_loss);
+    if (n_rest) atomicAdd(&n_sel[2 * tile + 1], n_rest);
+    if (sum) atomicAdd(covered, (u64)sum);
+  }
+}
+// chunks per tile from n_sel: lead[t] of loss columns, all[t] in total
+__global__ void plan_chunks(const int32_t* __restrict__ n_sel, int n_tiles, int32_t* lead, int32_t* all) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n_tiles) return;
+  lead[t] = (n_sel[2 * t] + kDenseCols - 1) / kDenseCols;
+  all[t] = lead[t] + (n_sel[2 * t + 1] + kDenseCols - 1) / kDenseCols;
+}
+// Block = tile: slots of the selected columns in column order (loss columns first), tcol (np in slots that are not
+// used), and per word of sel the slots before it: rank[2 w] loss columns, rank[2 w + 1] others.
+__global__ void __launch_bounds__(1024)
+plan_slots(const uint32_t* __restrict__ sel, const uint32_t* __restrict__ lossbits, int64_t words, int64_t np,
+           const int32_t* __restrict__ chunk_ptr, const int32_t* __restrict__ lead, int32_t* rank, int32_t* tcol) {
+  __shared__ int64_t ws[32];
+  const int tile = blockIdx.x;
+  const uint32_t* sw = sel + (int64_t)tile * words;
+  int32_t* rk = rank + (int64_t)tile * words * 2;
+  int32_t* tc = tcol + (int64_t)chunk_ptr[tile] * kDenseCols;
+  const int rest0 = lead[tile] * kDenseCols, slots = (chunk_ptr[tile + 1] - chunk_ptr[tile]) * kDenseCols;
+  int64_t run = 0;  // loss slots in the low half, others in the high half
+  for (int64_t w0 = 0; w0 < words; w0 += 1024) {
+    const int64_t w = w0 + threadIdx.x;
+    const unsigned m = w < words ? sw[w] : 0u, l = w < words ? lossbits[w] : 0u;
+    const int64_t mine = (int64_t)__popc(m & l) | ((int64_t)__popc(m & ~l) << 32);
+    int64_t total;
+    const int64_t before = run + block_inclusive_scan<1024>(mine, ws, &total) - mine;
+    if (w < words) {
+      int a = (int)(before & 0xFFFFFFFF), b = (int)(before >> 32);
+      rk[2 * w] = a;
+      rk[2 * w + 1] = b;
+      for (unsigned left = m; left; left &= left - 1) {
+        const int bit = __ffs(left) - 1;
+        const int slot = (l >> bit) & 1 ? a++ : rest0 + b++;
+        tc[slot] = (int32_t)(32 * w + bit);
+      }
+    }
+    run += total;
+  }
+  for (int i = (int)(run & 0xFFFFFFFF) + threadIdx.x; i < rest0; i += 1024) tc[i] = (int32_t)np;
+  for (int i = rest0 + (int)(run >> 32) + threadIdx.x; i < slots; i += 1024) tc[i] = (int32_t)np;
+}
+// A warp per row: the row's selected entries set their bits, the others are counted (by loss), or, with r_col given,
+// written: loss columns first, both in column order.
+__global__ void __launch_bounds__(256)
+plan_rows(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col, int64_t np, const int32_t* __restrict__ pos,
+          const uint32_t* __restrict__ sel, const uint32_t* __restrict__ lossbits, int64_t words,
+          const int32_t* __restrict__ rank, const int32_t* __restrict__ chunk_ptr, const int32_t* __restrict__ lead,
+          uint32_t* bits, int32_t* r_len, int32_t* r_loss, const int32_t* __restrict__ r_rowptr, int32_t* r_mid,
+          int32_t* r_col) {
+  const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (row >= np) return;
+  const int at = pos[row], tile = at / kDenseRows, r = at % kDenseRows;
+  const uint32_t* sw = sel + (int64_t)tile * words;
+  const int32_t* rk = rank + (int64_t)tile * words * 2;
+  const int64_t chunk0 = chunk_ptr[tile];
+  const int rest0 = lead[tile] * kDenseCols;
+  const int beg = rowptr[row], end = rowptr[row + 1];
+  int n_loss = 0, n_rest = 0;
+  const int out_loss = r_col ? r_rowptr[row] : 0, out_rest = r_col ? out_loss + r_loss[row] : 0;
+  for (int e0 = beg; e0 < end; e0 += 32) {
+    const int e = e0 + lane;
+    const int c = e < end ? __ldg(col + e) : 0;
+    const int w = c >> 5, bit = c & 31;
+    const unsigned m = sw[w], l = lossbits[w];
+    const bool dense = e < end && ((m >> bit) & 1), loss = (l >> bit) & 1;
+    if (dense && !r_col) {
+      const unsigned below = (1u << bit) - 1;
+      const int slot = loss ? rk[2 * w] + __popc(m & l & below) : rest0 + rk[2 * w + 1] + __popc(m & ~l & below);
+      const int k = slot % kDenseCols, kk = k & 31;
+      atomicOr(bits + ((chunk0 + slot / kDenseCols) * kDenseRows + r) * 2 + (k >> 5), 1u << ((kk >> 1) + 16 * (kk & 1)));
+    }
+    const unsigned bl = __ballot_sync(kFull, e < end && !dense && loss), br = __ballot_sync(kFull, e < end && !dense && !loss);
+    if (r_col && e < end && !dense) {
+      const unsigned below = (1u << lane) - 1;
+      r_col[loss ? out_loss + n_loss + __popc(bl & below) : out_rest + n_rest + __popc(br & below)] = c;
+    }
+    n_loss += __popc(bl);
+    n_rest += __popc(br);
+  }
+  if (lane == 0) {
+    if (r_col) {
+      r_mid[row] = out_rest;
+    } else {
+      r_len[row] = n_loss + n_rest;
+      r_loss[row] = n_loss;
+    }
+  }
+}
+
 // -------------------------------------------------------------- host side ---
 struct Builder {
   gcnsa_parts* P;
@@ -739,7 +914,138 @@ struct Builder {
   int run();
   void assign();
   void build_partition(int32_t p, int64_t n_owned);
+  void build_plan(DevPart& d, int64_t window);
 };
+
+// A plan pays where a chunk of 64 columns takes enough entries off the gathers: per 64 features a chunk costs one SM
+// about 1 300 clocks, an entry 3.4 of a gathering SM (see spmm_dense), and the split of X and the second pass over the
+// rows come on top.  Measured at 1 640 and 1 230 entries per chunk: F' = 128 365 -> 250 us (58 241 rows, 28 M entries)
+// and 435 -> 290 us (51 249 rows, 20.8 M entries); at 630 (245 000 rows, 12.6 M entries) the planned product is as slow
+// as the gathers.  A partition of fewer than kPlanMinNnz entries is a few microseconds of gathers, less than the
+// launches of a planned product cost.
+constexpr int64_t kPlanMinNnz = 1 << 19, kPlanEntriesPerChunk = 768;
+
+void Builder::build_plan(DevPart& d, int64_t window) {
+  const int64_t np = d.info.n, nnz = d.info.nnz, nt = d.info.n_train;
+  if (!ok() || nnz < kPlanMinNnz) return;
+  DensePlan& pl = d.plan;
+  const int64_t loss_tiles = ceil_div(nt, kDenseRows), n_tiles = loss_tiles + ceil_div(np - nt, kDenseRows);
+  const int64_t words = ceil_div(np, 32), windows = ceil_div(np, kPlanWindow);
+  if (n_tiles * kDenseRows >= (int64_t)INT32_MAX) return;
+  const size_t mark = tmp.size();
+  auto free_scratch = [&] {
+    cudaStreamSynchronize(s);
+    while (tmp.size() > mark) {
+      P->env.release(tmp.back());
+      tmp.pop_back();
+    }
+  };
+  const int64_t sort_tiles = std::max<int64_t>(1, ceil_div(np, kSortTile));
+  if (!tiles) {  // the host builder's partitions come without the scan scratch of run()
+    tiles_cap = ceil_div(std::max<int64_t>(std::max<int64_t>(np, n_tiles), 256 * sort_tiles) + 1, kScanTile) + 2;
+    tiles = scratch<int64_t>((size_t)tiles_cap);
+  }
+  int32_t* row_at = scratch<int32_t>((size_t)(n_tiles * kDenseRows));
+  int32_t* flags = scratch<int32_t>((size_t)np + 1);
+  int32_t* before = scratch<int32_t>((size_t)np + 1);
+  uint32_t* lossbits = scratch<uint32_t>((size_t)words);
+  uint32_t* sel = scratch<uint32_t>((size_t)(n_tiles * words));
+  int32_t* n_sel = scratch<int32_t>((size_t)(2 * n_tiles));
+  int32_t* lead = scratch<int32_t>((size_t)n_tiles + 1);
+  int32_t* all = scratch<int32_t>((size_t)n_tiles + 1);
+  u64* sums = scratch<u64>(4);
+  pl.pos = result<int32_t>((size_t)np);
+  pl.chunk_ptr = result<int32_t>((size_t)n_tiles + 1);
+  pl.loss_ptr = result<int32_t>((size_t)n_tiles + 1);
+  if (!ok()) return;
+  fill_ff(row_at, (size_t)(n_tiles * kDenseRows) * sizeof(int32_t));
+  zero(n_sel, (size_t)(2 * n_tiles) * sizeof(int32_t));
+  zero(sums, 4 * sizeof(u64));
+  plan_mask_flags<<<blocks_for(np, 256), 256, 0, s>>>(d.mask, np, flags);
+  launched("plan_mask_flags");
+  scan<int32_t>(flags, np, before);
+  plan_positions<<<blocks_for(np, 256), 256, 0, s>>>(d.mask, before, np, loss_tiles * kDenseRows, pl.pos, row_at);
+  launched("plan_positions");
+  plan_loss_bits<<<blocks_for(words * 32, 256), 256, 0, s>>>(d.mask, np, words, lossbits);
+  launched("plan_loss_bits");
+  const int smem = (int)((std::min<int64_t>(np, kPlanWindow) + 1) / 2 * 4);
+  cuda(cudaFuncSetAttribute(plan_select, cudaFuncAttributeMaxDynamicSharedMemorySize, kPlanWindow * 2), "plan_select");
+  if (!ok()) return;
+  plan_select<<<dim3((unsigned)n_tiles, (unsigned)windows), kPlanThreads, smem, s>>>(d.rowptr, d.col, np, row_at, lossbits,
+                                                                                     words, sel, n_sel, sums);
+  launched("plan_select");
+  plan_chunks<<<blocks_for(n_tiles, 256), 256, 0, s>>>(n_sel, (int)n_tiles, lead, all);
+  launched("plan_chunks");
+  const int64_t* total = scan<int32_t>(all, n_tiles, pl.chunk_ptr);
+  if (!ok()) return;
+  cuda(cudaMemcpyAsync(sums + 1, total, sizeof(int64_t), cudaMemcpyDeviceToDevice, s), "copy");
+  total = scan<int32_t>(lead, n_tiles, pl.loss_ptr);
+  if (!ok()) return;
+  cuda(cudaMemcpyAsync(sums + 2, total, sizeof(int64_t), cudaMemcpyDeviceToDevice, s), "copy");
+  cuda(cudaMemcpyAsync(sums + 3, pl.chunk_ptr + loss_tiles, sizeof(int32_t), cudaMemcpyDeviceToDevice, s), "copy");
+  u64 h[4];
+  read(h, sums, 4);
+  if (!ok()) return;
+  const int64_t covered = (int64_t)h[0], n_chunks = (int64_t)h[1];
+  if (n_chunks == 0 || covered < n_chunks * kPlanEntriesPerChunk) {
+    free_scratch();
+    return;
+  }
+  int32_t* rank = scratch<int32_t>((size_t)(n_tiles * words * 2));
+  int32_t* r_loss = scratch<int32_t>((size_t)np);
+  pl.tcol = result<int32_t>((size_t)(n_chunks * kDenseCols));
+  pl.bits = result<uint64_t>((size_t)(n_chunks * kDenseRows));
+  pl.r_rowptr = result<int32_t>((size_t)np + 1);
+  pl.r_mid = result<int32_t>((size_t)np);
+  pl.r_nnz = nnz - covered;
+  pl.r_col = result<int32_t>((size_t)pl.r_nnz);
+  pl.r_order = result<int32_t>((size_t)np);
+  pl.rm_order = result<int32_t>((size_t)nt);
+  uint32_t* k0 = scratch<uint32_t>((size_t)np);
+  int32_t* v0 = scratch<int32_t>((size_t)np);
+  uint32_t* k1 = scratch<uint32_t>((size_t)np);
+  int32_t* v1 = scratch<int32_t>((size_t)np);
+  int32_t* hist = scratch<int32_t>((size_t)(256 * sort_tiles + 1));
+  if (!ok()) return;
+  zero(pl.bits, (size_t)(n_chunks * kDenseRows) * sizeof(uint64_t));
+  plan_slots<<<(unsigned)n_tiles, 1024, 0, s>>>(sel, lossbits, words, np, pl.chunk_ptr, lead, rank, pl.tcol);
+  launched("plan_slots");
+  plan_rows<<<blocks_for(np * 32, 256), 256, 0, s>>>(d.rowptr, d.col, np, pl.pos, sel, lossbits, words, rank, pl.chunk_ptr,
+                                                     lead, (uint32_t*)pl.bits, flags, r_loss, nullptr, nullptr, nullptr);
+  launched("plan_rows");
+  scan<int32_t>(flags, np, pl.r_rowptr);
+  if (!ok()) return;
+  plan_rows<<<blocks_for(np * 32, 256), 256, 0, s>>>(d.rowptr, d.col, np, pl.pos, sel, lossbits, words, rank, pl.chunk_ptr,
+                                                     lead, nullptr, nullptr, r_loss, pl.r_rowptr, pl.r_mid, pl.r_col);
+  launched("plan_rows");
+  // processing orders of the remainder
+  length_keys<<<blocks_for(np, 256), 256, 0, s>>>(pl.r_rowptr, np, kRestLong, window, k0, v0);
+  launched("length_keys");
+  const int where = sort_pairs(k0, v0, k1, v1, np, order_key_bits(np, window), hist);
+  cuda(cudaMemcpyAsync(pl.r_order, where ? v1 : v0, (size_t)np * sizeof(int32_t), cudaMemcpyDeviceToDevice, s), "copy");
+  zero(sums, 4 * sizeof(u64));
+  count_long_rows<<<blocks_for(np, 256), 256, 0, s>>>(pl.r_rowptr, np, kRestLong, nullptr, sums);
+  launched("count_long_rows");
+  count_long_rows<<<blocks_for(np, 256), 256, 0, s>>>(pl.r_rowptr, np, kRestLong, d.mask, sums + 2);
+  launched("count_long_rows");
+  flag_carrying_in_order<<<blocks_for(np, 256), 256, 0, s>>>(pl.r_order, np, d.mask, flags);
+  launched("flag_carrying_in_order");
+  scan<int32_t>(flags, np, before);
+  scatter_flagged<<<blocks_for(np, 256), 256, 0, s>>>(flags, before, np, pl.r_order, pl.rm_order, 0);
+  launched("scatter_flagged");
+  u64 longs[4];
+  read(longs, sums, 4);
+  free_scratch();
+  if (!ok()) return;
+  pl.r_n_long = (int64_t)longs[0];
+  pl.rm_n_long = (int64_t)longs[2];
+  pl.n_rows = np;
+  pl.n_tiles = (int32_t)n_tiles;
+  pl.loss_tiles = (int32_t)loss_tiles;
+  pl.n_loss_chunks = (int64_t)h[2];
+  pl.loss_tile_chunks = (int64_t)(int32_t)h[3];
+  pl.n_chunks = n_chunks;
+}
 
 void Builder::assign() {
   const int64_t n = g->n;
@@ -980,6 +1286,7 @@ void Builder::build_partition(int32_t p, int64_t n_owned) {
   if (!ok()) return;
   d.members.assign(mem32.begin(), mem32.end());
   drop(members); drop(deg); drop(cnt);
+  build_plan(d, window);
 }
 
 int Builder::run() {
@@ -1074,6 +1381,12 @@ int build_device(gcnsa_parts* P, const gcnsa_graph* g, const gcnsa_part_opts* o)
   P->parts.assign((size_t)o->m, DevPart());
   P->n_max = 0;
   return b.run();
+}
+
+int build_dense_plan(gcnsa_parts* P, DevPart& d, int64_t window) {
+  Builder b{P, nullptr, nullptr, P->env.stream()};
+  b.build_plan(d, window);
+  return b.rc;
 }
 
 int debug_word_build(unsigned long long* out, bool clear) {

@@ -70,6 +70,7 @@ struct Lane {
   float* S[GCNSA_MAX_LAYERS] = {nullptr};      // A_hat H^{l-1} of layers that aggregate first
   float *tmp_a = nullptr, *tmp_b = nullptr, *dlogits = nullptr;
   void *ws = nullptr, *sc = nullptr;
+  void* dw = nullptr;              // workspace of the planned sparse products
   const float* s0_used = nullptr;  // A_hat H^0 the latest forward used (the cached one or S[0])
 };
 
@@ -102,7 +103,7 @@ struct gcnsa_model {
   // evaluation buffers (allocated on first gcnsa_evaluate)
   int32_t *ev_pred = nullptr, *ev_hits = nullptr;
   uint8_t* ev_mask = nullptr;
-  size_t ws_bytes = 0, sc_bytes = 0;
+  size_t ws_bytes = 0, sc_bytes = 0, dw_bytes = 0;
   int64_t ld_max = 0;
   int32_t last_forward = -1, accumulated = 0;
   int64_t last_n = 0;
@@ -343,6 +344,7 @@ int gcnsa_build_partitions(const gcnsa_env* env, const gcnsa_graph* g, const gcn
       if (!e2) e2 = launch_inv_sqrt_degree(s, hp.n, (const int32_t*)ddeg, d.dinv);
       if (e1 || e2) rc = cuda_fail((cudaError_t)(e1 ? e1 : e2), "normalize");
     }
+    if (rc == GCNSA_OK) rc = build_dense_plan(P, d, order_window_rows(opts->order_window, hp.n));
     // host staging vectors are reused: wait for the copies of this partition
     if (rc == GCNSA_OK) {
       cudaError_t e = cudaStreamSynchronize(s);
@@ -473,6 +475,10 @@ static bool alloc_lane(gcnsa_model* M, Lane& W, size_t act) {
   W.ws = get(std::max<size_t>(M->ws_bytes, 256));
   W.sc = get(std::max<size_t>(M->sc_bytes, 256));
   bool ok = W.tmp_a && W.tmp_b && W.dlogits && W.ws && W.sc;
+  if (ok && M->dw_bytes) {
+    W.dw = get(M->dw_bytes);
+    ok = W.dw != nullptr;
+  }
   for (int l = 0; l < M->L && ok; ++l) {
     W.H[l + 1] = get((size_t)M->n_max * GCNSA_LD(M->o.dims[l + 1]) * sizeof(float));
     ok = W.H[l + 1] != nullptr;
@@ -546,6 +552,10 @@ int gcnsa_model_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcn
     sc = std::max(sc, gemm_colsum_scratch(M->n_max, (int32_t)din));  // the fused bias gradient of the layer below
   }
   M->ws_bytes = ws; M->sc_bytes = sc;
+  if (opts->factored_norm)
+    for (const DevPart& d : parts->parts)
+      for (int l = 0; l < M->L; ++l)
+        M->dw_bytes = std::max(M->dw_bytes, spmm_planned_workspace(d.plan, std::min(opts->dims[l], opts->dims[l + 1])));
   M->lanes.resize((size_t)epoch_lanes(*opts, parts));
   for (size_t i = 0; i < M->lanes.size() && ok; ++i) {
     const size_t mark = M->owned.size();
@@ -614,14 +624,47 @@ int gcnsa_model_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcn
   return GCNSA_OK;
 }
 
+// Y = epi(A_hat X) or, transposed, epi(A_hat^T X) on partition d.  use: all rows and columns, the rows that carry loss
+// only, or only the columns that carry loss (X has zero rows elsewhere).  src_scaled: the rows of X have been
+// multiplied by d^-1/2 already (factored_norm), so the pattern of A + I is all the product needs besides a row scale.
+// With factored_norm a partition's plan takes the product where it has one; without it the stored values are read.
+static int sparse_product(gcnsa_model* M, Lane& W, void* s, const DevPart& d, DenseUse use, bool transposed, bool src_scaled,
+                          const float* x, int64_t ldx, int32_t f, int epi, const float* aux, int64_t ldaux, float* y,
+                          int64_t ldy) {
+  const int64_t n = d.info.n;
+  const bool fact = M->o.factored_norm != 0;
+  const int64_t rows = use == DenseUse::lossRows ? d.info.n_train : n;
+  const int64_t nnz = use == DenseUse::lossRows ? d.m_nnz : use == DenseUse::lossCols ? d.tm_nnz : d.info.nnz;
+  const bool values = !(fact && src_scaled);
+  const SpmmCost cost = spmm_cost(rows, use == DenseUse::lossCols ? d.info.n_train : n, nnz, f, values, epi == GCNSA_EPI_MASK);
+  // (gcnsa_evaluate may bring partitions the workspace was not sized for)
+  if (fact && d.plan.n_chunks > 0 && spmm_planned_workspace(d.plan, f) <= M->dw_bytes) {
+    M->prof_begin();
+    const int r = launch_spmm_planned(s, d.plan, use, rows, d.dinv, src_scaled ? nullptr : d.dinv, x, ldx, f, epi, aux, ldaux, y,
+                                      ldy, W.dw, SpmmBounds{n, n, d.info.nnz});
+    if (r > 0) return cuda_fail((cudaError_t)r, "launch_spmm_planned");
+    if (r == 0) {
+      M->prof_end(0, cost.bytes, cost.flops, cost.l1, cost.bytes_val);
+      return GCNSA_OK;
+    }
+  }
+  const int32_t* order = use == DenseUse::lossRows ? d.m_order : use == DenseUse::lossCols ? d.tm_order : transposed ? d.t_order : d.order;
+  const int64_t n_long = use == DenseUse::lossRows ? d.m_n_long : use == DenseUse::lossCols ? d.tm_n_long : transposed ? d.t_n_long : d.n_long;
+  const int32_t* rowptr = use == DenseUse::lossCols ? d.tm_rowptr : transposed ? d.t_rowptr : d.rowptr;
+  const int32_t* col = use == DenseUse::lossCols ? d.tm_col : transposed ? d.t_col : d.col;
+  const float* val = !values ? nullptr : use == DenseUse::lossCols ? d.tm_val : transposed ? d.t_val : d.val;
+  PROF_SPMM(M, cost, launch_spmm(s, rows, rowptr, col, val, values ? nullptr : d.dinv, order, n_long, x, ldx, f, epi, aux, ldaux,
+                                 y, ldy, SpmmBounds{n, n, use == DenseUse::lossCols ? d.tm_nnz : d.info.nnz}));
+  return GCNSA_OK;
+}
+
 // cache_ax: (re)computes A_hat X of partition p if its feature rows changed since the cached product was made
 static int ensure_ax(gcnsa_model* M, const gcnsa_parts* P, int32_t p) {
   if (M->ax_version[p] == P->x_version[p]) return GCNSA_OK;
   const DevPart& d = P->parts[p];
-  const int32_t din = M->o.dims[0];
-  PROF_SPMM(M, spmm_cost(d.info.n, d.info.n, d.info.nnz, din, true),
-       launch_spmm(M->env.e.stream, d.info.n, d.rowptr, d.col, d.val, nullptr, d.order, d.n_long, d.x, P->ldx, din,
-                   GCNSA_EPI_NONE, nullptr, 0, M->ax[p], P->ldx, SpmmBounds{d.info.n, d.info.n, d.info.nnz}));
+  const int rc = sparse_product(M, M->lanes[0], M->env.e.stream, d, DenseUse::all, false, false, d.x, P->ldx, M->o.dims[0],
+                                GCNSA_EPI_NONE, nullptr, 0, M->ax[p], P->ldx);
+  if (rc) return rc;
   M->ax_version[p] = P->x_version[p];
   return GCNSA_OK;
 }
@@ -635,11 +678,10 @@ static int check_model(const gcnsa_model* M, const gcnsa_parts* P) {
 // forward pass of partition p in the buffers of lane W on stream s; the partition's loss goes to loss_parts[p]
 static int forward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& W, void* s) {
   const DevPart& d = P->parts[p];
-  const int64_t n = d.info.n, nnz = d.info.nnz;
+  const int64_t n = d.info.n;
   const float* h = d.x;
   int64_t ldh = P->ldx;
   const bool fact = M->o.factored_norm != 0;
-  const float* rs = fact ? d.dinv : nullptr;
   for (int l = 0; l < M->L; ++l) {
     const int32_t din = M->o.dims[l], dout = M->o.dims[l + 1];
     const bool last = l == M->L - 1;
@@ -653,16 +695,10 @@ static int forward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& W
       PROF(M, 1, gemm_bytes(n, dout, din), 2.0 * n * dout * din,
            launch_gemm(s, M->o.gemm_mode, 0, 0, n, dout, din, h, ldh, w, M->w_ld[l], W.tmp_a, ldo, 0,
                        fact ? GCNSA_EPI_ROWSCALE : GCNSA_EPI_NONE, fact ? d.dinv : nullptr, 0, W.ws, M->ws_bytes));
-      const float* val = fact ? nullptr : d.val;
-      if (last && M->o.loss_rows_only && !M->all_rows_once) {
-        // training reads the logits of the rows that carry loss only: the other rows are not computed
-        PROF_SPMM(M, spmm_cost(d.info.n_train, n, d.m_nnz, dout, !fact),
-             launch_spmm(s, d.info.n_train, d.rowptr, d.col, val, rs, d.m_order, d.m_n_long, W.tmp_a, ldo, dout, epi, bias, 0,
-                         W.H[l + 1], ldo, SpmmBounds{n, n, nnz}));
-      } else {
-        PROF_SPMM(M, spmm_cost(n, n, nnz, dout, !fact),
-             launch_spmm(s, n, d.rowptr, d.col, val, rs, d.order, d.n_long, W.tmp_a, ldo, dout, epi, bias, 0, W.H[l + 1], ldo, SpmmBounds{n, n, nnz}));
-      }
+      // training reads the logits of the rows that carry loss only: the other rows are not computed
+      const DenseUse use = last && M->o.loss_rows_only && !M->all_rows_once ? DenseUse::lossRows : DenseUse::all;
+      const int rc = sparse_product(M, W, s, d, use, false, fact, W.tmp_a, ldo, dout, epi, bias, 0, W.H[l + 1], ldo);
+      if (rc) return rc;
     } else {
       const float* agg = W.S[l];
       if (l == 0 && M->o.cache_ax && P->uid == M->ax_uid) {
@@ -671,8 +707,8 @@ static int forward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& W
         if (rc) return rc;
         agg = M->ax[p];
       } else {
-        PROF_SPMM(M, spmm_cost(n, n, nnz, din, true),
-             launch_spmm(s, n, d.rowptr, d.col, d.val, nullptr, d.order, d.n_long, h, ldh, din, GCNSA_EPI_NONE, nullptr, 0, W.S[l], ldh, SpmmBounds{n, n, nnz}));
+        const int rc = sparse_product(M, W, s, d, DenseUse::all, false, false, h, ldh, din, GCNSA_EPI_NONE, nullptr, 0, W.S[l], ldh);
+        if (rc) return rc;
       }
       if (l == 0) W.s0_used = agg;
       PROF(M, 1, gemm_bytes(n, dout, din), 2.0 * n * dout * din,
@@ -692,10 +728,9 @@ static int forward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& W
 // to what is there when acc is 1
 static int backward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& W, void* s, float* grad, int acc) {
   const DevPart& d = P->parts[p];
-  const int64_t n = d.info.n, nnz = d.info.nnz;
+  const int64_t n = d.info.n;
   const float* g = W.dlogits;  // gradient w.r.t. Z^l, [n x LD(dims[l+1])]
   const bool fact = M->o.factored_norm != 0;
-  const float* rs = fact ? d.dinv : nullptr;
   bool bias_done = false, g_scaled = false;  // what the producer of g has done for this layer already
   for (int l = M->L - 1; l >= 0; --l) {
     const int32_t din = M->o.dims[l], dout = M->o.dims[l + 1];
@@ -725,16 +760,10 @@ static int backward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& 
         if (!scaled) PROF(M, 2, 8.0 * n * dout, 0.0, launch_scale_rows(s, n, dout, d.dinv, g, ldo, W.tmp_a, ldo));
         g = W.tmp_a;
       }
-      if (l == M->L - 1) {
-        // the logit gradient has zero rows outside T_p: only the non-zeros whose column carries loss contribute
-        PROF_SPMM(M, spmm_cost(n, d.info.n_train, d.tm_nnz, dout, !fact),
-             launch_spmm(s, n, d.tm_rowptr, d.tm_col, fact ? nullptr : d.tm_val, rs, d.tm_order, d.tm_n_long, g, ldo, dout,
-                         GCNSA_EPI_NONE, nullptr, 0, W.tmp_b, ldo, SpmmBounds{n, n, d.tm_nnz}));
-      } else {
-        PROF_SPMM(M, spmm_cost(n, n, nnz, dout, !fact),
-             launch_spmm(s, n, d.t_rowptr, d.t_col, fact ? nullptr : d.t_val, rs, d.t_order, d.t_n_long, g, ldo, dout,
-                         GCNSA_EPI_NONE, nullptr, 0, W.tmp_b, ldo, SpmmBounds{n, n, nnz}));
-      }
+      // the logit gradient has zero rows outside T_p: only the non-zeros whose column carries loss contribute
+      const int rc = sparse_product(M, W, s, d, l == M->L - 1 ? DenseUse::lossCols : DenseUse::all, true, fact, g, ldo, dout,
+                                    GCNSA_EPI_NONE, nullptr, 0, W.tmp_b, ldo);
+      if (rc) return rc;
       PROF(M, 1, gemm_bytes(din, dout, n), 2.0 * n * dout * din,
            launch_gemm(s, M->o.gemm_mode, 1, 0, din, dout, n, hprev, ldi, W.tmp_b, ldo, gw, M->w_ld[l], acc, GCNSA_EPI_NONE,
                        nullptr, 0, W.ws, M->ws_bytes));
@@ -766,15 +795,10 @@ static int backward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& 
         PROF(M, 1, gemm_bytes(n, din, dout), 2.0 * n * dout * din,
              launch_gemm(s, M->o.gemm_mode, 0, 1, n, din, dout, g, ldo, w, M->w_ld[l], W.tmp_b, ldi, 0,
                          fact ? GCNSA_EPI_ROWSCALE : GCNSA_EPI_NONE, fact ? d.dinv : nullptr, 0, W.ws, M->ws_bytes));
-        if (l == M->L - 1) {  // R = G W^T has the zero rows of G
-          PROF_SPMM(M, spmm_cost(n, d.info.n_train, d.tm_nnz, din, !fact, true),
-               launch_spmm(s, n, d.tm_rowptr, d.tm_col, fact ? nullptr : d.tm_val, rs, d.tm_order, d.tm_n_long, W.tmp_b, ldi, din,
-                           GCNSA_EPI_MASK, hprev, ldi, W.tmp_a, ldi, SpmmBounds{n, n, d.tm_nnz}));
-        } else {
-          PROF_SPMM(M, spmm_cost(n, n, nnz, din, !fact, true),
-               launch_spmm(s, n, d.t_rowptr, d.t_col, fact ? nullptr : d.t_val, rs, d.t_order, d.t_n_long, W.tmp_b, ldi, din,
-                           GCNSA_EPI_MASK, hprev, ldi, W.tmp_a, ldi, SpmmBounds{n, n, nnz}));
-        }
+        // (on the last layer R = G W^T has the zero rows of G)
+        const int rc = sparse_product(M, W, s, d, l == M->L - 1 ? DenseUse::lossCols : DenseUse::all, true, fact, W.tmp_b, ldi,
+                                      din, GCNSA_EPI_MASK, hprev, ldi, W.tmp_a, ldi);
+        if (rc) return rc;
         g = W.tmp_a;
       }
     }

@@ -103,6 +103,43 @@ int build_host(const gcnsa_graph* g, const gcnsa_part_opts* o, HostBuild* out);
 // 64-bit selection key (SplitMix64 finalizer applied word by word).
 uint64_t selection_key(uint64_t seed, uint64_t w0, uint64_t w1, uint64_t w2, uint64_t w3, uint64_t v);
 
+// ---- the plan of a partition's products on the tensor cores (kernels_spmm_dense.cu) ---
+// Rows are grouped into tiles of kDenseRows: first the rows that carry loss, then the others, each group in index order
+// (communities stay together) and filled up to whole tiles.  A column that at least kDenseMin of a tile's rows have an
+// entry in becomes one of the tile's columns: 1 bit per row, kDenseCols columns to a chunk, the columns that carry loss
+// in the leading chunks.  The entries in all other columns form the remainder CSR.  A + I is symmetric, so the plan
+// serves the transposed products as well; on the last layer these use the leading chunks only (its gradient has zero
+// rows elsewhere), and the forward product of the loss rows uses the leading tiles only.
+// kDenseMin: a column costs the tensor pipe 12 clocks of one SM per 64 features however few of its 256 bits are set,
+// an entry in the remainder a gather of 256 bytes, 3.4 clocks of one SM at the 21 TB/s the gathers reach.
+constexpr int kDenseRows = 256, kDenseCols = 64, kDenseMin = 4;
+struct DensePlan {
+  int64_t n_rows = 0;  // rows = columns of the matrix
+  int32_t n_tiles = 0, loss_tiles = 0;
+  int64_t n_chunks = 0, n_loss_chunks = 0, loss_tile_chunks = 0;  // all; leading ones of every tile; those of the loss tiles
+  int32_t* pos = nullptr;        // [n] where a row is: tile * kDenseRows + row of the tile
+  int32_t* chunk_ptr = nullptr;  // [n_tiles + 1] first chunk of a tile
+  int32_t* loss_ptr = nullptr;   // [n_tiles + 1] exclusive prefix of the tiles' leading (loss column) chunks
+  int32_t* tcol = nullptr;       // [n_chunks x kDenseCols] column of a slot, n_rows = none
+  uint64_t* bits = nullptr;      // [n_chunks x kDenseRows] slot k of a row: bit (k % 32) / 2 + 16 (k % 2) of half k / 32
+  int32_t *r_rowptr = nullptr, *r_mid = nullptr, *r_col = nullptr;  // remainder; [r_rowptr, r_mid): columns that carry loss
+  int64_t r_nnz = 0;
+  // processing orders of the remainder (as order_key has it, by remainder length) of all rows and of the loss rows;
+  // rows of kRestLong entries or more lead and get a thread block each
+  int32_t *r_order = nullptr, *rm_order = nullptr;
+  int64_t r_n_long = 0, rm_n_long = 0;
+};
+constexpr int64_t kRestLong = 256;
+enum class DenseUse { all, lossRows, lossCols };
+// what the remainder kernel needs to find the partial sums of a row (see spmm_dense)
+struct SpmmBase {
+  const float* pieces = nullptr;
+  const int32_t *pos = nullptr, *prefix = nullptr;
+  int nslab = 1, width = 16, per_cta = 1;
+  unsigned magic = 0;  // unit / per_cta = umulhi(unit, magic), 0 = divide
+  int q0 = 0;  // first float4 chunk of this launch
+};
+
 // ---- kernel launchers (all enqueue on `stream`, return a cudaError_t as int) ---
 // val == NULL: every stored entry counts as 1; row_scale (nullable): row i of the sum is multiplied by row_scale[i]
 // before the epilogue
@@ -110,6 +147,17 @@ uint64_t selection_key(uint64_t seed, uint64_t w0, uint64_t w1, uint64_t w2, uin
 int launch_spmm(void* stream, int64_t n_rows, const int32_t* rowptr, const int32_t* col, const float* val,
                 const float* row_scale, const int32_t* order, int64_t n_long, const float* x, int64_t ldx, int32_t f, int32_t epi, const float* aux,
                 int64_t ldaux, float* y, int64_t ldy, const SpmmBounds& bounds = SpmmBounds());
+// Y = epi(diag(row_scale) B diag(src_scale) X) through a partition's plan (both scales nullable); workspace:
+// spmm_planned_workspace(plan, f) bytes, 256-byte aligned.  Returns -1 when the plan cannot be used.
+int launch_spmm_planned(void* stream, const DensePlan& d, DenseUse use, int64_t n_rows, const float* row_scale,
+                        const float* src_scale, const float* x, int64_t ldx, int32_t f, int32_t epi, const float* aux,
+                        int64_t ldaux, float* y, int64_t ldy, void* workspace, const SpmmBounds& bounds);
+size_t spmm_planned_workspace(const DensePlan& d, int32_t f);
+// the remainder: row i adds its entries [rowptr[i], rowend[i]) and its partial sums
+int launch_spmm_rest(void* stream, int64_t n_rows, const int32_t* rowptr, const int32_t* rowend, const int32_t* col,
+                     const float* row_scale, const float* src_scale, const int32_t* order, int64_t n_long, const float* x,
+                     int64_t ldx, int32_t f, int32_t epi, const float* aux, int64_t ldaux, float* y, int64_t ldy,
+                     const SpmmBase& base, const SpmmBounds& bounds);
 int launch_gemm(void* stream, int32_t mode, int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k, const float* a,
                 int64_t lda, const float* b, int64_t ldb, float* c, int64_t ldc, int32_t accumulate, int32_t epi,
                 const float* aux, int64_t ldaux, void* workspace, size_t workspace_bytes);
@@ -140,6 +188,8 @@ int launch_gather_probe(void* stream, const float* x, int64_t ldx, int64_t n_row
                         int32_t rounds, float* out, int sms);
 int tc_status(int* out);  // error word of the tensor-core kernels (0 = no wait ran out)
 int tc_clear();           // sets that word back to 0
+int tc_status_gemm(int* out);  // the dense products' share of it
+int tc_clear_gemm();
 int launch_softmax_ce(void* stream, int64_t n, int32_t c, const float* logits, int64_t ld, const int32_t* y,
                       const uint8_t* mask, int64_t n_train, float* loss_dev, float* grad, int64_t ldg, void* scratch);
 size_t softmax_ce_scratch(int64_t n);

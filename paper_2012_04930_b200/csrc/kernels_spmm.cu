@@ -351,6 +351,153 @@ cudaError_t run(const Args& a) {
   return cudaGetLastError();
 }
 
+// ---- the remainder of a planned product ------------------------------------------------------------------------
+// Row = its partial sums from the tensor-core kernel plus its entries [rowptr, rowend) of the remainder CSR (SCALED:
+// each times the scale of its source row), then the epilogue of spmm_rows.  A row has few entries here (10 of 406 on
+// the 233 K-vertex graph, 17 of 50 on the 2.45 M-vertex one), so what counts is the chain of dependent loads, not the
+// gathers: the warp fetches 32 indices with one load and hands them round by shuffle, RU gathers per group are in flight
+// at once, and the partial sums are asked for before the first gather.
+template <int CH>
+__device__ __forceinline__ void load_pieces(float4 (&out)[CH], const SpmmBase& b, int row, int q_first, int q_step, int nvec) {
+  const int pos = __ldg(b.pos + row), t = pos / kDenseRows, w4 = b.width / 4;
+  const int first = __ldg(b.prefix + t), cnt = __ldg(b.prefix + t + 1) - first;
+#pragma unroll
+  for (int ch = 0; ch < CH; ++ch) {
+    out[ch] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int qq = q_first + ch * q_step;
+    if (cnt == 0 || qq >= nvec) continue;
+    const int Q = b.q0 + qq, slab = b.nslab > 1 ? Q / w4 : 0;
+    const unsigned u0 = b.nslab * first + slab * cnt, u1 = u0 + cnt - 1;
+    const int c0 = b.magic ? __umulhi(u0, b.magic) : u0 / b.per_cta, c1 = b.magic ? __umulhi(u1, b.magic) : u1 / b.per_cta;
+    const float4* src = reinterpret_cast<const float4*>(b.pieces) +
+                        ((int64_t)(t * b.nslab + slab + c0) * kDenseRows + (pos % kDenseRows)) * w4 + (Q - slab * w4);
+    out[ch] = __ldg(src);
+    for (int c = c0 + 1; c <= c1; ++c) {
+      src += (int64_t)kDenseRows * w4;
+      add4(out[ch], __ldg(src));
+    }
+  }
+}
+
+template <int G, int CH, int RU, bool SCALED>
+__device__ __forceinline__ void gather_range(float4 (&acc)[CH], int beg, int end, int g, int gl, int lane,
+                                             const int32_t* __restrict__ col, const float* __restrict__ sscale,
+                                             const float4* __restrict__ x, int64_t ldx4, int nvec GCNSA_DBG_PARAM) {
+  constexpr int NG = 32 / G;
+  for (int base = beg; base < end; base += 32) {
+    const int n = min(32, end - base);
+    const int mine = lane < n ? __ldg(col + base + lane) : 0;
+    const float msc = SCALED && lane < n ? __ldg(sscale + mine) : 1.f;
+    for (int k0 = 0; k0 < n; k0 += NG * RU) {
+      float4 v[RU][CH];
+#pragma unroll
+      for (int u = 0; u < RU; ++u) {
+        const int k = k0 + u * NG + g;
+        const int c = __shfl_sync(kFull, mine, k & 31);
+        bool live = k < n;
+#if GCNSA_DBG
+        if (live && dbg.src_rows >= 0) live = dbg_in(&g_dbg_spmm, c, 0, dbg.src_rows, kDbgColumn);
+#endif
+        const float4* xr = x + (int64_t)c * ldx4 + gl;
+#pragma unroll
+        for (int ch = 0; ch < CH; ++ch)
+          v[u][ch] = live && gl + ch * G < nvec ? __ldg(xr + ch * G) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+#pragma unroll
+      for (int u = 0; u < RU; ++u) {
+        const float sc = SCALED ? __shfl_sync(kFull, msc, (k0 + u * NG + g) & 31) : 1.f;
+#pragma unroll
+        for (int ch = 0; ch < CH; ++ch) {
+          if (SCALED) fma4(acc[ch], sc, v[u][ch]);
+          else add4(acc[ch], v[u][ch]);
+        }
+      }
+    }
+  }
+}
+
+template <int G, int CH, int RU, bool SCALED>
+__global__ void __launch_bounds__(256)
+spmm_rest(int n_long, int n_rows, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ rowend,
+          const int32_t* __restrict__ col, const float* __restrict__ sscale, const float* __restrict__ rscale,
+          const int32_t* __restrict__ order, const float4* __restrict__ x, int64_t ldx4, int nvec, int f, int epi,
+          const float* __restrict__ aux, int64_t ldaux, float* __restrict__ y, int64_t ldy, const SpmmBase base GCNSA_DBG_PARAM) {
+  constexpr int W = 8;
+  __shared__ float4 part[W][G * CH];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane / G, gl = lane % G;
+  const bool hub = (int)blockIdx.x < n_long;  // a hub row's entries are shared out to the warps of a block
+  const int w = hub ? (int)blockIdx.x : n_long + ((int)blockIdx.x - n_long) * W + warp;
+  if (w >= n_rows) return;
+  const int row = order ? __ldg(order + w) : w;
+#if GCNSA_DBG
+  if (dbg.mat_rows >= 0 && !dbg_in(&g_dbg_spmm, row, 0, dbg.mat_rows, kDbgOrderEntry)) return;  // hub: whole block alike
+#endif
+  int beg = __ldg(rowptr + row), end = __ldg(rowend + row);
+#if GCNSA_DBG
+  if (!dbg_in(&g_dbg_spmm, beg, 0, (long long)end + 1, kDbgRowRange)) return;
+  if (dbg.nnz >= 0 && !dbg_in(&g_dbg_spmm, end, 0, dbg.nnz + 1, kDbgRowRange)) return;
+#endif
+  float4 pieces[CH], acc[CH];
+  if (g == 0 && (!hub || warp == 0)) load_pieces<CH>(pieces, base, row, gl, G, nvec);
+#pragma unroll
+  for (int ch = 0; ch < CH; ++ch) acc[ch] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (hub) {
+    const int share = (end - beg + W - 1) / W;
+    beg = min(end, beg + warp * share);
+    end = min(end, beg + share);
+  }
+  gather_range<G, CH, RU, SCALED>(acc, beg, end, g, gl, lane, col, sscale, x, ldx4, nvec GCNSA_DBG_ARG);
+  fold_groups<G, CH>(acc);
+  if (hub) {
+    if (g == 0) {
+#pragma unroll
+      for (int ch = 0; ch < CH; ++ch) part[warp][gl + ch * G] = acc[ch];
+    }
+    __syncthreads();
+    if (warp != 0) return;
+  }
+  if (g != 0) return;
+  const float sc = rscale ? __ldg(rscale + row) : 1.f;
+#pragma unroll
+  for (int ch = 0; ch < CH; ++ch) {
+    const int qq = gl + ch * G;
+    if (qq >= nvec) continue;
+    float4 r = acc[ch];
+    if (hub) {
+#pragma unroll
+      for (int k = 1; k < W; ++k) add4(r, part[k][qq]);
+    }
+    add4(r, pieces[ch]);
+    if (rscale) { r.x *= sc; r.y *= sc; r.z *= sc; r.w *= sc; }
+    store_chunk(r, row, qq, f, epi, aux, ldaux, y, ldy);
+  }
+}
+
+struct RestArgs {
+  cudaStream_t s;
+  int n_rows, n_long;
+  const int32_t *rowptr, *rowend, *col, *order;
+  const float *sscale, *rscale;
+  int64_t ldx;
+  int epi;
+  int64_t ldaux, ldy;
+  SpmmBounds dbg;
+};
+template <int G, int CH, int RU>
+cudaError_t run_rest(const RestArgs& a, const float* x, int nvec, int f, const float* aux, float* y, const SpmmBase& base) {
+  const int grid = a.n_long + (a.n_rows - a.n_long + 7) / 8;
+  if (a.sscale)
+    spmm_rest<G, CH, RU, true><<<grid, 256, 0, a.s>>>(a.n_long, a.n_rows, a.rowptr, a.rowend, a.col, a.sscale, a.rscale, a.order,
+                                                      reinterpret_cast<const float4*>(x), a.ldx / 4, nvec, f, a.epi, aux, a.ldaux,
+                                                      y, a.ldy, base GCNSA_DBG_LAUNCH_ARG);
+  else
+    spmm_rest<G, CH, RU, false><<<grid, 256, 0, a.s>>>(a.n_long, a.n_rows, a.rowptr, a.rowend, a.col, nullptr, a.rscale, a.order,
+                                                       reinterpret_cast<const float4*>(x), a.ldx / 4, nvec, f, a.epi, aux,
+                                                       a.ldaux, y, a.ldy, base GCNSA_DBG_LAUNCH_ARG);
+  note_launch();
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 int launch_spmm(void* stream, int64_t n_rows, const int32_t* rowptr, const int32_t* col, const float* val,
@@ -388,6 +535,39 @@ int launch_spmm(void* stream, int64_t n_rows, const int32_t* rowptr, const int32
     else if (nv <= 96) e = run<32, 3, 2, 256, 3>(a);
     else if (nv <= 128) e = run<32, 4, 2, 256, 3>(a);
     else e = run<32, 5, 2, 256, 3>(a);
+    if (e != cudaSuccess) return (int)e;
+  }
+  return 0;
+}
+
+int launch_spmm_rest(void* stream, int64_t n_rows, const int32_t* rowptr, const int32_t* rowend, const int32_t* col,
+                     const float* row_scale, const float* src_scale, const int32_t* order, int64_t n_long, const float* x,
+                     int64_t ldx, int32_t f, int32_t epi, const float* aux, int64_t ldaux, float* y, int64_t ldy,
+                     const SpmmBase& base, const SpmmBounds& bounds) {
+  if (n_rows == 0 || f == 0) return 0;
+  RestArgs a;
+  a.dbg = bounds;
+  a.s = (cudaStream_t)stream;
+  a.n_rows = (int)n_rows;
+  a.n_long = order ? (int)std::min<int64_t>(std::max<int64_t>(n_long, 0), n_rows) : 0;
+  a.rowptr = rowptr; a.rowend = rowend; a.col = col; a.order = order;
+  a.sscale = src_scale; a.rscale = row_scale;
+  a.ldx = ldx; a.epi = epi; a.ldaux = ldaux; a.ldy = ldy;
+  const int nvec_total = (f + 3) / 4;
+  for (int v0 = 0; v0 < nvec_total; v0 += 128) {  // column slabs of at most 4 x 32 float4
+    SpmmBase b = base;
+    b.q0 = v0;
+    const int nv = std::min(128, nvec_total - v0), fs = std::min(f - 4 * v0, 4 * nv);
+    const float* xs = x + 4 * v0;
+    const float* as = aux ? aux + 4 * v0 : nullptr;
+    float* ys = y + 4 * v0;
+    cudaError_t e;
+    if (nv <= 4) e = run_rest<4, 1, 2>(a, xs, nv, fs, as, ys, b);
+    else if (nv <= 8) e = run_rest<8, 1, 4>(a, xs, nv, fs, as, ys, b);
+    else if (nv <= 16) e = run_rest<16, 1, 4>(a, xs, nv, fs, as, ys, b);
+    else if (nv <= 32) e = run_rest<32, 1, 8>(a, xs, nv, fs, as, ys, b);
+    else if (nv <= 64) e = run_rest<32, 2, 4>(a, xs, nv, fs, as, ys, b);
+    else e = run_rest<32, 4, 2>(a, xs, nv, fs, as, ys, b);
     if (e != cudaSuccess) return (int)e;
   }
   return 0;

@@ -39,6 +39,7 @@ struct DevPart {
   int64_t tm_nnz = 0, tm_n_long = 0;
   int32_t* y = nullptr;
   uint8_t* mask = nullptr;
+  DensePlan plan;  // n_chunks = 0: the partition's products are gathers alone
   std::vector<int64_t> members;
   std::vector<int32_t> depth;
   int64_t n_long = 0, t_n_long = 0;
@@ -75,6 +76,8 @@ namespace gcnsa {
 // arrays of g are HOST pointers; argument checks that need no device are done
 // by the caller.
 int build_device(gcnsa_parts* P, const gcnsa_graph* g, const gcnsa_part_opts* o);
+// the plan of the tensor-core products of one partition (d.plan) from its CSR and mask on the device
+int build_dense_plan(gcnsa_parts* P, DevPart& d, int64_t window);
 // Argument checks of gcnsa_build_partitions that need neither the graph's contents nor a device.
 int check_build_args(const gcnsa_graph* g, const gcnsa_part_opts* o);
 // Host check that the CSR is a simple symmetric graph with ascending rows and labels in range.

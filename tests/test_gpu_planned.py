@@ -1,0 +1,77 @@
+"""The products that run on the tensor cores through a partition's plan (256-row tiles of bits, a remainder of gathers),
+against a dense fp64 computation of the same layers."""
+import numpy as np
+import pytest
+import torch
+
+from gen import graphs
+from paper_2012_04930_b200 import gcnsa
+
+pytestmark = pytest.mark.gpu
+
+# fp32 sums of a few hundred terms (1e-6 of the largest entry) after dense products with a bound of 1e-5 of it
+TOL = 2e-5
+
+
+def _close(got, want, what):
+    got, want = torch.as_tensor(got, dtype=torch.float64), want.double().cpu()
+    err = ((got - want).abs().max() / want.abs().max()).item()
+    assert err <= TOL, (what, err)
+
+
+# widths of one to three slabs, each with the 16-, 32-, 48- and 64-wide kernel; rows that fill their tiles and rows that
+# do not; every, no and some rows with loss; a hidden layer that narrows and one that widens (source rows scaled while
+# they are split)
+@pytest.mark.parametrize("n,dims,mask_p", [
+    (3072, [20, 16], 0.5), (3001, [40, 7], 0.66), (2817, [40, 29], 0.66), (3001, [48, 41], 1.0), (2999, [70, 64], 0.3),
+    (3001, [130, 100], 0.66), (3010, [150, 130], 0.66), (3001, [90, 33, 9], 0.66), (3001, [24, 72, 40, 5], 0.5),
+    (3001, [40, 24, 7], 0.0)])
+def test_planned_products_match_fp64(n, dims, mask_p):
+    rowptr, col, comm = graphs.chung_lu_communities(n, 640_000, 2.1, 3, 0.93, 5)
+    rng = np.random.default_rng(n + dims[0])
+    x = rng.standard_normal((n, dims[0]), dtype=np.float32)
+    y = (comm % dims[-1]).astype(np.int32)
+    mask = (rng.random(n) < mask_p).astype(np.uint8)
+    w0 = [rng.standard_normal((a, b), dtype=np.float32) / np.float32(np.sqrt(a)) for a, b in zip(dims[:-1], dims[1:])]
+    env = gcnsa.make_env(0)
+    parts = gcnsa.Parts(env, rowptr, col, x, y, mask, dims[-1], 1, 0, 3)
+    A = torch.zeros((n, n), dtype=torch.float64)
+    A[np.repeat(np.arange(n), np.diff(rowptr)), torch.from_numpy(col.astype(np.int64))] = 1.0
+    A += torch.eye(n, dtype=torch.float64)
+    dinv = A.sum(1).rsqrt()
+    A = (dinv[:, None] * A * dinv[None, :]).cuda()
+    ws = [torch.from_numpy(w).double().cuda().requires_grad_() for w in w0]
+    acts, h = [], torch.from_numpy(x).double().cuda()
+    for l, w in enumerate(ws):
+        h = A @ (h @ w)
+        if l < len(ws) - 1:
+            h = torch.relu(h)
+        acts.append(h)
+    on = torch.from_numpy(mask).bool().cuda()
+    if mask.any():
+        torch.nn.functional.cross_entropy(h[on], torch.from_numpy(y).long().cuda()[on]).backward()
+    launches = {}
+    for loss_rows_only in (0, 1):
+        for fact in (0, 1):
+            m = gcnsa.Model(env, parts, dims, w0, loss_rows_only=loss_rows_only, factored_norm=fact, epoch_graph=0)
+            before = gcnsa.launch_count()
+            m.forward(0)
+            launches[fact] = gcnsa.launch_count() - before
+            m.backward(0)
+            if fact:
+                for l in range(1, len(dims)):
+                    got, want = m.get(gcnsa.GET_ACT, l, n), acts[l - 1].detach()
+                    if l == len(dims) - 1 and loss_rows_only:
+                        got, want = got[mask.astype(bool)], want[on]
+                    if want.numel():
+                        _close(got, want, ("H", l, loss_rows_only))
+                for l, w in enumerate(ws):
+                    g = m.get(gcnsa.GET_GRAD_W, l)
+                    if mask.any():
+                        _close(g, w.grad, ("dW", l, loss_rows_only))
+                    else:
+                        assert not g.any()
+            m.close()
+    assert launches[1] > launches[0], "the planned path did not run"
+    assert gcnsa.tc_status() == 0
+    parts.close()

@@ -22,8 +22,8 @@
 // tensor memory, the A operand; warps 16-23 fold finished accumulators into registers.
 //
 // The accumulator of the tensor core truncates when it adds: over the thousands of steps of a tile a bias of about
-// 1e-8 per step would pass the rounding of an fp32 sum.  So an accumulator only lives for kFold chunks and is then
-// added to the thread's running sums with a rounded fp32 add, while the MMAs work in a second accumulator.
+// 1e-8 per step would pass the rounding of an fp32 sum.  So an accumulator only lives for one unit and is then added to
+// the thread's running sums with a rounded fp32 add, while the MMAs work in a second accumulator.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -43,7 +43,6 @@ constexpr int kStagesB = 8;           // chunks whose source rows are in (or on 
 // registers per thread by role, in multiples of 8; their sum over the six warpgroups is what the launch gives (80 each)
 constexpr int kRegsLoad = 72, kRegsExpand = 48, kRegsFold = 120;
 static_assert(2 * (kRegsLoad + kRegsExpand + kRegsFold) <= 6 * 80, "setmaxnreg draws on the registers of the launch");
-constexpr int kFold = 2;              // chunks an accumulator lives for
 constexpr int kLineBytes = 8 * 1024;  // 64 columns x 128 bytes: 8 groups of 8 columns
 constexpr int kBitBytes = 2 * 1024;   // 256 rows x 64 bits
 
@@ -175,12 +174,12 @@ __global__ void __launch_bounds__(kThreads, 1) spmm_dense(const Params p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* full_a = reinterpret_cast<uint64_t*>(smem + L::BAR_OFF);  // A of the stage written (one arrival per expanding warp)
-  uint64_t* empty_a = full_a + kStagesA;                              // MMAs of the stage retired (one arrival per MMA warp, as acc_full)
-  uint64_t* full_b = empty_a + kStagesA;                              // lines landed
-  uint64_t* empty_b = full_b + kStagesB;
-  uint64_t* full_w = empty_b + kStagesB;                              // bits landed (one arrival + bytes)
-  uint64_t* acc_full = full_w + kStagesB;                             // accumulator complete
-  uint64_t* acc_empty = acc_full + 2;                                 // accumulator read back (one per folding warp)
+  uint64_t* full_b = full_a + kStagesA;                               // lines landed
+  uint64_t* full_w = full_b + kStagesB;                               // bits landed (one arrival + bytes)
+  // MMAs of a unit retired (one arrival per MMA warp): its A stage, its B stage and its accumulator change hands.  One
+  // commit says it to all three (with one each the commits were what an MMA warp spent most of its time on).
+  uint64_t* done = full_w + kStagesB;
+  uint64_t* acc_empty = done + kStagesB;                                // accumulator read back (one per folding warp)
   uint64_t* drain = acc_empty + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 2);
   int* abort_slot = reinterpret_cast<int*>(tmem_slot + 1);
@@ -190,19 +189,13 @@ __global__ void __launch_bounds__(kThreads, 1) spmm_dense(const Params p) {
   __syncthreads();
   if (*abort_slot != 0) return;
   if (threadIdx.x == 0) {
-    for (int i = 0; i < kStagesA; ++i) {
-      mbar_init(&full_a[i], kRowWarps);
-      mbar_init(&empty_a[i], 2);
-    }
+    for (int i = 0; i < kStagesA; ++i) mbar_init(&full_a[i], kRowWarps);
     for (int i = 0; i < kStagesB; ++i) {
       mbar_init(&full_b[i], 1);
-      mbar_init(&empty_b[i], 2);
       mbar_init(&full_w[i], 1);
+      mbar_init(&done[i], 2);
     }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&acc_full[b], 2);
-      mbar_init(&acc_empty[b], kRowWarps);
-    }
+    for (int b = 0; b < 2; ++b) mbar_init(&acc_empty[b], kRowWarps);
     mbar_init(&drain[0], 1);
     mbar_init(&drain[1], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -223,124 +216,121 @@ __global__ void __launch_bounds__(kThreads, 1) spmm_dense(const Params p) {
   const int n = max(0, min(p.total, (int)(blockIdx.x + 1) * p.per_cta) - (int)blockIdx.x * p.per_cta);
 
   if (warp < kExpandWarp0) {
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsLoad));
-  if (warp == 0 || warp == 7) {
-    // ---------------- MMA issuers ----------------
-    // The whole warp walks the units and one elected thread issues: loop counters, tensor-memory addresses and
-    // descriptors are then known to be the same in all lanes and stay in uniform registers (with the walk inside the
-    // elected branch every MMA moved its operands there first, 46 clocks each where the tensor pipe needs 32).
-    // D fp32, A and B bf16, A K-major (tensor memory), B MN-major, 128 x N
-    const int m = warp == 0 ? 0 : 1;
-    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(N >> 3) << 17) | (8u << 24);
-    const uint64_t b0 = desc_mn_bf16(smem_u32(smem));
-    const uint32_t tm = __shfl_sync(0xffffffffu, tmem_base, 0);
-    uint32_t seg = 0;
-    int c = 0, len = 0;  // where the item stands
-    bool ok = true;
-    int u = 0;
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsLoad));
+    if (warp == 0 || warp == 7) {
+      // ---------------- MMA issuers ----------------
+      // The whole warp walks the units and one elected thread issues: loop counters, tensor-memory addresses and
+      // descriptors are then known to be the same in all lanes and stay in uniform registers (with the walk inside the
+      // elected branch every MMA moved its operands there first, 46 clocks each where the tensor pipe needs 32).
+      // D fp32, A and B bf16, A K-major (tensor memory), B MN-major, 128 x N
+      const int m = warp == 0 ? 0 : 1;
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(N >> 3) << 17) | (8u << 24);
+      const uint64_t b0 = desc_mn_bf16(smem_u32(smem));
+      const uint32_t tm = __shfl_sync(0xffffffffu, tmem_base, 0);
+      bool ok = true;
+      int u = 0;
 #pragma unroll 1
-    for (; u < n; ++u) {
-      if (c == len) {
-        walk.next(p, it);
-        c = 0;
-        len = it.len;
-      }
-      const uint32_t sa = u % kStagesA, pa = (u / kStagesA) & 1, sb = u % kStagesB, pb = (u / kStagesB) & 1;
-      const bool first = c % kFold == 0, last = (c + 1) % kFold == 0 || c + 1 == len;
-      if (first) ok = mbar_wait(&acc_empty[seg & 1], ((seg >> 1) & 1) ^ 1, 24);
-      ok = ok && mbar_wait(&full_a[sa], pa, 25) && mbar_wait(&full_b[sb], pb, 26);
-      if (!__all_sync(0xffffffffu, ok)) break;
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint64_t bs = b0 + (uint64_t)((sb * L::STAGE) >> 4);
-      const uint32_t a = tm + A_COL0 + sa * 64 + m * 32;
-      const uint32_t d = tm + m * N + (__any_sync(0xffffffffu, seg & 1) ? ACC : 0);
-      const uint32_t old = __any_sync(0xffffffffu, !first);
-      if (elect_one()) {
+      for (; u < n; ++u) {
+        const uint32_t sa = u % kStagesA, pa = (u / kStagesA) & 1, sb = u % kStagesB, pb = (u / kStagesB) & 1;
+        const uint32_t b = u & 1, pe = ((u >> 1) & 1) ^ 1;
+        // the three questions are asked at once (their answers take 30 clocks each); only a no leads to a wait
+        const bool have_a = mbar_try_wait(&full_a[sa], pa), have_b = mbar_try_wait(&full_b[sb], pb),
+                   have_acc = mbar_try_wait(&acc_empty[b], pe);
+        if (!(have_a & have_b & have_acc))
+          ok = mbar_wait(&acc_empty[b], pe, 24) && mbar_wait(&full_a[sa], pa, 25) && mbar_wait(&full_b[sb], pb, 26);
+        if (!__all_sync(0xffffffffu, ok)) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint64_t bs = b0 + (uint64_t)((sb * L::STAGE) >> 4);
+        const uint32_t a = tm + A_COL0 + sa * 64 + m * 32;
+        const uint32_t d = tm + m * N + b * ACC;
+        if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk)
+          for (int kk = 0; kk < 4; ++kk)
 #pragma unroll
-          for (int t = 2; t >= 0; --t)  // small terms first
-            umma_bf16_ta(d, a + 8 * kk, bs + (uint64_t)((L::offset(t) + kk * 2048) >> 4), idesc,
-                         (kk == 0 && t == 2) ? old : 1u);
-        umma_commit(&empty_a[sa]);
-        umma_commit(&empty_b[sb]);
-        if (last) umma_commit(&acc_full[seg & 1]);
-      }
-      __syncwarp();
-      seg += last;
-      ++c;
-    }
-    if (u < n && u > 0) {  // a wait ran out: the MMAs issued so far must have retired before tensor memory is given back
-      if (elect_one()) umma_commit(&drain[m]);
-      const long long t0 = clock64();
-      while (!mbar_try_wait(&drain[m], 0) && clock64() - t0 < kSpinCycles) {
-      }
-    }
-  } else {
-    // ---------------- source rows: loading warp i takes units i, i + 6, ... ----------------
-    // eight lanes take the 16-byte pieces of a line, the four groups of eight lanes 16 columns each
-    const int q = lane >> 3, piece = lane & 7;
-    int g = warp - kLoadWarp0, done = 0, at = 0;  // done: units before the item `it`
-    bool have = walk.next(p, it), ok = true;
-    auto seek = [&]() {  // the item of unit g
-      while (have && g - done >= it.len) {
-        done += it.len;
-        have = walk.next(p, it);
-      }
-      at = g - done;
-      return have;
-    };
-    int4 idx[4];
-    auto indices = [&]() {
-      const int4* src = reinterpret_cast<const int4*>(p.tcol + (it.chunk + at) * 64) + 4 * q;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) idx[i] = __ldg(src + i);
-    };
-    if (seek()) indices();
-    while (have) {
-      const uint32_t s = g % kStagesB, ph = (g / kStagesB) & 1;
-      ok = __all_sync(0xffffffffu, mbar_wait(&empty_b[s], ph ^ 1, 22));
-      if (!ok) break;
-      uint8_t* stage = smem + s * L::STAGE;
-      if (elect_one()) {
-        mbar_expect_tx(&full_w[s], kBitBytes);
-        bulk_load(stage + L::COUNT * kLineBytes, p.bits + (it.chunk + at) * 256, kBitBytes, &full_w[s]);
-      }
-      __syncwarp();
-      const uint8_t* src = p.split + (int64_t)it.slab * L::COUNT * 128 + piece * 16;
-      const uint32_t dst = smem_u32(stage + q * 2048);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const int4& v = idx[i >> 2];
-        const int row = (i & 3) == 0 ? v.x : (i & 3) == 1 ? v.y : (i & 3) == 2 ? v.z : v.w;
-        const uint8_t* r = src + (int64_t)row * p.split_pitch;
-#pragma unroll
-        for (int line = 0; line < L::COUNT; ++line)
-          cp_async16(dst + line * kLineBytes + (i >> 3) * 1024 + (i & 7) * 128 + ((piece ^ (i & 7)) << 4), r + line * 128);
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-      g += kLoadWarps;
-      if (seek()) indices();  // on their way while the lines are
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // hand them to the tensor core
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&full_b[s]);
-    }
-    if (!ok || tc_error_now() != 0) {  // the bit copies already issued land before the CTA exits
-      const long long t0 = clock64();
-      for (int gi = g - kLoadWarps; gi >= 0 && gi > g - 3 * kLoadWarps; gi -= kLoadWarps)
-        while (!mbar_try_wait(&full_w[gi % kStagesB], (gi / kStagesB) & 1) && clock64() - t0 < kSpinCycles) {
+            for (int t = 2; t >= 0; --t)  // small terms first
+              umma_bf16_ta(d, a + 8 * kk, bs + (uint64_t)((L::offset(t) + kk * 2048) >> 4), idesc, kk != 0 || t != 2);
+          umma_commit(&done[sb]);
         }
+        __syncwarp();
+      }
+      if (u < n && u > 0) {  // a wait ran out: the MMAs issued so far must have retired before tensor memory is given back
+        if (elect_one()) umma_commit(&drain[m]);
+        const long long t0 = clock64();
+        while (!mbar_try_wait(&drain[m], 0) && clock64() - t0 < kSpinCycles) {
+        }
+      }
+    } else {
+      // ---------------- source rows: loading warp i takes units i, i + 6, ... ----------------
+      // eight lanes take the 16-byte pieces of a line, the four groups of eight lanes 16 columns each
+      const int q = lane >> 3, piece = lane & 7;
+      int g = warp - kLoadWarp0, before = 0, at = 0;  // before: units before the item `it`
+      bool have = walk.next(p, it), ok = true;
+      auto seek = [&]() {  // the item of unit g
+        while (have && g - before >= it.len) {
+          before += it.len;
+          have = walk.next(p, it);
+        }
+        at = g - before;
+        return have;
+      };
+      int4 idx[4];
+      auto indices = [&]() {
+        const int4* src = reinterpret_cast<const int4*>(p.tcol + (it.chunk + at) * 64) + 4 * q;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) idx[i] = __ldg(src + i);
+      };
+      if (seek()) indices();
+      while (have) {
+        const uint32_t s = g % kStagesB, ph = (g / kStagesB) & 1;
+        ok = __all_sync(0xffffffffu, mbar_wait(&done[s], ph ^ 1, 22));
+        if (!ok) break;
+        uint8_t* stage = smem + s * L::STAGE;
+        if (elect_one()) {
+          mbar_expect_tx(&full_w[s], kBitBytes);
+          bulk_load(stage + L::COUNT * kLineBytes, p.bits + (it.chunk + at) * 256, kBitBytes, &full_w[s]);
+        }
+        __syncwarp();
+        const uint8_t* src = p.split + (int64_t)it.slab * L::COUNT * 128 + piece * 16;
+        const uint32_t dst = smem_u32(stage + q * 2048);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          const int4& v = idx[i >> 2];
+          const int row = (i & 3) == 0 ? v.x : (i & 3) == 1 ? v.y : (i & 3) == 2 ? v.z : v.w;
+          const uint8_t* r = src + (int64_t)row * p.split_pitch;
+#pragma unroll
+          for (int line = 0; line < L::COUNT; ++line)
+            cp_async16(dst + line * kLineBytes + (i >> 3) * 1024 + (i & 7) * 128 + ((piece ^ (i & 7)) << 4), r + line * 128);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        g += kLoadWarps;
+        if (seek()) indices();  // on their way while the lines are
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // hand them to the tensor core
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&full_b[s]);
+      }
+      if (!ok || tc_error_now() != 0) {  // the bit copies already issued land before the CTA exits
+        const long long t0 = clock64();
+        for (int gi = g - kLoadWarps; gi >= 0 && gi > g - 3 * kLoadWarps; gi -= kLoadWarps)
+          while (!mbar_try_wait(&full_w[gi % kStagesB], (gi / kStagesB) & 1) && clock64() - t0 < kSpinCycles) {
+          }
+      }
     }
-  }
   } else if (warp < kFoldWarp0) {
     // ---------------- bits -> A ----------------
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsExpand));
     const int mt = (warp - kExpandWarp0) >> 2, q = warp & 3, row = mt * 128 + q * 32 + lane;
     const uint32_t lanes = tmem_base + ((uint32_t)(32 * q) << 16) + A_COL0 + mt * 32;
     for (int g = 0; g < n; ++g) {
-      const uint32_t s = g % kStagesA, ph = (g / kStagesA) & 1, sb = g % kStagesB, pb = (g / kStagesB) & 1;
-      if (!__all_sync(0xffffffffu, mbar_wait(&full_w[sb], pb, 27) && mbar_wait(&empty_a[s], ph ^ 1, 23))) break;
+      // the stage of A is free when the MMAs of unit g - kStagesA have retired
+      const uint32_t s = g % kStagesA, sb = g % kStagesB, pb = (g / kStagesB) & 1;
+      const int e = g + kStagesB - kStagesA;
+      uint64_t* freed = &done[e % kStagesB];
+      const uint32_t pf = (e / kStagesB + 1) & 1;
+      const bool have_w = mbar_try_wait(&full_w[sb], pb), have_a = mbar_try_wait(freed, pf);
+      bool ok = have_w & have_a;
+      if (!ok) ok = mbar_wait(&full_w[sb], pb, 27) && mbar_wait(freed, pf, 23);
+      if (!__all_sync(0xffffffffu, ok)) break;
       const uint64_t w = *reinterpret_cast<const uint64_t*>(smem + sb * L::STAGE + L::COUNT * kLineBytes + row * 8);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       // column j of A holds k = 2 j and 2 j + 1, bits j and j + 16 of a half of the word; a set bit lands on bit 14
@@ -364,28 +354,33 @@ __global__ void __launch_bounds__(kThreads, 1) spmm_dense(const Params p) {
     const int mt = (warp - kFoldWarp0) >> 2, q = warp & 3, row = mt * 128 + q * 32 + lane;
     const uint32_t lanes = tmem_base + ((uint32_t)(32 * q) << 16) + mt * N;
     float run[N];
-    uint32_t seg = 0;
+    uint32_t g = 0;
     bool ok = true;
     while (ok && walk.next(p, it)) {
 #pragma unroll
       for (int i = 0; i < N; ++i) run[i] = 0.f;
-      for (int c = 0; c < it.len; c += kFold, ++seg) {
-        const uint32_t b = seg & 1;
-        ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[b], (seg >> 1) & 1, 21));
+      for (int c = 0; c < it.len; ++c, ++g) {
+        const uint32_t b = g & 1;
+        ok = __all_sync(0xffffffffu, mbar_wait(&done[g % kStagesB], (g / kStagesB) & 1, 21));
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-        for (int n0 = 0; n0 < N; n0 += 16) {
-          uint32_t v[16];
+        for (int n0 = 0; n0 < N; n0 += 32) {  // two loads of 16 columns in flight
+          uint32_t v[16], w[16];
           tmem_ld16(lanes + b * ACC + n0, v);
+          if (n0 + 16 < N) tmem_ld16(lanes + b * ACC + n0 + 16, w);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          if (n0 + 16 == N) {
+          if (n0 + 32 >= N) {
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(&acc_empty[b]);
           }
 #pragma unroll
           for (int j = 0; j < 16; ++j) run[n0 + j] += __uint_as_float(v[j]);
+          if (n0 + 16 < N) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) run[n0 + 16 + j] += __uint_as_float(w[j]);
+          }
         }
       }
       if (!ok) break;

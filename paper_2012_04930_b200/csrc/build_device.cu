@@ -471,6 +471,27 @@ __global__ void gather_labels(const int32_t* __restrict__ members, int64_t np, i
   mask_out[i] = (i < lim && train_mask[v] != 0) ? 1 : 0;
 }
 
+// flag[k] = row order[k] has more than lo and at most hi entries
+__global__ void flag_by_length(const int32_t* __restrict__ order, int64_t n, const int32_t* __restrict__ rowptr, int64_t lo,
+                               int64_t hi, int32_t* flag) {
+  const int64_t k = global_thread();
+  if (k >= n) return;
+  const int32_t r = order[k];
+  const int64_t len = rowptr[r + 1] - rowptr[r];
+  flag[k] = len > lo && len <= hi;
+}
+// out[0] += entries whose column is more than an eighth of the matrix away from the row
+__global__ void count_far(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col, int64_t np, u64* out) {
+  const int64_t row = global_thread() >> 5;
+  if (row >= np) return;
+  int far = 0;
+  for (int e = rowptr[row] + lane_id(); e < rowptr[row + 1]; e += 32) {
+    const int64_t d = (int64_t)col[e] - row;
+    far += 8 * (d < 0 ? -d : d) > np;
+  }
+  far = warp_sum(far);
+  if (lane_id() == 0 && far) atomicAdd(out, (u64)far);
+}
 __global__ void flag_carrying_in_order(const int32_t* __restrict__ order, int64_t np, const uint8_t* __restrict__ carries,
                                        int32_t* flag) {
   const int64_t k = global_thread();
@@ -915,6 +936,7 @@ struct Builder {
   void assign();
   void build_partition(int32_t p, int64_t n_owned);
   void build_plan(DevPart& d, int64_t window);
+  void build_splits(DevPart& d);
 };
 
 // A plan pays where a chunk of 64 columns takes enough entries off the gathers: per 64 features a chunk costs one SM
@@ -924,6 +946,55 @@ struct Builder {
 // as the gathers.  A partition of fewer than kPlanMinNnz entries is a few microseconds of gathers, less than the
 // launches of a planned product cost.
 constexpr int64_t kPlanMinNnz = 1 << 19, kPlanEntriesPerChunk = 768;
+
+// The processing orders by row length (RowSplit in internal.h).
+void Builder::build_splits(DevPart& d) {
+  const int64_t np = d.info.n, nt = d.info.n_train;
+  if (!ok() || d.plan.n_chunks > 0 || np < kShortMinRows || d.info.nnz > np * kBlockRow) return;
+  if (!tiles) {
+    tiles_cap = ceil_div(np + 1, kScanTile) + 2;
+    tiles = scratch<int64_t>((size_t)tiles_cap);
+  }
+  const size_t mark = tmp.size();
+  int32_t* flags = scratch<int32_t>((size_t)np + 1);
+  int32_t* at = scratch<int32_t>((size_t)np + 1);
+  u64* far = scratch<u64>(1);
+  if (!ok()) return;
+  zero(far, sizeof(u64));
+  count_far<<<blocks_for(np * 32, 256), 256, 0, s>>>(d.rowptr, d.col, np, far);
+  launched("count_far");
+  u64 h_far = 0;
+  read(&h_far, far, 1);
+  struct One { RowSplit* split; const int32_t* order; int64_t n; const int32_t* rowptr; };
+  for (const One& o : {One{&d.split, d.order, np, d.rowptr}, One{&d.t_split, d.t_order, np, d.t_rowptr},
+                       One{&d.m_split, d.m_order, nt, d.rowptr}, One{&d.tm_split, d.tm_order, np, d.tm_rowptr}}) {
+    if (o.n < kShortMinRows) continue;
+    int32_t* out = result<int32_t>((size_t)o.n);
+    if (!ok()) return;
+    int64_t done[3] = {0, 0, 0}, at_out = 0;
+    const int64_t lo[3] = {kBlockRow, kShortRow, -1}, hi[3] = {INT64_MAX, kBlockRow, kShortRow};
+    for (int c = 0; c < 3; ++c) {
+      flag_by_length<<<blocks_for(o.n, 256), 256, 0, s>>>(o.order, o.n, o.rowptr, lo[c], hi[c], flags);
+      launched("flag_by_length");
+      const int64_t* total = scan<int32_t>(flags, o.n, at);
+      scatter_flagged<<<blocks_for(o.n, 256), 256, 0, s>>>(flags, at, o.n, o.order, out, at_out);
+      launched("scatter_flagged");
+      if (c < 2) at_out += scan_total(total);
+      done[c] = at_out;
+    }
+    if (!ok()) return;
+    if (2 * (o.n - done[1]) < o.n) continue;  // most rows keep a warp: the plain order serves as well
+    o.split->order = out;
+    o.split->n_long = done[0];
+    o.split->n_warp = done[1];
+    o.split->scattered = 2 * (int64_t)h_far > d.info.nnz;
+  }
+  cudaStreamSynchronize(s);
+  while (tmp.size() > mark) {
+    P->env.release(tmp.back());
+    tmp.pop_back();
+  }
+}
 
 void Builder::build_plan(DevPart& d, int64_t window) {
   const int64_t np = d.info.n, nnz = d.info.nnz, nt = d.info.n_train;
@@ -1287,6 +1358,7 @@ void Builder::build_partition(int32_t p, int64_t n_owned) {
   d.members.assign(mem32.begin(), mem32.end());
   drop(members); drop(deg); drop(cnt);
   build_plan(d, window);
+  build_splits(d);
 }
 
 int Builder::run() {
@@ -1386,6 +1458,7 @@ int build_device(gcnsa_parts* P, const gcnsa_graph* g, const gcnsa_part_opts* o)
 int build_dense_plan(gcnsa_parts* P, DevPart& d, int64_t window) {
   Builder b{P, nullptr, nullptr, P->env.stream()};
   b.build_plan(d, window);
+  b.build_splits(d);
   return b.rc;
 }
 

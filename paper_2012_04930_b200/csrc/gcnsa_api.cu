@@ -654,7 +654,8 @@ static int sparse_product(gcnsa_model* M, Lane& W, void* s, const DevPart& d, De
   const int32_t* col = use == DenseUse::lossCols ? d.tm_col : transposed ? d.t_col : d.col;
   const float* val = !values ? nullptr : use == DenseUse::lossCols ? d.tm_val : transposed ? d.t_val : d.val;
   PROF_SPMM(M, cost, launch_spmm(s, rows, rowptr, col, val, values ? nullptr : d.dinv, order, n_long, x, ldx, f, epi, aux, ldaux,
-                                 y, ldy, SpmmBounds{n, n, use == DenseUse::lossCols ? d.tm_nnz : d.info.nnz}));
+                                 y, ldy, SpmmBounds{n, n, use == DenseUse::lossCols ? d.tm_nnz : d.info.nnz},
+                                 use == DenseUse::lossRows ? d.m_split : use == DenseUse::lossCols ? d.tm_split : transposed ? d.t_split : d.split));
   return GCNSA_OK;
 }
 

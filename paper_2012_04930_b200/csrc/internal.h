@@ -103,6 +103,19 @@ int build_host(const gcnsa_graph* g, const gcnsa_part_opts* o, HostBuild* out);
 // 64-bit selection key (SplitMix64 finalizer applied word by word).
 uint64_t selection_key(uint64_t seed, uint64_t w0, uint64_t w1, uint64_t w2, uint64_t w3, uint64_t v);
 
+// ---- rows by length, where most rows are short: the processing order with the rows of more than kBlockRow entries
+// first, then those of more than kShortRow, then the others (each part in its order).  Rows [0, n_long) get a thread block
+// each, [n_long, n_warp) a warp, the rest a group of lanes (short_rows in kernels_spmm.cu).  From kShortMinRows rows on:
+// below that the launch is a handful of blocks per SM either way and a group's longer chain of loads costs more than the
+// fewer warps save (5 500 rows of 20 entries, 16 features: 4.8 us with a warp per row, 6.7 with a group; 13 200 rows: 10.3
+// and 6.7; 100 000 rows of 33: 43 and 16).
+constexpr int64_t kShortRow = 64, kBlockRow = 256, kShortMinRows = 10240;
+struct RowSplit {
+  int32_t* order = nullptr;  // NULL: not made
+  int64_t n_long = 0, n_warp = 0;
+  bool scattered = false;    // most entries lie far from the diagonal: neighbouring rows share few columns
+};
+
 // ---- the plan of a partition's products on the tensor cores (kernels_spmm_dense.cu) ---
 // Rows are grouped into tiles of kDenseRows: first the rows that carry loss, then the others, each group in index order
 // (communities stay together) and filled up to whole tiles.  A column that at least kDenseMin of a tile's rows have an
@@ -146,7 +159,8 @@ struct SpmmBase {
 // bounds: what the caller knows about the operands, checked by the kernels of the GCNSA_DEBUG build only
 int launch_spmm(void* stream, int64_t n_rows, const int32_t* rowptr, const int32_t* col, const float* val,
                 const float* row_scale, const int32_t* order, int64_t n_long, const float* x, int64_t ldx, int32_t f, int32_t epi, const float* aux,
-                int64_t ldaux, float* y, int64_t ldy, const SpmmBounds& bounds = SpmmBounds());
+                int64_t ldaux, float* y, int64_t ldy, const SpmmBounds& bounds = SpmmBounds(),
+                const RowSplit& split = RowSplit());
 // Y = epi(diag(row_scale) B diag(src_scale) X) through a partition's plan (both scales nullable); workspace:
 // spmm_planned_workspace(plan, f) bytes, 256-byte aligned.  Returns -1 when the plan cannot be used.
 int launch_spmm_planned(void* stream, const DensePlan& d, DenseUse use, int64_t n_rows, const float* row_scale,

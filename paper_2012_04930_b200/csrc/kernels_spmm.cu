@@ -224,13 +224,107 @@ __device__ __forceinline__ void store_chunk(float4 r, int row, int qq, int f, in
   reinterpret_cast<float4*>(y + (int64_t)row * ldy)[qq] = r;
 }
 
+// Rows of a few dozen entries (33 in the degree-32 random graph, 20 in the block models, four fifths of the rows of the
+// 2.45 M-vertex graph): with a warp per row the loads that depend on one another (order, row pointers, indices, rows) and
+// the folding of the groups' sums outweigh the gathers.  Here a group of G lanes owns a row, every lane CH float4 chunks
+// of it, so a warp works on 32 / G rows of one length class at a time and nothing is folded.  A group fetches the indices
+// of 16 (G < 16) or G entries with coalesced loads, the next ones while these are gathered, and hands them round by
+// shuffle; U gathers per lane are in flight.  w: the group's place in the processing order.
+template <int G, int CH, int U, bool UNIT>
+__device__ __forceinline__ void short_rows(int w, int n_rows, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
+                                           const float* __restrict__ val, const float* __restrict__ rscale,
+                                           const int32_t* __restrict__ order, const float4* __restrict__ x, int64_t ldx4, int nvec,
+                                           int f, int epi, const float* __restrict__ aux, int64_t ldaux, float* __restrict__ y,
+                                           int64_t ldy GCNSA_DBG_PARAM) {
+  constexpr int B = G < 16 ? 16 : G, L = B / G;  // entries per round, indices per lane
+  const int gl = threadIdx.x % G;
+  bool ok = w < n_rows;
+  if (!__any_sync(kFull, ok)) return;
+  int row = 0, beg = 0, n = 0;
+  if (ok) {
+    row = __ldg(order + w);
+#if GCNSA_DBG
+    ok = dbg.mat_rows < 0 || dbg_in(&g_dbg_spmm, row, 0, dbg.mat_rows, kDbgOrderEntry);
+#endif
+  }
+  if (ok) {
+    beg = __ldg(rowptr + row);
+    const int end = __ldg(rowptr + row + 1);
+#if GCNSA_DBG
+    ok = dbg_in(&g_dbg_spmm, beg, 0, (long long)end + 1, kDbgRowRange) &&
+         (dbg.nnz < 0 || dbg_in(&g_dbg_spmm, end, 0, dbg.nnz + 1, kDbgRowRange));
+#endif
+    if (ok) n = end - beg;
+  }
+  const int n_max = __reduce_max_sync(kFull, n);
+  float4 acc[CH];
+#pragma unroll
+  for (int ch = 0; ch < CH; ++ch) acc[ch] = make_float4(0.f, 0.f, 0.f, 0.f);
+  int nxt[L];
+  float nxt_v[L];
+  auto fetch = [&](int base) {
+#pragma unroll
+    for (int j = 0; j < L; ++j) {
+      const int k = base + j * G + gl;
+      nxt[j] = k < n ? __ldg(col + beg + k) : 0;
+      nxt_v[j] = !UNIT && k < n ? __ldg(val + beg + k) : 0.f;
+    }
+  };
+  fetch(0);
+  for (int base = 0; base < n_max; base += B) {
+    int mine[L];
+    float wgt[L];
+#pragma unroll
+    for (int j = 0; j < L; ++j) { mine[j] = nxt[j]; wgt[j] = nxt_v[j]; }
+    if (base + B < n_max) fetch(base + B);
+#pragma unroll
+    for (int k0 = 0; k0 < B; k0 += U) {
+      if (base + k0 >= n_max) break;  // all rows of the warp alike
+      float4 v[U][CH];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int k = k0 + u;
+        const int c = __shfl_sync(kFull, mine[k / G], k % G, G);
+        bool live = base + k < n;
+#if GCNSA_DBG
+        if (live && dbg.src_rows >= 0) live = dbg_in(&g_dbg_spmm, c, 0, dbg.src_rows, kDbgColumn);
+#endif
+        const float4* xr = x + (int64_t)c * ldx4 + gl;
+#pragma unroll
+        for (int ch = 0; ch < CH; ++ch)
+          v[u][ch] = live && gl + ch * G < nvec ? __ldg(xr + ch * G) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int k = k0 + u;
+        const float sv = UNIT ? 1.f : __shfl_sync(kFull, wgt[k / G], k % G, G);
+#pragma unroll
+        for (int ch = 0; ch < CH; ++ch) {
+          if (UNIT) add4(acc[ch], v[u][ch]);
+          else fma4(acc[ch], sv, v[u][ch]);
+        }
+      }
+    }
+  }
+  if (!ok) return;
+  const float sc = rscale ? __ldg(rscale + row) : 1.f;
+#pragma unroll
+  for (int ch = 0; ch < CH; ++ch) {
+    const int qq = gl + ch * G;
+    if (qq >= nvec) continue;
+    float4 r = acc[ch];
+    if (rscale) { r.x *= sc; r.y *= sc; r.z *= sc; r.w *= sc; }
+    store_chunk(r, row, qq, f, epi, aux, ldaux, y, ldy);
+  }
+}
+
 // Blocks [0, n_long): one thread block per long row order[b]; its TPB / 32 warps take equal parts of the row,
 // their sums meet in shared memory and are added in warp order (fixed order), so a hub row of thousands of
-// non-zeros is not one warp's serial chain.  Blocks after that: one warp per row order[n_long ..).  One launch,
-// longest rows dispatched first.
-template <int G, int CH, int U, int TPB, int MINB, bool UNIT>
+// non-zeros is not one warp's serial chain.  Blocks after that: one warp per row order[n_long .. n_warp), then a group of
+// lanes per row order[n_warp .. n_rows) (short_rows<SG, SCH, SU>).  One launch, longest rows dispatched first.
+template <int G, int CH, int U, int TPB, int MINB, bool UNIT, int SG, int SCH, int SU>
 __global__ void __launch_bounds__(TPB, MINB)
-spmm_rows(int n_long, int n_rows, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
+spmm_rows(int n_long, int n_warp, int n_rows, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
           const float* __restrict__ val, const float* __restrict__ rscale, const int32_t* __restrict__ order,
           const float4* __restrict__ x, int64_t ldx4,
           int nvec, int f, int vec_idx, int epi, const float* __restrict__ aux, int64_t ldaux, float* __restrict__ y,
@@ -288,8 +382,14 @@ spmm_rows(int n_long, int n_rows, const int32_t* __restrict__ rowptr, const int3
     }
     return;
   }
-  const int w = n_long + ((int)blockIdx.x - n_long) * W + warp;
-  if (w >= n_rows) return;
+  const int b = (int)blockIdx.x - n_long, b_short = b - (n_warp - n_long + W - 1) / W;
+  if (b_short >= 0) {
+    short_rows<SG, SCH, SU, UNIT>(n_warp + (b_short * W + warp) * (32 / SG) + lane / SG, n_rows, rowptr, col, val, rscale, order, x,
+                                  ldx4, nvec, f, epi, aux, ldaux, y, ldy GCNSA_DBG_ARG);
+    return;
+  }
+  const int w = n_long + b * W + warp;
+  if (w >= n_warp) return;
   const int row = order ? __ldg(order + w) : w;
 #if GCNSA_DBG
   if (dbg.mat_rows >= 0 && !dbg_in(&g_dbg_spmm, row, 0, dbg.mat_rows, kDbgOrderEntry)) return;  // whole warp alike
@@ -324,7 +424,7 @@ struct Args {
   const float* val;
   const float* rscale;
   const int32_t* order;
-  int n_long;
+  int n_long, n_warp;
   const float* x;
   int64_t ldx;
   int nvec, f, vec_idx, epi;
@@ -335,17 +435,18 @@ struct Args {
   SpmmBounds dbg;
 };
 
-template <int G, int CH, int U, int TPB, int MINB>
+template <int G, int CH, int U, int TPB, int MINB, int SG, int SCH, int SU>
 cudaError_t run(const Args& a) {
-  const int rows_per_block = TPB / 32;
-  const int grid = a.n_long + (a.n_rows - a.n_long + rows_per_block - 1) / rows_per_block;
+  const int rows_per_block = TPB / 32, short_per_block = rows_per_block * (32 / SG);
+  const int grid = a.n_long + (a.n_warp - a.n_long + rows_per_block - 1) / rows_per_block +
+                   (a.n_rows - a.n_warp + short_per_block - 1) / short_per_block;
   if (a.val)
-    spmm_rows<G, CH, U, TPB, MINB, false><<<grid, TPB, 0, a.s>>>(
-        a.n_long, a.n_rows, a.rowptr, a.col, a.val, a.rscale, a.order, reinterpret_cast<const float4*>(a.x), a.ldx / 4,
+    spmm_rows<G, CH, U, TPB, MINB, false, SG, SCH, SU><<<grid, TPB, 0, a.s>>>(
+        a.n_long, a.n_warp, a.n_rows, a.rowptr, a.col, a.val, a.rscale, a.order, reinterpret_cast<const float4*>(a.x), a.ldx / 4,
         a.nvec, a.f, a.vec_idx, a.epi, a.aux, a.ldaux, a.y, a.ldy GCNSA_DBG_LAUNCH_ARG);
   else
-    spmm_rows<G, CH, U, TPB, MINB, true><<<grid, TPB, 0, a.s>>>(
-        a.n_long, a.n_rows, a.rowptr, a.col, nullptr, a.rscale, a.order, reinterpret_cast<const float4*>(a.x), a.ldx / 4,
+    spmm_rows<G, CH, U, TPB, MINB, true, SG, SCH, SU><<<grid, TPB, 0, a.s>>>(
+        a.n_long, a.n_warp, a.n_rows, a.rowptr, a.col, nullptr, a.rscale, a.order, reinterpret_cast<const float4*>(a.x), a.ldx / 4,
         a.nvec, a.f, a.vec_idx, a.epi, a.aux, a.ldaux, a.y, a.ldy GCNSA_DBG_LAUNCH_ARG);
   note_launch();
   return cudaGetLastError();
@@ -502,7 +603,7 @@ cudaError_t run_rest(const RestArgs& a, const float* x, int nvec, int f, const f
 
 int launch_spmm(void* stream, int64_t n_rows, const int32_t* rowptr, const int32_t* col, const float* val,
                 const float* row_scale, const int32_t* order, int64_t n_long, const float* x, int64_t ldx, int32_t f, int32_t epi, const float* aux,
-                int64_t ldaux, float* y, int64_t ldy, const SpmmBounds& bounds) {
+                int64_t ldaux, float* y, int64_t ldy, const SpmmBounds& bounds, const RowSplit& split) {
   if (n_rows == 0 || f == 0) return 0;
   Args a;
   a.dbg = bounds;
@@ -510,13 +611,26 @@ int launch_spmm(void* stream, int64_t n_rows, const int32_t* rowptr, const int32
   a.n_rows = (int)n_rows;
   a.rowptr = rowptr; a.col = col; a.val = val; a.rscale = row_scale; a.order = order;
   a.n_long = order ? (int)std::min<int64_t>(std::max<int64_t>(n_long, 0), n_rows) : 0;
+  a.n_warp = (int)n_rows;
+  if (split.order) {
+    a.order = split.order;
+    a.n_long = (int)split.n_long;
+    a.n_warp = (int)split.n_warp;
+  }
   a.ldx = ldx; a.epi = epi; a.ldaux = ldaux; a.ldy = ldy;
   // 16-byte index loads need 16-byte aligned arrays; otherwise every quad goes element by element
   a.vec_idx = (((uintptr_t)col | (uintptr_t)val) & 15) == 0 ? 1 : 0;  // val == NULL (unit entries) counts as aligned
   const int nvec_total = (f + 3) / 4;
-  // column slabs of at most 5 x 32 float4 (640 floats) per launch
-  for (int v0 = 0; v0 < nvec_total; v0 += 160) {
-    a.nvec = min(160, nvec_total - v0);
+  // Column slabs of at most 5 x 32 float4 (640 floats) per launch.  Where the gathers have no locality, the gathered
+  // matrix is larger than L2 and its rows cut to 128 bytes are not (each die of the chip keeps its own copy of what its
+  // SMs read, so about 60 MB count), slabs of 8 float4 turn HBM reads into L2 hits: 400 000 rows of the degree-32 random
+  // graph, F' = 256: 1 128 -> 829 us, 128: 530 -> 410, 64: 206 -> 192.  Where neighbouring rows share their columns the
+  // slabs cost (245 000 rows of the 2.45 M-vertex graph, 256: 593 -> 764 us).
+  constexpr int64_t kL2 = 96 << 20, kL2Shared = 60 << 20;
+  const bool narrow = split.scattered && bounds.src_rows * nvec_total * 16 > kL2 && bounds.src_rows * 128 <= kL2Shared;
+  const int step = narrow ? 8 : 160;
+  for (int v0 = 0; v0 < nvec_total; v0 += step) {
+    a.nvec = std::min(step, nvec_total - v0);
     a.x = x + 4 * v0;
     a.y = y + 4 * v0;
     a.aux = aux ? aux + 4 * v0 : nullptr;  // bias and mask are both indexed by column
@@ -526,15 +640,15 @@ int launch_spmm(void* stream, int64_t n_rows, const int32_t* rowptr, const int32
     // MINB (blocks per SM the register allocation must allow) is part of the tuning: the kernel is bound by the
     // L1 data path, and about 32-40 resident warps per SM (64 resp. 48 registers a thread) measured fastest;
     // left alone the compiler unrolls to over 100 registers (16 warps), and at 32 registers (64 warps) L1 thrashes.
-    if (nv <= 4) e = run<4, 1, 2, 128, 10>(a);
-    else if (nv <= 8) e = run<4, 2, 2, 128, 10>(a);
-    else if (nv <= 12) e = run<4, 3, 2, 128, 10>(a);
-    else if (nv <= 16) e = run<8, 2, 2, 128, 10>(a);
-    else if (nv <= 32) e = run<32, 1, 4, 256, 4>(a);
-    else if (nv <= 64) e = run<32, 2, 4, 256, 4>(a);
-    else if (nv <= 96) e = run<32, 3, 2, 256, 3>(a);
-    else if (nv <= 128) e = run<32, 4, 2, 256, 3>(a);
-    else e = run<32, 5, 2, 256, 3>(a);
+    if (nv <= 4) e = run<4, 1, 2, 128, 10, 4, 1, 8>(a);
+    else if (nv <= 8) e = run<4, 2, 2, 128, 10, 8, 1, 8>(a);
+    else if (nv <= 12) e = run<4, 3, 2, 128, 10, 16, 1, 8>(a);
+    else if (nv <= 16) e = run<8, 2, 2, 128, 10, 16, 1, 8>(a);
+    else if (nv <= 32) e = run<32, 1, 4, 256, 4, 32, 1, 8>(a);
+    else if (nv <= 64) e = run<32, 2, 4, 256, 4, 32, 2, 4>(a);
+    else if (nv <= 96) e = run<32, 3, 2, 256, 3, 32, 3, 2>(a);
+    else if (nv <= 128) e = run<32, 4, 2, 256, 3, 32, 4, 2>(a);
+    else e = run<32, 5, 2, 256, 3, 32, 5, 2>(a);
     if (e != cudaSuccess) return (int)e;
   }
   return 0;

@@ -43,6 +43,7 @@ struct DevPart {
   std::vector<int64_t> members;
   std::vector<int32_t> depth;
   int64_t n_long = 0, t_n_long = 0;
+  RowSplit split, t_split, m_split, tm_split;  // of order, t_order, m_order, tm_order (partitions without a plan)
 };
 
 }  // namespace gcnsa
@@ -77,6 +78,7 @@ namespace gcnsa {
 // by the caller.
 int build_device(gcnsa_parts* P, const gcnsa_graph* g, const gcnsa_part_opts* o);
 // the plan of the tensor-core products of one partition (d.plan) from its CSR and mask on the device
+// or, where that does not pay, the split of its processing orders by row length
 int build_dense_plan(gcnsa_parts* P, DevPart& d, int64_t window);
 // Argument checks of gcnsa_build_partitions that need neither the graph's contents nor a device.
 int check_build_args(const gcnsa_graph* g, const gcnsa_part_opts* o);

@@ -75,3 +75,41 @@ def test_planned_products_match_fp64(n, dims, mask_p):
     assert launches[1] > launches[0], "the planned path did not run"
     assert gcnsa.tc_status() == 0
     parts.close()
+
+
+# rows of at most 64 entries go to a group of lanes, longer ones to a warp, those above 256 to a block; one width per
+# kernel shape, and a graph without locality whose gathered matrix exceeds L2 (column slabs)
+@pytest.mark.parametrize("n,width", [(12_003, 7), (12_003, 30), (12_003, 41), (12_003, 64), (12_003, 100), (12_003, 130),
+                                     (12_003, 300), (12_003, 400), (12_003, 520), (300_001, 101)])
+def test_rows_by_length_match_fp64(n, width):
+    if n < 100_000:
+        rowptr, col, _ = graphs.chung_lu_communities(n, 300_000, 2.1, 12, 0.7, 5)
+        assert (np.diff(rowptr) > 256).any() and (np.diff(rowptr) <= 64).mean() > 0.5
+    else:
+        rowptr, col = graphs.permutation_graph(n, 4, 5)
+    rng = np.random.default_rng(n + width)
+    x = rng.standard_normal((n, width), dtype=np.float32)
+    y = rng.integers(0, width, n).astype(np.int32)
+    mask = (rng.random(n) < 0.9).astype(np.uint8)
+    w0 = [np.eye(width, dtype=np.float32)]
+    env = gcnsa.make_env(0)
+    parts = gcnsa.Parts(env, rowptr, col, x, y, mask, width, 1, 0, 3)
+    ex = parts.export(0)
+    crow, ccol = (torch.from_numpy(ex[k].astype(np.int64)).cuda() for k in ("rowptr", "col"))
+    dinv = (crow[1:] - crow[:-1]).double().rsqrt()
+    pattern = torch.sparse_csr_tensor(crow, ccol, torch.ones(ccol.numel(), dtype=torch.float64, device="cuda"), size=(n, n))
+    on = mask.astype(bool)
+
+    def product(v):
+        return dinv[:, None] * (pattern @ (dinv[:, None] * v))
+
+    want = product(torch.from_numpy(x).double().cuda())
+    for fact in (0, 1):
+        m = gcnsa.Model(env, parts, [width, width], w0, use_bias=0, factored_norm=fact, epoch_graph=0)
+        m.forward(0)
+        _close(m.get(gcnsa.GET_ACT, 1, n)[on], want[torch.from_numpy(on).cuda()], ("logits", fact))
+        g = torch.from_numpy(m.get(gcnsa.GET_DLOGITS, 1, n)).double().cuda()
+        m.backward(0)
+        _close(m.get(gcnsa.GET_GRAD_W, 0), torch.from_numpy(x).double().cuda().T @ product(g), ("dW", fact))
+        m.close()
+    parts.close()

@@ -10,9 +10,9 @@
 //   - the graph induced on owned + sampled vertices (Section 4: all other edges
 //     are dropped) is written row by row, owned neighbours first, then sampled
 //     ones, the self-loop merged in, which is ascending local order;
-//   - the transposed CSR comes from a stable radix sort of (column, row) pairs,
-//     a real transpose that assumes nothing about symmetry;
-//   - rows are ordered hub rows first, then by descending length class (stable
+//   - the induced graph of a symmetric graph (check_symmetry) is symmetric, so
+//     its CSR with ascending rows is its own transposed CSR: same arrays;
+//   - rows are ordered hub rows first, then by descending length class (a stable
 //     radix sort), the loss rows and the transposed CSR over loss columns are
 //     compacted in order.
 // All integer work; results are bit-identical to the host builder's.  No kernel
@@ -21,9 +21,11 @@
 
 #include <algorithm>
 #include <cstring>
+#include <memory>
 #include <string>
 #include <vector>
 
+#include "host_upload.h"
 #include "internal.h"
 #include "parts.h"
 
@@ -423,17 +425,6 @@ __global__ void induced_fill(const int64_t* __restrict__ rp, const int32_t* __re
   if (lane == 0 && GCNSA_CHECK_WRITE(below, len, kDbgInducedWrite)) w[below] = (int32_t)i;
 }
 
-__global__ void expand_rows(const int32_t* __restrict__ rowptr, int64_t np, int32_t* rowid) {
-  const int64_t i = global_warp();
-  if (i >= np) return;
-  for (int32_t e = rowptr[i] + lane_id(); e < rowptr[i + 1]; e += 32) rowid[e] = (int32_t)i;
-}
-
-__global__ void count_columns(const int32_t* __restrict__ col, int64_t nnz, int32_t* cnt) {
-  const int64_t e = global_thread();
-  if (e < nnz) atomicAdd(&cnt[col[e]], 1);
-}
-
 // key[i] = order_key of row i (hub rows, then the others window by window, by descending length class), val[i] = i
 __global__ void length_keys(const int32_t* __restrict__ rowptr, int64_t np, int64_t thr, int64_t window, uint32_t* key,
                             int32_t* val) {
@@ -794,6 +785,8 @@ struct Builder {
   const gcnsa_part_opts* o;
   cudaStream_t s;
   std::vector<void*> tmp;  // scratch, released when the build ends
+  std::unique_ptr<HostUpload> loader;  // large pageable inputs
+  bool x_pending = false;              // the features are still on their way through the loader
   int rc = GCNSA_OK;
 
   // whole graph on the device
@@ -815,6 +808,7 @@ struct Builder {
   u64 h_words[8];
 
   ~Builder() {
+    loader.reset();  // its copies have ended before their targets are given back
     cudaStreamSynchronize(s);
     for (void* p : tmp) P->env.release(p);
   }
@@ -854,7 +848,8 @@ struct Builder {
   template <class T>
   T* upload(const T* host, size_t count) {
     T* d = scratch<T>(count);
-    if (d && count) cuda(cudaMemcpyAsync(d, host, count * sizeof(T), cudaMemcpyHostToDevice, s), "upload");
+    if (d && count && loader && HostUpload::pageable(host)) loader->add(d, host, 1, count * sizeof(T), count * sizeof(T));
+    else if (d && count) cuda(cudaMemcpyAsync(d, host, count * sizeof(T), cudaMemcpyHostToDevice, s), "upload");
     return d;
   }
   void zero(void* p, size_t bytes) {
@@ -944,8 +939,9 @@ struct Builder {
 // rows come on top.  Measured at 1 640 and 1 230 entries per chunk: F' = 128 365 -> 250 us (58 241 rows, 28 M entries)
 // and 435 -> 290 us (51 249 rows, 20.8 M entries); at 630 (245 000 rows, 12.6 M entries) the planned product is as slow
 // as the gathers.  A partition of fewer than kPlanMinNnz entries is a few microseconds of gathers, less than the
-// launches of a planned product cost.
-constexpr int64_t kPlanMinNnz = 1 << 19, kPlanEntriesPerChunk = 768;
+// launches of a planned product cost, and one with short rows is not looked at (a tile of 256 rows would have to meet the
+// same few hundred columns).
+constexpr int64_t kPlanMinNnz = 1 << 19, kPlanMinDegree = 40, kPlanEntriesPerChunk = 768;
 
 // The processing orders by row length (RowSplit in internal.h).
 void Builder::build_splits(DevPart& d) {
@@ -966,8 +962,8 @@ void Builder::build_splits(DevPart& d) {
   u64 h_far = 0;
   read(&h_far, far, 1);
   struct One { RowSplit* split; const int32_t* order; int64_t n; const int32_t* rowptr; };
-  for (const One& o : {One{&d.split, d.order, np, d.rowptr}, One{&d.t_split, d.t_order, np, d.t_rowptr},
-                       One{&d.m_split, d.m_order, nt, d.rowptr}, One{&d.tm_split, d.tm_order, np, d.tm_rowptr}}) {
+  for (const One& o : {One{&d.split, d.order, np, d.rowptr}, One{&d.m_split, d.m_order, nt, d.rowptr},
+                       One{&d.tm_split, d.tm_order, np, d.tm_rowptr}}) {
     if (o.n < kShortMinRows) continue;
     int32_t* out = result<int32_t>((size_t)o.n);
     if (!ok()) return;
@@ -989,6 +985,7 @@ void Builder::build_splits(DevPart& d) {
     o.split->n_warp = done[1];
     o.split->scattered = 2 * (int64_t)h_far > d.info.nnz;
   }
+  d.t_split = d.split;  // (the host builder's transposed CSR has the same rows)
   cudaStreamSynchronize(s);
   while (tmp.size() > mark) {
     P->env.release(tmp.back());
@@ -998,7 +995,7 @@ void Builder::build_splits(DevPart& d) {
 
 void Builder::build_plan(DevPart& d, int64_t window) {
   const int64_t np = d.info.n, nnz = d.info.nnz, nt = d.info.n_train;
-  if (!ok() || nnz < kPlanMinNnz) return;
+  if (!ok() || nnz < kPlanMinNnz || nnz < np * kPlanMinDegree) return;
   DensePlan& pl = d.plan;
   const int64_t loss_tiles = ceil_div(nt, kDenseRows), n_tiles = loss_tiles + ceil_div(np - nt, kDenseRows);
   const int64_t words = ceil_div(np, 32), windows = ceil_div(np, kPlanWindow);
@@ -1241,30 +1238,18 @@ void Builder::build_partition(int32_t p, int64_t n_owned) {
   induced_fill<<<pwb, 256, 0, s>>>(rp, col, members, np, n_owned, g2l, d.rowptr, d.col);
   launched("induced_fill");
 
-  // ---- transpose: stable sort of (column, row) by column
-  int bits = 1;
-  while (((int64_t)1 << bits) <= np) ++bits;  // keys are in [0, np]
-  const int64_t sort_tiles = std::max<int64_t>(1, ceil_div(nnz, kSortTile));
-  uint32_t* k0 = scratch<uint32_t>((size_t)nnz);
-  int32_t* v0 = scratch<int32_t>((size_t)nnz);
-  uint32_t* k1 = scratch<uint32_t>((size_t)nnz);
-  int32_t* v1 = scratch<int32_t>((size_t)nnz);
+  // ---- transposed CSR: the matrix is symmetric and its rows ascend, so it is the CSR itself
+  d.t_rowptr = d.rowptr;
+  d.t_col = d.col;
+  // scratch of the row sorts
+  const int64_t sort_tiles = std::max<int64_t>(1, ceil_div(np, kSortTile));
+  uint32_t* k0 = scratch<uint32_t>((size_t)np);
+  int32_t* v0 = scratch<int32_t>((size_t)np);
+  uint32_t* k1 = scratch<uint32_t>((size_t)np);
+  int32_t* v1 = scratch<int32_t>((size_t)np);
   int32_t* hist = scratch<int32_t>((size_t)(256 * sort_tiles + 1));
   int32_t* cnt = scratch<int32_t>((size_t)np + 1);
-  d.t_rowptr = result<int32_t>((size_t)np + 1);
-  d.t_col = result<int32_t>((size_t)nnz);
   if (!ok()) return;
-  cuda(cudaMemcpyAsync(k0, d.col, (size_t)nnz * sizeof(int32_t), cudaMemcpyDeviceToDevice, s), "copy");
-  expand_rows<<<pwb, 256, 0, s>>>(d.rowptr, np, v0);
-  launched("expand_rows");
-  zero(cnt, ((size_t)np + 1) * sizeof(int32_t));
-  count_columns<<<blocks_for(nnz, 256), 256, 0, s>>>(d.col, nnz, cnt);
-  launched("count_columns");
-  scan<int32_t>(cnt, np, d.t_rowptr);
-  {
-    const int where = sort_pairs(k0, v0, k1, v1, nnz, bits, hist);
-    cuda(cudaMemcpyAsync(d.t_col, where ? v1 : v0, (size_t)nnz * sizeof(int32_t), cudaMemcpyDeviceToDevice, s), "copy");
-  }
 
   // ---- labels, loss mask
   const int64_t lim = o->loss_on_halo ? np : n_owned;
@@ -1276,7 +1261,6 @@ void Builder::build_partition(int32_t p, int64_t n_owned) {
 
   // ---- processing orders (longest rows first, ties by row index) and hub-row counts
   d.order = result<int32_t>((size_t)np);
-  d.t_order = result<int32_t>((size_t)np);
   d.tm_order = result<int32_t>((size_t)np);
   d.tm_rowptr = result<int32_t>((size_t)np + 1);
   if (!ok()) return;
@@ -1289,11 +1273,9 @@ void Builder::build_partition(int32_t p, int64_t n_owned) {
   };
   const int64_t thr = long_row_threshold(nnz);
   make_order(d.rowptr, thr, d.order);
-  make_order(d.t_rowptr, thr, d.t_order);
+  d.t_order = d.order;
   zero(counters, 8 * sizeof(u64));
   count_long_rows<<<pvb, 256, 0, s>>>(d.rowptr, np, thr, nullptr, counters + 0);
-  launched("count_long_rows");
-  count_long_rows<<<pvb, 256, 0, s>>>(d.t_rowptr, np, thr, nullptr, counters + 2);
   launched("count_long_rows");
   count_long_rows<<<pvb, 256, 0, s>>>(d.rowptr, np, thr, d.mask, counters + 4);  // loss rows: [4] long ones, [5] entries
   launched("count_long_rows");
@@ -1325,29 +1307,30 @@ void Builder::build_partition(int32_t p, int64_t n_owned) {
   read(h_words, counters, 8);
   if (!ok()) return;
   d.n_long = (int64_t)h_words[0];
-  d.t_n_long = (int64_t)h_words[2];
+  d.t_n_long = d.n_long;
   d.m_n_long = (int64_t)h_words[4];
   d.m_nnz = (int64_t)h_words[5];
   d.tm_n_long = (int64_t)h_words[6];
 
-  // the sort scratch is the largest: give it back before the values and features are allocated
-  drop(k0); drop(v0); drop(k1); drop(v1); drop(hist);
-
   // ---- features in partition order
   d.x = result<float>((size_t)np * (size_t)P->ldx);
   if (!ok()) return;
+  if (x_pending) {
+    x_pending = false;
+    cuda(loader->finish(s), "upload of the features");
+    if (!ok()) return;
+  }
   gather_features<<<pwb, 256, 0, s>>>(x, g->f, members, np, d.x, P->ldx);
   launched("gather_features");
 
   // ---- D^-1/2 (A + I) D^-1/2: entry (i, j) and entry (j, i) of the transpose are both 1 / sqrt(d_i d_j)
   d.val = result<float>((size_t)nnz);
-  d.t_val = result<float>((size_t)nnz);
+  d.t_val = d.val;
   d.tm_val = result<float>((size_t)tm_nnz);
   d.dinv = result<float>((size_t)np);
   if (!ok()) return;
   int e = launch_normalize(s, np, d.rowptr, d.col, deg, d.val);
   if (!e) e = launch_inv_sqrt_degree(s, np, deg, d.dinv);
-  if (!e) e = launch_normalize(s, np, d.t_rowptr, d.t_col, deg, d.t_val);
   if (!e) e = launch_normalize(s, np, d.tm_rowptr, d.tm_col, deg, d.tm_val);
   if (e) { cuda((cudaError_t)e, "normalize"); return; }
 
@@ -1356,7 +1339,7 @@ void Builder::build_partition(int32_t p, int64_t n_owned) {
   read(mem32.data(), members, (size_t)np);
   if (!ok()) return;
   d.members.assign(mem32.begin(), mem32.end());
-  drop(members); drop(deg); drop(cnt);
+  for (void* t : std::initializer_list<void*>{members, deg, cnt, k0, v0, k1, v1, hist}) drop(t);
   build_plan(d, window);
   build_splits(d);
 }
@@ -1368,13 +1351,40 @@ int Builder::run() {
   const unsigned vb = blocks_for(n, 256), wb = blocks_for(n * 32, 256);
 
   // ---- the graph goes to the device once
+  const size_t x_bytes = (size_t)n * (size_t)g->f * sizeof(float);
+  if ((size_t)nnz * sizeof(int32_t) + x_bytes >= HostUpload::kWorthwhile &&
+      (HostUpload::pageable(g->col) || HostUpload::pageable(g->x))) {
+    loader.reset(new HostUpload(P->env.e.device));
+    if (!loader->open()) loader.reset();
+  }
   rp = upload(g->rowptr, (size_t)n + 1);
   col = upload(g->col, (size_t)nnz);
   y = upload(g->y, (size_t)n);
   train_mask = upload(g->train_mask, (size_t)n);
+  if (loader && ok()) {
+    cuda(loader->start(s), "upload of the graph");
+    if (ok()) cuda(loader->finish(s), "upload of the graph");
+  }
   err = scratch<u64>(1);
   counters = scratch<u64>(8);
   part = scratch<int32_t>((size_t)n);
+  if (!ok()) return rc;
+
+  // ---- features: uploaded dense, gathered per partition on the device; through the loader they travel while the graph is
+  // checked and partitioned
+  x = scratch<float>((size_t)n * (size_t)g->f);
+  if (!ok()) return rc;
+  if (loader && HostUpload::pageable(g->x)) {
+    loader->add(x, g->x, (size_t)n, (size_t)g->f * sizeof(float), (size_t)g->ldx * sizeof(float));
+    cuda(loader->start(s), "upload of the features");
+    x_pending = true;
+  } else if (g->ldx == g->f) {  // (a pageable copy row by row takes three times as long)
+    cuda(cudaMemcpyAsync(x, g->x, x_bytes, cudaMemcpyHostToDevice, s), "upload of the features");
+  } else {
+    cuda(cudaMemcpy2DAsync(x, (size_t)g->f * sizeof(float), g->x, (size_t)g->ldx * sizeof(float), (size_t)g->f * sizeof(float),
+                           (size_t)n, cudaMemcpyHostToDevice, s),
+         "upload of the features");
+  }
   if (!ok()) return rc;
 
   // ---- input checks (each needs what the one before it established)
@@ -1433,13 +1443,6 @@ int Builder::run() {
   read(n_owned.data(), owned_cnt, ms);
   read(P->part.data(), part, (size_t)n);
   if (!ok()) return rc;
-
-  // ---- features: uploaded dense, gathered per partition on the device
-  x = scratch<float>((size_t)n * (size_t)g->f);
-  if (!ok()) return rc;
-  cuda(cudaMemcpy2DAsync(x, (size_t)g->f * sizeof(float), g->x, (size_t)g->ldx * sizeof(float), (size_t)g->f * sizeof(float),
-                         (size_t)n, cudaMemcpyHostToDevice, s),
-       "upload of the features");
 
   for (int32_t p = 0; p < m && ok(); ++p) build_partition(p, (int64_t)n_owned[p]);
   if (ok()) cuda(cudaStreamSynchronize(s), "cudaStreamSynchronize");

@@ -207,6 +207,55 @@ splitk_reduce(int64_t M, int64_t N, int64_t n_pad, int splits, const float* __re
   *dst = accumulate ? *dst + t : t;
 }
 
+// The same sums in the same order, four columns a thread: rows of C and of the partial tiles that start on 16 bytes.
+// Four times fewer blocks, four slices in flight per thread (in the epochs of the GraphSAGE workers of a 116 K-vertex
+// graph 15.5 -> 8.3 us, in those of 20 000 vertices 9.5 -> 5.3, other branches running beside it).
+__global__ void __launch_bounds__(256)
+splitk_reduce_v4(int64_t total4, int64_t N, int n_pad4, int splits, const float4* __restrict__ partial, int64_t ldp4,
+                 int64_t slice4, float* __restrict__ c, int64_t ldc, int accumulate, int epi, const float* __restrict__ aux,
+                 int64_t ldaux) {
+  __shared__ float4 sh[8][32];
+  const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
+  const int64_t idx = (int64_t)blockIdx.x * 32 + lane;
+  const bool live = idx < total4;
+  const int64_t i = live ? idx / n_pad4 : 0;
+  const int q = live ? (int)(idx - i * n_pad4) : 0;
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (live) {
+    const float4* src = partial + i * ldp4 + q;
+#pragma unroll 4
+    for (int z = grp; z < splits; z += 8) {
+      const float4 t = __ldg(src + z * slice4);
+      s.x += t.x; s.y += t.y; s.z += t.z; s.w += t.w;
+    }
+  }
+  sh[grp][lane] = s;
+  __syncthreads();
+  if (grp != 0 || !live) return;
+  float4 t = sh[0][lane];
+#pragma unroll
+  for (int k = 1; k < 8; ++k) {
+    const float4 u = sh[k][lane];
+    t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
+  }
+  const int64_t j = 4 * q;
+  float* dst = c + i * ldc + j;
+  float r[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    if (j + e < N) {
+      r[e] = apply_epi(r[e], epi, aux, ldaux, i, j + e);
+    } else {
+      r[e] = 0.f;  // pad column
+    }
+  }
+  if (accumulate) {
+    const float4 o = *reinterpret_cast<const float4*>(dst);
+    r[0] += o.x; r[1] += o.y; r[2] += o.z; r[3] += o.w;
+  }
+  *reinterpret_cast<float4*>(dst) = make_float4(r[0], r[1], r[2], r[3]);
+}
+
 struct Plan {
   int bm, bn, splits;
   int64_t k_per_split;
@@ -271,6 +320,13 @@ int launch_splitk_reduce(void* stream, int64_t m, int64_t n, int splits, const f
                          int accumulate, int epi, const float* aux, int64_t ldaux) {
   const int64_t n_pad = std::min<int64_t>(ldc, (n + 3) / 4 * 4);
   const int64_t total = m * n_pad;
+  if (n_pad % 4 == 0 && ldp % 4 == 0 && ldc % 4 == 0 && (((uintptr_t)partial | (uintptr_t)c) & 15) == 0) {
+    splitk_reduce_v4<<<(unsigned)((total / 4 + 31) / 32), 256, 0, (cudaStream_t)stream>>>(
+        total / 4, n, (int)(n_pad / 4), splits, reinterpret_cast<const float4*>(partial), ldp / 4, m * ldp / 4, c, ldc, accumulate,
+        epi, aux, ldaux);
+    note_launch();
+    return (int)cudaGetLastError();
+  }
   splitk_reduce<<<(unsigned)((total + 31) / 32), 256, 0, (cudaStream_t)stream>>>(m, n, n_pad, splits, partial, ldp, c, ldc,
                                                                                   accumulate, epi, aux, ldaux);
   note_launch();

@@ -10,6 +10,7 @@
 #include <algorithm>
 
 #include "internal.h"
+#include "launch.h"
 
 namespace gcnsa {
 
@@ -51,6 +52,7 @@ __global__ void __launch_bounds__(kThreads)
 gemm_tile(int64_t M, int64_t N, int64_t K, int64_t k_per_split, const float* __restrict__ a, int64_t lda,
           const float* __restrict__ b, int64_t ldb, float* __restrict__ c, int64_t ldc, int accumulate, int epi,
           const float* __restrict__ aux, int64_t ldaux, float* __restrict__ partial) {
+  wait_for_predecessors();
   constexpr int TM = BM / 16, TN = BN / 16;
   constexpr int A_F4 = BM * BK / 4 / kThreads, B_F4 = BN * BK / 4 / kThreads;
   __shared__ __align__(16) float As[2][BK][BM + 4];
@@ -184,6 +186,7 @@ __global__ void __launch_bounds__(256)
 splitk_reduce(int64_t M, int64_t N, int64_t n_pad, int splits, const float* __restrict__ partial, int64_t ldp,
               float* __restrict__ c,
               int64_t ldc, int accumulate, int epi, const float* __restrict__ aux, int64_t ldaux) {
+  wait_for_predecessors();
   __shared__ float sh[8][32];
   const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
   const int64_t idx = (int64_t)blockIdx.x * 32 + lane;
@@ -214,6 +217,7 @@ __global__ void __launch_bounds__(256)
 splitk_reduce_v4(int64_t total4, int64_t N, int n_pad4, int splits, const float4* __restrict__ partial, int64_t ldp4,
                  int64_t slice4, float* __restrict__ c, int64_t ldc, int accumulate, int epi, const float* __restrict__ aux,
                  int64_t ldaux) {
+  wait_for_predecessors();
   __shared__ float4 sh[8][32];
   const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
   const int64_t idx = (int64_t)blockIdx.x * 32 + lane;
@@ -288,7 +292,7 @@ cudaError_t dispatch(cudaStream_t s, const Plan& p, bool ta, bool tb, bool vec, 
                      int epi, const float* aux, int64_t ldaux, float* partial) {
   dim3 grid((unsigned)((n + BN - 1) / BN), (unsigned)((m + BM - 1) / BM), (unsigned)p.splits);
 #define GCNSA_GEMM(TA, TB, V)                                                                                       \
-  gemm_tile<BM, BN, TA, TB, V><<<grid, kThreads, 0, s>>>(m, n, k, p.k_per_split, a, lda, b, ldb, c, ldc, accumulate, \
+  launch(gemm_tile<BM, BN, TA, TB, V>, grid, kThreads, 0, s, m, n, k, p.k_per_split, a, lda, b, ldb, c, ldc, accumulate, \
                                                          epi, aux, ldaux, partial)
   if (vec) {
     if (!ta && !tb) GCNSA_GEMM(false, false, true);
@@ -321,13 +325,13 @@ int launch_splitk_reduce(void* stream, int64_t m, int64_t n, int splits, const f
   const int64_t n_pad = std::min<int64_t>(ldc, (n + 3) / 4 * 4);
   const int64_t total = m * n_pad;
   if (n_pad % 4 == 0 && ldp % 4 == 0 && ldc % 4 == 0 && (((uintptr_t)partial | (uintptr_t)c) & 15) == 0) {
-    splitk_reduce_v4<<<(unsigned)((total / 4 + 31) / 32), 256, 0, (cudaStream_t)stream>>>(
+    launch(splitk_reduce_v4, (unsigned)((total / 4 + 31) / 32), 256, 0, (cudaStream_t)stream,
         total / 4, n, (int)(n_pad / 4), splits, reinterpret_cast<const float4*>(partial), ldp / 4, m * ldp / 4, c, ldc, accumulate,
         epi, aux, ldaux);
     note_launch();
     return (int)cudaGetLastError();
   }
-  splitk_reduce<<<(unsigned)((total + 31) / 32), 256, 0, (cudaStream_t)stream>>>(m, n, n_pad, splits, partial, ldp, c, ldc,
+  launch(splitk_reduce, (unsigned)((total + 31) / 32), 256, 0, (cudaStream_t)stream, m, n, n_pad, splits, partial, ldp, c, ldc,
                                                                                   accumulate, epi, aux, ldaux);
   note_launch();
   return (int)cudaGetLastError();

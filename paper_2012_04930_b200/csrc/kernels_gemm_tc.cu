@@ -34,6 +34,7 @@
 #include <mutex>
 
 #include "internal.h"
+#include "launch.h"
 #include "tc_device.h"
 
 namespace gcnsa {
@@ -209,7 +210,10 @@ gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   // a wait ran out in an earlier launch or in another CTA of this one: nothing is allocated, nothing is computed
   if (threadIdx.x == 0) *abort_slot = tc_error_now();
   __syncthreads();
-  if (*abort_slot != 0) return;
+  if (*abort_slot != 0) {
+    wait_for_predecessors();
+    return;
+  }
   if (threadIdx.x == 0) {
     for (int i = 0; i < NA; ++i) {
       mbar_init(&full_a[i], 1);
@@ -237,6 +241,7 @@ gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_base = *tmem_slot;
+  wait_for_predecessors();  // barriers and tensor memory are up; from here on global memory is read
 
   if (warp == 0 || warp == 2) {
     // ---------------- TMA producers: warp 0 streams A, warp 2 streams B ----------------
@@ -665,7 +670,7 @@ cudaError_t run_tc_shape(cudaStream_t s, const TcPlan& p, const CUtensorMap& ma,
                          int epi, const float* aux, int64_t ldaux, int64_t slice_stride, int vec_ok, int terms, float* colsum_partial, const float* post_scale) {
   cudaError_t e0 = cudaFuncSetAttribute(gemm_tf32x3<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_BYTES);
   if (e0 != cudaSuccess) return e0;
-  gemm_tf32x3<S><<<grid, kThreads, S::SMEM_BYTES, s>>>(ma, mb, m, n, p.k_blocks, p.kb_per_split, tiles_m, tiles_n, total,
+  launch(gemm_tf32x3<S>, grid, kThreads, S::SMEM_BYTES, s, ma, mb, m, n, p.k_blocks, p.kb_per_split, tiles_m, tiles_n, total,
                                                        c, ldc, accumulate, epi, aux, ldaux, slice_stride, vec_ok, terms, colsum_partial, post_scale);
   note_launch();
   return cudaGetLastError();

@@ -10,6 +10,7 @@
 #include <mutex>
 
 #include "internal.h"
+#include "launch.h"
 
 namespace gcnsa {
 
@@ -36,6 +37,7 @@ __global__ void __launch_bounds__(kCeWarps * 32)
 softmax_ce_rows(int64_t n, int c, const float* __restrict__ logits, int64_t ld, const int32_t* __restrict__ y,
                 const uint8_t* __restrict__ mask, float inv_nt, float* __restrict__ grad, int64_t ldg,
                 float* __restrict__ partial) {
+  wait_for_predecessors();
   __shared__ float sh[kCeWarps];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int ldg_cols = (int)min(ldg, (int64_t)((c + 3) / 4 * 4));
@@ -96,6 +98,7 @@ softmax_ce_rows(int64_t n, int c, const float* __restrict__ logits, int64_t ld, 
 }
 
 __global__ void loss_finalize(const float* __restrict__ partial, int count, float inv_nt, float* __restrict__ out) {
+  wait_for_predecessors();
   __shared__ float sh[256];
   float s = 0.f;
   for (int i = threadIdx.x; i < count; i += 256) s += partial[i];
@@ -109,6 +112,7 @@ __global__ void loss_finalize(const float* __restrict__ partial, int count, floa
 }
 
 __global__ void mean_kernel(const float* __restrict__ src, int count, float* __restrict__ dst) {
+  wait_for_predecessors();
   if (threadIdx.x == 0 && blockIdx.x == 0) {
     float s = 0.f;
     for (int i = 0; i < count; ++i) s += src[i];
@@ -120,6 +124,7 @@ __global__ void mean_kernel(const float* __restrict__ src, int count, float* __r
 __global__ void __launch_bounds__(256)
 colsum_partial(int64_t n, int f, const float* __restrict__ g, int64_t ldg, int64_t rows_per_block,
                float* __restrict__ partial) {
+  wait_for_predecessors();
   __shared__ float sh[8][33];
   const int64_t r0 = (int64_t)blockIdx.x * rows_per_block, r1 = min(n, r0 + rows_per_block);
   for (int j0 = 0; j0 < f; j0 += 32) {
@@ -147,6 +152,7 @@ template <int NV>
 __global__ void __launch_bounds__(256)
 colsum_partial_v4(int64_t n, int f, const float* g, int64_t ldg, int64_t rows_per_block, float* __restrict__ partial,
                   const float* __restrict__ rscale, float* scaled, int64_t lds) {
+  wait_for_predecessors();
   constexpr int RY = 256 / NV;
   __shared__ float4 sh[256];
   const int tx = threadIdx.x % NV, ty = threadIdx.x / NV;
@@ -189,6 +195,7 @@ colsum_partial_v4(int64_t n, int f, const float* g, int64_t ldg, int64_t rows_pe
 // block's partial in ascending order and the 8 sums are added in group order: fixed order.
 __global__ void __launch_bounds__(256)
 colsum_final(int f, int blocks, const float* __restrict__ partial, int64_t ldp, float* __restrict__ out, int accumulate) {
+  wait_for_predecessors();
   __shared__ float sh[8][32];
   const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
   const int j = blockIdx.x * 32 + lane;
@@ -207,6 +214,7 @@ colsum_final(int f, int blocks, const float* __restrict__ partial, int64_t ldp, 
 // Step counter and bias corrections kept on the device, so that a captured epoch can be replayed: state[0] = t
 // (as a float-exact integer in a double), state[1] = 1 / (1 - beta1^t), state[2] = 1 / (1 - beta2^t).
 __global__ void adam_advance(double* __restrict__ state, double b1, double b2) {
+  wait_for_predecessors();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   const double t = state[0] + 1.0;
   state[0] = t;
@@ -228,6 +236,7 @@ __device__ __forceinline__ float adam_delta(float g, float* __restrict__ m, floa
 __global__ void adam_kernel_dev(int64_t count, float* __restrict__ theta, float* __restrict__ gsum, float* __restrict__ m,
                                 float* __restrict__ v, float inv_m, float lr, float b1, float b2, float eps,
                                 const double* __restrict__ state) {
+  wait_for_predecessors();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const float c1 = (float)state[1], c2 = (float)state[2];
@@ -240,6 +249,7 @@ __global__ void adam_local_kernel_dev(int64_t count, const float* __restrict__ t
                                       float* __restrict__ m, float* __restrict__ v, float* __restrict__ acc, int first,
                                       float inv_m, float lr, float b1, float b2, float eps,
                                       const double* __restrict__ state) {
+  wait_for_predecessors();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const float c1 = (float)state[1], c2 = (float)state[2];
@@ -254,6 +264,7 @@ __global__ void adam_local_kernel_dev(int64_t count, const float* __restrict__ t
 __global__ void adam_parts_kernel(int64_t count, int n_parts, float* __restrict__ theta, const float* __restrict__ parts,
                                   float* __restrict__ m, float* __restrict__ v, float inv_m, float lr, float b1, float b2,
                                   float eps, const double* __restrict__ state) {
+  wait_for_predecessors();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const float c1 = (float)state[1], c2 = (float)state[2];
@@ -269,6 +280,7 @@ __global__ void adam_local_parts_kernel(int64_t count, int n_parts, float* __res
                                         const float* __restrict__ parts, float* __restrict__ m, float* __restrict__ v,
                                         float inv_m, float lr, float b1, float b2, float eps,
                                         const double* __restrict__ state) {
+  wait_for_predecessors();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const float c1 = (float)state[1], c2 = (float)state[2];
@@ -286,6 +298,7 @@ __global__ void adam_local_parts_kernel(int64_t count, int n_parts, float* __res
 __global__ void adam_kernel(int64_t count, float* __restrict__ theta, float* __restrict__ gsum, float* __restrict__ m,
                             float* __restrict__ v, float inv_m, float lr, float b1, float b2, float eps, float c1,
                             float c2) {
+  wait_for_predecessors();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const float g = gsum[i] * inv_m;
@@ -298,6 +311,7 @@ __global__ void adam_kernel(int64_t count, float* __restrict__ theta, float* __r
 __global__ void __launch_bounds__(kCeWarps * 32)
 argmax_hits_rows(int64_t n, int c, const float* __restrict__ logits, int64_t ld, const int32_t* __restrict__ y,
                  const uint8_t* __restrict__ mask, int32_t* __restrict__ pred, int32_t* __restrict__ hits) {
+  wait_for_predecessors();
   __shared__ int sh[kCeWarps];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   int count = 0;
@@ -332,6 +346,7 @@ argmax_hits_rows(int64_t n, int c, const float* __restrict__ logits, int64_t ld,
 __global__ void __launch_bounds__(256)
 normalize_rows(int64_t n_rows, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
                const int32_t* __restrict__ deg, float* __restrict__ val) {
+  wait_for_predecessors();
   const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   if (row >= n_rows) return;
   const int lane = threadIdx.x & 31;
@@ -352,11 +367,11 @@ int launch_softmax_ce(void* stream, int64_t n, int32_t c, const float* logits, i
   const int blocks = ce_blocks(n);
   const float inv_nt = n_train > 0 ? 1.0f / (float)n_train : 0.f;
   if (n > 0) {
-    softmax_ce_rows<<<blocks, kCeWarps * 32, 0, s>>>(n, c, logits, ld, y, mask, inv_nt, grad, ldg, (float*)scratch);
+    launch(softmax_ce_rows, blocks, kCeWarps * 32, 0, s, n, c, logits, ld, y, mask, inv_nt, grad, ldg, (float*)scratch);
     note_launch();
   }
   if (loss_dev) {
-    loss_finalize<<<1, 256, 0, s>>>((const float*)scratch, n > 0 ? blocks : 0, inv_nt, loss_dev);
+    launch(loss_finalize, 1, 256, 0, s, (const float*)scratch, n > 0 ? blocks : 0, inv_nt, loss_dev);
     note_launch();
   }
   return (int)cudaGetLastError();
@@ -379,17 +394,17 @@ int launch_colsum_scaled(void* stream, int64_t n, int32_t f, const float* g, int
   const bool side_ok = !side || ((((uintptr_t)scaled & 15) == 0) && (lds % 4 == 0));
   if ((((uintptr_t)g & 15) == 0) && (ldg % 4 == 0) && side_ok) {
     float* p = (float*)scratch;
-    if (nvec <= 8) colsum_partial_v4<8><<<blocks, 256, 0, s>>>(n, f, g, ldg, rpb, p, rscale, scaled, lds);
-    else if (nvec <= 16) colsum_partial_v4<16><<<blocks, 256, 0, s>>>(n, f, g, ldg, rpb, p, rscale, scaled, lds);
-    else if (nvec <= 32) colsum_partial_v4<32><<<blocks, 256, 0, s>>>(n, f, g, ldg, rpb, p, rscale, scaled, lds);
-    else colsum_partial_v4<64><<<blocks, 256, 0, s>>>(n, f, g, ldg, rpb, p, rscale, scaled, lds);
+    if (nvec <= 8) launch(colsum_partial_v4<8>, blocks, 256, 0, s, n, f, g, ldg, rpb, p, rscale, scaled, lds);
+    else if (nvec <= 16) launch(colsum_partial_v4<16>, blocks, 256, 0, s, n, f, g, ldg, rpb, p, rscale, scaled, lds);
+    else if (nvec <= 32) launch(colsum_partial_v4<32>, blocks, 256, 0, s, n, f, g, ldg, rpb, p, rscale, scaled, lds);
+    else launch(colsum_partial_v4<64>, blocks, 256, 0, s, n, f, g, ldg, rpb, p, rscale, scaled, lds);
   } else {
     // rows the vector kernel cannot take (unaligned base or pitch); the scaled side output exists in whole
     // float4 chunks only, so it cannot be produced for them
     if (side) return (int)cudaErrorMisalignedAddress;
-    colsum_partial<<<blocks, dim3(32, 8), 0, s>>>(n, f, g, ldg, rpb, (float*)scratch);
+    launch(colsum_partial, blocks, dim3(32, 8), 0, s, n, f, g, ldg, rpb, (float*)scratch);
   }
-  colsum_final<<<(f + 31) / 32, 256, 0, s>>>(f, blocks, (const float*)scratch, f, out, accumulate);
+  launch(colsum_final, (f + 31) / 32, 256, 0, s, f, blocks, (const float*)scratch, f, out, accumulate);
   note_launch(2);
   return (int)cudaGetLastError();
 }
@@ -399,14 +414,14 @@ int launch_adam(void* stream, int64_t count, float* theta, float* gsum, float* m
   if (count == 0) return 0;
   const double c1 = 1.0 / (1.0 - std::pow((double)beta1, (double)t));
   const double c2 = 1.0 / (1.0 - std::pow((double)beta2, (double)t));
-  adam_kernel<<<(unsigned)((count + 255) / 256), 256, 0, (cudaStream_t)stream>>>(count, theta, gsum, m, v, inv_m, lr,
+  launch(adam_kernel, (unsigned)((count + 255) / 256), 256, 0, (cudaStream_t)stream, count, theta, gsum, m, v, inv_m, lr,
                                                                                 beta1, beta2, eps, (float)c1, (float)c2);
   note_launch();
   return (int)cudaGetLastError();
 }
 
 int launch_adam_advance(void* stream, double* state, float beta1, float beta2) {
-  adam_advance<<<1, 32, 0, (cudaStream_t)stream>>>(state, (double)beta1, (double)beta2);
+  launch(adam_advance, 1, 32, 0, (cudaStream_t)stream, state, (double)beta1, (double)beta2);
   note_launch();
   return (int)cudaGetLastError();
 }
@@ -414,7 +429,7 @@ int launch_adam_advance(void* stream, double* state, float beta1, float beta2) {
 int launch_adam_dev(void* stream, int64_t count, float* theta, float* gsum, float* m, float* v, float inv_m, float lr,
                     float beta1, float beta2, float eps, const double* state) {
   if (count == 0) return 0;
-  adam_kernel_dev<<<(unsigned)((count + 255) / 256), 256, 0, (cudaStream_t)stream>>>(count, theta, gsum, m, v, inv_m, lr,
+  launch(adam_kernel_dev, (unsigned)((count + 255) / 256), 256, 0, (cudaStream_t)stream, count, theta, gsum, m, v, inv_m, lr,
                                                                                     beta1, beta2, eps, state);
   note_launch();
   return (int)cudaGetLastError();
@@ -423,7 +438,7 @@ int launch_adam_dev(void* stream, int64_t count, float* theta, float* gsum, floa
 int launch_adam_local_dev(void* stream, int64_t count, const float* theta, float* gsum, float* m, float* v, float* acc,
                           int first, float inv_m, float lr, float beta1, float beta2, float eps, const double* state) {
   if (count == 0) return 0;
-  adam_local_kernel_dev<<<(unsigned)((count + 255) / 256), 256, 0, (cudaStream_t)stream>>>(
+  launch(adam_local_kernel_dev, (unsigned)((count + 255) / 256), 256, 0, (cudaStream_t)stream,
       count, theta, gsum, m, v, acc, first, inv_m, lr, beta1, beta2, eps, state);
   note_launch();
   return (int)cudaGetLastError();
@@ -432,7 +447,7 @@ int launch_adam_local_dev(void* stream, int64_t count, const float* theta, float
 int launch_adam_parts(void* stream, int64_t count, int n_parts, float* theta, const float* parts, float* m, float* v,
                       float inv_m, float lr, float beta1, float beta2, float eps, const double* state) {
   if (count == 0) return 0;
-  adam_parts_kernel<<<(unsigned)((count + 255) / 256), 256, 0, (cudaStream_t)stream>>>(count, n_parts, theta, parts, m, v,
+  launch(adam_parts_kernel, (unsigned)((count + 255) / 256), 256, 0, (cudaStream_t)stream, count, n_parts, theta, parts, m, v,
                                                                                       inv_m, lr, beta1, beta2, eps, state);
   note_launch();
   return (int)cudaGetLastError();
@@ -441,7 +456,7 @@ int launch_adam_parts(void* stream, int64_t count, int n_parts, float* theta, co
 int launch_adam_local_parts(void* stream, int64_t count, int n_parts, float* theta, const float* parts, float* m, float* v,
                             float inv_m, float lr, float beta1, float beta2, float eps, const double* state) {
   if (count == 0) return 0;
-  adam_local_parts_kernel<<<(unsigned)((count + 255) / 256), 256, 0, (cudaStream_t)stream>>>(
+  launch(adam_local_parts_kernel, (unsigned)((count + 255) / 256), 256, 0, (cudaStream_t)stream,
       count, n_parts, theta, parts, m, v, inv_m, lr, beta1, beta2, eps, state);
   note_launch();
   return (int)cudaGetLastError();
@@ -452,7 +467,7 @@ int launch_argmax_hits(void* stream, int64_t n, int32_t c, const float* logits, 
   const int blocks = ce_blocks(n);
   *n_blocks_out = blocks;
   if (n == 0) return 0;
-  argmax_hits_rows<<<blocks, kCeWarps * 32, 0, (cudaStream_t)stream>>>(n, c, logits, ld, y, mask, pred, hits);
+  launch(argmax_hits_rows, blocks, kCeWarps * 32, 0, (cudaStream_t)stream, n, c, logits, ld, y, mask, pred, hits);
   note_launch();
   return (int)cudaGetLastError();
 }
@@ -460,19 +475,20 @@ int launch_argmax_hits(void* stream, int64_t n, int32_t c, const float* logits, 
 int launch_normalize(void* stream, int64_t n_rows, const int32_t* rowptr, const int32_t* col, const int32_t* deg,
                      float* val) {
   if (n_rows == 0) return 0;
-  normalize_rows<<<(unsigned)((n_rows + 7) / 8), 256, 0, (cudaStream_t)stream>>>(n_rows, rowptr, col, deg, val);
+  launch(normalize_rows, (unsigned)((n_rows + 7) / 8), 256, 0, (cudaStream_t)stream, n_rows, rowptr, col, deg, val);
   note_launch();
   return (int)cudaGetLastError();
 }
 
 // dinv[i] = 1 / sqrt(deg[i]): the diagonal of D^-1/2 (degrees of A + I, so deg >= 1)
 __global__ void inv_sqrt_degree(int64_t n, const int32_t* __restrict__ deg, float* __restrict__ dinv) {
+  wait_for_predecessors();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) dinv[i] = 1.0f / sqrtf((float)deg[i]);
 }
 int launch_inv_sqrt_degree(void* stream, int64_t n, const int32_t* deg, float* dinv) {
   if (n == 0) return 0;
-  inv_sqrt_degree<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(n, deg, dinv);
+  launch(inv_sqrt_degree, (unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream, n, deg, dinv);
   note_launch();
   return (int)cudaGetLastError();
 }
@@ -480,6 +496,7 @@ int launch_inv_sqrt_degree(void* stream, int64_t n, const int32_t* deg, float* d
 // dst[i, :] = scale[i] * src[i, :] over nvec float4 per row (dst may be src)
 __global__ void scale_rows(int64_t n, int nvec, const float* __restrict__ scale, const float4* src, int64_t lds4,
                            float4* dst, int64_t ldd4) {
+  wait_for_predecessors();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= n * nvec) return;
   const int64_t i = idx / nvec;
@@ -494,13 +511,14 @@ int launch_scale_rows(void* stream, int64_t n, int32_t f, const float* scale, co
   if (n == 0 || f == 0) return 0;
   const int nvec = (f + 3) / 4;
   const int64_t total = n * nvec;
-  scale_rows<<<(unsigned)((total + 255) / 256), 256, 0, (cudaStream_t)stream>>>(
+  launch(scale_rows, (unsigned)((total + 255) / 256), 256, 0, (cudaStream_t)stream,
       n, nvec, scale, reinterpret_cast<const float4*>(src), lds / 4, reinterpret_cast<float4*>(dst), ldd / 4);
   note_launch();
   return (int)cudaGetLastError();
 }
 
 __global__ void repitch_rows(int64_t n, int f, const float* __restrict__ src, float* __restrict__ dst, int64_t ld) {
+  wait_for_predecessors();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= n * f) return;
   const int64_t i = idx / f, j = idx - i * f;
@@ -510,13 +528,13 @@ __global__ void repitch_rows(int64_t n, int f, const float* __restrict__ src, fl
 int launch_repitch(void* stream, int64_t n, int32_t f, const float* src, float* dst, int64_t ld) {
   if (n == 0 || f == 0) return 0;
   const int64_t total = n * f;
-  repitch_rows<<<(unsigned)((total + 255) / 256), 256, 0, (cudaStream_t)stream>>>(n, f, src, dst, ld);
+  launch(repitch_rows, (unsigned)((total + 255) / 256), 256, 0, (cudaStream_t)stream, n, f, src, dst, ld);
   note_launch();
   return (int)cudaGetLastError();
 }
 
 int launch_mean(void* stream, const float* src, int count, float* dst) {
-  mean_kernel<<<1, 32, 0, (cudaStream_t)stream>>>(src, count, dst);
+  launch(mean_kernel, 1, 32, 0, (cudaStream_t)stream, src, count, dst);
   note_launch();
   return (int)cudaGetLastError();
 }

@@ -19,6 +19,7 @@
 
 #include "debug_check.h"
 #include "internal.h"
+#include "launch.h"
 
 namespace gcnsa {
 
@@ -329,6 +330,7 @@ spmm_rows(int n_long, int n_warp, int n_rows, const int32_t* __restrict__ rowptr
           const float4* __restrict__ x, int64_t ldx4,
           int nvec, int f, int vec_idx, int epi, const float* __restrict__ aux, int64_t ldaux, float* __restrict__ y,
           int64_t ldy GCNSA_DBG_PARAM) {
+  wait_for_predecessors();
   constexpr int NG = 32 / G;
   constexpr int W = TPB / 32;
   __shared__ float4 part[W][G * CH];
@@ -441,11 +443,11 @@ cudaError_t run(const Args& a) {
   const int grid = a.n_long + (a.n_warp - a.n_long + rows_per_block - 1) / rows_per_block +
                    (a.n_rows - a.n_warp + short_per_block - 1) / short_per_block;
   if (a.val)
-    spmm_rows<G, CH, U, TPB, MINB, false, SG, SCH, SU><<<grid, TPB, 0, a.s>>>(
+    launch(spmm_rows<G, CH, U, TPB, MINB, false, SG, SCH, SU>, grid, TPB, 0, a.s,
         a.n_long, a.n_warp, a.n_rows, a.rowptr, a.col, a.val, a.rscale, a.order, reinterpret_cast<const float4*>(a.x), a.ldx / 4,
         a.nvec, a.f, a.vec_idx, a.epi, a.aux, a.ldaux, a.y, a.ldy GCNSA_DBG_LAUNCH_ARG);
   else
-    spmm_rows<G, CH, U, TPB, MINB, true, SG, SCH, SU><<<grid, TPB, 0, a.s>>>(
+    launch(spmm_rows<G, CH, U, TPB, MINB, true, SG, SCH, SU>, grid, TPB, 0, a.s,
         a.n_long, a.n_warp, a.n_rows, a.rowptr, a.col, nullptr, a.rscale, a.order, reinterpret_cast<const float4*>(a.x), a.ldx / 4,
         a.nvec, a.f, a.vec_idx, a.epi, a.aux, a.ldaux, a.y, a.ldy GCNSA_DBG_LAUNCH_ARG);
   note_launch();
@@ -523,6 +525,7 @@ spmm_rest(int n_long, int n_rows, const int32_t* __restrict__ rowptr, const int3
           const int32_t* __restrict__ col, const float* __restrict__ sscale, const float* __restrict__ rscale,
           const int32_t* __restrict__ order, const float4* __restrict__ x, int64_t ldx4, int nvec, int f, int epi,
           const float* __restrict__ aux, int64_t ldaux, float* __restrict__ y, int64_t ldy, const SpmmBase base GCNSA_DBG_PARAM) {
+  wait_for_predecessors();
   constexpr int W = 8;
   __shared__ float4 part[W][G * CH];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane / G, gl = lane % G;
@@ -588,11 +591,11 @@ template <int G, int CH, int RU>
 cudaError_t run_rest(const RestArgs& a, const float* x, int nvec, int f, const float* aux, float* y, const SpmmBase& base) {
   const int grid = a.n_long + (a.n_rows - a.n_long + 7) / 8;
   if (a.sscale)
-    spmm_rest<G, CH, RU, true><<<grid, 256, 0, a.s>>>(a.n_long, a.n_rows, a.rowptr, a.rowend, a.col, a.sscale, a.rscale, a.order,
+    launch(spmm_rest<G, CH, RU, true>, grid, 256, 0, a.s, a.n_long, a.n_rows, a.rowptr, a.rowend, a.col, a.sscale, a.rscale, a.order,
                                                       reinterpret_cast<const float4*>(x), a.ldx / 4, nvec, f, a.epi, aux, a.ldaux,
                                                       y, a.ldy, base GCNSA_DBG_LAUNCH_ARG);
   else
-    spmm_rest<G, CH, RU, false><<<grid, 256, 0, a.s>>>(a.n_long, a.n_rows, a.rowptr, a.rowend, a.col, nullptr, a.rscale, a.order,
+    launch(spmm_rest<G, CH, RU, false>, grid, 256, 0, a.s, a.n_long, a.n_rows, a.rowptr, a.rowend, a.col, nullptr, a.rscale, a.order,
                                                        reinterpret_cast<const float4*>(x), a.ldx / 4, nvec, f, a.epi, aux,
                                                        a.ldaux, y, a.ldy, base GCNSA_DBG_LAUNCH_ARG);
   note_launch();

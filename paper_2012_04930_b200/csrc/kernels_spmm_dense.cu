@@ -30,6 +30,7 @@
 #include <mutex>
 
 #include "internal.h"
+#include "launch.h"
 #include "tc_device.h"
 
 namespace gcnsa {
@@ -187,7 +188,10 @@ __global__ void __launch_bounds__(kThreads, 1) spmm_dense(const Params p) {
 
   if (threadIdx.x == 0) *abort_slot = tc_error_now();
   __syncthreads();
-  if (*abort_slot != 0) return;
+  if (*abort_slot != 0) {
+    wait_for_predecessors();
+    return;
+  }
   if (threadIdx.x == 0) {
     for (int i = 0; i < kStagesA; ++i) mbar_init(&full_a[i], kRowWarps);
     for (int i = 0; i < kStagesB; ++i) {
@@ -208,6 +212,7 @@ __global__ void __launch_bounds__(kThreads, 1) spmm_dense(const Params p) {
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_base = *tmem_slot;
+  wait_for_predecessors();  // barriers and tensor memory are up; from here on global memory is read
 
   Walk walk;
   walk.start(p);
@@ -410,6 +415,7 @@ __device__ __forceinline__ float lower_part(float x) { return x - __uint_as_floa
 __global__ void __launch_bounds__(256)
 split_rows(int64_t n, const float4* __restrict__ x, int64_t ldx4, int nvec, const float* __restrict__ xscale, int groups,
            int groups_per_slab, int step, int lines, uint4* __restrict__ out) {
+  wait_for_predecessors();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (n + 1) * groups) return;
   const int64_t row = i / groups;
@@ -470,7 +476,7 @@ template <int N>
 cudaError_t run(cudaStream_t s, int grid, const Params& p) {
   cudaError_t e = cudaFuncSetAttribute(spmm_dense<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, Lines<N>::SMEM);
   if (e != cudaSuccess) return e;
-  spmm_dense<N><<<grid, kThreads, Lines<N>::SMEM, s>>>(p);
+  launch(spmm_dense<N>, grid, kThreads, Lines<N>::SMEM, s, p);
   note_launch();
   return cudaGetLastError();
 }
@@ -505,7 +511,7 @@ int launch_spmm_planned(void* stream, const DensePlan& d, DenseUse use, int64_t 
     uint8_t* split = (uint8_t*)workspace + pieces_bytes(d, sl);
     const int gps = sl.width / 8, groups = gps * sl.n;
     const int64_t threads = (d.n_rows + 1) * groups;
-    split_rows<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(d.n_rows, reinterpret_cast<const float4*>(x), ldx / 4,
+    launch(split_rows, (unsigned)((threads + 255) / 256), 256, 0, s, d.n_rows, reinterpret_cast<const float4*>(x), ldx / 4,
                                                                  (f + 3) / 4, src_scale, groups, gps, sl.step, sl.lines,
                                                                  reinterpret_cast<uint4*>(split));
     note_launch();

@@ -28,6 +28,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "launch.h"
 #include "parts.h"
 
 namespace gcnsa {
@@ -60,6 +61,7 @@ inline unsigned blocks_for(int64_t items, int per_block) {
 // ---------------------------------------------------------------- batches ---
 // keys[i] = key(seed; 4, p, epoch, 0; list[i])
 __global__ void sage_keys(const int32_t* __restrict__ list, int64_t n, u64 prefix, u64* __restrict__ keys) {
+  wait_for_predecessors();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) keys[i] = mix64s(prefix ^ (u64)list[i]);
 }
@@ -67,6 +69,7 @@ __global__ void sage_keys(const int32_t* __restrict__ list, int64_t n, u64 prefi
 // permutation.  Brute force over tiles of keys in shared memory: n^2 comparisons, a millisecond at n = 10^5.
 __global__ void __launch_bounds__(256)
 sage_rank(const int32_t* __restrict__ list, const u64* __restrict__ keys, int64_t n, int32_t* __restrict__ order) {
+  wait_for_predecessors();
   __shared__ u64 tile[1024];
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const u64 mine = i < n ? keys[i] : 0ull;
@@ -99,6 +102,7 @@ __global__ void __launch_bounds__(kSampleWarps * 32)
 sage_sample(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col, const int32_t* __restrict__ vs,
             int64_t n_v, int r, u64 seed, u64 p, u64 epoch_layer, const int64_t* __restrict__ batch_state,
             int32_t* __restrict__ out, int32_t* __restrict__ cnt) {
+  wait_for_predecessors();
   // recorded batches: the epoch is read from the batch state, epoch_layer then carries the layer only
   if (batch_state) epoch_layer += (u64)batch_state[1] * 256;
   __shared__ u64 cand_key[kSampleWarps][kCand];
@@ -215,6 +219,7 @@ __global__ void __launch_bounds__(256)
 sage_concat_mean(const float* __restrict__ src, int64_t ld_src, int f, const int32_t* __restrict__ self_idx,
                  const int32_t* __restrict__ samp, const int32_t* __restrict__ cnt, int r, int64_t slot_base,
                  int64_t n_rows, float* __restrict__ out, int64_t ld) {
+  wait_for_predecessors();
   const int lvec = (int)(ld / 4), nvec = (f + 3) / 4;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= n_rows * lvec) return;
@@ -243,6 +248,7 @@ sage_concat_mean(const float* __restrict__ src, int64_t ld_src, int f, const int
 
 __global__ void sage_gather_labels(const int32_t* __restrict__ y, const int32_t* __restrict__ targets, int64_t nb,
                                    int32_t* __restrict__ yb) {
+  wait_for_predecessors();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < nb) yb[i] = y[targets[i]];
 }
@@ -252,6 +258,7 @@ __global__ void sage_gather_labels(const int32_t* __restrict__ y, const int32_t*
 // samples, of which each sample receives 1 / count.  ReLU'(z) = [h > 0].
 __global__ void sage_hidden_grad(const float* __restrict__ dcat, const float* __restrict__ h1, const int32_t* __restrict__ cnt2,
                                  int64_t nb, int r2, int64_t ldh, int64_t n_rows, float* __restrict__ dz1) {
+  wait_for_predecessors();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= n_rows * ldh) return;
   const int64_t j = idx / ldh, c = idx - j * ldh;
@@ -269,6 +276,7 @@ __global__ void sage_hidden_grad(const float* __restrict__ dcat, const float* __
 // out[0] += number of source rows the [self | mean] kernel reads for these rows: 1 + cnt per row that has a vertex
 __global__ void sage_count_reads(const int32_t* __restrict__ self_idx, const int32_t* __restrict__ cnt, int64_t n_rows,
                                  u64* out) {
+  wait_for_predecessors();
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int c = 0;
   if (j < n_rows && (!self_idx || self_idx[j] >= 0)) c = 1 + cnt[j];
@@ -281,11 +289,13 @@ __global__ void sage_count_reads(const int32_t* __restrict__ self_idx, const int
 // Batch state of the recorded batches: [0] = index of the batch in flight, [1] = epoch.  A replayed graph cannot
 // take new kernel arguments, so the batch's first kernel advances the index itself and copies the batch's targets.
 __global__ void sage_set_state(int64_t* state, int64_t b, int64_t epoch) {
+  wait_for_predecessors();
   state[0] = b;
   state[1] = epoch;
 }
 // one block: every thread reads the old index before thread 0 writes the new one
 __global__ void sage_begin_batch(int64_t* state, const int32_t* __restrict__ order, int batch, int32_t* __restrict__ targets) {
+  wait_for_predecessors();
   const int64_t b = state[0] + 1;
   __syncthreads();
   for (int i = threadIdx.x; i < batch; i += blockDim.x) targets[i] = order[b * batch + i];
@@ -293,10 +303,12 @@ __global__ void sage_begin_batch(int64_t* state, const int32_t* __restrict__ ord
 }
 
 __global__ void sage_loss_add(float* acc, const float* loss, float weight) {
+  wait_for_predecessors();
   if (threadIdx.x == 0 && blockIdx.x == 0) acc[0] += loss[0] * weight;
 }
 // dst[0] = part[0] * scale; part[0] = 0: a worker's epoch is over
 __global__ void sage_loss_fold(float* dst, float* part, float scale) {
+  wait_for_predecessors();
   if (threadIdx.x == 0 && blockIdx.x == 0) {
     dst[0] = part[0] * scale;
     part[0] = 0.f;
@@ -307,6 +319,7 @@ __global__ void sage_loss_fold(float* dst, float* part, float scale) {
 __global__ void sage_param_mean(int64_t count, int m, const float* copies, float* __restrict__ theta, float* work,
                                 float scale, const float* __restrict__ loss_parts,
                                 float* __restrict__ loss) {
+  wait_for_predecessors();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < count) {
     float acc = 0.f;
@@ -434,9 +447,9 @@ int ensure_order(gcnsa_sage* S, const gcnsa_parts* P, int32_t p, int64_t epoch, 
   const int64_t nt = d.info.n_train;
   if (nt > 0) {
     const u64 prefix = key_prefix(S->o.seed, kTagBatch, (u64)p, (u64)epoch, 0);
-    sage_keys<<<blocks_for(nt, 256), 256, 0, s>>>(d.m_order, nt, prefix, W.keys);
+    launch(sage_keys, blocks_for(nt, 256), 256, 0, s, d.m_order, nt, prefix, W.keys);
     SLAUNCHED("sage_keys");
-    sage_rank<<<blocks_for(nt, 256), 256, 0, s>>>(d.m_order, W.keys, nt, W.order);
+    launch(sage_rank, blocks_for(nt, 256), 256, 0, s, d.m_order, W.keys, nt, W.order);
     SLAUNCHED("sage_rank");
   }
   W.order_p = p; W.order_epoch = epoch; W.order_uid = P->uid;
@@ -467,35 +480,35 @@ int run_batch(gcnsa_sage* S, const gcnsa_parts* P, int32_t p, int64_t epoch, int
   const int64_t* state = recorded ? W.batch_state : nullptr;
   const u64 ep = recorded ? 0 : (u64)epoch * 256;
   if (recorded) {
-    sage_begin_batch<<<1, 256, 0, s>>>(W.batch_state, W.order, (int)B, W.b1);
+    launch(sage_begin_batch, 1, 256, 0, s, W.batch_state, W.order, (int)B, W.b1);
     SLAUNCHED("sage_begin_batch");
   } else {
     SCK(cudaMemcpyAsync(W.b1, targets, (size_t)nb * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
   }
   if (r2 > 0) {
-    sage_sample<<<blocks_for(nb * 32, kSampleWarps * 32), kSampleWarps * 32, 0, s>>>(d.rowptr, d.col, W.b1, nb, r2, S->o.seed, (u64)p,
+    launch(sage_sample, blocks_for(nb * 32, kSampleWarps * 32), kSampleWarps * 32, 0, s, d.rowptr, d.col, W.b1, nb, r2, S->o.seed, (u64)p,
                                                         ep + 2, state, W.b1 + nb, W.cnt2);
     SLAUNCHED("sage_sample");
   } else {
     SCK(cudaMemsetAsync(W.cnt2, 0, (size_t)nb * sizeof(int32_t), s));
   }
   if (r1 > 0) {
-    sage_sample<<<blocks_for(rows1 * 32, kSampleWarps * 32), kSampleWarps * 32, 0, s>>>(d.rowptr, d.col, W.b1, rows1, r1, S->o.seed, (u64)p,
+    launch(sage_sample, blocks_for(rows1 * 32, kSampleWarps * 32), kSampleWarps * 32, 0, s, d.rowptr, d.col, W.b1, rows1, r1, S->o.seed, (u64)p,
                                                            ep + 1, state, W.s1, W.cnt1);
     SLAUNCHED("sage_sample");
   } else {
     SCK(cudaMemsetAsync(W.cnt1, 0, (size_t)rows1 * sizeof(int32_t), s));
   }
   if (S->prof_on) {
-    sage_count_reads<<<blocks_for(rows1, 256), 256, 0, s>>>(W.b1, W.cnt1, rows1, S->read_rows);
+    launch(sage_count_reads, blocks_for(rows1, 256), 256, 0, s, W.b1, W.cnt1, rows1, S->read_rows);
     SLAUNCHED("sage_count_reads");
-    sage_count_reads<<<blocks_for(nb, 256), 256, 0, s>>>(nullptr, W.cnt2, nb, S->read_rows + 1);
+    launch(sage_count_reads, blocks_for(nb, 256), 256, 0, s, nullptr, W.cnt2, nb, S->read_rows + 1);
     SLAUNCHED("sage_count_reads");
   }
   S->prof_end(2, 0.0, 0.0);
   // ---- hidden layer: H1 = relu([x_v | mean x_u] [W_self ; W_neigh] + b)
   S->prof_begin();
-  sage_concat_mean<<<blocks_for(rows1 * (S->ldf / 4), 256), 256, 0, s>>>(d.x, P->ldx, (int)S->f, W.b1, W.s1, W.cnt1, r1, 0, rows1,
+  launch(sage_concat_mean, blocks_for(rows1 * (S->ldf / 4), 256), 256, 0, s, d.x, P->ldx, (int)S->f, W.b1, W.s1, W.cnt1, r1, 0, rows1,
                                                               W.cat1, S->ldf);
   SLAUNCHED("sage_concat_mean");
   S->prof_end(0, 8.0 * (double)rows1 * (double)S->ldf, 0.0);  // the rows written; the rows read are counted on the device
@@ -507,7 +520,7 @@ int run_batch(gcnsa_sage* S, const gcnsa_parts* P, int32_t p, int64_t epoch, int
   S->prof_end(1, 0.0, fl1);
   // ---- output layer: logits = [h_v | mean h_u] [W_self ; W_neigh] + b, the samples of vertex i in slots nb + i r2 + s
   S->prof_begin();
-  sage_concat_mean<<<blocks_for(nb * (S->ldh / 4), 256), 256, 0, s>>>(W.h1, S->ldh, (int)S->h, nullptr, nullptr, W.cnt2, r2, nb, nb,
+  launch(sage_concat_mean, blocks_for(nb * (S->ldh / 4), 256), 256, 0, s, W.h1, S->ldh, (int)S->h, nullptr, nullptr, W.cnt2, r2, nb, nb,
                                                            W.cat2, S->ldh);
   SLAUNCHED("sage_concat_mean");
   S->prof_end(0, 8.0 * (double)nb * (double)S->ldh, 0.0);
@@ -517,10 +530,10 @@ int run_batch(gcnsa_sage* S, const gcnsa_parts* P, int32_t p, int64_t epoch, int
   S->prof_end(1, 0.0, fl2);
   // ---- loss over the batch and its gradient
   S->prof_begin();
-  sage_gather_labels<<<blocks_for(nb, 256), 256, 0, s>>>(d.y, W.b1, nb, W.yb);
+  launch(sage_gather_labels, blocks_for(nb, 256), 256, 0, s, d.y, W.b1, nb, W.yb);
   SLAUNCHED("sage_gather_labels");
   SCKL(launch_softmax_ce(sv, nb, (int32_t)S->c, W.logits, S->ldc, W.yb, S->ones, nb, W.loss, W.g, S->ldc, W.sc));
-  sage_loss_add<<<1, 32, 0, s>>>(W.loss + 1, W.loss, (float)nb);
+  launch(sage_loss_add, 1, 32, 0, s, W.loss + 1, W.loss, (float)nb);
   SLAUNCHED("sage_loss_add");
   S->prof_end(2, 0.0, 0.0);
   // ---- backward
@@ -533,7 +546,7 @@ int run_batch(gcnsa_sage* S, const gcnsa_parts* P, int32_t p, int64_t epoch, int
   S->prof_end(1, 0.0, 2.0 * fl2);
   S->prof_begin();
   SCKL(launch_colsum(sv, nb, (int32_t)S->c, W.g, S->ldc, gr + S->b2_off, 0, W.sc));
-  sage_hidden_grad<<<blocks_for(rows1 * S->ldh, 256), 256, 0, s>>>(W.dcat2, W.h1, W.cnt2, nb, std::max(r2, 1), S->ldh, rows1,
+  launch(sage_hidden_grad, blocks_for(rows1 * S->ldh, 256), 256, 0, s, W.dcat2, W.h1, W.cnt2, nb, std::max(r2, 1), S->ldh, rows1,
                                                                   W.dz1);
   SLAUNCHED("sage_hidden_grad");
   S->prof_end(2, 0.0, 0.0);
@@ -818,7 +831,7 @@ int gcnsa_sage_epoch(gcnsa_sage* S, const gcnsa_parts* P, float* loss_dev) {
       if (r == GCNSA_OK) r = ensure_batch_graph(S, P, p, W, st);
       if (r) return r;
       if (S->batch_exec[p]) {
-        sage_set_state<<<1, 1, 0, st>>>(W.batch_state, -1, S->epoch);
+        launch(sage_set_state, 1, 1, 0, st, W.batch_state, -1, S->epoch);
         SLAUNCHED("sage_set_state");
         a.nreplay = nfull;
       }
@@ -828,7 +841,7 @@ int gcnsa_sage_epoch(gcnsa_sage* S, const gcnsa_parts* P, float* loss_dev) {
   auto finish = [&](int lane) -> int {
     const int32_t p = at[lane].p;
     const int64_t nt = P->parts[p].info.n_train;
-    sage_loss_fold<<<1, 32, 0, stream_of(lane)>>>(S->loss_parts + p, S->lanes[lane].loss + 1,
+    launch(sage_loss_fold, 1, 32, 0, stream_of(lane), S->loss_parts + p, S->lanes[lane].loss + 1,
                                                   nt > 0 ? 1.0f / ((float)nt * (float)P->m) : 0.f);
     SLAUNCHED("sage_loss_fold");
     return GCNSA_OK;
@@ -880,7 +893,7 @@ int gcnsa_sage_epoch(gcnsa_sage* S, const gcnsa_parts* P, float* loss_dev) {
     SCK(cudaStreamWaitEvent(s, S->join_ev[i - 1], 0));
   }
   S->work_p = P->m - 1;
-  sage_param_mean<<<blocks_for(S->count, 256), 256, 0, s>>>(S->count, P->m, S->copies, S->theta,
+  launch(sage_param_mean, blocks_for(S->count, 256), 256, 0, s, S->count, P->m, S->copies, S->theta,
                                                             S->copies + (size_t)S->work_p * S->count, 1.0f / (float)P->m,
                                                             S->loss_parts, S->loss);
   SLAUNCHED("sage_param_mean");

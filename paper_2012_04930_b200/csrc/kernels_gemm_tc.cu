@@ -44,10 +44,13 @@ namespace {
 constexpr int BM = 128, BK = 32;
 // warps: 0 loads A, 1 issues the MMAs (and owns tensor memory), 2 loads B, 3 idle, 4-11 split the operands (two
 // groups of four: a warp may only touch the quarter warp % 4 of tensor memory's lanes), 12-15 run the epilogue
-constexpr int kSplitWarp0 = 4, kSplitWarps = 8, kSplitGroups = 2, kEpiWarp0 = 12, kEpiWarps = 4;
-constexpr int kThreads = 32 * (kEpiWarp0 + kEpiWarps);
+// (12-19 the masked one)
+constexpr int kSplitWarp0 = 4, kSplitWarps = 8, kSplitGroups = 2, kEpiWarp0 = 12;
 constexpr int EPI_PITCH = 36;                               // floats per row of an epilogue patch
-constexpr int EPI_BYTES = kEpiWarps * 32 * EPI_PITCH * 4;   // 18 KiB
+// registers per thread by role with eight epilogue warps, in multiples of 8; their sum over the five warpgroups is what
+// the launch gives (96 each)
+constexpr int kRegsIssue = 48, kRegsSplit = 80, kRegsEpi = 136;
+static_assert(kRegsIssue + 2 * kRegsSplit + 2 * kRegsEpi <= 5 * 96, "setmaxnreg draws on the registers of the launch");
 constexpr int A_BYTES = BM * BK * 4;                        // 16 KiB
 
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
@@ -141,11 +144,14 @@ __device__ __forceinline__ void split_buffer(const uint8_t* hi_buf, uint8_t* lo_
 // accumulator.  With the issuing thread behind elect.sync the tensor pipe sets the pace (see elect_one); behind
 // `lane == 0` an instruction cost it 97 clocks whether 128 or 256 columns wide.  51 249 x 128 x 602: 57 -> 47 us,
 // 269 498 x 256 x 256: 201 -> 151 us, 256 x 256 x 269 498: 169 -> 151 us (L2 flushed).
-template <int BN_, bool A_MN_, bool B_MN_, bool DB_>
+template <int BN_, bool A_MN_, bool B_MN_, bool DB_, bool MASKED_ = false>
 struct Shape {
   static constexpr int BN = BN_;
   static constexpr bool A_MN = A_MN_, B_MN = B_MN_, DB = DB_;
   static constexpr int B_BYTES = BN * BK * 4;
+  static constexpr bool MASKED = MASKED_;                 // the epilogue of masked_epilogue
+  static constexpr int EPI_WARPS = MASKED ? 8 : 4, THREADS = 32 * (kEpiWarp0 + EPI_WARPS);
+  static constexpr int EPI_BYTES = EPI_WARPS * 32 * (MASKED ? 32 : EPI_PITCH) * 4;
   static constexpr int NBUF = DB ? 2 : 1;                 // accumulator buffers
   static constexpr bool MERGED = BN == 64 || !DB;
   static constexpr int ACC_COLS = MERGED ? 2 * BN : BN;   // columns of one buffer
@@ -178,11 +184,147 @@ __device__ __forceinline__ Work decode_work(int w, int tiles_m, int tiles_n, int
   return k;
 }
 
+// a load that stays where it is written: hoisted above the accumulator's read-back, the mask of the next step would need
+// registers while the accumulator is in them
+__device__ __forceinline__ float4 load_here(const float* p) {
+  float4 v;
+  asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
+  return v;
+}
+
+// C = (A B^T) .* [mask > 0] (+ C), column sums of the masked product to colsum_partial, rows scaled by post_scale
+// afterwards: what warps 12..19 do where a CTA has several items and C takes float4 stores.  The mask has the size of C and
+// comes from memory, and four warps that each read a step of it ahead keep 16 KB an SM on the way: too little, the
+// epilogue set the pace at 9 us per 128 x 128 tile with k = 47, whose MMAs take one.  So two warps share a quarter of tensor memory's lanes
+// and take its steps of 32 columns in turn (warps 12-15 the even ones, 16-19 the odd ones), and each has the mask of its
+// next step - of the next item after the last one - on the way as soon as the previous one is in a word of bits.  Registers
+// decide the rest: with 112 / 128 / 136 a thread (and spills of 120 / 20 / 0 bytes) 245 000 x 256 x 32 takes 184 / 160 / 145
+// us, with four warps 192 us; a plain copy kernel that reads two matrices and writes one takes 117 us.
+// With column sums: 245 000 x 256 x 47: 223 -> 175 us, 245 000 x 256 x 256: 255 -> 210, 58 241 x 128 x 41: 46 -> 40,
+// 245 000 x 47 x 256: 103 -> 83 (L2 full of dirty lines before each call).  Without a
+// mask there is nothing to keep on the way (245 000 x 256 x 256: 145 us with four warps, 157 with eight), and a CTA with a
+// single item is done later with this code (5 000 x 64 x 20 in a chain of launches: 4.7 -> 5.2 us): both stay with four.
+template <class S>
+__device__ __forceinline__ void masked_epilogue(int w_epi, int lane, uint32_t tmem_base, float* tile, uint64_t* acc_full,
+                                                uint64_t* acc_empty, int M, int N, int tiles_n, int total_work,
+                                                float* __restrict__ c, int64_t ldc, int accumulate,
+                                                const float* __restrict__ mask, int64_t ldmask, int terms,
+                                                float* __restrict__ colsum_partial, const float* __restrict__ post_scale) {
+  constexpr int BN = S::BN, NBUF = S::NBUF;
+  const int quad = w_epi & 3, first_c0 = 32 * (w_epi >> 2);
+  const int lr = lane >> 3, lc = (lane & 7) * 4;
+  const int n_pad = (int)min(ldc, ((int64_t)N + 3) / 4 * 4);  // C's pad columns [N, n_pad) are written as zeros
+  float4 mk[8];
+  auto load_mask = [&](bool there, int row0, int col) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      mk[i] = there && row0 + 4 * i < M && col < n_pad ? load_here(mask + (int64_t)(row0 + 4 * i) * ldmask + col) : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  // one factor per row: thread = row here, eight rows per thread below
+  auto load_factor = [&](int row) { return post_scale && row < M ? __ldg(post_scale + row) : 1.f; };
+  int m0 = (int)blockIdx.x / tiles_n * BM, n0 = (int)blockIdx.x % tiles_n * BN;  // (rows and columns are below 2^31)
+  float next_factor = load_factor(m0 + quad * 32 + lane);
+  load_mask(true, m0 + quad * 32 + lr, n0 + first_c0 + lc);
+  uint32_t item = 0;
+  for (int w = blockIdx.x; w < total_work; w += gridDim.x, ++item) {
+    const uint32_t ab = item % NBUF, aph = (item / NBUF) & 1;
+    const int nw = w + (int)gridDim.x;
+    const bool more = nw < total_work;
+    const int row_base = m0 + quad * 32, m1 = more ? nw / tiles_n * BM : 0, n1 = nw % tiles_n * BN;
+    float ps[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) ps[i] = __shfl_sync(0xffffffffu, next_factor, lr + 4 * i);
+    if (more) next_factor = load_factor(m1 + quad * 32 + lane);
+    if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[ab], aph, 5))) break;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t acc = tmem_base + ((uint32_t)(quad * 32) << 16) + ab * S::ACC_COLS;
+    const int last_c0 = ((min(BN, N - n0) + 31) / 32 - 1) * 32;
+    if (first_c0 > last_c0) {  // a single step, which the other warp of this quarter takes
+      if (lane == 0) mbar_arrive(&acc_empty[ab]);
+      load_mask(more, m1 + quad * 32 + lr, n1 + first_c0 + lc);
+    }
+#pragma unroll 1
+    for (int c0 = first_c0; c0 <= last_c0; c0 += 64) {
+      const bool last = c0 + 64 > last_c0;
+      uint32_t bits = 0;  // taken before the accumulator: mask and accumulator are never in registers together
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        bits |= ((mk[i].x > 0.f ? 1u : 0u) | (mk[i].y > 0.f ? 2u : 0u) | (mk[i].z > 0.f ? 4u : 0u) | (mk[i].w > 0.f ? 8u : 0u))
+                << (4 * i);
+      uint32_t v[32];
+      tmem_ld32(acc + (uint32_t)c0, v);
+      if constexpr (S::MERGED) {
+        if (terms == 3) {  // the second accumulator: A_hi B_lo
+          uint32_t u[32];
+          tmem_ld32(acc + (uint32_t)(BN + c0), u);
+#pragma unroll
+          for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + __uint_as_float(u[j]));
+        }
+      }
+      if (last) {  // the warp's part of the accumulator is in registers
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&acc_empty[ab]);
+      }
+      // thread = row; chunk j (16 bytes) of row r at position j ^ (r % 8): rows and columns both spread over all banks
+#pragma unroll
+      for (int j = 0; j < 32; j += 4)
+        *reinterpret_cast<uint4*>(tile + lane * 32 + (j ^ ((lane & 7) << 2))) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+      __syncwarp();
+      load_mask(!last || more, (last ? m1 : m0) + quad * 32 + lr, (last ? n1 + first_c0 : n0 + c0 + 64) + lc);
+      const int col = n0 + c0 + lc;
+      const unsigned inside = __ballot_sync(0xffffffffu, col < n_pad);
+      if (col < n_pad) {
+        // col is a multiple of 4 below n_pad; of the float4 that straddles N the columns past it are pad (zeros)
+        const int keep = min(4, N - col);
+        bits &= 0x11111111u * ((1u << keep) - 1);
+        float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int h = 0; h < 8; h += 4) {  // four rows at a time: registers
+          float4 a4[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            a4[i] = *reinterpret_cast<const float4*>(tile + (lr + 4 * (h + i)) * 32 + (lc ^ ((lr + 4 * (i & 1)) << 2)));
+          float* const dst = c + (int64_t)(row_base + lr + 4 * h) * ldc + col;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const uint32_t b = bits >> (4 * (h + i));
+            a4[i].x = (b & 1u) ? a4[i].x : 0.f; a4[i].y = (b & 2u) ? a4[i].y : 0.f;
+            a4[i].z = (b & 4u) ? a4[i].z : 0.f; a4[i].w = (b & 8u) ? a4[i].w : 0.f;
+            // (rows past M are zero rows of A: they add nothing to the column sums)
+            cs.x += a4[i].x; cs.y += a4[i].y; cs.z += a4[i].z; cs.w += a4[i].w;
+            a4[i].x *= ps[h + i]; a4[i].y *= ps[h + i]; a4[i].z *= ps[h + i]; a4[i].w *= ps[h + i];
+            if (row_base + lr + 4 * (h + i) < M) {
+              float4* const o = reinterpret_cast<float4*>(dst + 4 * i * ldc);
+              if (accumulate) {
+                const float4 was = *o;
+                a4[i].x += was.x; a4[i].y += was.y; a4[i].z += was.z; a4[i].w += was.w;
+              }
+              *o = a4[i];
+            }
+          }
+        }
+        if (colsum_partial) {  // the 4 threads that share these columns; one row of partial sums per lane quarter
+#pragma unroll
+          for (int o = 8; o <= 16; o <<= 1) {
+            cs.x += __shfl_xor_sync(inside, cs.x, o); cs.y += __shfl_xor_sync(inside, cs.y, o);
+            cs.z += __shfl_xor_sync(inside, cs.z, o); cs.w += __shfl_xor_sync(inside, cs.w, o);
+          }
+          if (lr == 0) *reinterpret_cast<float4*>(colsum_partial + ((int64_t)(m0 / BM) * 4 + quad) * n_pad + col) = cs;
+        }
+      }
+      __syncwarp();  // the patch is rewritten by the next step
+    }
+    m0 = m1;
+    n0 = n1;
+  }
+}
+
 // One CTA per SM walks the work items (tile x k-slice) blockIdx.x, blockIdx.x + gridDim.x, ...; the rings and the
 // accumulator buffers keep their phase across items, so that the loads, the split and the MMAs of item i + 1 run
 // while warps 12-15 turn the accumulator of item i around.
 template <class S>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(S::THREADS, 1)
 gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, int64_t M, int64_t N,
             int k_blocks, int k_blocks_per_split, int tiles_m, int tiles_n, int total_work, float* __restrict__ c,
             int64_t ldc, int accumulate, int epi, const float* __restrict__ aux, int64_t ldaux,
@@ -226,7 +368,7 @@ gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     }
     for (int b = 0; b < NBUF; ++b) {
       mbar_init(&acc_full[b], 1);
-      mbar_init(&acc_empty[b], kEpiWarps);
+      mbar_init(&acc_empty[b], S::EPI_WARPS);
     }
     mbar_init(drain, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -243,6 +385,7 @@ gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   const uint32_t tmem_base = *tmem_slot;
   wait_for_predecessors();  // barriers and tensor memory are up; from here on global memory is read
 
+  if (S::MASKED && warp < kSplitWarp0) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsIssue));
   if (warp == 0 || warp == 2) {
     // ---------------- TMA producers: warp 0 streams A, warp 2 streams B ----------------
     if (elect_one()) {
@@ -349,6 +492,7 @@ gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   } else if (warp >= kSplitWarp0 && warp < kSplitWarp0 + kSplitWarps) {
     // ---------------- operand split (warps 4..11): group 0 takes the even k-blocks, group 1 the odd ones ----------
     // thread = row 32 q + lane of the A tile (q = the lane quarter of tensor memory this warp may touch)
+    if (S::MASKED) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsSplit));
     const int q = warp & 3, group = (warp - kSplitWarp0) >> 2, row = 32 * q + lane;
     const int tg = row;  // index among the 128 threads of the group
     uint32_t g = 0;
@@ -400,6 +544,12 @@ gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         if (lane == 0) mbar_arrive(&split[s]);
       }
     }
+  } else if (S::MASKED && warp >= kEpiWarp0) {
+    // ---------------- masked epilogue (warps 12..19) ----------------
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsEpi));
+    float* tile = reinterpret_cast<float*>(smem + S::EPI_OFF) + (warp - kEpiWarp0) * (32 * 32);
+    masked_epilogue<S>(warp - kEpiWarp0, lane, tmem_base, tile, acc_full, acc_empty, (int)M, (int)N, tiles_n, total_work, c, ldc,
+                       accumulate, aux, ldaux, terms, colsum_partial, post_scale);
   } else if (warp >= kEpiWarp0) {
     // ---------------- epilogue (warps 12..15) ----------------
     // A warp owns the 32 rows of its lane quarter of tensor memory and walks the tile's columns 32 at a time: read
@@ -670,7 +820,7 @@ cudaError_t run_tc_shape(cudaStream_t s, const TcPlan& p, const CUtensorMap& ma,
                          int epi, const float* aux, int64_t ldaux, int64_t slice_stride, int vec_ok, int terms, float* colsum_partial, const float* post_scale) {
   cudaError_t e0 = cudaFuncSetAttribute(gemm_tf32x3<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_BYTES);
   if (e0 != cudaSuccess) return e0;
-  launch(gemm_tf32x3<S>, grid, kThreads, S::SMEM_BYTES, s, ma, mb, m, n, p.k_blocks, p.kb_per_split, tiles_m, tiles_n, total,
+  launch(gemm_tf32x3<S>, grid, S::THREADS, S::SMEM_BYTES, s, ma, mb, m, n, p.k_blocks, p.kb_per_split, tiles_m, tiles_n, total,
                                                        c, ldc, accumulate, epi, aux, ldaux, slice_stride, vec_ok, terms, colsum_partial, post_scale);
   note_launch();
   return cudaGetLastError();
@@ -685,6 +835,12 @@ cudaError_t run_tc(cudaStream_t s, const TcPlan& p, const CUtensorMap& ma, const
   if (total >= (1LL << 31)) return cudaErrorInvalidValue;
   const int grid = (int)std::min<int64_t>(total, sm_count());
   // a second accumulator buffer pays only when a CTA has more than one work item
+  if constexpr (!A_MN && !B_MN) {  // (the layouts of the gradient product Q W^T, where masks are met)
+    if (total > grid && epi == GCNSA_EPI_MASK && vec_ok && p.splits == 1 && std::max(m, n) < (1LL << 31) - 2 * BM)
+      return run_tc_shape<Shape<BN, A_MN, B_MN, true, true>>(s, p, ma, mb, m, n, (int)tiles_m, (int)tiles_n, (int)total, grid,
+                                                             c, ldc, accumulate, epi, aux, ldaux, slice_stride, vec_ok, terms,
+                                                             colsum_partial, post_scale);
+  }
   if (total > grid)
     return run_tc_shape<Shape<BN, A_MN, B_MN, true>>(s, p, ma, mb, m, n, (int)tiles_m, (int)tiles_n, (int)total, grid, c,
                                                      ldc, accumulate, epi, aux, ldaux, slice_stride, vec_ok, terms, colsum_partial, post_scale);

@@ -508,3 +508,27 @@ def test_gather_probe_gathers_the_documented_rows(hit_every):
             gcnsa.op_gather_probe(_dev(x), n_rows, kw["window_rows"], kw["hit_every"], kw["rounds"], out)
     with pytest.raises(gcnsa.GcnsaError):
         gcnsa.op_gather_probe(_dev(x), n_rows, window, hit_every, rounds, out[:8])
+
+
+@pytest.mark.parametrize("m,n,k", [(30_011, 20, 33), (20_000, 130, 36), (40_003, 37, 5), (19_100, 256, 64)])
+@pytest.mark.parametrize("accumulate", [0, 1])
+def test_masked_product_with_several_items_per_cta(m, n, k, accumulate):
+    """C (+)= (A W^T) .* [mask > 0] where a CTA takes more tiles than one, so that eight warps share the epilogue: a
+    tile with a single step of 32 columns (which one of two warps takes), a second tile two columns wide, a float4
+    that straddles the last column, an even number of steps, a last row tile of 59, 32, 67 and 28 rows.  Operands are
+    small whole numbers over 8: products and sums are exact in fp32 and in the three-term split, so the result is too."""
+    rng = np.random.default_rng(m + n)
+    a = (rng.integers(-8, 9, (m, k)) / 8).astype(np.float32)
+    wt = (rng.integers(-8, 9, (n, k)) / 8).astype(np.float32)
+    mk = rng.integers(-1, 2, (m, n)).astype(np.float32)
+    c0 = (rng.integers(-8, 9, (m, n)) / 8).astype(np.float32)
+    want = (a @ wt.T) * (mk > 0) + (c0 if accumulate else 0)
+    ad, bd, md = _padded(a, _ld(k)), _padded(wt, _ld(k)), _padded(mk, _ld(n))
+    cd = _padded(c0, _ld(n))
+    ws = torch.empty(gcnsa.op_gemm_workspace(0, 1, m, n, k, gcnsa.GEMM_TF32X3) // 4 + 64, device="cuda")
+    tc0, fb0 = gcnsa.gemm_path_counts()
+    gcnsa.op_gemm(ad, bd, cd, m, n, k, tb=1, epi=gcnsa.EPI_MASK, aux=md, accumulate=accumulate, workspace=ws,
+                  mode=gcnsa.GEMM_TF32X3)
+    assert gcnsa.gemm_path_counts() == (tc0 + 1, fb0) and gcnsa.tc_status() == 0
+    assert np.array_equal(cd[:, :n].cpu().numpy(), want)
+    assert torch.all(cd[:, n:] == 0)

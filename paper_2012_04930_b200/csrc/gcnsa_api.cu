@@ -69,6 +69,7 @@ struct Lane {
   float* H[GCNSA_MAX_LAYERS + 1] = {nullptr};  // H[l], l >= 1
   float* S[GCNSA_MAX_LAYERS] = {nullptr};      // A_hat H^{l-1} of layers that aggregate first
   float *tmp_a = nullptr, *tmp_b = nullptr, *dlogits = nullptr;
+  float* ce_sums = nullptr;        // partial column sums of dlogits (the last layer's bias gradient), where the softmax makes them
   void *ws = nullptr, *sc = nullptr;
   void* dw = nullptr;              // workspace of the planned sparse products
   const float* s0_used = nullptr;  // A_hat H^0 the latest forward used (the cached one or S[0])
@@ -472,9 +473,10 @@ static bool alloc_lane(gcnsa_model* M, Lane& W, size_t act) {
   W.tmp_a = get(act);
   W.tmp_b = get(act);
   W.dlogits = get((size_t)M->n_max * GCNSA_LD(M->o.dims[M->L]) * sizeof(float));
+  W.ce_sums = get(std::max<size_t>(ce_sums_scratch(M->o.dims[M->L]), 256));
   W.ws = get(std::max<size_t>(M->ws_bytes, 256));
   W.sc = get(std::max<size_t>(M->sc_bytes, 256));
-  bool ok = W.tmp_a && W.tmp_b && W.dlogits && W.ws && W.sc;
+  bool ok = W.tmp_a && W.tmp_b && W.dlogits && W.ce_sums && W.ws && W.sc;
   if (ok && M->dw_bytes) {
     W.dw = get(M->dw_bytes);
     ok = W.dw != nullptr;
@@ -720,8 +722,19 @@ static int forward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& W
     ldh = ldo;
   }
   const int64_t ldc = GCNSA_LD(P->c);
-  PROF(M, 2, 8.0 * n * P->c + 5.0 * n, 0.0,
-       launch_softmax_ce(s, n, P->c, h, ldc, d.y, d.mask, d.info.n_train, M->loss_parts + p, W.dlogits, ldc, W.sc));
+  // the backward pass wants the column sums of the logit gradient (a bias) and, with factored_norm and a last layer that
+  // multiplies by W first, diag(dinv) times it in tmp_a (free by now): made while the gradient is in registers
+  CeSide side;
+  if (ce_by_groups(P->c)) {
+    if (M->o.use_bias) side.sums = W.ce_sums;
+    if (fact && M->transform_first[M->L - 1]) {
+      side.row_scale = d.dinv;
+      side.scaled = W.tmp_a;
+      side.lds = ldc;
+    }
+  }
+  PROF(M, 2, (side.scaled ? 12.0 : 8.0) * n * P->c + 5.0 * n, 0.0,
+       launch_softmax_ce(s, n, P->c, h, ldc, d.y, d.mask, d.info.n_train, M->loss_parts + p, W.dlogits, ldc, W.sc, side));
   return GCNSA_OK;
 }
 
@@ -744,6 +757,10 @@ static int backward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& 
     bool scaled = false;
     if (bias_done) {  // the masked product of the layer above has added the column sums (and scaled g) already
       scaled = g_scaled;
+    } else if (l == M->L - 1 && ce_by_groups(dout)) {  // the softmax kernel has made the partial sums and the scaled copy
+      scaled = fact && M->transform_first[l];
+      if (M->o.use_bias)
+        PROF(M, 2, 0.0, 0.0, launch_ce_sums(s, n, dout, W.ce_sums, grad + M->b_off[l], acc));
     } else if (M->o.use_bias) {
       if (fact && M->transform_first[l]) {
         PROF(M, 2, 12.0 * n * dout, 0.0,

@@ -204,9 +204,21 @@ int tc_status(int* out);  // error word of the tensor-core kernels (0 = no wait 
 int tc_clear();           // sets that word back to 0
 int tc_status_gemm(int* out);  // the dense products' share of it
 int tc_clear_gemm();
+// What the softmax kernel can write beside the gradient while that is in registers; rows on 16-byte boundaries only.
+struct CeSide {
+  const float* row_scale = nullptr;
+  float* scaled = nullptr;  // row_scale[r] * grad[r, :], rows lds floats apart
+  int64_t lds = 0;
+  float* sums = nullptr;    // partial column sums (ce_sums_scratch bytes) for launch_ce_sums
+};
 int launch_softmax_ce(void* stream, int64_t n, int32_t c, const float* logits, int64_t ld, const int32_t* y,
-                      const uint8_t* mask, int64_t n_train, float* loss_dev, float* grad, int64_t ldg, void* scratch);
+                      const uint8_t* mask, int64_t n_train, float* loss_dev, float* grad, int64_t ldg, void* scratch,
+                      const CeSide& side = CeSide{});
 size_t softmax_ce_scratch(int64_t n);
+// out[j] (+)= column sums of the gradient whose partial sums launch_softmax_ce(side.sums) left (same n, c)
+int launch_ce_sums(void* stream, int64_t n, int32_t c, const float* sums, float* out, int32_t accumulate);
+size_t ce_sums_scratch(int32_t c);  // bytes of CeSide::sums
+bool ce_by_groups(int32_t c);       // whether the kernel takes c columns with a CeSide
 int launch_colsum(void* stream, int64_t n, int32_t f, const float* g, int64_t ldg, float* out, int32_t accumulate,
                   void* scratch);
 // the same sums, and on the way scaled[i, :] = rscale[i] * g[i, :] (scaled may be g)

@@ -31,8 +31,107 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
-// One warp per row.  grad row = (softmax - onehot) * inv_nt for masked rows,
-// zero otherwise; block partial of sum(lse - z_y) goes to partial[blockIdx.x].
+// Rows that lie on 16-byte boundaries and have at most 256 columns: G lanes hold a row as NV float4 each, a warp works on
+// 32 / G rows at a time.  grad row = (softmax - onehot) * inv_nt for masked rows, zero otherwise; block partial of
+// sum(lse - z_y) goes to partial[blockIdx.x].  While the gradient is in registers the kernel also writes
+// row_scale[r] * grad (if `scaled`; what the last layer's transposed sparse product reads) and this block's column sums,
+// row blockIdx.x of `sums` (the bias gradient): a kernel for these would read the whole gradient again.
+// What holds it up is the chain of loads, shuffles and exponentials of a row, so it wants many warps more than many rows
+// a warp: 245 000 x 47 takes 50 us with one row a group and five blocks an SM, 51 / 58 us with two / four rows and four /
+// three blocks.  Gradient, scaled copy and sums, against a warp per row and a second kernel for the other two: 245 000 x
+// 47: 108 -> 50 us, 400 000 x 256: 407 -> 215, 46 593 x 41: 30 -> 17.
+constexpr int kSumBlocks = 740;  // 5 x 148
+template <int G, int NV>
+__global__ void __launch_bounds__(kCeWarps * 32, 5)
+softmax_ce_groups(int64_t n, int c, const float* __restrict__ logits, int64_t ld, const int32_t* __restrict__ y,
+                  const uint8_t* __restrict__ mask, float inv_nt, float* __restrict__ grad, int64_t ldg,
+                  float* __restrict__ partial, const float* __restrict__ row_scale, float* __restrict__ scaled, int64_t lds,
+                  float* __restrict__ sums) {
+  wait_for_predecessors();
+  constexpr int RW = 32 / G;
+  __shared__ float4 sh[NV][kCeWarps * 32];
+  __shared__ float sh_loss[kCeWarps];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, g = lane % G, sub = lane / G;
+  const int nq = (c + 3) / 4;
+  float4 cs[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) cs[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+  float loss = 0.f;
+  for (int64_t base = ((int64_t)blockIdx.x * kCeWarps + wib) * RW; base < n;
+       base += (int64_t)gridDim.x * kCeWarps * RW) {
+    const int64_t row = base + sub;
+    const bool in = row < n, on = in && mask[row] != 0;
+    const int yi = in ? y[row] : 0;
+    const float sc = in && scaled ? __ldg(row_scale + row) : 0.f;
+    float z[4 * NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const int q = v * G + g;
+      float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (in && q < nq) t = __ldg(reinterpret_cast<const float4*>(logits + row * ld) + q);
+      z[4 * v + 0] = 4 * q + 0 < c ? t.x : -INFINITY;
+      z[4 * v + 1] = 4 * q + 1 < c ? t.y : -INFINITY;
+      z[4 * v + 2] = 4 * q + 2 < c ? t.z : -INFINITY;
+      z[4 * v + 3] = 4 * q + 3 < c ? t.w : -INFINITY;
+    }
+    // the label's logit: lane (yi / 4) % G of the row's group holds it, in the float4 and component that yi names
+    const int label_k = 4 * (yi / (4 * G)) + (yi & 3);
+    float mine = z[0], mx = z[0];
+#pragma unroll
+    for (int k = 1; k < 4 * NV; ++k) {
+      mx = fmaxf(mx, z[k]);
+      mine = k == label_k ? z[k] : mine;
+    }
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, o));
+    const float zy = __shfl_sync(kFull, mine, sub * G + ((yi >> 2) & (G - 1)));
+    float se = 0.f;
+#pragma unroll
+    for (int k = 0; k < 4 * NV; ++k) {
+      z[k] = expf(z[k] - mx);
+      se += z[k];
+    }
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) se += __shfl_xor_sync(kFull, se, o);
+    const float inv_se = 1.f / se;
+    if (g == 0 && on) loss += (mx + logf(se)) - zy;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const int q = v * G + g;
+      float d[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        d[k] = on ? (z[4 * v + k] * inv_se - (4 * q + k == yi ? 1.f : 0.f)) * inv_nt : 0.f;
+      cs[v].x += d[0]; cs[v].y += d[1]; cs[v].z += d[2]; cs[v].w += d[3];
+      if (in && q < nq) {
+        *(reinterpret_cast<float4*>(grad + row * ldg) + q) = make_float4(d[0], d[1], d[2], d[3]);
+        if (scaled)
+          *(reinterpret_cast<float4*>(scaled + row * lds) + q) =
+              make_float4(sc * d[0], sc * d[1], sc * d[2], sc * d[3]);
+      }
+    }
+  }
+  loss = warp_sum(loss);
+  if (lane == 0) sh_loss[wib] = loss;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) sh[v][threadIdx.x] = cs[v];
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float s = 0.f;
+    for (int i = 0; i < kCeWarps; ++i) s += sh_loss[i];
+    partial[blockIdx.x] = s;
+  }
+  if (sums && (int)threadIdx.x < nq) {  // the block's groups in a fixed order
+    float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k = 0; k < kCeWarps * RW; ++k) {
+      const float4 u = sh[threadIdx.x / G][k * G + threadIdx.x % G];
+      t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
+    }
+    reinterpret_cast<float4*>(sums + (int64_t)blockIdx.x * 4 * nq)[threadIdx.x] = t;
+  }
+}
+
+// Every other row: a warp per row, the row read three times.
 __global__ void __launch_bounds__(kCeWarps * 32)
 softmax_ce_rows(int64_t n, int c, const float* __restrict__ logits, int64_t ld, const int32_t* __restrict__ y,
                 const uint8_t* __restrict__ mask, float inv_nt, float* __restrict__ grad, int64_t ldg,
@@ -44,30 +143,6 @@ softmax_ce_rows(int64_t n, int c, const float* __restrict__ logits, int64_t ld, 
   float loss = 0.f;
   for (int64_t row = (int64_t)blockIdx.x * kCeWarps + wib; row < n; row += (int64_t)gridDim.x * kCeWarps) {
     float* gr = grad + row * ldg;
-    if (c <= 64) {
-      // the row lives in two registers per lane; logits, label and mask are fetched together (no load waits for
-      // another), the same sums in the same order as the general path below
-      const float* z = logits + row * ld;
-      const bool on = mask[row] != 0;
-      const int yi = y[row];
-      const int j0 = lane, j1 = lane + 32;
-      const float z0 = j0 < c ? z[j0] : -INFINITY, z1 = j1 < c ? z[j1] : -INFINITY;
-      if (!on) {
-        for (int j = lane; j < ldg_cols; j += 32) gr[j] = 0.f;
-        continue;
-      }
-      const float mx = warp_max(fmaxf(z0, z1));
-      float se = 0.f;
-      if (j0 < c) se += expf(z0 - mx);
-      if (j1 < c) se += expf(z1 - mx);
-      se = warp_sum(se);
-      const float inv_se = 1.f / se;
-      if (j0 < ldg_cols) gr[j0] = j0 < c ? (expf(z0 - mx) * inv_se - (j0 == yi ? 1.f : 0.f)) * inv_nt : 0.f;
-      if (j1 < ldg_cols) gr[j1] = j1 < c ? (expf(z1 - mx) * inv_se - (j1 == yi ? 1.f : 0.f)) * inv_nt : 0.f;
-      const float zy = __shfl_sync(kFull, yi < 32 ? z0 : z1, yi & 31);
-      if (lane == 0) loss += (mx + logf(se)) - zy;
-      continue;
-    }
     if (!mask[row]) {
       for (int j = lane; j < ldg_cols; j += 32) gr[j] = 0.f;
       continue;
@@ -191,23 +266,25 @@ colsum_partial_v4(int64_t n, int f, const float* g, int64_t ldg, int64_t rows_pe
   }
 }
 
-// out[j] (+)= sum over blocks of partial[b][j] (rows ldp floats apart).  A block covers 32 columns; its 8 thread groups add every 8th
-// block's partial in ascending order and the 8 sums are added in group order: fixed order.
-__global__ void __launch_bounds__(256)
+// out[j] (+)= sum over blocks of partial[b][j] (rows ldp floats apart).  A block covers 32 columns; its 16 warps add every
+// 16th block's partial in ascending order, eight loads under way, and the 16 sums are added in warp order: fixed order.
+constexpr int kFinalWarps = 16;
+__global__ void __launch_bounds__(kFinalWarps * 32)
 colsum_final(int f, int blocks, const float* __restrict__ partial, int64_t ldp, float* __restrict__ out, int accumulate) {
   wait_for_predecessors();
-  __shared__ float sh[8][32];
+  __shared__ float sh[kFinalWarps][32];
   const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
   const int j = blockIdx.x * 32 + lane;
   float s = 0.f;
   if (j < f)
-    for (int b = grp; b < blocks; b += 8) s += partial[(int64_t)b * ldp + j];
+#pragma unroll 8
+    for (int b = grp; b < blocks; b += kFinalWarps) s += partial[(int64_t)b * ldp + j];
   sh[grp][lane] = s;
   __syncthreads();
   if (grp != 0 || j >= f) return;
   float t = sh[0][lane];
 #pragma unroll
-  for (int q = 1; q < 8; ++q) t += sh[q][lane];
+  for (int q = 1; q < kFinalWarps; ++q) t += sh[q][lane];
   out[j] = accumulate ? out[j] + t : t;
 }
 
@@ -359,16 +436,51 @@ int colsum_blocks(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t
 
 }  // namespace
 
+bool ce_by_groups(int32_t c) { return c >= 1 && c <= 256; }
+
+static int ce_group_blocks(int64_t n, int32_t c) {
+  const int64_t rows = kCeWarps * (c <= 32 ? 4 : c <= 64 ? 2 : 1);
+  return (int)std::max<int64_t>(1, std::min<int64_t>((n + rows - 1) / rows, kSumBlocks));
+}
+
+size_t ce_sums_scratch(int32_t c) { return (size_t)kSumBlocks * (size_t)((c + 3) / 4 * 4) * sizeof(float); }
+
+int launch_ce_sums(void* stream, int64_t n, int32_t c, const float* sums, float* out, int32_t accumulate) {
+  launch(colsum_final, (c + 31) / 32, kFinalWarps * 32, 0, (cudaStream_t)stream, c, n > 0 ? ce_group_blocks(n, c) : 0, sums,
+         (c + 3) / 4 * 4, out, accumulate);
+  note_launch();
+  return (int)cudaGetLastError();
+}
+
 size_t softmax_ce_scratch(int64_t n) { return (size_t)ce_blocks(n) * sizeof(float); }
 
 int launch_softmax_ce(void* stream, int64_t n, int32_t c, const float* logits, int64_t ld, const int32_t* y,
-                      const uint8_t* mask, int64_t n_train, float* loss_dev, float* grad, int64_t ldg, void* scratch) {
+                      const uint8_t* mask, int64_t n_train, float* loss_dev, float* grad, int64_t ldg, void* scratch,
+                      const CeSide& side) {
   cudaStream_t s = (cudaStream_t)stream;
-  const int blocks = ce_blocks(n);
+  int blocks = ce_blocks(n);
   const float inv_nt = n_train > 0 ? 1.0f / (float)n_train : 0.f;
-  if (n > 0) {
-    launch(softmax_ce_rows, blocks, kCeWarps * 32, 0, s, n, c, logits, ld, y, mask, inv_nt, grad, ldg, (float*)scratch);
-    note_launch();
+  auto aligned = [](const void* p, int64_t pitch) { return ((uintptr_t)p & 15) == 0 && pitch % 4 == 0; };
+  if (ce_by_groups(c) && aligned(logits, ld) && aligned(grad, ldg) && ldg >= (c + 3) / 4 * 4 && aligned(side.scaled, side.lds) &&
+      aligned(side.sums, 0)) {
+    blocks = ce_group_blocks(n, c);
+    if (n > 0) {
+      auto go = [&](auto kernel) {
+        launch(kernel, blocks, kCeWarps * 32, 0, s, n, c, logits, ld, y, mask, inv_nt, grad, ldg, (float*)scratch,
+               side.row_scale, side.scaled, side.lds, side.sums);
+      };
+      if (c <= 32) go(softmax_ce_groups<8, 1>);
+      else if (c <= 64) go(softmax_ce_groups<16, 1>);
+      else if (c <= 128) go(softmax_ce_groups<32, 1>);
+      else go(softmax_ce_groups<32, 2>);
+      note_launch();
+    }
+  } else {
+    if (side.scaled || side.sums) return (int)cudaErrorMisalignedAddress;
+    if (n > 0) {
+      launch(softmax_ce_rows, blocks, kCeWarps * 32, 0, s, n, c, logits, ld, y, mask, inv_nt, grad, ldg, (float*)scratch);
+      note_launch();
+    }
   }
   if (loss_dev) {
     launch(loss_finalize, 1, 256, 0, s, (const float*)scratch, n > 0 ? blocks : 0, inv_nt, loss_dev);
@@ -404,7 +516,7 @@ int launch_colsum_scaled(void* stream, int64_t n, int32_t f, const float* g, int
     if (side) return (int)cudaErrorMisalignedAddress;
     launch(colsum_partial, blocks, dim3(32, 8), 0, s, n, f, g, ldg, rpb, (float*)scratch);
   }
-  launch(colsum_final, (f + 31) / 32, 256, 0, s, f, blocks, (const float*)scratch, f, out, accumulate);
+  launch(colsum_final, (f + 31) / 32, kFinalWarps * 32, 0, s, f, blocks, (const float*)scratch, f, out, accumulate);
   note_launch(2);
   return (int)cudaGetLastError();
 }

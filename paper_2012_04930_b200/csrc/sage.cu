@@ -351,7 +351,7 @@ struct SageLane {
   uint64_t order_uid = 0;
   // the batch
   int32_t *b1 = nullptr, *cnt2 = nullptr, *s1 = nullptr, *cnt1 = nullptr, *yb = nullptr;
-  float *cat1 = nullptr, *h1 = nullptr, *cat2 = nullptr, *logits = nullptr, *g = nullptr, *dcat2 = nullptr, *dz1 = nullptr;
+  float *cat1 = nullptr, *h1 = nullptr, *cat2 = nullptr, *logits = nullptr, *g = nullptr, *dcat2 = nullptr, *dz1 = nullptr, *ce_sums = nullptr;
   float* loss = nullptr;  // [0] batch loss, [1] sum over the worker's batches
   int64_t* batch_state = nullptr;
   void *ws = nullptr, *sc = nullptr;
@@ -532,7 +532,9 @@ int run_batch(gcnsa_sage* S, const gcnsa_parts* P, int32_t p, int64_t epoch, int
   S->prof_begin();
   launch(sage_gather_labels, blocks_for(nb, 256), 256, 0, s, d.y, W.b1, nb, W.yb);
   SLAUNCHED("sage_gather_labels");
-  SCKL(launch_softmax_ce(sv, nb, (int32_t)S->c, W.logits, S->ldc, W.yb, S->ones, nb, W.loss, W.g, S->ldc, W.sc));
+  CeSide side;  // the partial column sums of the logit gradient come with it
+  if (ce_by_groups((int32_t)S->c)) side.sums = W.ce_sums;
+  SCKL(launch_softmax_ce(sv, nb, (int32_t)S->c, W.logits, S->ldc, W.yb, S->ones, nb, W.loss, W.g, S->ldc, W.sc, side));
   launch(sage_loss_add, 1, 32, 0, s, W.loss + 1, W.loss, (float)nb);
   SLAUNCHED("sage_loss_add");
   S->prof_end(2, 0.0, 0.0);
@@ -545,7 +547,11 @@ int run_batch(gcnsa_sage* S, const gcnsa_parts* P, int32_t p, int64_t epoch, int
                    GCNSA_EPI_NONE, nullptr, 0, W.ws, S->ws_bytes));
   S->prof_end(1, 0.0, 2.0 * fl2);
   S->prof_begin();
-  SCKL(launch_colsum(sv, nb, (int32_t)S->c, W.g, S->ldc, gr + S->b2_off, 0, W.sc));
+  if (side.sums) {
+    SCKL(launch_ce_sums(sv, nb, (int32_t)S->c, W.ce_sums, gr + S->b2_off, 0));
+  } else {
+    SCKL(launch_colsum(sv, nb, (int32_t)S->c, W.g, S->ldc, gr + S->b2_off, 0, W.sc));
+  }
   launch(sage_hidden_grad, blocks_for(rows1 * S->ldh, 256), 256, 0, s, W.dcat2, W.h1, W.cnt2, nb, std::max(r2, 1), S->ldh, rows1,
                                                                   W.dz1);
   SLAUNCHED("sage_hidden_grad");
@@ -677,7 +683,7 @@ int gcnsa_sage_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcns
         {(void**)&W.cat1, f4 * (size_t)(S->max_rows1 * 2 * S->ldf)}, {(void**)&W.h1, f4 * (size_t)(S->max_rows1 * S->ldh)},
         {(void**)&W.cat2, f4 * (size_t)(B * 2 * S->ldh)}, {(void**)&W.logits, f4 * (size_t)(B * S->ldc)},
         {(void**)&W.g, f4 * (size_t)(B * S->ldc)}, {(void**)&W.dcat2, f4 * (size_t)(B * 2 * S->ldh)},
-        {(void**)&W.dz1, f4 * (size_t)(S->max_rows1 * S->ldh)}, {(void**)&W.loss, f4 * 2},
+        {(void**)&W.dz1, f4 * (size_t)(S->max_rows1 * S->ldh)}, {(void**)&W.ce_sums, ce_sums_scratch((int32_t)S->c)}, {(void**)&W.loss, f4 * 2},
         {(void**)&W.batch_state, sizeof(int64_t) * 2}, {&W.ws, ws}, {&W.sc, std::max<size_t>(sc, 256)}};
   };
   cudaStream_t s = S->env.stream();

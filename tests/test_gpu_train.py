@@ -5,6 +5,8 @@ seeded inputs.
 Bars: bit-exact partition assignment, sampled vertex sets, CSR and transposed
 CSR indices; fp32 tensors within 1e-4 * max|reference| after one step; epoch
 loss within 1e-3 relative at every epoch."""
+import copy
+
 import numpy as np
 import pytest
 import torch
@@ -498,3 +500,38 @@ def test_cached_aggregated_features_give_the_same_training(epoch_graph, small_wl
                what="H1 after the feature rows changed")
         assert abs(la.item() - lb.item()) <= 1e-5 * abs(lb.item())
         cached.close(); plain.close(); parts.close()
+
+
+@pytest.mark.parametrize("c", [1, 32, 33, 64, 65, 128, 129, 256, 257])
+def test_last_layer_gradients_for_every_number_of_classes(tiny_wl, c):
+    """The softmax kernel holds a row in 8, 16 or 32 lanes, one or two float4 each (up to 32, 64, 128, 256 columns), and
+    writes the scaled copy and the partial column sums the last layer's backward pass starts from; wider rows take the
+    row kernel and the column-sum kernel.  Loss, logit gradient, dW and db against the checker, at the bars of the
+    other tests (fp32 sums over at most a partition's rows)."""
+    w = copy.copy(tiny_wl)
+    rng = np.random.default_rng(c)
+    f, h = w.dims[0], 300
+    w.dims = [f, h, c]
+    w.y = rng.integers(0, c, len(w.y)).astype(np.int32)
+    w.w0 = [(rng.standard_normal(s) / np.sqrt(s[0])).astype(np.float32) for s in ((f, h), (h, c))]
+    w.b0 = [rng.standard_normal(s).astype(np.float32) * 0.1 for s in (h, c)]
+    env, parts, model = _make(w, gemm_mode=gcnsa.GEMM_TF32X3, factored_norm=1)
+    _, rparts = oracle.build_partitions(w.rowptr, w.col, w.m, w.overlap_ppm, w.seed, w.part_mode, w.user_part)
+    ws, bs = [a.astype(np.float64) for a in w.w0], [b.astype(np.float64) for b in w.b0]
+    gw, gb = [np.zeros_like(a) for a in ws], [np.zeros_like(b) for b in bs]
+    loss = torch.zeros(1, device="cuda")
+    for p, pt in enumerate(rparts):
+        fw = oracle.forward(pt, w.x[pt.members], ws, bs, w.y[pt.members], w.train_mask[pt.members], w.loss_on_halo)
+        model.forward(p, loss.data_ptr())
+        assert abs(loss.item() - fw["loss"]) <= 1e-5 * max(abs(fw["loss"]), 1e-6)
+        h_gpu = [model.get(gcnsa.GET_ACT, l, rows=pt.n) for l in (1, 2)]
+        bw = oracle.backward(pt, fw, ws, w.y[pt.members], relu_on=_relu_decisions(fw, h_gpu[:-1]))
+        _close(model.get(gcnsa.GET_DLOGITS, rows=pt.n), bw["G"][1], what=f"p{p} dlogits")
+        model.backward(p)
+        for l in range(2):
+            gw[l] += bw["dW"][l]; gb[l] += bw["db"][l]
+    for l in range(2):
+        _close(model.get(gcnsa.GET_GRAD_W, l), gw[l], what=f"dW{l}")
+        _close(model.get(gcnsa.GET_GRAD_B, l), gb[l], what=f"db{l}")
+    assert gcnsa.tc_status() == 0
+    model.close(); parts.close()

@@ -191,7 +191,7 @@ int launch_gemm_mask_colsum(void* stream, int32_t mode, int32_t ta, int32_t tb, 
                             const float* mask, int64_t ldmask, const float* row_scale, float* out, int32_t accumulate,
                             void* scratch, void* workspace, size_t workspace_bytes);
 size_t gemm_colsum_scratch(int64_t m, int32_t n);
-int64_t gemm_tc_colsum_rows(int64_t m);
+int64_t gemm_tc_colsum_rows(int32_t ta, int32_t tb, int64_t m, int64_t n);
 size_t gemm_tc_workspace(int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k);
 int launch_splitk_reduce(void* stream, int64_t m, int64_t n, int splits, const float* partial, int64_t ldp, float* c,
                          int64_t ldc,
@@ -225,6 +225,9 @@ int launch_colsum(void* stream, int64_t n, int32_t f, const float* g, int64_t ld
 int launch_colsum_scaled(void* stream, int64_t n, int32_t f, const float* g, int64_t ldg, float* out, int32_t accumulate,
                          void* scratch, const float* rscale, float* scaled, int64_t lds);
 size_t colsum_scratch(int64_t n, int32_t f);
+// the same sums over rows that are partial sums already: one launch where they are few
+int launch_sum_rows(void* stream, int64_t n, int32_t f, const float* g, int64_t ldg, float* out, int32_t accumulate,
+                    void* scratch);
 int launch_adam(void* stream, int64_t count, float* theta, float* gsum, float* m, float* v, float inv_m, float lr,
                 float beta1, float beta2, float eps, int64_t t);
 // pred[i] = argmax_j logits[i, j] (lowest j on ties); hits[b] = per-block count of masked rows with pred == y

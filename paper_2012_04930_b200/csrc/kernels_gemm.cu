@@ -377,15 +377,15 @@ int launch_gemm(void* stream, int32_t mode, int32_t ta, int32_t tb, int64_t m, i
   return 0;
 }
 
-// the rows of partial sums the product's epilogue writes (one per epilogue warp and row tile), 256-byte rounded
+// the rows of partial sums the product's epilogue writes (at most one per lane quarter and row tile), 256-byte rounded
 static size_t fused_partial_bytes(int64_t m, int32_t n) {
-  return ((size_t)gemm_tc_colsum_rows(m) * (size_t)((n + 3) / 4 * 4) * sizeof(float) + 255) / 256 * 256;
+  return ((size_t)gemm_tc_colsum_rows(1, 0, m, n) * (size_t)((n + 3) / 4 * 4) * sizeof(float) + 255) / 256 * 256;
 }
 
 // ... followed by the scratch of the column-sum kernels that add those rows up; or, when the product runs
 // unfused, the scratch of the column sums over C itself
 size_t gemm_colsum_scratch(int64_t m, int32_t n) {
-  return std::max(fused_partial_bytes(m, n) + colsum_scratch(gemm_tc_colsum_rows(m), n), colsum_scratch(m, n));
+  return std::max(fused_partial_bytes(m, n) + colsum_scratch(gemm_tc_colsum_rows(1, 0, m, n), n), colsum_scratch(m, n));
 }
 
 int launch_gemm_mask_colsum(void* stream, int32_t mode, int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k,
@@ -398,9 +398,8 @@ int launch_gemm_mask_colsum(void* stream, int32_t mode, int32_t ta, int32_t tb, 
                                  workspace_bytes, mode == GCNSA_GEMM_TF32 ? 1 : 3, (float*)scratch, row_scale);
     if (r == 0) {
       note_gemm_path(true);
-      // thousands of partial rows for a tall product: the column-sum kernels add them in their fixed order
-      return launch_colsum(stream, gemm_tc_colsum_rows(m), n, (const float*)scratch, (n + 3) / 4 * 4, out, accumulate,
-                           (uint8_t*)scratch + fused_partial_bytes(m, n));
+      return launch_sum_rows(stream, gemm_tc_colsum_rows(ta, tb, m, n), n, (const float*)scratch, (n + 3) / 4 * 4, out,
+                             accumulate, (uint8_t*)scratch + fused_partial_bytes(m, n));
     }
     if (r > 0) return r;
   }

@@ -200,8 +200,8 @@ __device__ __forceinline__ float4 load_here(const float* p) {
 // next step - of the next item after the last one - on the way as soon as the previous one is in a word of bits.  Registers
 // decide the rest: with 112 / 128 / 136 a thread (and spills of 120 / 20 / 0 bytes) 245 000 x 256 x 32 takes 184 / 160 / 145
 // us, with four warps 192 us; a plain copy kernel that reads two matrices and writes one takes 117 us.
-// With column sums: 245 000 x 256 x 47: 223 -> 175 us, 245 000 x 256 x 256: 255 -> 210, 58 241 x 128 x 41: 46 -> 40,
-// 245 000 x 47 x 256: 103 -> 83 (L2 full of dirty lines before each call).  Without a
+// With column sums: 245 000 x 256 x 47: 223 -> 169 us, 245 000 x 256 x 256: 255 -> 202, 58 241 x 128 x 41: 46 -> 40,
+// 245 000 x 47 x 256: 103 -> 81 (L2 full of dirty lines before each call).  Without a
 // mask there is nothing to keep on the way (245 000 x 256 x 256: 145 us with four warps, 157 with eight), and a CTA with a
 // single item is done later with this code (5 000 x 64 x 20 in a chain of launches: 4.7 -> 5.2 us): both stay with four.
 template <class S>
@@ -225,6 +225,10 @@ __device__ __forceinline__ void masked_epilogue(int w_epi, int lane, uint32_t tm
   int m0 = (int)blockIdx.x / tiles_n * BM, n0 = (int)blockIdx.x % tiles_n * BN;  // (rows and columns are below 2^31)
   float next_factor = load_factor(m0 + quad * 32 + lane);
   load_mask(true, m0 + quad * 32 + lr, n0 + first_c0 + lc);
+  // Where the grid is a multiple of the tiles in a row of C, all items of a CTA lie in the same columns, and the column sums
+  // run on from item to item in one row of `colsum_partial` per CTA and lane quarter, which the warp reads and writes itself
+  // (fixed order).  Else every row tile has its own row.
+  const bool running = gridDim.x % tiles_n == 0;
   uint32_t item = 0;
   for (int w = blockIdx.x; w < total_work; w += gridDim.x, ++item) {
     const uint32_t ab = item % NBUF, aph = (item / NBUF) & 1;
@@ -246,6 +250,11 @@ __device__ __forceinline__ void masked_epilogue(int w_epi, int lane, uint32_t tm
 #pragma unroll 1
     for (int c0 = first_c0; c0 <= last_c0; c0 += 64) {
       const bool last = c0 + 64 > last_c0;
+      const int col = n0 + c0 + lc;
+      float4* const sums = reinterpret_cast<float4*>(
+          colsum_partial + ((int64_t)(running ? (int)blockIdx.x / tiles_n : m0 / BM) * 4 + quad) * n_pad + col);
+      float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (colsum_partial && running && item > 0 && lr == 0 && col < n_pad) cs = *sums;
       uint32_t bits = 0;  // taken before the accumulator: mask and accumulator are never in registers together
 #pragma unroll
       for (int i = 0; i < 8; ++i)
@@ -272,13 +281,11 @@ __device__ __forceinline__ void masked_epilogue(int w_epi, int lane, uint32_t tm
         *reinterpret_cast<uint4*>(tile + lane * 32 + (j ^ ((lane & 7) << 2))) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
       __syncwarp();
       load_mask(!last || more, (last ? m1 : m0) + quad * 32 + lr, (last ? n1 + first_c0 : n0 + c0 + 64) + lc);
-      const int col = n0 + c0 + lc;
       const unsigned inside = __ballot_sync(0xffffffffu, col < n_pad);
       if (col < n_pad) {
         // col is a multiple of 4 below n_pad; of the float4 that straddles N the columns past it are pad (zeros)
         const int keep = min(4, N - col);
         bits &= 0x11111111u * ((1u << keep) - 1);
-        float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int h = 0; h < 8; h += 4) {  // four rows at a time: registers
           float4 a4[4];
@@ -310,7 +317,7 @@ __device__ __forceinline__ void masked_epilogue(int w_epi, int lane, uint32_t tm
             cs.x += __shfl_xor_sync(inside, cs.x, o); cs.y += __shfl_xor_sync(inside, cs.y, o);
             cs.z += __shfl_xor_sync(inside, cs.z, o); cs.w += __shfl_xor_sync(inside, cs.w, o);
           }
-          if (lr == 0) *reinterpret_cast<float4*>(colsum_partial + ((int64_t)(m0 / BM) * 4 + quad) * n_pad + col) = cs;
+          if (lr == 0) *sums = cs;
         }
       }
       __syncwarp();  // the patch is rewritten by the next step
@@ -826,6 +833,11 @@ cudaError_t run_tc_shape(cudaStream_t s, const TcPlan& p, const CUtensorMap& ma,
   return cudaGetLastError();
 }
 
+// several items per CTA and the layouts of the gradient product Q W^T, where masks are met (rows and columns in 32 bits)
+bool takes_masked_epilogue(bool a_mn, bool b_mn, int64_t m, int64_t n, bool several) {
+  return several && !a_mn && !b_mn && std::max(m, n) < (1LL << 31) - 2 * BM;
+}
+
 template <int BN, bool A_MN, bool B_MN>
 cudaError_t run_tc(cudaStream_t s, const TcPlan& p, const CUtensorMap& ma, const CUtensorMap& mb, int64_t m, int64_t n,
                    float* c, int64_t ldc, int accumulate, int epi, const float* aux, int64_t ldaux, int64_t slice_stride,
@@ -835,8 +847,8 @@ cudaError_t run_tc(cudaStream_t s, const TcPlan& p, const CUtensorMap& ma, const
   if (total >= (1LL << 31)) return cudaErrorInvalidValue;
   const int grid = (int)std::min<int64_t>(total, sm_count());
   // a second accumulator buffer pays only when a CTA has more than one work item
-  if constexpr (!A_MN && !B_MN) {  // (the layouts of the gradient product Q W^T, where masks are met)
-    if (total > grid && epi == GCNSA_EPI_MASK && vec_ok && p.splits == 1 && std::max(m, n) < (1LL << 31) - 2 * BM)
+  if constexpr (!A_MN && !B_MN) {
+    if (epi == GCNSA_EPI_MASK && vec_ok && p.splits == 1 && takes_masked_epilogue(A_MN, B_MN, m, n, total > grid))
       return run_tc_shape<Shape<BN, A_MN, B_MN, true, true>>(s, p, ma, mb, m, n, (int)tiles_m, (int)tiles_n, (int)total, grid,
                                                              c, ldc, accumulate, epi, aux, ldaux, slice_stride, vec_ok, terms,
                                                              colsum_partial, post_scale);
@@ -860,8 +872,13 @@ cudaError_t run_tc_major(bool a_mn, bool b_mn, cudaStream_t s, const TcPlan& p, 
 
 }  // namespace
 
-// rows of column partial sums the fused epilogue writes: one per epilogue warp and row tile
-int64_t gemm_tc_colsum_rows(int64_t m) { return (m + BM - 1) / BM * 4; }
+// rows of column partial sums the fused epilogue writes: one per lane quarter and row tile, or, where masked_epilogue sums
+// on over the items of a CTA, per lane quarter and CTA in a column of tiles
+int64_t gemm_tc_colsum_rows(int32_t ta, int32_t tb, int64_t m, int64_t n) {
+  const int64_t tiles_m = (m + BM - 1) / BM, tiles_n = (n + tc_plan(m, n, 1).bn - 1) / tc_plan(m, n, 1).bn, sms = sm_count();
+  const bool several = takes_masked_epilogue(ta != 0, tb == 0, m, n, tiles_m * tiles_n > sms);
+  return several && sms % tiles_n == 0 ? sms / tiles_n * 4 : tiles_m * 4;
+}
 
 size_t gemm_tc_workspace(int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k) {
   (void)ta; (void)tb;  // operands are read in the layout they have: no transposed copies to make room for

@@ -532,3 +532,24 @@ def test_masked_product_with_several_items_per_cta(m, n, k, accumulate):
     assert gcnsa.gemm_path_counts() == (tc0 + 1, fb0) and gcnsa.tc_status() == 0
     assert np.array_equal(cd[:, :n].cpu().numpy(), want)
     assert torch.all(cd[:, n:] == 0)
+
+
+@pytest.mark.parametrize("m,n,k", [(7_000, 300, 24), (38_100, 300, 12), (19_100, 400, 16), (19_100, 128, 8), (2_000, 64, 8)])
+def test_column_sums_of_a_masked_product_by_cta_and_by_tile(m, n, k):
+    """The partial column sums of the masked product: a row per CTA where the grid is a multiple of the tiles across C
+    (1, 4), a row per row tile where it is not (3; few rows and rows for two stages) or a CTA has one tile.  Whole
+    numbers over 8, sums below 2^24 / 64: exact in fp32 in any order."""
+    rng = np.random.default_rng(m + n)
+    a = (rng.integers(-4, 5, (m, k)) / 8).astype(np.float32)
+    wt = (rng.integers(-4, 5, (n, k)) / 8).astype(np.float32)
+    mk = rng.integers(-1, 2, (m, n)).astype(np.float32)
+    base = (a @ wt.T) * (mk > 0)
+    cd = torch.full((m, _ld(n)), 7.0, device="cuda")
+    out = torch.full((n,), 3.0, device="cuda")
+    ws = torch.empty(gcnsa.op_gemm_workspace(0, 1, m, n, k, gcnsa.GEMM_TF32X3) // 4 + 64, device="cuda")
+    sc = torch.empty(gcnsa.op_gemm_mask_colsum_scratch(m, n) // 4, device="cuda")
+    for accumulate in (1, 0):
+        gcnsa.op_gemm_mask_colsum(_padded(a, _ld(k)), _padded(wt, _ld(k)), cd, m, n, k, _padded(mk, _ld(n)), out, tb=1,
+                                  accumulate=accumulate, scratch=sc, workspace=ws, mode=gcnsa.GEMM_TF32X3)
+        assert np.array_equal(out.cpu().numpy(), base.astype(np.float64).sum(0) + (3 if accumulate else 0))
+    assert np.array_equal(cd[:, :n].cpu().numpy(), base) and gcnsa.tc_status() == 0

@@ -1105,9 +1105,16 @@ int gcnsa_model_get(const gcnsa_model* M, int32_t what, int32_t layer, void* hos
     return fail(GCNSA_ERR_ARG, "unknown tensor id");
   }
   if (bytes != (size_t)(M->last_n * cols) * sizeof(float)) return fail(GCNSA_ERR_ARG, "byte count does not match the tensor");
-  if (M->last_n > 0)
-    CK(cudaMemcpy2DAsync(host_dst, (size_t)cols * sizeof(float), src, (size_t)GCNSA_LD(cols) * sizeof(float),
-                         (size_t)cols * sizeof(float), (size_t)M->last_n, cudaMemcpyDeviceToHost, M->env.stream()));
+  if (M->last_n > 0 && cols > 0) {
+    // A strided copy to the host goes row by row (rows of 80 bytes: 21 GB/s), a dense one at 55 GB/s: rows without padding
+    // are one piece, others are packed on the device first (tmp_b: no pass leaves anything there).  An evaluation that
+    // fetches the logits: 116 483 x 41 1 595 -> 1 336 us, 20 000 x 20 201 -> 162, x 41 246 -> 209, x 5 165 -> 160.
+    if (GCNSA_LD(cols) != cols) {
+      CKL(launch_pack_rows(M->env.e.stream, M->last_n, cols, src, GCNSA_LD(cols), M->lanes[0].tmp_b));
+      src = M->lanes[0].tmp_b;
+    }
+    CK(cudaMemcpyAsync(host_dst, src, bytes, cudaMemcpyDeviceToHost, M->env.stream()));
+  }
   CK(cudaStreamSynchronize(M->env.stream()));
   return GCNSA_OK;
 }
@@ -1158,15 +1165,18 @@ int gcnsa_evaluate(gcnsa_model* M, const gcnsa_parts* P, int32_t p, const uint8_
   if (!M->ev_hits) M->ev_hits = (int32_t*)M->dalloc(4096 * sizeof(int32_t));
   if (!M->ev_mask) M->ev_mask = (uint8_t*)M->dalloc((size_t)M->n_max);
   if (!M->ev_pred || !M->ev_hits || !M->ev_mask) return fail(GCNSA_ERR_OOM, "device allocation failed");
-  M->all_rows_once = true;
-  int rc = gcnsa_forward(M, P, p, nullptr);   // also checks that the model fits these partitions
-  M->all_rows_once = false;
+  int rc = check_model(M, P);
   if (rc) return rc;
-  M->last_forward = -1;                       // an evaluation pass is not followed by a backward pass
   const DevPart& d = P->parts[p];
   const int64_t n = d.info.n;
   cudaStream_t s = M->env.stream();
+  // (before the forward pass: a copy from pageable memory holds the host up, and behind the pass the device would wait)
   if (mask_host && n > 0) CK(cudaMemcpyAsync(M->ev_mask, mask_host, (size_t)n, cudaMemcpyHostToDevice, s));
+  M->all_rows_once = true;
+  rc = gcnsa_forward(M, P, p, nullptr);
+  M->all_rows_once = false;
+  if (rc) return rc;
+  M->last_forward = -1;                       // an evaluation pass is not followed by a backward pass
   int blocks = 0;
   CKL(launch_argmax_hits(s, n, P->c, M->lanes[0].H[M->L], GCNSA_LD(P->c), d.y, mask_host ? M->ev_mask : nullptr, M->ev_pred,
                          M->ev_hits, &blocks));

@@ -218,6 +218,8 @@ size_t softmax_ce_scratch(int64_t n);
 // out[j] (+)= column sums of the gradient whose partial sums launch_softmax_ce(side.sums) left (same n, c)
 int launch_ce_sums(void* stream, int64_t n, int32_t c, const float* sums, float* out, int32_t accumulate);
 size_t ce_sums_scratch(int32_t c);  // bytes of CeSide::sums
+// dst[i * cols + j] = src[i * ld + j]
+int launch_pack_rows(void* stream, int64_t n, int64_t cols, const float* src, int64_t ld, float* dst);
 bool ce_by_groups(int32_t c);       // whether the kernel takes c columns with a CeSide
 int launch_colsum(void* stream, int64_t n, int32_t f, const float* g, int64_t ldg, float* out, int32_t accumulate,
                   void* scratch);

@@ -431,10 +431,24 @@ normalize_rows(int64_t n_rows, const int32_t* __restrict__ rowptr, const int32_t
   for (int e = rowptr[row] + lane; e < rowptr[row + 1]; e += 32) val[e] = 1.0f / sqrtf(di * (float)deg[col[e]]);
 }
 
+__global__ void __launch_bounds__(256)
+pack_rows(int64_t count, int64_t cols, const float* __restrict__ src, int64_t ld, float* __restrict__ dst) {
+  wait_for_predecessors();
+  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (i < count) dst[i] = src[i / cols * ld + i % cols];
+}
+
 int ce_blocks(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + kCeWarps - 1) / kCeWarps, kCeBlocksMax)); }
 int colsum_blocks(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + 63) / 64, 296)); }
 
 }  // namespace
+
+int launch_pack_rows(void* stream, int64_t n, int64_t cols, const float* src, int64_t ld, float* dst) {
+  const int64_t count = n * cols;
+  launch(pack_rows, (unsigned)((count + 255) / 256), 256, 0, (cudaStream_t)stream, count, cols, src, ld, dst);
+  note_launch();
+  return (int)cudaGetLastError();
+}
 
 bool ce_by_groups(int32_t c) { return c >= 1 && c <= 256; }
 

@@ -1022,11 +1022,11 @@ int gcnsa_epoch_host(gcnsa_model* M, gcnsa_parts* P, const float* const* x_host,
   if (!P->copy_stream) {  // first use: copy stream, events, two staging buffers
     CK(cudaStreamCreateWithFlags(&P->copy_stream, cudaStreamNonBlocking));
     P->ready.resize((size_t)P->m);
-    P->consumed.resize((size_t)P->m);
-    for (int32_t p = 0; p < P->m; ++p) {
-      CK(cudaEventCreateWithFlags(&P->ready[p], cudaEventDisableTiming));
-      CK(cudaEventCreateWithFlags(&P->consumed[p], cudaEventDisableTiming));
-      CK(cudaEventRecord(P->consumed[p], s));
+    for (int32_t p = 0; p < P->m; ++p) CK(cudaEventCreateWithFlags(&P->ready[p], cudaEventDisableTiming));
+    P->consumed.resize(2);
+    for (cudaEvent_t& e : P->consumed) {
+      CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+      CK(cudaEventRecord(e, s));
     }
   }
   for (int b = 0; b < 2; ++b) {  // (a call that ran out of memory here leaves what it got for the next one)
@@ -1034,24 +1034,27 @@ int gcnsa_epoch_host(gcnsa_model* M, gcnsa_parts* P, const float* const* x_host,
     P->staging[b] = (float*)P->dalloc((size_t)std::max<int64_t>(P->n_max, 1) * (size_t)P->f * sizeof(float));
     if (!P->staging[b]) return fail(GCNSA_ERR_OOM, "device allocation failed");
   }
-  // uploads run on their own stream, one partition ahead of the compute stream:
-  // dense host rows -> staging buffer -> padded device rows
+  // Uploads run back to back on their own stream, two staging buffers ahead of the compute stream, which spreads the dense
+  // rows over the padded device rows itself: on the copy stream that kernel stood between two copies (58 241 x 602 in four
+  // partitions: 45 us each).  The epoch takes the copies (2.8 ms at 50 GB/s) and the last partition's passes: 3.45 -> 3.28 ms.
+  auto copy_in = [&](int32_t p) {
+    cudaError_t e = cudaStreamWaitEvent(P->copy_stream, P->consumed[p & 1], 0);  // the buffer's previous rows have been read
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(P->staging[p & 1], x_host[p], (size_t)P->parts[p].info.n * (size_t)P->f * sizeof(float),
+                          cudaMemcpyHostToDevice, P->copy_stream);
+    return e == cudaSuccess ? cudaEventRecord(P->ready[p], P->copy_stream) : e;
+  };
+  for (int32_t p = 0; p < std::min(P->m, 2); ++p) CK(copy_in(p));
   for (int32_t p = 0; p < P->m; ++p) {
-    DevPart& d = P->parts[p];
-    CK(cudaStreamWaitEvent(P->copy_stream, P->consumed[p], 0));  // the previous reader of X_p has finished
-    float* st = P->staging[p & 1];
-    CK(cudaMemcpyAsync(st, x_host[p], (size_t)d.info.n * (size_t)P->f * sizeof(float), cudaMemcpyHostToDevice,
-                       P->copy_stream));
-    CKL(launch_repitch(P->copy_stream, d.info.n, P->f, st, d.x, P->ldx));
-    P->x_version[p] += 1;
-    CK(cudaEventRecord(P->ready[p], P->copy_stream));
-  }
-  for (int32_t p = 0; p < P->m; ++p) {
+    const DevPart& d = P->parts[p];
     CK(cudaStreamWaitEvent(s, P->ready[p], 0));
+    CKL(launch_copy_rows(s, d.info.n, P->f, P->staging[p & 1], P->f, d.x, P->ldx));
+    P->x_version[p] += 1;
+    CK(cudaEventRecord(P->consumed[p & 1], s));
+    if (p + 2 < P->m) CK(copy_in(p + 2));
     rc = forward_lane(M, P, p, M->lanes[0], s);
     if (rc == GCNSA_OK) rc = backward_lane(M, P, p, M->lanes[0], s, M->gparts + (size_t)p * M->count, 0);
     if (rc) return rc;
-    CK(cudaEventRecord(P->consumed[p], s));
   }
   PROF(M, 2, 0.0, 0.0, launch_adam_advance(s, M->adam_state, M->o.beta1, M->o.beta2));  // t -> t + 1
   rc = optimizer_step(M, s);
@@ -1110,7 +1113,7 @@ int gcnsa_model_get(const gcnsa_model* M, int32_t what, int32_t layer, void* hos
     // are one piece, others are packed on the device first (tmp_b: no pass leaves anything there).  An evaluation that
     // fetches the logits: 116 483 x 41 1 595 -> 1 336 us, 20 000 x 20 201 -> 162, x 41 246 -> 209, x 5 165 -> 160.
     if (GCNSA_LD(cols) != cols) {
-      CKL(launch_pack_rows(M->env.e.stream, M->last_n, cols, src, GCNSA_LD(cols), M->lanes[0].tmp_b));
+      CKL(launch_copy_rows(M->env.e.stream, M->last_n, cols, src, GCNSA_LD(cols), M->lanes[0].tmp_b, cols));
       src = M->lanes[0].tmp_b;
     }
     CK(cudaMemcpyAsync(host_dst, src, bytes, cudaMemcpyDeviceToHost, M->env.stream()));

@@ -218,8 +218,8 @@ size_t softmax_ce_scratch(int64_t n);
 // out[j] (+)= column sums of the gradient whose partial sums launch_softmax_ce(side.sums) left (same n, c)
 int launch_ce_sums(void* stream, int64_t n, int32_t c, const float* sums, float* out, int32_t accumulate);
 size_t ce_sums_scratch(int32_t c);  // bytes of CeSide::sums
-// dst[i * cols + j] = src[i * ld + j]
-int launch_pack_rows(void* stream, int64_t n, int64_t cols, const float* src, int64_t ld, float* dst);
+// dst[i * ldd + j] = src[i * lds + j], j < cols
+int launch_copy_rows(void* stream, int64_t n, int64_t cols, const float* src, int64_t lds, float* dst, int64_t ldd);
 bool ce_by_groups(int32_t c);       // whether the kernel takes c columns with a CeSide
 int launch_colsum(void* stream, int64_t n, int32_t f, const float* g, int64_t ldg, float* out, int32_t accumulate,
                   void* scratch);
@@ -255,7 +255,6 @@ int launch_inv_sqrt_degree(void* stream, int64_t n, const int32_t* deg, float* d
 int launch_scale_rows(void* stream, int64_t n, int32_t f, const float* scale, const float* src, int64_t lds, float* dst,
                       int64_t ldd);
 // dst[i * ld + j] = src[i * f + j]: dense rows into padded rows
-int launch_repitch(void* stream, int64_t n, int32_t f, const float* src, float* dst, int64_t ld);
 int launch_mean(void* stream, const float* src, int count, float* dst);  // dst[0] = mean(src[0..count))
 
 }  // namespace gcnsa

@@ -230,7 +230,8 @@ void gcnsa_model_opts_default(gcnsa_model_opts* opts);
  * once and every step above runs in CUDA kernels: checks of the input graph,
  * the assignment, the breadth-first levels of Algorithm 1 for all other
  * partitions at once, the key selection (a radix select over the 64-bit keys),
- * the induced rows, the transpose (a stable radix sort by column) and the row
+ * the induced rows, the transpose (the matrix itself, as the induced graph is
+ * symmetric) and the row
  * orders.  The host only reads back sizes to allocate the results.  Needs
  * about 8 (n + nnz) + 4 n f bytes of device memory for the inputs plus 24 bytes
  * per non-zero of the largest partition as scratch, released before returning.
@@ -545,7 +546,7 @@ int gcnsa_tc_clear(void);
  * Section 4.1 checks every row of the processing order, every row range and
  * every gathered column index against the sizes of the extended partition, and
  * the kernels of gcnsa_build_partitions that scatter by computed positions
- * (induced rows of Section 3.1, the radix sort behind the transpose, the
+ * (induced rows of Section 3.1, the radix sort behind the row orders, the
  * transposed CSR over the loss columns) check every write position.  A failed
  * check records what it saw and skips the access; nothing traps.
  * *enabled_host = 1 in the checking build, 0 otherwise (then the rest is 0).

@@ -456,9 +456,8 @@ cudaError_t run(const Args& a) {
 
 // ---- the remainder of a planned product ------------------------------------------------------------------------
 // Row = its partial sums from the tensor-core kernel plus its entries [rowptr, rowend) of the remainder CSR (SCALED:
-// each times the scale of its source row), then the epilogue of spmm_rows.  A row has few entries here (10 of 406 on
-// the 233 K-vertex graph, 17 of 50 on the 2.45 M-vertex one), so what counts is the chain of dependent loads, not the
-// gathers: the warp fetches 32 indices with one load and hands them round by shuffle, RU gathers per group are in flight
+// each times the scale of its source row), then the epilogue of spmm_rows.  A row has few entries here (a few
+// per cent of its own on the 233 K-vertex graph), so what counts is the chain of dependent loads as much as the gathers: the warp fetches 32 indices with one load and hands them round by shuffle, RU gathers per group are in flight
 // at once, and the partial sums are asked for before the first gather.
 template <int CH>
 __device__ __forceinline__ void load_pieces(float4 (&out)[CH], const SpmmBase& b, int row, int q_first, int q_step, int nvec) {

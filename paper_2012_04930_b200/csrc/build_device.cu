@@ -1000,6 +1000,11 @@ void Builder::build_plan(DevPart& d, int64_t window) {
   const int64_t loss_tiles = ceil_div(nt, kDenseRows), n_tiles = loss_tiles + ceil_div(np - nt, kDenseRows);
   const int64_t words = ceil_div(np, 32), windows = ceil_div(np, kPlanWindow);
   if (n_tiles * kDenseRows >= (int64_t)INT32_MAX) return;
+  const int64_t sort_tiles = std::max<int64_t>(1, ceil_div(np, kSortTile));
+  if (!tiles) {  // the host builder's partitions come without the scan scratch of run(); build_splits uses it after this
+    tiles_cap = ceil_div(std::max<int64_t>(std::max<int64_t>(np, n_tiles), 256 * sort_tiles) + 1, kScanTile) + 2;
+    tiles = scratch<int64_t>((size_t)tiles_cap);
+  }
   const size_t mark = tmp.size();
   auto free_scratch = [&] {
     cudaStreamSynchronize(s);
@@ -1008,11 +1013,6 @@ void Builder::build_plan(DevPart& d, int64_t window) {
       tmp.pop_back();
     }
   };
-  const int64_t sort_tiles = std::max<int64_t>(1, ceil_div(np, kSortTile));
-  if (!tiles) {  // the host builder's partitions come without the scan scratch of run()
-    tiles_cap = ceil_div(std::max<int64_t>(std::max<int64_t>(np, n_tiles), 256 * sort_tiles) + 1, kScanTile) + 2;
-    tiles = scratch<int64_t>((size_t)tiles_cap);
-  }
   int32_t* row_at = scratch<int32_t>((size_t)(n_tiles * kDenseRows));
   int32_t* flags = scratch<int32_t>((size_t)np + 1);
   int32_t* before = scratch<int32_t>((size_t)np + 1);

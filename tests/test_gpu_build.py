@@ -223,3 +223,28 @@ def test_empty_partition_and_edgeless_graph_build_and_train():
                 model.close()
         assert max(losses) - min(losses) <= 1e-5 * max(abs(l) for l in losses)
         dev.close(); host.close()
+
+
+def test_builders_agree_where_a_plan_is_looked_for_and_rejected():
+    """A graph without shared columns but dense enough to be looked at for a plan (mean degree 52, above 2^19 entries): no
+    plan is kept, and the row lists made after that are the same from both builders, so the products are bit for bit."""
+    n = 12_003
+    rowptr, col = graphs.permutation_graph(n, 26, 5)
+    assert col.size + n >= 1 << 19 and col.size >= 40 * n
+    rng = np.random.default_rng(8)
+    x = rng.standard_normal((n, 24)).astype(np.float32)
+    y = rng.integers(0, 9, n).astype(np.int32)
+    mask = (rng.random(n) < 0.6).astype(np.uint8)
+    w0 = [rng.standard_normal((24, 9)).astype(np.float32)]
+    got = []
+    for builder in (gcnsa.BUILD_DEVICE, gcnsa.BUILD_HOST):
+        parts = _build(builder, rowptr, col, x, y, mask, 9, 1, 0, 3, gcnsa.PART_RANGE, None, 1)
+        sched = parts.export_schedule(0)
+        model = gcnsa.Model(gcnsa.make_env(0), parts, [24, 9], w0, loss_rows_only=0, epoch_graph=0)
+        model.forward(0)
+        model.backward(0)
+        got.append([sched[k] for k in sorted(sched)] + [model.get(gcnsa.GET_ACT, 1, n), model.get(gcnsa.GET_GRAD_W, 0)])
+        model.close()
+        parts.close()
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)

@@ -845,6 +845,34 @@ struct Builder {
     if (!p) { rc = fail(GCNSA_ERR_OOM, "device allocation failed"); return nullptr; }
     return (T*)p;
   }
+  void keep(void* p) {  // a scratch buffer that the partitions keep
+    P->owned.push_back(p);
+    tmp.erase(std::find(tmp.begin(), tmp.end(), p));
+  }
+  // Plans and splits only save time: where memory for one is not to be had, the partition goes without it.  Scratch that
+  // make() has not kept is handed back; make() keeps nothing before all it needs has been obtained.
+  template <class F>
+  void optional(F&& make) {
+    if (!ok()) return;
+    const size_t mark = tmp.size();
+    const bool own_tiles = !tiles;
+    make();
+    if (rc == GCNSA_ERR_OOM) rc = GCNSA_OK;
+    if (tmp.size() > mark) cudaStreamSynchronize(s);
+    while (tmp.size() > mark) {
+      P->env.release(tmp.back());
+      tmp.pop_back();
+    }
+    if (own_tiles) {  // (the host builder's partitions come without the scan scratch of run())
+      tiles = nullptr;
+      tiles_cap = 0;
+    }
+  }
+  void scan_scratch(int64_t entries) {
+    if (tiles) return;
+    tiles_cap = ceil_div(entries + 1, kScanTile) + 2;
+    tiles = scratch<int64_t>((size_t)tiles_cap);
+  }
   template <class T>
   T* upload(const T* host, size_t count) {
     T* d = scratch<T>(count);
@@ -932,6 +960,10 @@ struct Builder {
   void build_partition(int32_t p, int64_t n_owned);
   void build_plan(DevPart& d, int64_t window);
   void build_splits(DevPart& d);
+  void build_extras(DevPart& d, int64_t window) {
+    optional([&] { build_plan(d, window); });
+    optional([&] { build_splits(d); });
+  }
 };
 
 // A plan pays where a chunk of 64 columns takes enough entries off the gathers: per 64 features a chunk costs one SM
@@ -946,12 +978,8 @@ constexpr int64_t kPlanMinNnz = 1 << 19, kPlanMinDegree = 40, kPlanEntriesPerChu
 // The processing orders by row length (RowSplit in internal.h).
 void Builder::build_splits(DevPart& d) {
   const int64_t np = d.info.n, nt = d.info.n_train;
-  if (!ok() || d.plan.n_chunks > 0 || np < kShortMinRows || d.info.nnz > np * kBlockRow) return;
-  if (!tiles) {
-    tiles_cap = ceil_div(np + 1, kScanTile) + 2;
-    tiles = scratch<int64_t>((size_t)tiles_cap);
-  }
-  const size_t mark = tmp.size();
+  if (d.plan.n_chunks > 0 || np < kShortMinRows || d.info.nnz > np * kBlockRow) return;
+  scan_scratch(np);
   int32_t* flags = scratch<int32_t>((size_t)np + 1);
   int32_t* at = scratch<int32_t>((size_t)np + 1);
   u64* far = scratch<u64>(1);
@@ -961,11 +989,12 @@ void Builder::build_splits(DevPart& d) {
   launched("count_far");
   u64 h_far = 0;
   read(&h_far, far, 1);
-  struct One { RowSplit* split; const int32_t* order; int64_t n; const int32_t* rowptr; };
-  for (const One& o : {One{&d.split, d.order, np, d.rowptr}, One{&d.m_split, d.m_order, nt, d.rowptr},
-                       One{&d.tm_split, d.tm_order, np, d.tm_rowptr}}) {
+  struct One { RowSplit* split; const int32_t* order; int64_t n; const int32_t* rowptr; RowSplit made; };
+  One ones[] = {{&d.split, d.order, np, d.rowptr, {}}, {&d.m_split, d.m_order, nt, d.rowptr, {}},
+                {&d.tm_split, d.tm_order, np, d.tm_rowptr, {}}};
+  for (One& o : ones) {
     if (o.n < kShortMinRows) continue;
-    int32_t* out = result<int32_t>((size_t)o.n);
+    int32_t* out = scratch<int32_t>((size_t)o.n);
     if (!ok()) return;
     int64_t done[3] = {0, 0, 0}, at_out = 0;
     const int64_t lo[3] = {kBlockRow, kShortRow, -1}, hi[3] = {INT64_MAX, kBlockRow, kShortRow};
@@ -980,39 +1009,27 @@ void Builder::build_splits(DevPart& d) {
     }
     if (!ok()) return;
     if (2 * (o.n - done[1]) < o.n) continue;  // most rows keep a warp: the plain order serves as well
-    o.split->order = out;
-    o.split->n_long = done[0];
-    o.split->n_warp = done[1];
-    o.split->scattered = 2 * (int64_t)h_far > d.info.nnz;
+    o.made.order = out;
+    o.made.n_long = done[0];
+    o.made.n_warp = done[1];
+    o.made.scattered = 2 * (int64_t)h_far > d.info.nnz;
+  }
+  for (One& o : ones) {
+    if (o.made.order) keep(o.made.order);
+    *o.split = o.made;
   }
   d.t_split = d.split;  // (the host builder's transposed CSR has the same rows)
-  cudaStreamSynchronize(s);
-  while (tmp.size() > mark) {
-    P->env.release(tmp.back());
-    tmp.pop_back();
-  }
 }
 
 void Builder::build_plan(DevPart& d, int64_t window) {
   const int64_t np = d.info.n, nnz = d.info.nnz, nt = d.info.n_train;
-  if (!ok() || nnz < kPlanMinNnz || nnz < np * kPlanMinDegree) return;
-  DensePlan& pl = d.plan;
+  if (nnz < kPlanMinNnz || nnz < np * kPlanMinDegree) return;
+  DensePlan pl;
   const int64_t loss_tiles = ceil_div(nt, kDenseRows), n_tiles = loss_tiles + ceil_div(np - nt, kDenseRows);
   const int64_t words = ceil_div(np, 32), windows = ceil_div(np, kPlanWindow);
   if (n_tiles * kDenseRows >= (int64_t)INT32_MAX) return;
   const int64_t sort_tiles = std::max<int64_t>(1, ceil_div(np, kSortTile));
-  if (!tiles) {  // the host builder's partitions come without the scan scratch of run(); build_splits uses it after this
-    tiles_cap = ceil_div(std::max<int64_t>(std::max<int64_t>(np, n_tiles), 256 * sort_tiles) + 1, kScanTile) + 2;
-    tiles = scratch<int64_t>((size_t)tiles_cap);
-  }
-  const size_t mark = tmp.size();
-  auto free_scratch = [&] {
-    cudaStreamSynchronize(s);
-    while (tmp.size() > mark) {
-      P->env.release(tmp.back());
-      tmp.pop_back();
-    }
-  };
+  scan_scratch(std::max<int64_t>(std::max<int64_t>(np, n_tiles), 256 * sort_tiles));
   int32_t* row_at = scratch<int32_t>((size_t)(n_tiles * kDenseRows));
   int32_t* flags = scratch<int32_t>((size_t)np + 1);
   int32_t* before = scratch<int32_t>((size_t)np + 1);
@@ -1022,9 +1039,9 @@ void Builder::build_plan(DevPart& d, int64_t window) {
   int32_t* lead = scratch<int32_t>((size_t)n_tiles + 1);
   int32_t* all = scratch<int32_t>((size_t)n_tiles + 1);
   u64* sums = scratch<u64>(4);
-  pl.pos = result<int32_t>((size_t)np);
-  pl.chunk_ptr = result<int32_t>((size_t)n_tiles + 1);
-  pl.loss_ptr = result<int32_t>((size_t)n_tiles + 1);
+  pl.pos = scratch<int32_t>((size_t)np);
+  pl.chunk_ptr = scratch<int32_t>((size_t)n_tiles + 1);
+  pl.loss_ptr = scratch<int32_t>((size_t)n_tiles + 1);
   if (!ok()) return;
   fill_ff(row_at, (size_t)(n_tiles * kDenseRows) * sizeof(int32_t));
   zero(n_sel, (size_t)(2 * n_tiles) * sizeof(int32_t));
@@ -1055,20 +1072,17 @@ void Builder::build_plan(DevPart& d, int64_t window) {
   read(h, sums, 4);
   if (!ok()) return;
   const int64_t covered = (int64_t)h[0], n_chunks = (int64_t)h[1];
-  if (n_chunks == 0 || covered < n_chunks * kPlanEntriesPerChunk) {
-    free_scratch();
-    return;
-  }
+  if (n_chunks == 0 || covered < n_chunks * kPlanEntriesPerChunk) return;
   int32_t* rank = scratch<int32_t>((size_t)(n_tiles * words * 2));
   int32_t* r_loss = scratch<int32_t>((size_t)np);
-  pl.tcol = result<int32_t>((size_t)(n_chunks * kDenseCols));
-  pl.bits = result<uint64_t>((size_t)(n_chunks * kDenseRows));
-  pl.r_rowptr = result<int32_t>((size_t)np + 1);
-  pl.r_mid = result<int32_t>((size_t)np);
+  pl.tcol = scratch<int32_t>((size_t)(n_chunks * kDenseCols));
+  pl.bits = scratch<uint64_t>((size_t)(n_chunks * kDenseRows));
+  pl.r_rowptr = scratch<int32_t>((size_t)np + 1);
+  pl.r_mid = scratch<int32_t>((size_t)np);
   pl.r_nnz = nnz - covered;
-  pl.r_col = result<int32_t>((size_t)pl.r_nnz);
-  pl.r_order = result<int32_t>((size_t)np);
-  pl.rm_order = result<int32_t>((size_t)nt);
+  pl.r_col = scratch<int32_t>((size_t)pl.r_nnz);
+  pl.r_order = scratch<int32_t>((size_t)np);
+  pl.rm_order = scratch<int32_t>((size_t)nt);
   uint32_t* k0 = scratch<uint32_t>((size_t)np);
   int32_t* v0 = scratch<int32_t>((size_t)np);
   uint32_t* k1 = scratch<uint32_t>((size_t)np);
@@ -1103,7 +1117,6 @@ void Builder::build_plan(DevPart& d, int64_t window) {
   launched("scatter_flagged");
   u64 longs[4];
   read(longs, sums, 4);
-  free_scratch();
   if (!ok()) return;
   pl.r_n_long = (int64_t)longs[0];
   pl.rm_n_long = (int64_t)longs[2];
@@ -1113,6 +1126,10 @@ void Builder::build_plan(DevPart& d, int64_t window) {
   pl.n_loss_chunks = (int64_t)h[2];
   pl.loss_tile_chunks = (int64_t)(int32_t)h[3];
   pl.n_chunks = n_chunks;
+  for (void* b : std::initializer_list<void*>{pl.pos, pl.chunk_ptr, pl.loss_ptr, pl.tcol, pl.bits, pl.r_rowptr, pl.r_mid, pl.r_col,
+                                              pl.r_order, pl.rm_order})
+    keep(b);
+  d.plan = pl;
 }
 
 void Builder::assign() {
@@ -1340,8 +1357,7 @@ void Builder::build_partition(int32_t p, int64_t n_owned) {
   if (!ok()) return;
   d.members.assign(mem32.begin(), mem32.end());
   for (void* t : std::initializer_list<void*>{members, deg, cnt, k0, v0, k1, v1, hist}) drop(t);
-  build_plan(d, window);
-  build_splits(d);
+  build_extras(d, window);
 }
 
 int Builder::run() {
@@ -1460,8 +1476,7 @@ int build_device(gcnsa_parts* P, const gcnsa_graph* g, const gcnsa_part_opts* o)
 
 int build_dense_plan(gcnsa_parts* P, DevPart& d, int64_t window) {
   Builder b{P, nullptr, nullptr, P->env.stream()};
-  b.build_plan(d, window);
-  b.build_splits(d);
+  b.build_extras(d, window);
   return b.rc;
 }
 

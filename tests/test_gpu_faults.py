@@ -9,7 +9,7 @@ import numpy as np
 import pytest
 import torch
 
-from gen import configs
+from gen import configs, graphs
 from paper_2012_04930_b200 import gcnsa
 
 pytestmark = pytest.mark.gpu
@@ -19,16 +19,17 @@ class FailingAllocator:
     """gcnsa_env callbacks on top of torch's caching allocator; call number `fail_at` (1-based) returns NULL."""
 
     def __init__(self):
-        self.calls, self.fail_at, self.live = 0, 0, {}
+        self.calls, self.fail_at, self.on, self.live = 0, 0, False, {}
         self.alloc_cb = gcnsa.ALLOC_FN(self._alloc)
         self.free_cb = gcnsa.FREE_FN(self._free)
 
-    def arm(self, fail_at):
-        self.calls, self.fail_at = 0, fail_at
+    def arm(self, fail_at, on=False):
+        """on: every call from number fail_at on is refused, not that one alone."""
+        self.calls, self.fail_at, self.on = 0, fail_at, on
 
     def _alloc(self, nbytes, user):
         self.calls += 1
-        if self.calls == self.fail_at:
+        if self.calls == self.fail_at or (self.on and self.calls > self.fail_at):
             return None
         p = torch.cuda.caching_allocator_alloc(int(nbytes), stream=torch.cuda.current_stream())
         self.live[p] = int(nbytes)
@@ -126,4 +127,67 @@ def test_out_of_memory_while_creating_and_using_a_model(agg_mode, cache_ax, tiny
     assert held <= set(alloc.live) and len(set(alloc.live) - held) <= 2   # the partitions and their two staging buffers
     parts.close()
     torch.cuda.synchronize()
+    assert not alloc.live
+
+
+def _planned_graph(n, target_nnz):
+    rowptr, col, comm = graphs.chung_lu_communities(n, target_nnz, 2.1, 3, 0.93, 5)
+    rng = np.random.default_rng(n)
+    return (rowptr, col, rng.standard_normal((n, 20)).astype(np.float32), (comm % 7).astype(np.int32),
+            (rng.random(n) < 0.9).astype(np.uint8), 7, 1, 0, 3)
+
+
+@pytest.mark.parametrize("builder", [gcnsa.BUILD_DEVICE, gcnsa.BUILD_HOST])
+@pytest.mark.parametrize("n,target_nnz", [(3001, 640_000), (12_003, 300_000)])
+def test_no_memory_for_a_plan_or_for_row_lists_is_no_failure(builder, n, target_nnz):
+    """The plan of the tensor-core products (first graph) and the row lists by length (second graph) only save time: where
+    one of their allocations is refused, alone or with all after it, the build succeeds and the products are right."""
+    alloc = FailingAllocator()
+    env = alloc.env()
+    small = _planned_graph(200, 2000)
+    alloc.arm(0)
+    gcnsa.Parts(env, *small, builder=builder).close()
+    required = alloc.calls                     # with one partition, the same for every graph
+    args = _planned_graph(n, target_nnz)
+    w0 = [np.random.default_rng(1).standard_normal((20, 7)).astype(np.float32)]
+
+    def logits(parts):
+        m = gcnsa.Model(gcnsa.make_env(0), parts, [20, 7], w0, loss_rows_only=0, epoch_graph=0)
+        m.forward(0)
+        out = m.get(gcnsa.GET_ACT, 1, n)
+        m.close()
+        return out
+
+    alloc.arm(0)
+    parts = gcnsa.Parts(env, *args, builder=builder)
+    total, want, full = alloc.calls, logits(parts), len(alloc.live)
+    parts.close()
+    assert total >= required + 6 and not alloc.live
+    for k in range(required + 1, total + 1):
+        for on in (False, True):
+            alloc.arm(k, on)
+            parts = gcnsa.Parts(env, *args, builder=builder)
+            assert len(alloc.live) <= full
+            if on:
+                # sums of up to a few hundred terms in another order, and another rounding of the three terms
+                assert np.abs(logits(parts) - want).max() <= 2e-5 * np.abs(want).max(), k
+            parts.close()
+            assert not alloc.live, k
+
+
+def test_a_rejected_plan_keeps_no_memory():
+    """A graph that is looked at for a plan and gets none holds as many buffers as one that is not looked at."""
+    alloc = FailingAllocator()
+    env = alloc.env()
+    small = gcnsa.Parts(env, *_planned_graph(200, 2000))
+    held = len(alloc.live)
+    small.close()
+    n = 10_001
+    rowptr, col = graphs.permutation_graph(n, 27, 5)
+    assert col.size + n >= 1 << 19
+    rng = np.random.default_rng(2)
+    parts = gcnsa.Parts(env, rowptr, col, rng.standard_normal((n, 4)).astype(np.float32), np.zeros(n, np.int32),
+                        np.ones(n, np.uint8), 2, 1, 0, 3)
+    assert len(alloc.live) == held
+    parts.close()
     assert not alloc.live

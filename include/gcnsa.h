@@ -233,8 +233,9 @@ void gcnsa_model_opts_default(gcnsa_model_opts* opts);
  * the induced rows, the transpose (the matrix itself, as the induced graph is
  * symmetric) and the row
  * orders.  The host only reads back sizes to allocate the results.  Needs
- * about 8 (n + nnz) + 4 n f bytes of device memory for the inputs plus 24 bytes
- * per non-zero of the largest partition as scratch, released before returning.
+ * about 37 n + 4 nnz + 4 n f bytes of device memory for the inputs and the
+ * vertices' states, plus as scratch at most 24 bytes per non-zero and 64 per
+ * row of the largest partition, all released before returning.
  * GCNSA_BUILD_HOST computes the structure on the host cores instead.
  */
 int gcnsa_build_partitions(const gcnsa_env* env, const gcnsa_graph* g, const gcnsa_part_opts* opts,

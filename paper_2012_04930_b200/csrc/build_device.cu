@@ -973,6 +973,10 @@ struct Builder {
 // 12.6 M entries) the planned product is as slow as the gathers.  A partition of fewer than kPlanMinNnz entries is a few microseconds of gathers, less than the
 // launches of a planned product cost, and one with short rows is not looked at (a tile of 256 rows would have to meet the
 // same few hundred columns).
+// kPlanScratch: a plan's tables of tiles x columns (sel, rank: np^2 / 683 bytes) are held to this many bytes per entry of
+// the matrix, what the header states.  Larger partitions (655 000 rows and more at mean degree 40, 5.7 million at 350)
+// would pay gigabytes to be looked at, 2.45 million rows 8.8 GB, 20 million 586 GB: they are gathered.
+constexpr int64_t kPlanScratch = 24;
 constexpr int64_t kPlanMinNnz = 1 << 19, kPlanMinDegree = 40, kPlanEntriesPerChunk = 768;
 
 // The processing orders by row length (RowSplit in internal.h).
@@ -1027,7 +1031,7 @@ void Builder::build_plan(DevPart& d, int64_t window) {
   DensePlan pl;
   const int64_t loss_tiles = ceil_div(nt, kDenseRows), n_tiles = loss_tiles + ceil_div(np - nt, kDenseRows);
   const int64_t words = ceil_div(np, 32), windows = ceil_div(np, kPlanWindow);
-  if (n_tiles * kDenseRows >= (int64_t)INT32_MAX) return;
+  if (n_tiles * kDenseRows >= (int64_t)INT32_MAX || 12 * n_tiles * words > kPlanScratch * nnz) return;
   const int64_t sort_tiles = std::max<int64_t>(1, ceil_div(np, kSortTile));
   scan_scratch(std::max<int64_t>(std::max<int64_t>(np, n_tiles), 256 * sort_tiles));
   int32_t* row_at = scratch<int32_t>((size_t)(n_tiles * kDenseRows));

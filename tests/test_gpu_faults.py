@@ -191,3 +191,29 @@ def test_a_rejected_plan_keeps_no_memory():
     assert len(alloc.live) == held
     parts.close()
     assert not alloc.live
+
+
+def test_scratch_of_the_build_stays_within_the_stated_bound():
+    """A partition so large for its degree that the tables of a plan would outgrow its matrix: it is not looked at (no
+    request is larger than the graph's own arrays), and the scratch of the whole build is what gcnsa.h states."""
+    n, f = 720_001, 4
+    rowptr, col = graphs.permutation_graph(n, 21, 5)
+    assert col.size >= 40 * n
+    rng = np.random.default_rng(2)
+
+    class Recorder(FailingAllocator):
+        peak = largest = 0
+
+        def _alloc(self, nbytes, user):
+            p = super()._alloc(nbytes, user)
+            self.largest, self.peak = max(self.largest, int(nbytes)), max(self.peak, sum(self.live.values()))
+            return p
+
+    alloc = Recorder()
+    parts = gcnsa.Parts(alloc.env(), rowptr, col, rng.standard_normal((n, f)).astype(np.float32), np.zeros(n, np.int32),
+                        np.ones(n, np.uint8), 2, 1, 0, 3)
+    nnz = parts.info(0).nnz
+    assert alloc.largest <= 4 * (nnz + n + 1)
+    scratch = alloc.peak - sum(alloc.live.values())
+    assert scratch <= 37 * n + 4 * col.size + 4 * n * f + 24 * nnz + 64 * n + (8 << 20)
+    parts.close()

@@ -607,6 +607,7 @@ int gcnsa_model_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcn
   for (Lane& W : M->lanes) {
     if (e == cudaSuccess) e = cudaMemsetAsync(W.tmp_a, 0, act, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(W.tmp_b, 0, act, s);
+    if (e == cudaSuccess && W.dw) e = cudaMemsetAsync(W.dw, 0, kPlannedHead, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(W.dlogits, 0, (size_t)M->n_max * GCNSA_LD(parts->c) * sizeof(float), s);
     for (int l = 0; l < M->L && e == cudaSuccess; ++l) {
       e = cudaMemsetAsync(W.H[l + 1], 0, (size_t)M->n_max * GCNSA_LD(opts->dims[l + 1]) * sizeof(float), s);
@@ -639,11 +640,13 @@ static int sparse_product(gcnsa_model* M, Lane& W, void* s, const DevPart& d, De
   const int64_t nnz = use == DenseUse::lossRows ? d.m_nnz : use == DenseUse::lossCols ? d.tm_nnz : d.info.nnz;
   const bool values = !(fact && src_scaled);
   const SpmmCost cost = spmm_cost(rows, use == DenseUse::lossCols ? d.info.n_train : n, nnz, f, values, epi == GCNSA_EPI_MASK);
+  const int32_t* rowptr = use == DenseUse::lossCols ? d.tm_rowptr : transposed ? d.t_rowptr : d.rowptr;
+  const int32_t* col = use == DenseUse::lossCols ? d.tm_col : transposed ? d.t_col : d.col;
   // (gcnsa_evaluate may bring partitions the workspace was not sized for)
   if (fact && d.plan.n_chunks > 0 && spmm_planned_workspace(d.plan, f) <= M->dw_bytes) {
     M->prof_begin();
-    const int r = launch_spmm_planned(s, d.plan, use, rows, d.dinv, src_scaled ? nullptr : d.dinv, x, ldx, f, epi, aux, ldaux, y,
-                                      ldy, W.dw, SpmmBounds{n, n, d.info.nnz});
+    const int r = launch_spmm_planned(s, d.plan, use, rows, rowptr, col, d.dinv, src_scaled ? nullptr : d.dinv, x, ldx, f, epi,
+                                      aux, ldaux, y, ldy, W.dw, SpmmBounds{n, n, use == DenseUse::lossCols ? d.tm_nnz : d.info.nnz});
     if (r > 0) return cuda_fail((cudaError_t)r, "launch_spmm_planned");
     if (r == 0) {
       M->prof_end(0, cost.bytes, cost.flops, cost.l1, cost.bytes_val);
@@ -652,8 +655,6 @@ static int sparse_product(gcnsa_model* M, Lane& W, void* s, const DevPart& d, De
   }
   const int32_t* order = use == DenseUse::lossRows ? d.m_order : use == DenseUse::lossCols ? d.tm_order : transposed ? d.t_order : d.order;
   const int64_t n_long = use == DenseUse::lossRows ? d.m_n_long : use == DenseUse::lossCols ? d.tm_n_long : transposed ? d.t_n_long : d.n_long;
-  const int32_t* rowptr = use == DenseUse::lossCols ? d.tm_rowptr : transposed ? d.t_rowptr : d.rowptr;
-  const int32_t* col = use == DenseUse::lossCols ? d.tm_col : transposed ? d.t_col : d.col;
   const float* val = !values ? nullptr : use == DenseUse::lossCols ? d.tm_val : transposed ? d.t_val : d.val;
   PROF_SPMM(M, cost, launch_spmm(s, rows, rowptr, col, val, values ? nullptr : d.dinv, order, n_long, x, ldx, f, epi, aux, ldaux,
                                  y, ldy, SpmmBounds{n, n, use == DenseUse::lossCols ? d.tm_nnz : d.info.nnz},

@@ -151,6 +151,10 @@ struct SpmmBase {
   int nslab = 1, width = 16, per_cta = 1;
   unsigned magic = 0;  // unit / per_cta = umulhi(unit, magic), 0 = divide
   int q0 = 0;  // first float4 chunk of this launch
+  // *beyond != 0: X has values the tensor cores cannot take; the rows are then gathered from the matrix itself
+  const int* beyond = nullptr;
+  const int32_t *all_rowptr = nullptr, *all_col = nullptr;
+  int64_t all_nnz = -1;
 };
 
 // ---- kernel launchers (all enqueue on `stream`, return a cudaError_t as int) ---
@@ -161,9 +165,12 @@ int launch_spmm(void* stream, int64_t n_rows, const int32_t* rowptr, const int32
                 const float* row_scale, const int32_t* order, int64_t n_long, const float* x, int64_t ldx, int32_t f, int32_t epi, const float* aux,
                 int64_t ldaux, float* y, int64_t ldy, const SpmmBounds& bounds = SpmmBounds(),
                 const RowSplit& split = RowSplit());
-// Y = epi(diag(row_scale) B diag(src_scale) X) through a partition's plan (both scales nullable); workspace:
-// spmm_planned_workspace(plan, f) bytes, 256-byte aligned.  Returns -1 when the plan cannot be used.
-int launch_spmm_planned(void* stream, const DensePlan& d, DenseUse use, int64_t n_rows, const float* row_scale,
+// Y = epi(diag(row_scale) B diag(src_scale) X) through a partition's plan (both scales nullable; rowptr, col: B itself,
+// restricted to the loss columns for DenseUse::lossCols); workspace: spmm_planned_workspace(plan, f) bytes, 256-byte
+// aligned, the first kPlannedHead of them zero before the first product.  Returns -1 when the plan cannot be used.
+constexpr size_t kPlannedHead = 256;
+int launch_spmm_planned(void* stream, const DensePlan& d, DenseUse use, int64_t n_rows, const int32_t* rowptr,
+                        const int32_t* col, const float* row_scale,
                         const float* src_scale, const float* x, int64_t ldx, int32_t f, int32_t epi, const float* aux,
                         int64_t ldaux, float* y, int64_t ldy, void* workspace, const SpmmBounds& bounds);
 size_t spmm_planned_workspace(const DensePlan& d, int32_t f);

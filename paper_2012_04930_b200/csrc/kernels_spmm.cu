@@ -532,18 +532,21 @@ spmm_rest(int n_long, int n_rows, const int32_t* __restrict__ rowptr, const int3
   const int w = hub ? (int)blockIdx.x : n_long + ((int)blockIdx.x - n_long) * W + warp;
   if (w >= n_rows) return;
   const int row = order ? __ldg(order + w) : w;
+  const bool whole = base.beyond && __ldcg(base.beyond) != 0;  // no partial sums: all entries of the row
 #if GCNSA_DBG
   if (dbg.mat_rows >= 0 && !dbg_in(&g_dbg_spmm, row, 0, dbg.mat_rows, kDbgOrderEntry)) return;  // hub: whole block alike
 #endif
-  int beg = __ldg(rowptr + row), end = __ldg(rowend + row);
+  int beg = __ldg((whole ? base.all_rowptr : rowptr) + row), end = __ldg((whole ? base.all_rowptr + 1 : rowend) + row);
+  if (whole) col = base.all_col;
 #if GCNSA_DBG
+  const int64_t nnz = whole ? base.all_nnz : dbg.nnz;
   if (!dbg_in(&g_dbg_spmm, beg, 0, (long long)end + 1, kDbgRowRange)) return;
-  if (dbg.nnz >= 0 && !dbg_in(&g_dbg_spmm, end, 0, dbg.nnz + 1, kDbgRowRange)) return;
+  if (nnz >= 0 && !dbg_in(&g_dbg_spmm, end, 0, nnz + 1, kDbgRowRange)) return;
 #endif
   float4 pieces[CH], acc[CH];
-  if (g == 0 && (!hub || warp == 0)) load_pieces<CH>(pieces, base, row, gl, G, nvec);
 #pragma unroll
-  for (int ch = 0; ch < CH; ++ch) acc[ch] = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int ch = 0; ch < CH; ++ch) pieces[ch] = acc[ch] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (g == 0 && (!hub || warp == 0) && !whole) load_pieces<CH>(pieces, base, row, gl, G, nvec);
   if (hub) {
     const int share = (end - beg + W - 1) / W;
     beg = min(end, beg + warp * share);

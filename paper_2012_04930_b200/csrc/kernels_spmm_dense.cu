@@ -24,6 +24,11 @@
 // The accumulator of the tensor core truncates when it adds: over the thousands of steps of a tile a bias of about
 // 1e-8 per step would pass the rounding of an fp32 sum.  So an accumulator only lives for one unit and is then added to
 // the thread's running sums with a rounded fp32 add, while the MMAs work in a second accumulator.
+//
+// A bit that is not set is a 0 that multiplies the source row, a set one a 2, and the split subtracts: with Inf or NaN in
+// a source row all rows of the tiles that list its column would be NaN, and sums above half of the largest fp32 would
+// overflow.  split_rows looks for such values (not finite, or 2^96 and more: below that twice the sum of 2^31 terms is
+// finite) and leaves a word for spmm_rest, which then takes all entries of every row as gathers and no partial sums.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -121,6 +126,7 @@ struct Params {
   int64_t split_pitch;
   int per_cta, total;        // units
   float* pieces;             // [(tiles x nslab + CTAs)][256][N]
+  int* beyond;               // [0] set by split_rows: values the MMAs cannot take; moved to [1] for spmm_rest
 };
 
 // A CTA's run of units, tile by tile and slab by slab.
@@ -213,6 +219,10 @@ __global__ void __launch_bounds__(kThreads, 1) spmm_dense(const Params p) {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_base = *tmem_slot;
   wait_for_predecessors();  // barriers and tensor memory are up; from here on global memory is read
+  if (blockIdx.x == 0 && threadIdx.x == 0) {  // the word is 0 again before the next product's split_rows runs
+    p.beyond[1] = p.beyond[0];
+    p.beyond[0] = 0;
+  }
 
   Walk walk;
   walk.start(p);
@@ -408,13 +418,18 @@ __device__ __forceinline__ uint32_t upper_halves(float lo, float hi) {
   return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
 }
 // x minus its upper half: exact, and the result has at most 16 (then 8) significant bits
+__device__ __forceinline__ uint32_t magnitude(const float4& v) {
+  return max(max(__float_as_uint(v.x) & 0x7FFFFFFFu, __float_as_uint(v.y) & 0x7FFFFFFFu),
+             max(__float_as_uint(v.z) & 0x7FFFFFFFu, __float_as_uint(v.w) & 0x7FFFFFFFu));
+}
+constexpr uint32_t kBeyond = (127u + 96u) << 23;  // the word of 2^96; Inf and NaN lie above
 __device__ __forceinline__ float lower_part(float x) { return x - __uint_as_float(__float_as_uint(x) & 0xFFFF0000u); }
 
 // The three bf16 terms of (xscale[i] times) every row, in the lines spmm_dense gathers; row n is zero (the row of slots
 // that are not used).  A thread takes 8 features.
 __global__ void __launch_bounds__(256)
 split_rows(int64_t n, const float4* __restrict__ x, int64_t ldx4, int nvec, const float* __restrict__ xscale, int groups,
-           int groups_per_slab, int step, int lines, uint4* __restrict__ out) {
+           int groups_per_slab, int step, int lines, uint4* __restrict__ out, int* __restrict__ beyond) {
   wait_for_predecessors();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (n + 1) * groups) return;
@@ -431,6 +446,7 @@ split_rows(int64_t n, const float4* __restrict__ x, int64_t ldx4, int nvec, cons
       b.x *= sc; b.y *= sc; b.z *= sc; b.w *= sc;
     }
   }
+  if (max(magnitude(a), magnitude(b)) >= kBeyond) *beyond = 1;
   const int slabs = groups / groups_per_slab;
   uint4* dst = out + (row * slabs + slab) * lines * 8 + in;
 #pragma unroll
@@ -486,11 +502,12 @@ cudaError_t run(cudaStream_t s, int grid, const Params& p) {
 size_t spmm_planned_workspace(const DensePlan& d, int32_t f) {
   if (d.n_chunks == 0) return 0;
   const Slabs sl = slabs_of(f);
-  return pieces_bytes(d, sl) + (size_t)(d.n_rows + 1) * sl.n * sl.lines * 128;
+  return kPlannedHead + pieces_bytes(d, sl) + (size_t)(d.n_rows + 1) * sl.n * sl.lines * 128;
 }
 
 // -1: too many units to count in an int (the caller then gathers)
-int launch_spmm_planned(void* stream, const DensePlan& d, DenseUse use, int64_t n_rows, const float* row_scale,
+int launch_spmm_planned(void* stream, const DensePlan& d, DenseUse use, int64_t n_rows, const int32_t* rowptr,
+                        const int32_t* col, const float* row_scale,
                         const float* src_scale, const float* x, int64_t ldx, int32_t f, int32_t epi, const float* aux,
                         int64_t ldaux, float* y, int64_t ldy, void* workspace, const SpmmBounds& bounds) {
   if (n_rows == 0 || f == 0) return 0;
@@ -499,7 +516,9 @@ int launch_spmm_planned(void* stream, const DensePlan& d, DenseUse use, int64_t 
   const int64_t total = us.chunks * sl.n;
   if (total >= INT32_MAX / 2) return -1;
   SpmmBase base;
-  base.pieces = (const float*)workspace;
+  int* beyond = (int*)workspace;
+  float* pieces = (float*)((uint8_t*)workspace + kPlannedHead);
+  base.pieces = pieces;
   base.pos = d.pos;
   base.prefix = us.prefix;
   base.nslab = sl.n;
@@ -508,12 +527,12 @@ int launch_spmm_planned(void* stream, const DensePlan& d, DenseUse use, int64_t 
   if (total > 0) {
     cudaStream_t s = (cudaStream_t)stream;
     const int sms = sm_count();
-    uint8_t* split = (uint8_t*)workspace + pieces_bytes(d, sl);
+    uint8_t* split = (uint8_t*)pieces + pieces_bytes(d, sl);
     const int gps = sl.width / 8, groups = gps * sl.n;
     const int64_t threads = (d.n_rows + 1) * groups;
     launch(split_rows, (unsigned)((threads + 255) / 256), 256, 0, s, d.n_rows, reinterpret_cast<const float4*>(x), ldx / 4,
                                                                  (f + 3) / 4, src_scale, groups, gps, sl.step, sl.lines,
-                                                                 reinterpret_cast<uint4*>(split));
+                                                                 reinterpret_cast<uint4*>(split), beyond);
     note_launch();
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return (int)e;
@@ -522,7 +541,12 @@ int launch_spmm_planned(void* stream, const DensePlan& d, DenseUse use, int64_t 
     p.prefix = us.prefix; p.chunk_ptr = d.chunk_ptr; p.tcol = d.tcol; p.bits = d.bits;
     p.total = (int)total;
     p.per_cta = (int)((total + sms - 1) / sms);
-    p.pieces = (float*)workspace;
+    p.pieces = pieces;
+    p.beyond = beyond;
+    base.beyond = beyond + 1;
+    base.all_rowptr = rowptr;
+    base.all_col = col;
+    base.all_nnz = bounds.nnz;
     p.split = split;
     p.split_pitch = (int64_t)sl.n * sl.lines * 128;
     base.per_cta = p.per_cta;

@@ -77,6 +77,68 @@ def test_planned_products_match_fp64(n, dims, mask_p):
     parts.close()
 
 
+def _reference(rowptr, col, n):
+    A = torch.zeros((n, n), dtype=torch.float64)
+    A[np.repeat(np.arange(n), np.diff(rowptr)), torch.from_numpy(col.astype(np.int64))] = 1.0
+    A += torch.eye(n, dtype=torch.float64)
+    dinv = A.sum(1).rsqrt()
+    return (dinv[:, None] * A * dinv[None, :]).cuda()
+
+
+# what a source row does to the rows that do not have it as a neighbour (nothing), and to sums between half of the largest
+# fp32 number and that number (they are finite); one layer that multiplies first and one that aggregates first
+@pytest.mark.parametrize("dims", [[16, 16], [16, 20], [80, 80]])
+@pytest.mark.parametrize("loss_rows_only", [0, 1])
+def test_planned_products_with_values_that_are_not_finite_or_very_large(dims, loss_rows_only):
+    n = 3001
+    rowptr, col, comm = graphs.chung_lu_communities(n, 640_000, 2.1, 3, 0.93, 5)
+    rng = np.random.default_rng(7)
+    x = rng.standard_normal((n, dims[0]), dtype=np.float32)
+    mask = (rng.random(n) < 0.66).astype(np.uint8)
+    w0 = [np.eye(dims[0], dims[1], dtype=np.float32)]
+    env = gcnsa.make_env(0)
+    parts = gcnsa.Parts(env, rowptr, col, x, (comm % 3).astype(np.int32), mask, dims[1], 1, 0, 3)
+    A = _reference(rowptr, col, n)
+    m = gcnsa.Model(env, parts, dims, w0, use_bias=0, loss_rows_only=loss_rows_only, epoch_graph=0)
+    rows = mask.astype(bool) if loss_rows_only else np.ones(n, bool)
+
+    def forward(values):
+        values = np.ascontiguousarray(values)
+        parts.set_features(0, values.ctypes.data)
+        before = gcnsa.launch_count()
+        m.forward(0)
+        assert gcnsa.launch_count() - before >= 5, "the planned path did not run"
+        return m.get(gcnsa.GET_ACT, 1, n)[rows]
+
+    clean = forward(x)
+    v = int(np.argmin(np.diff(rowptr)))
+    near = np.zeros(n, bool)
+    near[col[rowptr[v]:rowptr[v + 1]]] = True
+    near[v] = True
+    assert 0 < near[rows].sum() < rows.sum() // 2
+    for bad in (np.inf, -np.inf, np.nan):
+        broken = x.copy()
+        broken[v, 3] = bad
+        got = forward(broken)
+        assert not np.isfinite(got[near[rows]][:, 3]).any()
+        # (the same sums in another order and another rounding of the three terms)
+        assert np.abs(got[~near[rows]] - clean[~near[rows]]).max() <= 2e-5 * np.abs(clean).max()
+        assert np.array_equal(forward(x), clean), "the next product is planned again"
+    # sums of about 0.9 of the largest fp32 number, before the rows are scaled by d^-1/2
+    big = np.abs(x)
+    deg = torch.from_numpy(np.diff(rowptr) + 1).double().cuda().sqrt()
+    top = (deg[:, None] * (A @ torch.from_numpy(big).double().cuda())).max().item()
+    big *= np.float32(0.9 * np.finfo(np.float32).max / top)
+    want = (A @ torch.from_numpy(big).double().cuda()) @ torch.from_numpy(w0[0]).double().cuda()
+    _close(forward(big), want[torch.from_numpy(rows).cuda()], "large values")
+    # and values whose terms are subnormal: the planned product's absolute error is that of the smallest normal number
+    tiny = x * np.float32(2.0 ** -112)
+    want = (A @ torch.from_numpy(tiny).double().cuda()) @ torch.from_numpy(w0[0]).double().cuda()
+    _close(forward(tiny), want[torch.from_numpy(rows).cuda()], "small values")
+    m.close()
+    parts.close()
+
+
 # rows of at most 64 entries go to a group of lanes, longer ones to a warp, those above 256 to a block; one width per
 # kernel shape, and a graph without locality whose gathered matrix exceeds L2 (column slabs)
 @pytest.mark.parametrize("n,width", [(12_003, 7), (12_003, 30), (12_003, 41), (12_003, 64), (12_003, 100), (12_003, 130),

@@ -477,10 +477,6 @@ static bool alloc_lane(gcnsa_model* M, Lane& W, size_t act) {
   W.ws = get(std::max<size_t>(M->ws_bytes, 256));
   W.sc = get(std::max<size_t>(M->sc_bytes, 256));
   bool ok = W.tmp_a && W.tmp_b && W.dlogits && W.ce_sums && W.ws && W.sc;
-  if (ok && M->dw_bytes) {
-    W.dw = get(M->dw_bytes);
-    ok = W.dw != nullptr;
-  }
   for (int l = 0; l < M->L && ok; ++l) {
     W.H[l + 1] = get((size_t)M->n_max * GCNSA_LD(M->o.dims[l + 1]) * sizeof(float));
     ok = W.H[l + 1] != nullptr;
@@ -596,6 +592,9 @@ int gcnsa_model_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcn
     }
   }
   if (!ok) return fail_free(fail(GCNSA_ERR_OOM, "device allocation failed"));
+  // the workspace of the planned products; a lane without one gathers
+  for (Lane& W : M->lanes)
+    if (M->dw_bytes) W.dw = M->dalloc(M->dw_bytes);
   cudaStream_t s = M->env.stream();
   cudaError_t e = cudaMemsetAsync(M->theta, 0, pbytes, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(M->gsum, 0, pbytes, s);
@@ -643,7 +642,7 @@ static int sparse_product(gcnsa_model* M, Lane& W, void* s, const DevPart& d, De
   const int32_t* rowptr = use == DenseUse::lossCols ? d.tm_rowptr : transposed ? d.t_rowptr : d.rowptr;
   const int32_t* col = use == DenseUse::lossCols ? d.tm_col : transposed ? d.t_col : d.col;
   // (gcnsa_evaluate may bring partitions the workspace was not sized for)
-  if (fact && d.plan.n_chunks > 0 && spmm_planned_workspace(d.plan, f) <= M->dw_bytes) {
+  if (fact && d.plan.n_chunks > 0 && W.dw && spmm_planned_workspace(d.plan, f) <= M->dw_bytes) {
     M->prof_begin();
     const int r = launch_spmm_planned(s, d.plan, use, rows, rowptr, col, d.dinv, src_scaled ? nullptr : d.dinv, x, ldx, f, epi,
                                       aux, ldaux, y, ldy, W.dw, SpmmBounds{n, n, use == DenseUse::lossCols ? d.tm_nnz : d.info.nnz});

@@ -217,3 +217,32 @@ def test_scratch_of_the_build_stays_within_the_stated_bound():
     scratch = alloc.peak - sum(alloc.live.values())
     assert scratch <= 37 * n + 4 * col.size + 4 * n * f + 24 * nnz + 64 * n + (8 << 20)
     parts.close()
+
+
+@pytest.mark.parametrize("agg_mode,cache_ax", [(gcnsa.AGG_GRAD_AVG, 0), (gcnsa.AGG_PARAM_AVG, 1)])
+def test_a_model_without_memory_for_planned_products_gathers(agg_mode, cache_ax):
+    """The workspace of the planned products is asked for after everything a model needs; without it the model trains on
+    the gathers, with the losses of a model that has it up to rounding."""
+    alloc = FailingAllocator()
+    env = alloc.env()
+    args = _planned_graph(3001, 640_000)
+    parts = gcnsa.Parts(gcnsa.make_env(0), *args)
+    rng = np.random.default_rng(1)
+    w0 = [rng.standard_normal(s).astype(np.float32) / np.float32(np.sqrt(s[0])) for s in ((20, 12), (12, 7))]
+    losses = {}
+    for fail_at in (0, -1):      # -1: the last allocation of the first round
+        alloc.arm(0 if fail_at == 0 else calls)
+        m = gcnsa.Model(env, parts, [20, 12, 7], w0, agg_mode=agg_mode, cache_ax=cache_ax, epoch_graph=0)
+        calls = alloc.calls
+        loss = torch.zeros(1, device="cuda")
+        before = gcnsa.launch_count()
+        out = []
+        for _ in range(3):
+            m.epoch(loss.data_ptr())
+            out.append(loss.item())
+        losses[fail_at] = out, gcnsa.launch_count() - before
+        m.close()
+        assert not alloc.live
+    assert losses[-1][1] < losses[0][1], "planned products take more launches than gathers"
+    assert np.allclose(losses[0][0], losses[-1][0], rtol=1e-4)
+    parts.close()

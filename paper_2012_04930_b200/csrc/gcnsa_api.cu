@@ -460,16 +460,26 @@ static int copy_param(const gcnsa_model* M, float* base, int32_t layer, bool is_
 // 20.8 M entries per partition every sparse product fills the chip by itself and two of them at once evict each
 // other's source rows from L1 and L2 (233 K vertices, 5 partitions: 7.1 ms with one lane, 8.1 with two, 9.0 with
 // five); at 10 M entries two lanes gain 1 % and four lose 3 % (2.45 M vertices), which does not pay for the memory.
+// What counts beside the entries is the rows: a lane is activations and work buffers for all of them.  Eight partitions
+// without locality, one lane against eight: 8 000 rows of 8 entries, 64 wide (7 MB a lane) 587 -> 251 us per epoch, 64 000
+// rows (58 MB) 1 161 -> 954; three layers of 256, 32 000 rows (156 MB) 2 727 -> 2 508, 64 000 rows (294 MB) 4 871 -> 4 800,
+// 125 000 rows of 4 entries (556 MB) 9 101 -> 9 407, 250 000 rows (1.1 GB) 18 010 -> 18 240.  So the lanes after the first
+// together take at most 1 GB: seven of 146 MB, three of 294 MB, none of more than 1 GB.
 constexpr int64_t kMaxLanes = 8, kLaneNnz = 4 << 20;
-static int epoch_lanes(const gcnsa_model_opts& o, const gcnsa_parts* parts) {
+constexpr size_t kLaneBytes = (size_t)1 << 30;
+static int epoch_lanes(const gcnsa_model* M, const gcnsa_parts* parts, size_t lane_bytes) {
   int64_t nnz_max = 0;
   for (const DevPart& d : parts->parts) nnz_max = std::max<int64_t>(nnz_max, d.info.nnz);
-  if (!o.epoch_graph || nnz_max > kLaneNnz) return 1;
-  return (int)std::max<int64_t>(1, std::min<int64_t>(parts->m, kMaxLanes));
+  if (!M->o.epoch_graph || M->env.stream() == nullptr || nnz_max > kLaneNnz) return 1;  // (the default stream records nothing)
+  return (int)std::min<int64_t>(std::min<int64_t>(parts->m, kMaxLanes), 1 + (int64_t)(kLaneBytes / lane_bytes));
 }
 
-static bool alloc_lane(gcnsa_model* M, Lane& W, size_t act) {
-  auto get = [&](size_t bytes) { return (float*)M->dalloc(bytes); };
+// one lane's buffers; *bytes (nullable) grows by what was asked for
+static bool alloc_lane(gcnsa_model* M, Lane& W, size_t act, size_t* bytes_out = nullptr) {
+  auto get = [&](size_t bytes) {
+    if (bytes_out) *bytes_out += bytes;
+    return (float*)M->dalloc(bytes);
+  };
   W.tmp_a = get(act);
   W.tmp_b = get(act);
   W.dlogits = get((size_t)M->n_max * GCNSA_LD(M->o.dims[M->L]) * sizeof(float));
@@ -554,20 +564,9 @@ int gcnsa_model_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcn
     for (const DevPart& d : parts->parts)
       for (int l = 0; l < M->L; ++l)
         M->dw_bytes = std::max(M->dw_bytes, spmm_planned_workspace(d.plan, std::min(opts->dims[l], opts->dims[l + 1])));
-  M->lanes.resize((size_t)epoch_lanes(*opts, parts));
-  for (size_t i = 0; i < M->lanes.size() && ok; ++i) {
-    const size_t mark = M->owned.size();
-    ok = alloc_lane(M, M->lanes[i], act);
-    if (!ok && i > 0) {  // lanes after the first only make a recorded epoch faster
-      while (M->owned.size() > mark) {
-        M->env.release(M->owned.back());
-        M->owned.pop_back();
-      }
-      M->lanes.resize(i);
-      ok = true;
-      break;
-    }
-  }
+  M->lanes.resize(1);
+  size_t lane_bytes = M->dw_bytes;
+  ok = ok && alloc_lane(M, M->lanes[0], act, &lane_bytes);
   if (ok && opts->cache_ax) {
     M->ax.assign((size_t)parts->m, nullptr);
     M->ax_version.assign((size_t)parts->m, 0);
@@ -592,9 +591,20 @@ int gcnsa_model_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcn
     }
   }
   if (!ok) return fail_free(fail(GCNSA_ERR_OOM, "device allocation failed"));
-  // the workspace of the planned products; a lane without one gathers
-  for (Lane& W : M->lanes)
-    if (M->dw_bytes) W.dw = M->dalloc(M->dw_bytes);
+  // from here on what a model can do without: the workspace of the planned products (without it the products are gathers),
+  // and the lanes after the first, which only make a recorded epoch faster
+  if (M->dw_bytes && !(M->lanes[0].dw = M->dalloc(M->dw_bytes))) M->dw_bytes = 0;
+  M->lanes.resize((size_t)epoch_lanes(M, parts, lane_bytes));
+  for (size_t i = 1; i < M->lanes.size(); ++i) {
+    const size_t mark = M->owned.size();
+    Lane& W = M->lanes[i];
+    if (alloc_lane(M, W, act) && (!M->dw_bytes || (W.dw = M->dalloc(M->dw_bytes)))) continue;
+    while (M->owned.size() > mark) {
+      M->env.release(M->owned.back());
+      M->owned.pop_back();
+    }
+    M->lanes.resize(i);
+  }
   cudaStream_t s = M->env.stream();
   cudaError_t e = cudaMemsetAsync(M->theta, 0, pbytes, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(M->gsum, 0, pbytes, s);
@@ -642,7 +652,7 @@ static int sparse_product(gcnsa_model* M, Lane& W, void* s, const DevPart& d, De
   const int32_t* rowptr = use == DenseUse::lossCols ? d.tm_rowptr : transposed ? d.t_rowptr : d.rowptr;
   const int32_t* col = use == DenseUse::lossCols ? d.tm_col : transposed ? d.t_col : d.col;
   // (gcnsa_evaluate may bring partitions the workspace was not sized for)
-  if (fact && d.plan.n_chunks > 0 && W.dw && spmm_planned_workspace(d.plan, f) <= M->dw_bytes) {
+  if (fact && d.plan.n_chunks > 0 && spmm_planned_workspace(d.plan, f) <= M->dw_bytes) {
     M->prof_begin();
     const int r = launch_spmm_planned(s, d.plan, use, rows, rowptr, col, d.dinv, src_scaled ? nullptr : d.dinv, x, ldx, f, epi,
                                       aux, ldaux, y, ldy, W.dw, SpmmBounds{n, n, use == DenseUse::lossCols ? d.tm_nnz : d.info.nnz});

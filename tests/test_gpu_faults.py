@@ -246,3 +246,66 @@ def test_a_model_without_memory_for_planned_products_gathers(agg_mode, cache_ax)
     assert losses[-1][1] < losses[0][1], "planned products take more launches than gathers"
     assert np.allclose(losses[0][0], losses[-1][0], rtol=1e-4)
     parts.close()
+
+
+def _sparse_parts(env, m, rows, f, c):
+    """m partitions of the same ring of `rows` vertices: few entries, many rows."""
+    rp, cl = graphs.from_edge_list(rows, np.stack([np.arange(rows), (np.arange(rows) + 1) % rows], 1))
+    rowptr = np.concatenate([[0], np.cumsum(np.tile(np.diff(rp), m))])
+    col = (np.tile(cl.astype(np.int64), m) + np.repeat(np.arange(m) * rows, cl.size)).astype(np.int32)
+    rng = np.random.default_rng(m)
+    x = rng.standard_normal((m * rows, f)).astype(np.float32)
+    return gcnsa.Parts(env, rowptr, col, x, np.zeros(m * rows, np.int32), np.ones(m * rows, np.uint8), c, m, 0, 3)
+
+
+def test_side_by_side_partitions_take_bounded_memory():
+    """The buffers with which a recorded epoch runs partitions side by side: at most 1 GiB above the model of a caller who
+    records nothing, whatever the rows; none on the default stream, which cannot be recorded."""
+    rng = np.random.default_rng(1)
+    for rows, dims in ((1000, [16, 8, 3]), (40_000, [256, 256, 3])):
+        w0 = [rng.standard_normal(s).astype(np.float32) * 0.05 for s in zip(dims[:-1], dims[1:])]
+        held = {}
+        for name, stream, graph in (("plain", torch.cuda.Stream(), 0), ("recorded", torch.cuda.Stream(), 1),
+                                    ("default", torch.cuda.default_stream(), 1)):
+            with torch.cuda.stream(stream):
+                alloc = FailingAllocator()
+                env = alloc.env()
+                parts = _sparse_parts(gcnsa.make_env(0), 8, rows, dims[0], dims[-1])
+                m = gcnsa.Model(env, parts, dims, w0, epoch_graph=graph)
+                held[name] = sum(alloc.live.values())
+                m.close()
+                parts.close()
+        assert held["default"] == held["plain"]
+        assert held["plain"] < held["recorded"] <= held["plain"] + (1 << 30)
+
+
+@pytest.mark.parametrize("agg_mode,cache_ax", [(gcnsa.AGG_GRAD_AVG, 1), (gcnsa.AGG_PARAM_AVG, 0)])
+def test_buffers_a_model_needs_come_before_those_that_save_time(agg_mode, cache_ax):
+    """An allocator with just the memory of a model that records nothing: the same model that records is created too."""
+
+    class Budget(FailingAllocator):
+        room = 1 << 62
+
+        def _alloc(self, nbytes, user):
+            if sum(self.live.values()) + nbytes > self.room:
+                return None
+            return super()._alloc(nbytes, user)
+
+    rng = np.random.default_rng(1)
+    dims = [32, 16, 3]
+    w0 = [rng.standard_normal(s).astype(np.float32) * 0.05 for s in zip(dims[:-1], dims[1:])]
+    with torch.cuda.stream(torch.cuda.Stream()):
+        parts = _sparse_parts(gcnsa.make_env(0), 8, 3000, dims[0], dims[-1])
+        alloc = Budget()
+        env = alloc.env()
+        losses = []
+        for graph in (0, 1):
+            m = gcnsa.Model(env, parts, dims, w0, agg_mode=agg_mode, cache_ax=cache_ax, epoch_graph=graph)
+            alloc.room = min(alloc.room, sum(alloc.live.values()))
+            loss = torch.zeros(1, device="cuda")
+            for _ in range(2):
+                m.epoch(loss.data_ptr())
+            losses.append(loss.item())
+            m.close()
+        assert losses[0] == losses[1] and not alloc.live
+        parts.close()

@@ -916,16 +916,16 @@ struct Fork {
   }
 };
 
-// the step from the gradients of all partitions in gparts
+// the step from the gradients of all partitions in gparts, on top of what gcnsa_model_set has left in the gradient sum
 static int optimizer_step(gcnsa_model* M, cudaStream_t s) {
   const float inv_m = 1.0f / (float)M->m;
   if (M->o.agg_mode == GCNSA_AGG_PARAM_AVG)
     PROF(M, 2, 32.0 * M->count * M->m, 0.0,
-         launch_adam_local_parts(s, M->count, M->m, M->theta, M->gparts, M->am_parts, M->av_parts, inv_m, M->o.lr,
+         launch_adam_local_parts(s, M->count, M->m, M->theta, M->gsum, M->gparts, M->am_parts, M->av_parts, inv_m, M->o.lr,
                                  M->o.beta1, M->o.beta2, M->o.eps, M->adam_state));
   else
     PROF(M, 2, (24.0 + 4.0 * M->m) * M->count, 0.0,
-         launch_adam_parts(s, M->count, M->m, M->theta, M->gparts, M->am, M->av, inv_m, M->o.lr, M->o.beta1, M->o.beta2,
+         launch_adam_parts(s, M->count, M->m, M->theta, M->gsum, M->gparts, M->am, M->av, inv_m, M->o.lr, M->o.beta1, M->o.beta2,
                            M->o.eps, M->adam_state));
   return GCNSA_OK;
 }

@@ -249,12 +249,12 @@ int launch_adam_dev(void* stream, int64_t count, float* theta, float* gsum, floa
 // one partition's own Adam step from theta (not written): acc (+)= theta_p * inv_m; gsum cleared
 int launch_adam_local_dev(void* stream, int64_t count, const float* theta, float* gsum, float* m, float* v, float* acc,
                           int first, float inv_m, float lr, float beta1, float beta2, float eps, const double* state);
-// the same over the gradients of all partitions of an epoch, parts[p * count + i], added in partition order
-int launch_adam_parts(void* stream, int64_t count, int n_parts, float* theta, const float* parts, float* m, float* v,
-                      float inv_m, float lr, float beta1, float beta2, float eps, const double* state);
+// the same over the gradients of all partitions of an epoch, parts[p * count + i], added to gsum in partition order
+int launch_adam_parts(void* stream, int64_t count, int n_parts, float* theta, float* gsum, const float* parts, float* m,
+                      float* v, float inv_m, float lr, float beta1, float beta2, float eps, const double* state);
 // parameter averaging: theta becomes the mean over the partitions of their own steps (moments m, v: [n_parts x count])
-int launch_adam_local_parts(void* stream, int64_t count, int n_parts, float* theta, const float* parts, float* m, float* v,
-                            float inv_m, float lr, float beta1, float beta2, float eps, const double* state);
+int launch_adam_local_parts(void* stream, int64_t count, int n_parts, float* theta, float* gsum, const float* parts, float* m,
+                            float* v, float inv_m, float lr, float beta1, float beta2, float eps, const double* state);
 int launch_normalize(void* stream, int64_t n_rows, const int32_t* rowptr, const int32_t* col, const int32_t* deg,
                      float* val);
 int launch_inv_sqrt_degree(void* stream, int64_t n, const int32_t* deg, float* dinv);  // dinv[i] = 1 / sqrt(deg[i])

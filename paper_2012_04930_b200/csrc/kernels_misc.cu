@@ -336,16 +336,24 @@ __global__ void adam_local_kernel_dev(int64_t count, const float* __restrict__ t
   gsum[i] = 0.f;
 }
 
-// The optimizer over the gradients of all partitions of an epoch, parts[p * count + i], added in partition order: the
-// sums adam_kernel_dev finds in gsum when the backward passes add into one buffer, so the same result bit for bit.
-__global__ void adam_parts_kernel(int64_t count, int n_parts, float* __restrict__ theta, const float* __restrict__ parts,
+// what the caller has put into the gradient sum before the epoch (zero otherwise); the step clears it
+__device__ __forceinline__ float take(float* __restrict__ gsum) {
+  const float g = *gsum;
+  if (g != 0.f) *gsum = 0.f;
+  return g;
+}
+
+// The optimizer over the gradients of all partitions of an epoch, parts[p * count + i], added to gsum in partition order:
+// the sums adam_kernel_dev finds in gsum when the backward passes add into it, so the same result bit for bit.
+__global__ void adam_parts_kernel(int64_t count, int n_parts, float* __restrict__ theta, float* __restrict__ gsum,
+                                  const float* __restrict__ parts,
                                   float* __restrict__ m, float* __restrict__ v, float inv_m, float lr, float b1, float b2,
                                   float eps, const double* __restrict__ state) {
   wait_for_predecessors();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const float c1 = (float)state[1], c2 = (float)state[2];
-  float sum = 0.f;
+  float sum = take(gsum + i);
   for (int p = 0; p < n_parts; ++p) sum += parts[(int64_t)p * count + i];
   const float g = sum * inv_m;
   theta[i] -= adam_delta(g, m + i, v + i, lr, b1, b2, eps, c1, c2);
@@ -353,7 +361,7 @@ __global__ void adam_parts_kernel(int64_t count, int n_parts, float* __restrict_
 
 // Parameter averaging (Section 3.2): every partition's own Adam step from theta with its own moments, theta becomes
 // the mean of the results, added in partition order.
-__global__ void adam_local_parts_kernel(int64_t count, int n_parts, float* __restrict__ theta,
+__global__ void adam_local_parts_kernel(int64_t count, int n_parts, float* __restrict__ theta, float* __restrict__ gsum,
                                         const float* __restrict__ parts, float* __restrict__ m, float* __restrict__ v,
                                         float inv_m, float lr, float b1, float b2, float eps,
                                         const double* __restrict__ state) {
@@ -365,7 +373,7 @@ __global__ void adam_local_parts_kernel(int64_t count, int n_parts, float* __res
   float acc = 0.f;
   for (int p = 0; p < n_parts; ++p) {
     const int64_t k = (int64_t)p * count + i;
-    const float g = parts[k];
+    const float g = p == 0 ? take(gsum + i) + parts[k] : parts[k];
     const float th = __fmul_rn(th0 - adam_delta(g, m + k, v + k, lr, b1, b2, eps, c1, c2), inv_m);
     acc = p == 0 ? th : __fadd_rn(acc, th);
   }
@@ -594,20 +602,20 @@ int launch_adam_local_dev(void* stream, int64_t count, const float* theta, float
   return (int)cudaGetLastError();
 }
 
-int launch_adam_parts(void* stream, int64_t count, int n_parts, float* theta, const float* parts, float* m, float* v,
-                      float inv_m, float lr, float beta1, float beta2, float eps, const double* state) {
+int launch_adam_parts(void* stream, int64_t count, int n_parts, float* theta, float* gsum, const float* parts, float* m,
+                      float* v, float inv_m, float lr, float beta1, float beta2, float eps, const double* state) {
   if (count == 0) return 0;
-  launch(adam_parts_kernel, (unsigned)((count + 255) / 256), 256, 0, (cudaStream_t)stream, count, n_parts, theta, parts, m, v,
-                                                                                      inv_m, lr, beta1, beta2, eps, state);
+  launch(adam_parts_kernel, (unsigned)((count + 255) / 256), 256, 0, (cudaStream_t)stream, count, n_parts, theta, gsum, parts, m,
+                                                                                      v, inv_m, lr, beta1, beta2, eps, state);
   note_launch();
   return (int)cudaGetLastError();
 }
 
-int launch_adam_local_parts(void* stream, int64_t count, int n_parts, float* theta, const float* parts, float* m, float* v,
-                            float inv_m, float lr, float beta1, float beta2, float eps, const double* state) {
+int launch_adam_local_parts(void* stream, int64_t count, int n_parts, float* theta, float* gsum, const float* parts, float* m,
+                            float* v, float inv_m, float lr, float beta1, float beta2, float eps, const double* state) {
   if (count == 0) return 0;
   launch(adam_local_parts_kernel, (unsigned)((count + 255) / 256), 256, 0, (cudaStream_t)stream,
-      count, n_parts, theta, parts, m, v, inv_m, lr, beta1, beta2, eps, state);
+      count, n_parts, theta, gsum, parts, m, v, inv_m, lr, beta1, beta2, eps, state);
   note_launch();
   return (int)cudaGetLastError();
 }

@@ -535,3 +535,42 @@ def test_last_layer_gradients_for_every_number_of_classes(tiny_wl, c):
         _close(model.get(gcnsa.GET_GRAD_B, l), gb[l], what=f"db{l}")
     assert gcnsa.tc_status() == 0
     model.close(); parts.close()
+
+
+@pytest.mark.parametrize("agg_mode", [gcnsa.AGG_GRAD_AVG, gcnsa.AGG_PARAM_AVG])
+def test_a_gradient_set_before_an_epoch_is_part_of_its_sum(tiny_wl, agg_mode):
+    """gcnsa_model_set may put a gradient into the sum (a penalty on the weights, say): the epoch that follows adds the
+    partitions' gradients to it and clears it, bit for bit as the calls step by step do."""
+    w = tiny_wl
+    rng = np.random.default_rng(5)
+    extra = {(what, l): rng.standard_normal(s).astype(np.float32) for l, (a, b) in enumerate(zip(w.dims[:-1], w.dims[1:]))
+             for what, s in ((gcnsa.GET_GRAD_W, (a, b)), (gcnsa.GET_GRAD_B, (b,)))}
+    results = []
+    for how in ("steps", "plain", "recorded", "host"):
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            env = gcnsa.make_env(0)
+            parts = gcnsa.Parts(env, w.rowptr, w.col, w.x, w.y, w.train_mask, w.dims[-1], w.m, w.overlap_ppm, w.seed,
+                                w.part_mode, w.user_part, w.loss_on_halo)
+            model = gcnsa.Model(env, parts, w.dims, w.w0, w.b0, lr=w.lr, agg_mode=agg_mode, epoch_graph=how == "recorded")
+            for e in range(3):
+                if e != 1:
+                    for (what, l), g in extra.items():
+                        model.set(what, l, g)
+                if how == "steps":
+                    for p in range(w.m):
+                        model.forward(p)
+                        model.backward(p)
+                    model.step()
+                elif how == "host":
+                    xs = [np.ascontiguousarray(w.x[parts.members(p)]) for p in range(w.m)]
+                    model.epoch_host([x.ctypes.data for x in xs], np.zeros(1, np.float32))
+                else:
+                    model.epoch()
+                assert not any(model.get(what, l).any() for what, l in extra)
+            results.append([model.get(what, l) for what in (gcnsa.GET_W, gcnsa.GET_B, gcnsa.GET_ADAM_M_W) for l in range(2)])
+            model.close()
+            parts.close()
+    for other in results[1:]:
+        for a, b in zip(results[0], other):
+            assert np.array_equal(a, b)

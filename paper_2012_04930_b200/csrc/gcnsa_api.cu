@@ -99,7 +99,7 @@ struct gcnsa_model {
   std::vector<int64_t> ax_version;  // x_version of the partition the product was computed from (0 = none yet)
   uint64_t ax_uid = 0;
   std::vector<Lane> lanes;        // at least one
-  float* gparts = nullptr;        // [m x count]: the gradient of every partition of an epoch
+  float* gparts = nullptr;        // [m x count]: the gradient of every partition of an epoch; NULL: they go into gsum
   float* loss_parts = nullptr;
   // evaluation buffers (allocated on first gcnsa_evaluate)
   int32_t *ev_pred = nullptr, *ev_hits = nullptr;
@@ -464,13 +464,15 @@ static int copy_param(const gcnsa_model* M, float* base, int32_t layer, bool is_
 // without locality, one lane against eight: 8 000 rows of 8 entries, 64 wide (7 MB a lane) 587 -> 251 us per epoch, 64 000
 // rows (58 MB) 1 161 -> 954; three layers of 256, 32 000 rows (156 MB) 2 727 -> 2 508, 64 000 rows (294 MB) 4 871 -> 4 800,
 // 125 000 rows of 4 entries (556 MB) 9 101 -> 9 407, 250 000 rows (1.1 GB) 18 010 -> 18 240.  So the lanes after the first
-// together take at most 1 GB: seven of 146 MB, three of 294 MB, none of more than 1 GB.
+// together take at most 1 GB: seven of 146 MB, three of 294 MB, none of more than 1 GB.  Lanes need a gradient buffer per
+// partition; models with as many partitions and parameters that these would pass kGradBytes add into one sum instead, one
+// partition after the other.
 constexpr int64_t kMaxLanes = 8, kLaneNnz = 4 << 20;
-constexpr size_t kLaneBytes = (size_t)1 << 30;
+constexpr size_t kLaneBytes = (size_t)1 << 30, kGradBytes = (size_t)64 << 20;
 static int epoch_lanes(const gcnsa_model* M, const gcnsa_parts* parts, size_t lane_bytes) {
   int64_t nnz_max = 0;
   for (const DevPart& d : parts->parts) nnz_max = std::max<int64_t>(nnz_max, d.info.nnz);
-  if (!M->o.epoch_graph || M->env.stream() == nullptr || nnz_max > kLaneNnz) return 1;  // (the default stream records nothing)
+  if (!M->o.epoch_graph || M->env.stream() == nullptr || nnz_max > kLaneNnz || !M->gparts) return 1;  // (the default stream records nothing)
   return (int)std::min<int64_t>(std::min<int64_t>(parts->m, kMaxLanes), 1 + (int64_t)(kLaneBytes / lane_bytes));
 }
 
@@ -546,10 +548,10 @@ int gcnsa_model_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcn
   M->theta = (float*)M->dalloc(pbytes); M->gsum = (float*)M->dalloc(pbytes);
   M->am = (float*)M->dalloc(pbytes);    M->av = (float*)M->dalloc(pbytes);
   const size_t act = (size_t)M->n_max * (size_t)M->ld_max * sizeof(float);
-  M->gparts = (float*)M->dalloc(pbytes * (size_t)M->m);
   M->loss_parts = (float*)M->dalloc((size_t)(M->m + 1) * sizeof(float));
   M->adam_state = (double*)M->dalloc(4 * sizeof(double));
-  bool ok = M->theta && M->gsum && M->am && M->av && M->gparts && M->loss_parts && M->adam_state;
+  bool ok = M->theta && M->gsum && M->am && M->av && M->loss_parts && M->adam_state;
+  if (ok && pbytes * (size_t)M->m <= kGradBytes) ok = (M->gparts = (float*)M->dalloc(pbytes * (size_t)M->m)) != nullptr;
   size_t ws = 0, sc = softmax_ce_scratch(M->n_max);
   for (int l = 0; l < M->L; ++l) {
     const int64_t din = opts->dims[l], dout = opts->dims[l + 1];
@@ -610,7 +612,7 @@ int gcnsa_model_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcn
   if (e == cudaSuccess) e = cudaMemsetAsync(M->gsum, 0, pbytes, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(M->am, 0, pbytes, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(M->av, 0, pbytes, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(M->gparts, 0, pbytes * (size_t)M->m, s);
+  if (e == cudaSuccess && M->gparts) e = cudaMemsetAsync(M->gparts, 0, pbytes * (size_t)M->m, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(M->loss_parts, 0, (size_t)(M->m + 1) * sizeof(float), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(M->adam_state, 0, 4 * sizeof(double), s);
   for (Lane& W : M->lanes) {
@@ -847,6 +849,15 @@ int gcnsa_forward(gcnsa_model* M, const gcnsa_parts* P, int32_t p, float* loss_d
   return GCNSA_OK;
 }
 
+// this partition's own optimizer step from the aggregated parameters (Section 3.2), folded into the mean
+static int local_step(gcnsa_model* M, int32_t p, bool first) {
+  PROF(M, 2, 32.0 * M->count, 0.0,
+       launch_adam_local_dev(M->env.e.stream, M->count, M->theta, M->gsum, M->am_parts + (size_t)p * M->count,
+                             M->av_parts + (size_t)p * M->count, M->theta_acc, first, 1.0f / (float)M->m, M->o.lr, M->o.beta1,
+                             M->o.beta2, M->o.eps, M->adam_state));
+  return GCNSA_OK;
+}
+
 int gcnsa_backward(gcnsa_model* M, const gcnsa_parts* P, int32_t p) {
   if (!M || !P || p < 0 || p >= P->m) return fail(GCNSA_ERR_ARG, "bad partition index or NULL");
   if (M->last_forward != p) return fail(GCNSA_ERR_ORDER, "gcnsa_backward needs gcnsa_forward on the same partition first");
@@ -855,16 +866,25 @@ int gcnsa_backward(gcnsa_model* M, const gcnsa_parts* P, int32_t p) {
   const int rc = backward_lane(M, P, p, M->lanes[0], s, M->gsum, 1);
   if (rc) return rc;
   if (M->o.agg_mode == GCNSA_AGG_PARAM_AVG) {
-    // this partition's own optimizer step from the aggregated parameters (Section 3.2), folded into the mean
     if (M->accumulated == 0)  // t -> t + 1 once per epoch
       PROF(M, 2, 0.0, 0.0, launch_adam_advance(s, M->adam_state, M->o.beta1, M->o.beta2));
-    PROF(M, 2, 32.0 * M->count, 0.0,
-         launch_adam_local_dev(s, M->count, M->theta, M->gsum, M->am_parts + (size_t)p * M->count,
-                               M->av_parts + (size_t)p * M->count, M->theta_acc, M->accumulated == 0,
-                               1.0f / (float)M->m, M->o.lr, M->o.beta1, M->o.beta2, M->o.eps, M->adam_state));
+    const int rs = local_step(M, p, M->accumulated == 0);
+    if (rs) return rs;
   }
   M->last_forward = -1;
   M->accumulated += 1;
+  return GCNSA_OK;
+}
+
+// the step from the gradient sum, or the mean of the partitions' own steps as the new parameters
+static int sum_step(gcnsa_model* M) {
+  if (M->o.agg_mode == GCNSA_AGG_PARAM_AVG) {
+    CK(cudaMemcpyAsync(M->theta, M->theta_acc, (size_t)M->count * sizeof(float), cudaMemcpyDeviceToDevice, M->env.stream()));
+    return GCNSA_OK;
+  }
+  PROF(M, 2, 28.0 * M->count, 0.0,
+       launch_adam_dev(M->env.e.stream, M->count, M->theta, M->gsum, M->am, M->av, 1.0f / (float)M->m, M->o.lr,
+                       M->o.beta1, M->o.beta2, M->o.eps, M->adam_state));
   return GCNSA_OK;
 }
 
@@ -872,15 +892,10 @@ int gcnsa_step(gcnsa_model* M) {
   if (!M) return fail(GCNSA_ERR_ARG, "model is NULL");
   if (M->accumulated != M->m) return fail(GCNSA_ERR_ORDER, "gcnsa_step needs one backward pass per partition");
   M->t += 1;
-  if (M->o.agg_mode == GCNSA_AGG_PARAM_AVG) {
-    CK(cudaMemcpyAsync(M->theta, M->theta_acc, (size_t)M->count * sizeof(float), cudaMemcpyDeviceToDevice, M->env.stream()));
-    M->accumulated = 0;
-    return GCNSA_OK;
-  }
-  PROF(M, 2, 0.0, 0.0, launch_adam_advance(M->env.e.stream, M->adam_state, M->o.beta1, M->o.beta2));  // t -> t + 1
-  PROF(M, 2, 28.0 * M->count, 0.0,
-       launch_adam_dev(M->env.e.stream, M->count, M->theta, M->gsum, M->am, M->av, 1.0f / (float)M->m, M->o.lr,
-                       M->o.beta1, M->o.beta2, M->o.eps, M->adam_state));
+  if (M->o.agg_mode != GCNSA_AGG_PARAM_AVG)
+    PROF(M, 2, 0.0, 0.0, launch_adam_advance(M->env.e.stream, M->adam_state, M->o.beta1, M->o.beta2));  // t -> t + 1
+  const int rc = sum_step(M);
+  if (rc) return rc;
   M->accumulated = 0;
   return GCNSA_OK;
 }
@@ -916,8 +931,18 @@ struct Fork {
   }
 };
 
+// forward and backward pass of partition p of an epoch in lane W
+static int epoch_partition(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& W, cudaStream_t s) {
+  int rc = forward_lane(M, P, p, W, s);
+  if (rc) return rc;
+  if (M->gparts) return backward_lane(M, P, p, W, s, M->gparts + (size_t)p * M->count, 0);
+  rc = backward_lane(M, P, p, W, s, M->gsum, 1);
+  return rc == GCNSA_OK && M->o.agg_mode == GCNSA_AGG_PARAM_AVG ? local_step(M, p, p == 0) : rc;
+}
+
 // the step from the gradients of all partitions in gparts, on top of what gcnsa_model_set has left in the gradient sum
 static int optimizer_step(gcnsa_model* M, cudaStream_t s) {
+  if (!M->gparts) return sum_step(M);
   const float inv_m = 1.0f / (float)M->m;
   if (M->o.agg_mode == GCNSA_AGG_PARAM_AVG)
     PROF(M, 2, 32.0 * M->count * M->m, 0.0,
@@ -930,8 +955,8 @@ static int optimizer_step(gcnsa_model* M, cudaStream_t s) {
   return GCNSA_OK;
 }
 
-// One epoch: forward and backward of every partition, each with a gradient buffer of its own, then the optimizer over
-// all of them.  fork == NULL: everything on the model's stream, partition after partition.  Otherwise lane i takes
+// One epoch: forward and backward of every partition, each with a gradient buffer of its own (see kGradBytes), then the
+// optimizer over all of them.  fork == NULL: everything on the model's stream, partition after partition.  Otherwise lane i takes
 // partitions ..., i counted from the last one backwards in steps of the number of lanes (so lane 0 ends with the
 // activations of the last partition, as without lanes) on a branch of its own; the sums are added in partition order
 // in both cases, so the results are the same bit for bit.
@@ -944,12 +969,11 @@ static int epoch_body(gcnsa_model* M, const gcnsa_parts* P, float* loss_dev, For
   cudaStream_t aux = fork ? fork->side[lanes - 1] : s;
   if (fork)
     for (cudaStream_t st : fork->side) CK(fork->edge(s, st));
-  PROF(M, 2, 0.0, 0.0, launch_adam_advance(aux, M->adam_state, M->o.beta1, M->o.beta2));  // t -> t + 1
+  // t -> t + 1 (the steps of the partitions, where they come one by one, are on s)
+  PROF(M, 2, 0.0, 0.0, launch_adam_advance(M->gparts ? aux : s, M->adam_state, M->o.beta1, M->o.beta2));
   for (int32_t p = 0; p < P->m; ++p) {
     const int lane = (P->m - 1 - p) % lanes;
-    rc = forward_lane(M, P, p, M->lanes[lane], stream_of(lane));
-    if (rc == GCNSA_OK)
-      rc = backward_lane(M, P, p, M->lanes[lane], stream_of(lane), M->gparts + (size_t)p * M->count, 0);
+    rc = epoch_partition(M, P, p, M->lanes[lane], stream_of(lane));
     if (rc) return rc;
   }
   if (fork)
@@ -1055,6 +1079,7 @@ int gcnsa_epoch_host(gcnsa_model* M, gcnsa_parts* P, const float* const* x_host,
     return e == cudaSuccess ? cudaEventRecord(P->ready[p], P->copy_stream) : e;
   };
   for (int32_t p = 0; p < std::min(P->m, 2); ++p) CK(copy_in(p));
+  PROF(M, 2, 0.0, 0.0, launch_adam_advance(s, M->adam_state, M->o.beta1, M->o.beta2));  // t -> t + 1
   for (int32_t p = 0; p < P->m; ++p) {
     const DevPart& d = P->parts[p];
     CK(cudaStreamWaitEvent(s, P->ready[p], 0));
@@ -1062,11 +1087,9 @@ int gcnsa_epoch_host(gcnsa_model* M, gcnsa_parts* P, const float* const* x_host,
     P->x_version[p] += 1;
     CK(cudaEventRecord(P->consumed[p & 1], s));
     if (p + 2 < P->m) CK(copy_in(p + 2));
-    rc = forward_lane(M, P, p, M->lanes[0], s);
-    if (rc == GCNSA_OK) rc = backward_lane(M, P, p, M->lanes[0], s, M->gparts + (size_t)p * M->count, 0);
+    rc = epoch_partition(M, P, p, M->lanes[0], s);
     if (rc) return rc;
   }
-  PROF(M, 2, 0.0, 0.0, launch_adam_advance(s, M->adam_state, M->o.beta1, M->o.beta2));  // t -> t + 1
   rc = optimizer_step(M, s);
   if (rc) return rc;
   M->last_forward = -1;

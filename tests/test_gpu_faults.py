@@ -279,6 +279,41 @@ def test_side_by_side_partitions_take_bounded_memory():
         assert held["plain"] < held["recorded"] <= held["plain"] + (1 << 30)
 
 
+def test_many_partitions_of_a_large_model_share_one_gradient_sum():
+    """The gradients of the partitions of an epoch are kept apart up to 64 MB; beyond that the memory of a model does not
+    grow with the number of partitions times its parameters, and an epoch is bit for bit that of the calls step by step."""
+    rng = np.random.default_rng(1)
+    dims = [4000, 64, 3]
+    w0 = [rng.standard_normal(s).astype(np.float32) * 0.05 for s in zip(dims[:-1], dims[1:])]
+    with torch.cuda.stream(torch.cuda.Stream()):
+        held = {}
+        for m in (1, 100):
+            parts = _sparse_parts(gcnsa.make_env(0), m, 50, dims[0], dims[-1])
+            alloc = FailingAllocator()
+            model = gcnsa.Model(alloc.env(), parts, dims, w0, epoch_graph=0)
+            held[m] = sum(alloc.live.values())
+            model.close()
+        assert held[100] <= held[1]
+        for agg_mode in (gcnsa.AGG_GRAD_AVG, gcnsa.AGG_PARAM_AVG):
+            got = []
+            for how in ("steps", "plain", "recorded"):
+                model = gcnsa.Model(gcnsa.make_env(0), parts, dims, w0, agg_mode=agg_mode, epoch_graph=how == "recorded")
+                for _ in range(3):
+                    if how != "steps":
+                        model.epoch()
+                        continue
+                    for p in range(100):
+                        model.forward(p)
+                        model.backward(p)
+                    model.step()
+                got.append([model.get(what, l) for what in (gcnsa.GET_W, gcnsa.GET_B) for l in range(2)])
+                model.close()
+            for other in got[1:]:
+                for x, y in zip(got[0], other):
+                    assert np.array_equal(x, y)
+        parts.close()
+
+
 @pytest.mark.parametrize("agg_mode,cache_ax", [(gcnsa.AGG_GRAD_AVG, 1), (gcnsa.AGG_PARAM_AVG, 0)])
 def test_buffers_a_model_needs_come_before_those_that_save_time(agg_mode, cache_ax):
     """An allocator with just the memory of a model that records nothing: the same model that records is created too."""

@@ -598,10 +598,13 @@ int gcnsa_sage_destroy(gcnsa_sage* S) {
 // two dozen kernels of a batch are a chain of microseconds on a fraction of the SMs, so workers side by side overlap
 // (116 K vertices, 5 workers, batches of 256: 63.2 ms per epoch with one lane, 47.7 with two, 38.4 with four, 29.9
 // with five; 20 000 vertices, 4 workers: 7.7 -> 4.2 ms).  Larger batches fill the chip by themselves and their lanes
-// would cost gigabytes.
-static int sage_lanes(int32_t m, int64_t max_rows1) {
+// would cost gigabytes.  The lanes after the first take at most 1 GB (a batch of 2 816 rows of 602 features 17 MB each; with
+// fan-outs in the thousands the sample lists alone can be half a gigabyte).  The default stream runs one worker at a time.
+static int sage_lanes(int32_t m, int64_t max_rows1, size_t lane_bytes, cudaStream_t s) {
   constexpr int64_t kLaneRows = 32768;
-  return max_rows1 > kLaneRows ? 1 : std::max(1, std::min<int>(m, 8));
+  constexpr size_t kLaneBytes = (size_t)1 << 30;
+  if (max_rows1 > kLaneRows || s == nullptr) return 1;
+  return (int)std::min<int64_t>(std::min<int>(m, 8), 1 + (int64_t)(kLaneBytes / lane_bytes));
 }
 
 int gcnsa_sage_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcnsa_sage_opts* opts,
@@ -697,7 +700,10 @@ int gcnsa_sage_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcns
     return (int)GCNSA_OK;
   };
   int rc = obtain(wants);
-  S->lanes.resize((size_t)sage_lanes(S->m, S->max_rows1));
+  S->lanes.resize(1);
+  size_t lane_bytes = 0;
+  for (const Want& w : lane_wants(S->lanes[0])) lane_bytes += std::max<size_t>(w.bytes, 256);
+  S->lanes.resize((size_t)sage_lanes(S->m, S->max_rows1, lane_bytes, s));
   for (size_t i = 0; i < S->lanes.size() && rc == GCNSA_OK; ++i) {
     const size_t mark = S->owned.size();
     rc = obtain(lane_wants(S->lanes[i]));

@@ -344,3 +344,24 @@ def test_buffers_a_model_needs_come_before_those_that_save_time(agg_mode, cache_
             m.close()
         assert losses[0] == losses[1] and not alloc.live
         parts.close()
+
+
+def test_workers_side_by_side_take_bounded_memory():
+    """GraphSAGE: the buffers of the workers after the first, at most 1 GiB together; none on the default stream."""
+    dims = [16, 8, 3]
+    rng = np.random.default_rng(1)
+    ws = [rng.standard_normal(s).astype(np.float32) * 0.05 for s in zip(dims[:-1], dims[1:])]
+    held = {}
+    for fanout, batch in (((2000, 1), 16_000), ((4, 3), 64)):   # a quarter of a gigabyte of sample lists a worker; little
+        for name, stream in (("own", torch.cuda.Stream()), ("default", torch.cuda.default_stream())):
+            with torch.cuda.stream(stream):
+                alloc = FailingAllocator()
+                parts = _sparse_parts(gcnsa.make_env(0), 8, 300, dims[0], dims[-1])
+                model = gcnsa.Sage(alloc.env(), parts, dims, ws, ws, fanout=fanout, batch=batch)
+                held[name] = sum(alloc.live.values())
+                model.epoch()
+                stream.synchronize()
+                model.close()
+                parts.close()
+                assert not alloc.live
+        assert held["default"] < held["own"] <= held["default"] + (1 << 30)

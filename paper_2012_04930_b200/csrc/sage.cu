@@ -377,7 +377,8 @@ struct gcnsa_sage {
   cudaEvent_t fork_ev = nullptr;
   std::vector<cudaEvent_t> join_ev;
   int work_p = 0;                // whose copy GCNSA_SAGE_WORK_* and the step-by-step calls address
-  int64_t last_nb = 0, last_rows1 = 0;
+  int64_t last_nb = 0, last_rows1 = 0;  // the latest batch, in the buffers of lane last_lane
+  int last_lane = 0;
   // recorded full-size batch of every worker (batch_graph): keyed by the partitions object
   std::vector<cudaGraphExec_t> batch_exec;
   std::vector<int> batch_kernels;
@@ -773,6 +774,7 @@ int gcnsa_sage_batch(gcnsa_sage* S, const gcnsa_parts* P, int32_t p, int64_t epo
     SCK(cudaMemcpyAsync(S->copies + (size_t)p * S->count, S->copies + (size_t)S->work_p * S->count,
                         (size_t)S->count * sizeof(float), cudaMemcpyDeviceToDevice, s));
   S->work_p = p;
+  S->last_lane = 0;
   SageLane& W = S->lanes[0];
   rc = run_batch(S, P, p, epoch, b, apply != 0, W, s);
   if (rc) return rc;
@@ -834,7 +836,7 @@ int gcnsa_sage_epoch(gcnsa_sage* S, const gcnsa_parts* P, float* loss_dev) {
     a.p = p; a.b = 0; a.nbatch = n_batches(S, P, p); a.nreplay = 0;
     // the worker starts the epoch from the aggregated parameters (Section 3.2)
     SCK(cudaMemcpyAsync(S->copies + (size_t)p * S->count, S->theta, pb, cudaMemcpyDeviceToDevice, st));
-    SCK(cudaMemsetAsync(W.loss, 0, 2 * sizeof(float), st));
+    SCK(cudaMemsetAsync(W.loss + 1, 0, sizeof(float), st));
     // the worker's full-size batches are one kernel sequence with the same shapes: recorded once per worker and
     // replayed, the batch index advancing on the device; the ragged last batch runs as plain launches
     const int64_t nfull = P->parts[p].info.n_train / S->o.batch;
@@ -893,12 +895,14 @@ int gcnsa_sage_epoch(gcnsa_sage* S, const gcnsa_parts* P, float* loss_dev) {
       }
     }
   }
-  {  // the shape of the last worker's last batch is what gcnsa_sage_batch_export describes
-    const int64_t nt = P->parts[P->m - 1].info.n_train;
-    if (nt > 0) {
-      S->last_nb = nt - (n_batches(S, P, P->m - 1) - 1) * S->o.batch;
-      S->last_rows1 = S->last_nb * (1 + S->o.fanout[1]);
-    }
+  // what gcnsa_sage_batch_export describes: the last batch of the last worker that has any
+  for (int32_t p = P->m - 1; p >= 0; --p) {
+    const int64_t nt = P->parts[p].info.n_train;
+    if (nt == 0) continue;
+    S->last_nb = nt - (n_batches(S, P, p) - 1) * S->o.batch;
+    S->last_rows1 = S->last_nb * (1 + S->o.fanout[1]);
+    S->last_lane = (P->m - 1 - p) % lanes;
+    break;
   }
   for (int i = 1; i < lanes; ++i) {
     SCK(cudaEventRecord(S->join_ev[i - 1], stream_of(i)));
@@ -963,7 +967,7 @@ int gcnsa_sage_batch_export(const gcnsa_sage* S, const gcnsa_sage_batch_host* ds
   cudaStream_t s = S->env.stream();
   const size_t nb = (size_t)S->last_nb, rows1 = (size_t)S->last_rows1;
   const size_t r1 = (size_t)S->o.fanout[0];
-  const SageLane& W = S->lanes[0];
+  const SageLane& W = S->lanes[S->last_lane];
   if (dst->vertices && rows1) SCK(cudaMemcpyAsync(dst->vertices, W.b1, rows1 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   if (dst->count2 && nb) SCK(cudaMemcpyAsync(dst->count2, W.cnt2, nb * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   if (dst->samples1 && rows1 && r1)
@@ -989,7 +993,7 @@ static int sage_param(const gcnsa_sage* S, int32_t what, int32_t layer, float** 
   if (layer < 0 || layer > 1) return fail(GCNSA_ERR_ARG, "layer out of range");
   const int kind = what % 3, which = what / 3;  // kind: self, neighbour, bias; which: aggregated, working copy, gradient
   float* buf = which == 0 ? S->theta : which == 1 ? S->copies + (size_t)S->work_p * S->count
-                          : which == 2 ? S->lanes[0].grad : nullptr;
+                          : which == 2 ? S->lanes[S->last_lane].grad : nullptr;
   if (!buf || what < 0) return fail(GCNSA_ERR_ARG, "unknown tensor id");
   const int64_t din = layer == 0 ? S->f : S->h, dout = layer == 0 ? S->h : S->c;
   const int64_t ldin = layer == 0 ? S->ldf : S->ldh, ldo = layer == 0 ? S->ldh : S->ldc;

@@ -233,6 +233,38 @@ def test_workers_side_by_side_equal_workers_one_after_another(tiny_wl, m):
         assert np.array_equal(b0[key], b1[key]), key
 
 
+@pytest.mark.parametrize("idle", [1, 2, 3])
+def test_latest_batch_of_an_epoch_whose_last_workers_have_none(tiny_wl, idle):
+    """The last `idle` of four workers have no training vertices: after an epoch the export describes the last batch of the
+    last worker that has any, workers side by side as one after another (default stream)."""
+    w = tiny_wl
+    n = w.rowptr.size - 1
+    user = (np.arange(n) * 4 // n).astype(np.int32)
+    mask = ((user < 4 - idle) & (np.arange(n) % 3 > 0)).astype(np.uint8)
+    dims = [w.dims[0], 16, w.dims[-1]]
+    ws, wn, bs = configs.sage_weights(dims, 3)
+    got = []
+    for stream in (torch.cuda.default_stream(), torch.cuda.Stream()):
+        with torch.cuda.stream(stream):
+            env = gcnsa.make_env(0)
+            parts = gcnsa.Parts(env, w.rowptr, w.col, w.x, w.y, mask, w.dims[-1], 4, 100_000, 5, gcnsa.PART_USER, user,
+                                loss_on_halo=0)
+            assert [parts.info(p).n_train > 0 for p in range(4)] == [True] * (4 - idle) + [False] * idle
+            model = gcnsa.Sage(env, parts, dims, ws, wn, bs, fanout=(4, 3), batch=64, seed=9)
+            for _ in range(2):
+                model.epoch()
+            got.append(model.batch_export())
+            model.run_batch(0, 0, 0)
+            got.append(model.batch_export())
+            got.append({"grad": model.get(gcnsa.SAGE_GRAD_W_SELF, 0)})
+            assert got[-1]["grad"].any()
+            model.close()
+            parts.close()
+    for one, other in zip(got[:3], got[3:]):
+        for key in one:
+            assert np.array_equal(one[key], other[key]), key
+
+
 def test_runs_are_bitwise_reproducible_and_arguments_are_checked(tiny_wl):
     w = tiny_wl
     outs = []

@@ -860,41 +860,51 @@ int gcnsa_sage_epoch(gcnsa_sage* S, const gcnsa_parts* P, float* loss_dev) {
     SLAUNCHED("sage_loss_fold");
     return GCNSA_OK;
   };
-  int open = 0;
-  for (int i = 0; i < lanes; ++i) {
-    const int32_t first = (P->m - 1 - i) % lanes;  // the smallest p with (m - 1 - p) % lanes == i
-    rc = begin(i, first);
-    if (rc) return rc;
-    ++open;
-  }
-  while (open > 0) {  // one batch of every lane in turn, so that all streams are fed
+  auto workers = [&]() -> int {
+    int open = 0;
     for (int i = 0; i < lanes; ++i) {
-      At& a = at[i];
-      if (a.p < 0) continue;
-      if (a.b < a.nreplay) {
-        SCK(cudaGraphLaunch(S->batch_exec[a.p], stream_of(i)));
-        note_launch(S->batch_kernels[a.p]);
-        S->last_nb = S->o.batch;
-        S->last_rows1 = (int64_t)S->o.batch * (1 + S->o.fanout[1]);
-        ++a.b;
-      } else if (a.b < a.nbatch) {
-        rc = run_batch(S, P, a.p, S->epoch, a.b, true, S->lanes[i], stream_of(i));
-        if (rc) return rc;
-        ++a.b;
-      }
-      if (a.b < a.nbatch) continue;
-      rc = finish(i);
-      if (rc) return rc;
-      const int32_t next = a.p + lanes;
-      if (next < P->m) {
-        rc = begin(i, next);
-        if (rc) return rc;
-      } else {
-        a.p = -1;
-        --open;
+      const int32_t first = (P->m - 1 - i) % lanes;  // the smallest p with (m - 1 - p) % lanes == i
+      const int r = begin(i, first);
+      if (r) return r;
+      ++open;
+    }
+    while (open > 0) {  // one batch of every lane in turn, so that all streams are fed
+      for (int i = 0; i < lanes; ++i) {
+        At& a = at[i];
+        if (a.p < 0) continue;
+        if (a.b < a.nreplay) {
+          SCK(cudaGraphLaunch(S->batch_exec[a.p], stream_of(i)));
+          note_launch(S->batch_kernels[a.p]);
+          S->last_nb = S->o.batch;
+          S->last_rows1 = (int64_t)S->o.batch * (1 + S->o.fanout[1]);
+          ++a.b;
+        } else if (a.b < a.nbatch) {
+          const int r = run_batch(S, P, a.p, S->epoch, a.b, true, S->lanes[i], stream_of(i));
+          if (r) return r;
+          ++a.b;
+        }
+        if (a.b < a.nbatch) continue;
+        int r = finish(i);
+        if (r) return r;
+        const int32_t next = a.p + lanes;
+        if (next < P->m) {
+          r = begin(i, next);
+          if (r) return r;
+        } else {
+          a.p = -1;
+          --open;
+        }
       }
     }
+    return GCNSA_OK;
+  };
+  rc = workers();
+  // (also when a worker has failed: what the others have been given ends before what follows on the caller's stream)
+  for (int i = 1; i < lanes; ++i) {
+    SCK(cudaEventRecord(S->join_ev[i - 1], stream_of(i)));
+    SCK(cudaStreamWaitEvent(s, S->join_ev[i - 1], 0));
   }
+  if (rc) return rc;
   // what gcnsa_sage_batch_export describes: the last batch of the last worker that has any
   for (int32_t p = P->m - 1; p >= 0; --p) {
     const int64_t nt = P->parts[p].info.n_train;
@@ -903,10 +913,6 @@ int gcnsa_sage_epoch(gcnsa_sage* S, const gcnsa_parts* P, float* loss_dev) {
     S->last_rows1 = S->last_nb * (1 + S->o.fanout[1]);
     S->last_lane = (P->m - 1 - p) % lanes;
     break;
-  }
-  for (int i = 1; i < lanes; ++i) {
-    SCK(cudaEventRecord(S->join_ev[i - 1], stream_of(i)));
-    SCK(cudaStreamWaitEvent(s, S->join_ev[i - 1], 0));
   }
   S->work_p = P->m - 1;
   launch(sage_param_mean, blocks_for(S->count, 256), 256, 0, s, S->count, P->m, S->copies, S->theta,

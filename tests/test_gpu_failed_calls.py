@@ -1,0 +1,123 @@
+"""Calls of the runtime that fail in the middle of an epoch, made on the host: the library's objects are linked a second
+time with a few runtime functions wrapped, a chosen kernel launch returns an error without being made, and what the
+library does with its streams after that is counted.  Runs in a child process (a process loads one build); nothing
+here faults, traps or hangs the GPU."""
+import json
+import os
+import subprocess
+import sys
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+if ROOT not in sys.path:
+    sys.path.insert(0, ROOT)
+
+pytestmark = pytest.mark.gpu
+
+SHIM = r"""
+#include <cuda_runtime.h>
+static int fail_at = 0, calls = 0, pending = 0, failed = 0, waits = 0, syncs = 0;
+static cudaStream_t own = nullptr;
+extern "C" {
+// launch number `at` (1-based, 0 = none) from now on fails; events are counted from then on
+void shim_arm(int at, void* stream) { fail_at = at; calls = pending = failed = waits = syncs = 0; own = (cudaStream_t)stream; }
+int shim_launches() { return calls; }
+int shim_waits_of_own() { return waits; }    // waits given to the caller's stream after the failure
+int shim_syncs_of_others() { return syncs; }  // other streams waited for on the host after the failure
+cudaError_t __real_cudaLaunchKernelExC(const cudaLaunchConfig_t*, const void*, void**);
+cudaError_t __real_cudaGetLastError();
+cudaError_t __real_cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned);
+cudaError_t __real_cudaStreamSynchronize(cudaStream_t);
+cudaError_t __wrap_cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void** a) {
+  if (++calls == fail_at) { pending = failed = 1; return cudaErrorLaunchOutOfResources; }
+  return __real_cudaLaunchKernelExC(c, f, a);
+}
+cudaError_t __wrap_cudaGetLastError() {
+  if (pending) { pending = 0; return cudaErrorLaunchOutOfResources; }
+  return __real_cudaGetLastError();
+}
+cudaError_t __wrap_cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t e, unsigned f) {
+  if (failed && s == own) ++waits;
+  return __real_cudaStreamWaitEvent(s, e, f);
+}
+cudaError_t __wrap_cudaStreamSynchronize(cudaStream_t s) {
+  if (failed && s != own) ++syncs;
+  return __real_cudaStreamSynchronize(s);
+}
+}
+"""
+WRAPPED = ("cudaLaunchKernelExC", "cudaGetLastError", "cudaStreamWaitEvent", "cudaStreamSynchronize")
+
+
+def _run(scenario, tmp_path):
+    from paper_2012_04930_b200 import build
+    build.build()
+    shim = tmp_path / "shim.cpp"
+    shim.write_text(SHIM)
+    objs = []
+    for src in build.sources():
+        obj = build._object(src, False)
+        if not os.path.exists(obj):
+            obj = str(tmp_path / (os.path.basename(src) + ".o"))
+            subprocess.check_call(["nvcc", *build._flags(False, False), "-c", "-o", obj, src])
+        objs.append(obj)
+    lib = str(tmp_path / "libgcnsa_wrapped.so")
+    subprocess.check_call(["nvcc", *build._ARCH, "-Xcompiler", "-fPIC", "-shared", "-o", lib, str(shim), *objs,
+                           *[a for f in WRAPPED for a in ("-Xlinker", f"--wrap={f}")]])
+    child = subprocess.run([sys.executable, os.path.abspath(__file__), scenario, lib], capture_output=True, text=True,
+                           timeout=300)
+    assert child.returncode == 0, child.stderr[-2000:]
+    return json.loads(child.stdout.strip().splitlines()[-1])
+
+
+def _child(scenario):
+    import numpy as np
+    import torch
+    from gen import configs
+    from paper_2012_04930_b200 import gcnsa
+    w = configs.small()
+    L, out = gcnsa.lib(), []
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        env = gcnsa.make_env(0)
+        parts = gcnsa.Parts(env, w.rowptr, w.col, w.x, w.y, w.train_mask, w.dims[-1], w.m, w.overlap_ppm, w.seed,
+                            w.part_mode, w.user_part, w.loss_on_halo)
+        dims = [w.dims[0], 16, w.dims[-1]]
+        ws, wn, bs = configs.sage_weights(dims, 3)
+        model = gcnsa.Sage(env, parts, dims, ws, wn, bs, batch=256, batch_graph=0)
+        call = model.epoch
+        call()
+        L.shim_arm(0, stream.cuda_stream)
+        call()
+        total = L.shim_launches()
+        for at in (2, total // 3, total // 2, total - 40):
+            L.shim_arm(at, stream.cuda_stream)
+            try:
+                call()
+                code = 0
+            except gcnsa.GcnsaError as e:
+                code = e.code
+            out.append([code, L.shim_waits_of_own(), L.shim_syncs_of_others()])
+            stream.synchronize()
+        L.shim_arm(0, stream.cuda_stream)
+        call()                       # and the object is usable
+        stream.synchronize()
+        model.close()
+        parts.close()
+    print(json.dumps({"m": w.m, "out": out, "err_cuda": gcnsa.ERR_CUDA}))
+
+
+def test_a_failed_sage_epoch_joins_its_workers(tmp_path):
+    """The workers' streams are joined to the caller's however an epoch ends: one wait each after the failure."""
+    got = _run("sage", tmp_path)
+    for code, waits, _ in got["out"]:
+        assert code == got["err_cuda"]
+        assert waits == got["m"] - 1
+
+
+if __name__ == "__main__":
+    if len(sys.argv) == 3:
+        from paper_2012_04930_b200 import gcnsa
+        gcnsa.use_library(sys.argv[2])
+        _child(sys.argv[1])

@@ -1078,20 +1078,26 @@ int gcnsa_epoch_host(gcnsa_model* M, gcnsa_parts* P, const float* const* x_host,
                           cudaMemcpyHostToDevice, P->copy_stream);
     return e == cudaSuccess ? cudaEventRecord(P->ready[p], P->copy_stream) : e;
   };
-  for (int32_t p = 0; p < std::min(P->m, 2); ++p) CK(copy_in(p));
-  PROF(M, 2, 0.0, 0.0, launch_adam_advance(s, M->adam_state, M->o.beta1, M->o.beta2));  // t -> t + 1
-  for (int32_t p = 0; p < P->m; ++p) {
-    const DevPart& d = P->parts[p];
-    CK(cudaStreamWaitEvent(s, P->ready[p], 0));
-    CKL(launch_copy_rows(s, d.info.n, P->f, P->staging[p & 1], P->f, d.x, P->ldx));
-    P->x_version[p] += 1;
-    CK(cudaEventRecord(P->consumed[p & 1], s));
-    if (p + 2 < P->m) CK(copy_in(p + 2));
-    rc = epoch_partition(M, P, p, M->lanes[0], s);
-    if (rc) return rc;
+  auto epoch = [&]() -> int {
+    for (int32_t p = 0; p < std::min(P->m, 2); ++p) CK(copy_in(p));
+    PROF(M, 2, 0.0, 0.0, launch_adam_advance(s, M->adam_state, M->o.beta1, M->o.beta2));  // t -> t + 1
+    for (int32_t p = 0; p < P->m; ++p) {
+      const DevPart& d = P->parts[p];
+      CK(cudaStreamWaitEvent(s, P->ready[p], 0));
+      CKL(launch_copy_rows(s, d.info.n, P->f, P->staging[p & 1], P->f, d.x, P->ldx));
+      P->x_version[p] += 1;
+      CK(cudaEventRecord(P->consumed[p & 1], s));
+      if (p + 2 < P->m) CK(copy_in(p + 2));
+      const int r = epoch_partition(M, P, p, M->lanes[0], s);
+      if (r) return r;
+    }
+    return optimizer_step(M, s);
+  };
+  rc = epoch();
+  if (rc) {  // copies may be on their way: the caller's buffers are not read after the call
+    cudaStreamSynchronize(P->copy_stream);
+    return rc;
   }
-  rc = optimizer_step(M, s);
-  if (rc) return rc;
   M->last_forward = -1;
   M->last_n = P->parts[P->m - 1].info.n;
   M->t += 1;

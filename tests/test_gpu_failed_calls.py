@@ -83,15 +83,21 @@ def _child(scenario):
         env = gcnsa.make_env(0)
         parts = gcnsa.Parts(env, w.rowptr, w.col, w.x, w.y, w.train_mask, w.dims[-1], w.m, w.overlap_ppm, w.seed,
                             w.part_mode, w.user_part, w.loss_on_halo)
-        dims = [w.dims[0], 16, w.dims[-1]]
-        ws, wn, bs = configs.sage_weights(dims, 3)
-        model = gcnsa.Sage(env, parts, dims, ws, wn, bs, batch=256, batch_graph=0)
-        call = model.epoch
+        if scenario == "sage":
+            dims = [w.dims[0], 16, w.dims[-1]]
+            ws, wn, bs = configs.sage_weights(dims, 3)
+            model = gcnsa.Sage(env, parts, dims, ws, wn, bs, batch=256, batch_graph=0)
+            call = model.epoch
+        else:
+            model = gcnsa.Model(env, parts, w.dims, w.w0, w.b0, lr=w.lr)
+            xs = [torch.from_numpy(w.x[parts.members(p)]).pin_memory() for p in range(w.m)]
+            loss = np.zeros(1, np.float32)
+            call = lambda: model.epoch_host([x.data_ptr() for x in xs], loss)  # noqa: E731
         call()
         L.shim_arm(0, stream.cuda_stream)
         call()
         total = L.shim_launches()
-        for at in (2, total // 3, total // 2, total - 40):
+        for at in (2, total // 3, total // 2, total - total // 20):
             L.shim_arm(at, stream.cuda_stream)
             try:
                 call()
@@ -114,6 +120,14 @@ def test_a_failed_sage_epoch_joins_its_workers(tmp_path):
     for code, waits, _ in got["out"]:
         assert code == got["err_cuda"]
         assert waits == got["m"] - 1
+
+
+def test_a_failed_epoch_from_host_buffers_reads_them_no_longer(tmp_path):
+    """The copies of the caller's buffers have ended when a failed call returns: their stream is waited for."""
+    got = _run("host", tmp_path)
+    for code, _, syncs in got["out"]:
+        assert code == got["err_cuda"]
+        assert syncs == 1
 
 
 if __name__ == "__main__":

@@ -1374,7 +1374,8 @@ int gcnsa_op_gemm_mask_colsum(void* stream, int32_t mode, int32_t ta, int32_t tb
     return fail(GCNSA_ERR_ARG, "unknown gemm mode");
   if (n > 0 && !out) return fail(GCNSA_ERR_ARG, "NULL pointer");
   if (m == 0 || n == 0) {
-    if (n > 0 && !accumulate) CK(cudaMemsetAsync(out, 0, (size_t)n * sizeof(float), (cudaStream_t)stream));
+    CKL(launch_gemm_mask_colsum(stream, mode, ta, tb, m, n, k, a, lda, b, ldb, c, ldc, mask, ldmask, row_scale, out, accumulate,
+                                scratch, workspace, workspace_bytes));
     return GCNSA_OK;
   }
   if (!c || !mask || (k > 0 && (!a || !b))) return fail(GCNSA_ERR_ARG, "NULL pointer");

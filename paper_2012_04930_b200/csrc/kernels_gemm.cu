@@ -392,7 +392,9 @@ int launch_gemm_mask_colsum(void* stream, int32_t mode, int32_t ta, int32_t tb, 
                             const float* a, int64_t lda, const float* b, int64_t ldb, float* c, int64_t ldc,
                             const float* mask, int64_t ldmask, const float* row_scale, float* out, int32_t accumulate,
                             void* scratch, void* workspace, size_t workspace_bytes) {
-  if (m == 0 || n == 0) return 0;
+  if (n == 0) return 0;
+  if (m == 0)  // no rows: sums of nothing
+    return accumulate ? 0 : (int)cudaMemsetAsync(out, 0, (size_t)n * sizeof(float), (cudaStream_t)stream);
   if (mode != GCNSA_GEMM_FP32 && k > 0) {
     const int r = launch_gemm_tc(stream, ta, tb, m, n, k, a, lda, b, ldb, c, ldc, 0, GCNSA_EPI_MASK, mask, ldmask, workspace,
                                  workspace_bytes, mode == GCNSA_GEMM_TF32 ? 1 : 3, (float*)scratch, row_scale);

@@ -574,3 +574,33 @@ def test_a_gradient_set_before_an_epoch_is_part_of_its_sum(tiny_wl, agg_mode):
     for other in results[1:]:
         for a, b in zip(results[0], other):
             assert np.array_equal(a, b)
+
+
+def test_an_empty_partition_leaves_no_bias_gradient_of_other_partitions(tiny_wl):
+    """One model trained in turn on two cuts of a graph, the second with an empty partition: that partition adds nothing to
+    the sum, so an epoch is bit for bit that of the calls step by step."""
+    w = tiny_wl
+    n = w.rowptr.size - 1
+    even = (np.arange(n) * 3 // n).astype(np.int32)
+    got = []
+    for how in ("steps", "epoch"):
+        env = gcnsa.make_env(0)
+        cuts = [gcnsa.Parts(env, w.rowptr, w.col, w.x, w.y, w.train_mask, w.dims[-1], 3, 0, 5, gcnsa.PART_USER, user)
+                for user in (np.zeros(n, np.int32), even, np.where(even == 1, 2, even).astype(np.int32))]
+        assert cuts[2].info(1).n == 0
+        model = gcnsa.Model(env, cuts[0], w.dims, w.w0, w.b0, lr=w.lr, epoch_graph=0)
+        for parts in (cuts[1], cuts[2], cuts[2]):
+            model.parts = parts
+            if how == "epoch":
+                model.epoch()
+                continue
+            for p in range(3):
+                model.forward(p)
+                model.backward(p)
+            model.step()
+        got.append([model.get(what, l) for what in (gcnsa.GET_W, gcnsa.GET_B, gcnsa.GET_ADAM_M_B) for l in range(2)])
+        model.close()
+        for parts in cuts:
+            parts.close()
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)

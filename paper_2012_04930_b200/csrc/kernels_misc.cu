@@ -100,8 +100,8 @@ softmax_ce_groups(int64_t n, int c, const float* __restrict__ logits, int64_t ld
       const int q = v * G + g;
       float d[4];
 #pragma unroll
-      for (int k = 0; k < 4; ++k)
-        d[k] = on ? (z[4 * v + k] * inv_se - (4 * q + k == yi ? 1.f : 0.f)) * inv_nt : 0.f;
+      for (int k = 0; k < 4; ++k)  // (pad columns are zeros also where the row's sum is not finite)
+        d[k] = on && 4 * q + k < c ? (z[4 * v + k] * inv_se - (4 * q + k == yi ? 1.f : 0.f)) * inv_nt : 0.f;
       cs[v].x += d[0]; cs[v].y += d[1]; cs[v].z += d[2]; cs[v].w += d[3];
       if (in && q < nq) {
         *(reinterpret_cast<float4*>(grad + row * ldg) + q) = make_float4(d[0], d[1], d[2], d[3]);

@@ -242,6 +242,27 @@ def test_softmax_cross_entropy_extreme_logits():
     assert abs(loss.item() - (2e4 + np.log1p(np.exp(-10.0) + np.exp(-20.0))) / 2) < 1e-2
 
 
+@pytest.mark.parametrize("c", [3, 33, 65, 130, 257])
+def test_softmax_cross_entropy_of_rows_that_are_not_finite(c):
+    """A row with NaN or infinite logits has a gradient that is not finite in its own columns only: pad columns are zeros,
+    and other rows are what they are without it."""
+    rng = np.random.default_rng(c)
+    z = rng.standard_normal((6, c)).astype(np.float32)
+    y, mask = _dev(rng.integers(0, c, 6).astype(np.int32)), _dev(np.array([1, 1, 1, 1, 1, 0], np.uint8))
+    sc = torch.empty(64, device="cuda")
+    ld = _ld(c) + 4
+    grads = []
+    for bad in (False, True):
+        if bad:
+            z[0], z[2, 1], z[4, 0], z[5] = -np.inf, np.nan, np.inf, np.nan
+        gd, loss = torch.full((6, ld), 9.0, device="cuda"), torch.empty(1, device="cuda")
+        gcnsa.op_softmax_ce(_padded(z, ld), c, y, mask, 5, loss, gd, sc)
+        grads.append(gd)
+        assert torch.all(gd[:, c:(c + 3) // 4 * 4] == 0) and torch.all(gd[:, (c + 3) // 4 * 4:] == 9.0)
+    assert torch.equal(grads[0][[1, 3, 5]], grads[1][[1, 3, 5]])
+    assert not torch.isfinite(grads[1][[0, 2, 4]][:, :c]).all(1).any()
+
+
 @pytest.mark.parametrize("n,f", [(1, 1), (1000, 41), (50_001, 128), (300, 602)])
 def test_colsum(n, f):
     rng = np.random.default_rng(n)

@@ -387,7 +387,9 @@ int gcnsa_sage_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcns
 /* One epoch (Section 3.2): for every partition the worker's copy is set to the
  * aggregated parameters and takes one Adam step per batch; afterwards the
  * aggregated parameters become the mean of the copies.  loss_dev: nullable
- * DEVICE float, the epoch loss.  Asynchronous on the stream. */
+ * DEVICE float, the epoch loss.  Asynchronous on the stream.  parts may be other
+ * partitions than the model was created for, as many of them and none with more
+ * training vertices than the largest of those (GCNSA_ERR_ARG otherwise). */
 int gcnsa_sage_epoch(gcnsa_sage* model, const gcnsa_parts* parts, float* loss_dev);
 int gcnsa_sage_get_epoch(const gcnsa_sage* model, int64_t* epoch_out); /* epochs run so far = index of the next */
 /* Timing of the batches with CUDA events on the model's stream, as

@@ -364,6 +364,7 @@ struct gcnsa_sage {
   int64_t f = 0, h = 0, c = 0, ldf = 0, ldh = 0, ldc = 0;
   int64_t count = 0, w1_off = 0, b1_off = 0, w2_off = 0, b2_off = 0;  // flat parameter layout
   int64_t max_rows1 = 0;  // batch (1 + r2): rows of the hidden layer per batch
+  int64_t nt_max = 1;     // training vertices of the partition that has most
   int64_t epoch = 0;
   // parameters: aggregated; per worker its copy and its moments ([m x count] each)
   float *theta = nullptr, *copies = nullptr, *am = nullptr, *av = nullptr;
@@ -437,7 +438,9 @@ int cuda_err(cudaError_t e, const char* what) { return fail(GCNSA_ERR_CUDA, std:
 
 int check_model(const gcnsa_sage* S, const gcnsa_parts* P) {
   if (!S || !P) return fail(GCNSA_ERR_ARG, "NULL argument");
-  if (P->m != S->m || P->f != S->f || P->c != S->c) return fail(GCNSA_ERR_ARG, "model was created for other partitions");
+  bool fits = P->m == S->m && P->f == S->f && P->c == S->c;
+  for (const DevPart& d : P->parts) fits = fits && d.info.n_train <= S->nt_max;  // the batch order of a partition
+  if (!fits) return fail(GCNSA_ERR_ARG, "model was created for other partitions");
   return GCNSA_OK;
 }
 
@@ -645,8 +648,7 @@ int gcnsa_sage_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcns
   S->count = off;
   const int64_t B = opts->batch, r1 = opts->fanout[0], r2 = opts->fanout[1];
   S->max_rows1 = B * (1 + r2);
-  int64_t nt_max = 1;
-  for (int32_t p = 0; p < parts->m; ++p) nt_max = std::max<int64_t>(nt_max, parts->parts[p].info.n_train);
+  for (const DevPart& d : parts->parts) S->nt_max = std::max<int64_t>(S->nt_max, d.info.n_train);
   auto fail_free = [&](int code) {
     const std::string keep = gcnsa_last_error();
     gcnsa_sage_destroy(S);
@@ -680,7 +682,7 @@ int gcnsa_sage_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcns
                              {(void**)&S->ones, (size_t)B}, {(void**)&S->read_rows, sizeof(u64) * 2}};
   auto lane_wants = [&](SageLane& W) {
     return std::vector<Want>{
-        {(void**)&W.grad, pb}, {(void**)&W.keys, sizeof(u64) * (size_t)nt_max}, {(void**)&W.order, i4 * (size_t)nt_max},
+        {(void**)&W.grad, pb}, {(void**)&W.keys, sizeof(u64) * (size_t)S->nt_max}, {(void**)&W.order, i4 * (size_t)S->nt_max},
         {(void**)&W.b1, i4 * (size_t)S->max_rows1}, {(void**)&W.cnt2, i4 * (size_t)B},
         {(void**)&W.s1, i4 * (size_t)(S->max_rows1 * std::max<int64_t>(r1, 1))},
         {(void**)&W.cnt1, i4 * (size_t)S->max_rows1}, {(void**)&W.yb, i4 * (size_t)B},

@@ -265,6 +265,29 @@ def test_latest_batch_of_an_epoch_whose_last_workers_have_none(tiny_wl, idle):
             assert np.array_equal(one[key], other[key]), key
 
 
+def test_partitions_with_more_training_vertices_than_the_model_has_room_for_are_refused(tiny_wl):
+    w = tiny_wl
+    n = w.rowptr.size - 1
+    dims = [w.dims[0], 16, w.dims[-1]]
+    ws, wn, bs = configs.sage_weights(dims, 3)
+    env = gcnsa.make_env(0)
+    few, more = (gcnsa.Parts(env, w.rowptr, w.col, w.x, w.y, (np.arange(n) % k == 0).astype(np.uint8), w.dims[-1], 2, 0, 5)
+                 for k in (3, 2))
+    model = gcnsa.Sage(env, few, dims, ws, wn, bs, batch=64)
+    model.epoch()
+    model.parts = more
+    for call in (model.epoch, lambda: model.run_batch(0, 0, 0), lambda: model.n_batches(0)):
+        with pytest.raises(gcnsa.GcnsaError) as ei:
+            call()
+        assert ei.value.code == gcnsa.ERR_ARG
+    other = gcnsa.Sage(env, more, dims, ws, wn, bs, batch=64)
+    other.parts = few
+    other.epoch()
+    torch.cuda.synchronize()
+    for closing in (model, other, few, more):
+        closing.close()
+
+
 def test_runs_are_bitwise_reproducible_and_arguments_are_checked(tiny_wl):
     w = tiny_wl
     outs = []

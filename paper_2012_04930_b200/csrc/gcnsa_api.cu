@@ -267,15 +267,20 @@ int gcnsa_build_partitions(const gcnsa_env* env, const gcnsa_graph* g, const gcn
   P->env.e = *env;
   P->m = opts->m; P->f = g->f; P->c = g->c; P->n = g->n; P->ldx = GCNSA_LD(g->f);
   P->builder = opts->builder;
-  P->x_version.assign((size_t)opts->m, 1);
   static std::atomic<uint64_t> next_uid{1};
   P->uid = next_uid.fetch_add(1);
   if (!on_host) {
-    rc = build_device(P, g, opts);
+    try {
+      P->x_version.assign((size_t)opts->m, 1);
+      rc = build_device(P, g, opts);
+    } catch (const std::bad_alloc&) {  // (the builder has joined its threads and handed its scratch back)
+      rc = fail(GCNSA_ERR_OOM, "host allocation failed");
+    }
     if (rc) return build_failed(P, rc);
     *out = P;
     return GCNSA_OK;
   }
+  P->x_version.assign((size_t)opts->m, 1);
   P->part.swap(hb.part);
   P->parts.resize((size_t)opts->m);
   cudaStream_t s = P->env.stream();

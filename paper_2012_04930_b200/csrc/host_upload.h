@@ -9,7 +9,7 @@
 #include <atomic>
 #include <cstdint>
 #include <cstring>
-#include <system_error>
+#include <exception>
 #include <thread>
 #include <vector>
 
@@ -81,7 +81,7 @@ class HostUpload {
     for (int t = 0; t < kThreads; ++t) {
       try {
         threads_.emplace_back([this, t] { work(t); });
-      } catch (const std::system_error&) {
+      } catch (const std::exception&) {  // no thread, or no memory for one
         break;
       }
     }

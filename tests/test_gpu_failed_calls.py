@@ -17,6 +17,7 @@ pytestmark = pytest.mark.gpu
 
 SHIM = r"""
 #include <cuda_runtime.h>
+#include <new>
 static int fail_at = 0, calls = 0, pending = 0, failed = 0, waits = 0, syncs = 0;
 static cudaStream_t own = nullptr;
 extern "C" {
@@ -25,6 +26,15 @@ void shim_arm(int at, void* stream) { fail_at = at; calls = pending = failed = w
 int shim_launches() { return calls; }
 int shim_waits_of_own() { return waits; }    // waits given to the caller's stream after the failure
 int shim_syncs_of_others() { return syncs; }  // other streams waited for on the host after the failure
+// operator new number `at` from now on, on this thread, throws
+static thread_local int new_at = 0, news = 0;
+void shim_arm_new(int at) { new_at = at; news = 0; }
+int shim_news() { return news; }
+void* __real__Znwm(size_t);
+void* __wrap__Znwm(size_t n) {
+  if (++news == new_at) throw std::bad_alloc();
+  return __real__Znwm(n);
+}
 cudaError_t __real_cudaLaunchKernelExC(const cudaLaunchConfig_t*, const void*, void**);
 cudaError_t __real_cudaGetLastError();
 cudaError_t __real_cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned);
@@ -47,7 +57,7 @@ cudaError_t __wrap_cudaStreamSynchronize(cudaStream_t s) {
 }
 }
 """
-WRAPPED = ("cudaLaunchKernelExC", "cudaGetLastError", "cudaStreamWaitEvent", "cudaStreamSynchronize")
+WRAPPED = ("cudaLaunchKernelExC", "cudaGetLastError", "cudaStreamWaitEvent", "cudaStreamSynchronize", "_Znwm")
 
 
 def _run(scenario, tmp_path):
@@ -69,6 +79,39 @@ def _run(scenario, tmp_path):
                            timeout=300)
     assert child.returncode == 0, child.stderr[-2000:]
     return json.loads(child.stdout.strip().splitlines()[-1])
+
+
+def _child_build():
+    """A build whose k-th host allocation fails, for every k; inputs large enough to go through the upload threads."""
+    import numpy as np
+    from gen import graphs
+    from paper_2012_04930_b200 import gcnsa
+    n, f = 20_000, 900
+    rowptr, col = graphs.permutation_graph(n, 3, 5)
+    x = np.random.default_rng(0).standard_normal((n, f)).astype(np.float32)
+    assert x.nbytes + col.nbytes >= 64 << 20
+    L, env, codes = gcnsa.lib(), gcnsa.make_env(0), []
+
+    def build():
+        return gcnsa.Parts(env, rowptr, col, x, np.zeros(n, np.int32), np.ones(n, np.uint8), 2, 2, 100_000, 3)
+
+    build().close()
+    L.shim_arm_new(0)
+    build().close()
+    total = L.shim_news()
+    for at in range(total, 0, -1):
+        L.shim_arm_new(at)
+        try:
+            parts = build()
+            codes.append(0)
+        except gcnsa.GcnsaError as e:
+            codes.append(e.code)
+            L.shim_arm_new(0)
+            continue
+        L.shim_arm_new(0)
+        assert np.array_equal(parts.features(0), x[parts.members(0)])
+        parts.close()
+    print(json.dumps({"total": total, "codes": codes, "oom": gcnsa.ERR_OOM}))
 
 
 def _child(scenario):
@@ -130,8 +173,13 @@ def test_a_failed_epoch_from_host_buffers_reads_them_no_longer(tmp_path):
         assert syncs == 1
 
 
+def test_no_host_memory_while_building_is_an_error_code(tmp_path):
+    got = _run("build", tmp_path)
+    assert got["total"] > 10 and set(got["codes"]) <= {0, got["oom"]} and got["oom"] in got["codes"], got
+
+
 if __name__ == "__main__":
     if len(sys.argv) == 3:
         from paper_2012_04930_b200 import gcnsa
         gcnsa.use_library(sys.argv[2])
-        _child(sys.argv[1])
+        _child_build() if sys.argv[1] == "build" else _child(sys.argv[1])

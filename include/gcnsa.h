@@ -550,12 +550,15 @@ int gcnsa_tc_clear(void);
  * every gathered column index against the sizes of the extended partition, and
  * the kernels of gcnsa_build_partitions that scatter by computed positions
  * (induced rows of Section 3.1, the radix sort behind the row orders, the
- * transposed CSR over the loss columns) check every write position.  A failed
- * check records what it saw and skips the access; nothing traps.
+ * transposed CSR over the loss columns, the plan of the tensor-core products)
+ * check every write position.  A planned product checks the rows it fetches and
+ * the places of its partial sums.  A failed check records what it saw and skips
+ * the access; nothing traps.
  * *enabled_host = 1 in the checking build, 0 otherwise (then the rest is 0).
  * *code_host = 0 when every check passed, else 1 = processing-order entry,
  * 2 = row range, 3 = column index, 4 = induced-row write, 5 = sort scatter,
- * 6 = loss-column write; *value_host = the offending value.  Synchronizes the
+ * 6 = loss-column write, 7 = slot of a plan, 8 = remainder write of a plan,
+ * 9 = partial sum of a planned product; *value_host = the offending value.  Synchronizes the
  * device and clears the record.  HOST pointers. */
 int gcnsa_debug_status(int32_t* enabled_host, int32_t* code_host, int64_t* value_host);
 

@@ -609,10 +609,11 @@ __global__ void __launch_bounds__(kSortWarps * 32) sort_scatter(const uint32_t* 
 
 // positions: loss rows in index order from 0, the others in index order from `rest0` (a multiple of kDenseRows)
 __global__ void plan_positions(const uint8_t* __restrict__ mask, const int32_t* __restrict__ before, int64_t np,
-                               int64_t rest0, int32_t* pos, int32_t* row_at) {
+                               int64_t rest0, int64_t limit, int32_t* pos, int32_t* row_at) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= np) return;
   const int64_t at = mask[i] ? before[i] : rest0 + (i - before[i]);  // before = exclusive scan of the mask
+  if (!GCNSA_CHECK_WRITE(at, limit, kDbgPlanSlot)) return;
   pos[i] = (int32_t)at;
   row_at[at] = (int32_t)i;
 }
@@ -721,7 +722,7 @@ plan_slots(const uint32_t* __restrict__ sel, const uint32_t* __restrict__ lossbi
       for (unsigned left = m; left; left &= left - 1) {
         const int bit = __ffs(left) - 1;
         const int slot = (l >> bit) & 1 ? a++ : rest0 + b++;
-        tc[slot] = (int32_t)(32 * w + bit);
+        if (GCNSA_CHECK_WRITE(slot, slots, kDbgPlanSlot)) tc[slot] = (int32_t)(32 * w + bit);
       }
     }
     run += total;
@@ -758,12 +759,14 @@ plan_rows(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col, i
       const unsigned below = (1u << bit) - 1;
       const int slot = loss ? rk[2 * w] + __popc(m & l & below) : rest0 + rk[2 * w + 1] + __popc(m & ~l & below);
       const int k = slot % kDenseCols, kk = k & 31;
-      atomicOr(bits + ((chunk0 + slot / kDenseCols) * kDenseRows + r) * 2 + (k >> 5), 1u << ((kk >> 1) + 16 * (kk & 1)));
+      if (GCNSA_CHECK_WRITE(slot, (chunk_ptr[tile + 1] - chunk0) * kDenseCols, kDbgPlanSlot))
+        atomicOr(bits + ((chunk0 + slot / kDenseCols) * kDenseRows + r) * 2 + (k >> 5), 1u << ((kk >> 1) + 16 * (kk & 1)));
     }
     const unsigned bl = __ballot_sync(kFull, e < end && !dense && loss), br = __ballot_sync(kFull, e < end && !dense && !loss);
     if (r_col && e < end && !dense) {
       const unsigned below = (1u << lane) - 1;
-      r_col[loss ? out_loss + n_loss + __popc(bl & below) : out_rest + n_rest + __popc(br & below)] = c;
+      const int to = loss ? out_loss + n_loss + __popc(bl & below) : out_rest + n_rest + __popc(br & below);
+      if (GCNSA_CHECK_WRITE(to, r_rowptr[row + 1], kDbgPlanRest)) r_col[to] = c;
     }
     n_loss += __popc(bl);
     n_rest += __popc(br);
@@ -1053,7 +1056,8 @@ void Builder::build_plan(DevPart& d, int64_t window) {
   plan_mask_flags<<<blocks_for(np, 256), 256, 0, s>>>(d.mask, np, flags);
   launched("plan_mask_flags");
   scan<int32_t>(flags, np, before);
-  plan_positions<<<blocks_for(np, 256), 256, 0, s>>>(d.mask, before, np, loss_tiles * kDenseRows, pl.pos, row_at);
+  plan_positions<<<blocks_for(np, 256), 256, 0, s>>>(d.mask, before, np, loss_tiles * kDenseRows, n_tiles * kDenseRows,
+                                                     pl.pos, row_at);
   launched("plan_positions");
   plan_loss_bits<<<blocks_for(words * 32, 256), 256, 0, s>>>(d.mask, np, words, lossbits);
   launched("plan_loss_bits");

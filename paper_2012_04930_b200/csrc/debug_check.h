@@ -16,6 +16,9 @@ constexpr int kDbgColumn = 3;        // a column index outside [0, source rows)
 constexpr int kDbgInducedWrite = 4;  // induced rows: a write position outside the row
 constexpr int kDbgSortWrite = 5;     // radix sort: a scatter position outside [0, n)
 constexpr int kDbgLossColWrite = 6;  // transposed CSR over the loss columns: a write position outside the row
+constexpr int kDbgPlanSlot = 7;      // plan of the tensor-core products: a row or column slot outside its tile's chunks
+constexpr int kDbgPlanRest = 8;      // plan: a write position outside the row's part of the remainder
+constexpr int kDbgPartialSum = 9;    // planned product: a partial sum outside the workspace
 
 // Bounds a caller knows about the operands of one sparse product; -1 = not known, not checked.
 struct SpmmBounds {
@@ -41,5 +44,6 @@ __device__ __forceinline__ bool dbg_in(unsigned long long* word, long long v, lo
 // Host side, one reader per translation unit that has a word (0 when the checks are compiled out).
 int debug_word_spmm(unsigned long long* out, bool clear);
 int debug_word_build(unsigned long long* out, bool clear);
+int debug_word_dense(unsigned long long* out, bool clear);
 
 }  // namespace gcnsa

@@ -1333,10 +1333,11 @@ int gcnsa_debug_status(int32_t* enabled_host, int32_t* code_host, int64_t* value
   *code_host = 0;
   *value_host = 0;
   CK(cudaDeviceSynchronize());
-  unsigned long long w[2] = {0ull, 0ull};
+  unsigned long long w[3] = {0ull, 0ull, 0ull};
   CKL(debug_word_spmm(&w[0], true));
   CKL(debug_word_build(&w[1], true));
-  const unsigned long long first = w[0] ? w[0] : w[1];
+  CKL(debug_word_dense(&w[2], true));
+  const unsigned long long first = w[0] ? w[0] : w[1] ? w[1] : w[2];
   *code_host = (int32_t)(first >> 56);
   *value_host = (int64_t)(first & 0x00ffffffffffffffull);
   return GCNSA_OK;

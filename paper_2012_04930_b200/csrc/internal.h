@@ -154,7 +154,7 @@ struct SpmmBase {
   // *beyond != 0: X has values the tensor cores cannot take; the rows are then gathered from the matrix itself
   const int* beyond = nullptr;
   const int32_t *all_rowptr = nullptr, *all_col = nullptr;
-  int64_t all_nnz = -1;
+  int64_t all_nnz = -1, n_pieces = -1;  // (checked by the GCNSA_DEBUG build)
 };
 
 // ---- kernel launchers (all enqueue on `stream`, return a cudaError_t as int) ---

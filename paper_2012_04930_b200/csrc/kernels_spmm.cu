@@ -471,6 +471,9 @@ __device__ __forceinline__ void load_pieces(float4 (&out)[CH], const SpmmBase& b
     const int Q = b.q0 + qq, slab = b.nslab > 1 ? Q / w4 : 0;
     const unsigned u0 = b.nslab * first + slab * cnt, u1 = u0 + cnt - 1;
     const int c0 = b.magic ? __umulhi(u0, b.magic) : u0 / b.per_cta, c1 = b.magic ? __umulhi(u1, b.magic) : u1 / b.per_cta;
+#if GCNSA_DBG
+    if (!dbg_in(&g_dbg_spmm, (long long)t * b.nslab + slab + c1, t * b.nslab + slab + c0, b.n_pieces, kDbgPartialSum)) continue;
+#endif
     const float4* src = reinterpret_cast<const float4*>(b.pieces) +
                         ((int64_t)(t * b.nslab + slab + c0) * kDenseRows + (pos % kDenseRows)) * w4 + (Q - slab * w4);
     out[ch] = __ldg(src);

@@ -34,6 +34,7 @@
 #include <algorithm>
 #include <mutex>
 
+#include "debug_check.h"
 #include "internal.h"
 #include "launch.h"
 #include "tc_device.h"
@@ -41,6 +42,10 @@
 namespace gcnsa {
 
 namespace {
+
+#if GCNSA_DBG
+GCNSA_DBG_WORD(g_dbg_dense);
+#endif
 
 constexpr int kLoadWarp0 = 1, kLoadWarps = 6, kExpandWarp0 = 8, kFoldWarp0 = 16, kRowWarps = 8;
 constexpr int kThreads = 32 * (kFoldWarp0 + kRowWarps);
@@ -126,6 +131,7 @@ struct Params {
   int64_t split_pitch;
   int per_cta, total;        // units
   float* pieces;             // [(tiles x nslab + CTAs)][256][N]
+  int64_t rows, n_pieces;    // (checked by the GCNSA_DEBUG build)
   int* beyond;               // [0] set by split_rows: values the MMAs cannot take; moved to [1] for spmm_rest
 };
 
@@ -310,7 +316,10 @@ __global__ void __launch_bounds__(kThreads, 1) spmm_dense(const Params p) {
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
           const int4& v = idx[i >> 2];
-          const int row = (i & 3) == 0 ? v.x : (i & 3) == 1 ? v.y : (i & 3) == 2 ? v.z : v.w;
+          int row = (i & 3) == 0 ? v.x : (i & 3) == 1 ? v.y : (i & 3) == 2 ? v.z : v.w;
+#if GCNSA_DBG
+          if (!dbg_in(&g_dbg_dense, row, 0, p.rows + 1, kDbgColumn)) row = (int)p.rows;  // the row of zeros
+#endif
           const uint8_t* r = src + (int64_t)row * p.split_pitch;
 #pragma unroll
           for (int line = 0; line < L::COUNT; ++line)
@@ -399,6 +408,9 @@ __global__ void __launch_bounds__(kThreads, 1) spmm_dense(const Params p) {
         }
       }
       if (!ok) break;
+#if GCNSA_DBG
+      if (!dbg_in(&g_dbg_dense, it.piece, 0, p.n_pieces, kDbgPartialSum)) continue;
+#endif
       float4* dst = reinterpret_cast<float4*>(p.pieces + ((int64_t)it.piece * 256 + row) * N);
 #pragma unroll
       for (int c = 0; c < N / 4; ++c)
@@ -542,6 +554,8 @@ int launch_spmm_planned(void* stream, const DensePlan& d, DenseUse use, int64_t 
     p.total = (int)total;
     p.per_cta = (int)((total + sms - 1) / sms);
     p.pieces = pieces;
+    p.rows = d.n_rows;
+    p.n_pieces = base.n_pieces = (int64_t)d.n_tiles * sl.n + sms;
     p.beyond = beyond;
     base.beyond = beyond + 1;
     base.all_rowptr = rowptr;
@@ -562,6 +576,21 @@ int launch_spmm_planned(void* stream, const DensePlan& d, DenseUse use, int64_t 
                           row_scale, src_scale, use == DenseUse::lossRows ? d.rm_order : d.r_order,
                           use == DenseUse::lossRows ? d.rm_n_long : d.r_n_long, x, ldx, f, epi, aux, ldaux, y, ldy, base,
                           SpmmBounds{bounds.mat_rows, bounds.src_rows, d.r_nnz});
+}
+
+int debug_word_dense(unsigned long long* out, bool clear) {
+  *out = 0ull;
+#if GCNSA_DBG
+  cudaError_t e = cudaMemcpyFromSymbol(out, g_dbg_dense, sizeof(*out));
+  if (e == cudaSuccess && clear) {
+    const unsigned long long zero = 0ull;
+    e = cudaMemcpyToSymbol(g_dbg_dense, &zero, sizeof(zero));
+  }
+  return (int)e;
+#else
+  (void)clear;
+  return 0;
+#endif
 }
 
 int tc_status(int* out) {

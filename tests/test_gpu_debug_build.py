@@ -2,8 +2,9 @@
 once on the regular library (this process) and once on libgcnsa_debug.so (a
 child process, because a process loads one build), and must give bit-identical
 results with no check recorded.  The scenario: the tiny workload trained in
-the plain and in the measured configuration, and partition builds of random
-graphs under every assignment mode."""
+the plain and in the measured configuration, partition builds of random
+graphs under every assignment mode, and training on graphs whose products run
+through a plan and on one whose rows are split by length."""
 import hashlib
 import json
 import os
@@ -68,6 +69,20 @@ def scenario():
         builds.append(_digest(arrays))
         parts.close()
     out["builds"] = builds
+    out["planned"] = []
+    for n, target, widths in ((3001, 640_000, [40, 24, 7]), (3001, 640_000, [20, 33, 130]), (12_003, 300_000, [40, 24, 7])):
+        rowptr, col, comm = graphs.chung_lu_communities(n, target, 2.1, 3, 0.93, 5)
+        x = rng.standard_normal((n, widths[0])).astype(np.float32)
+        mask = (rng.random(n) < 0.7).astype(np.uint8)
+        w0 = [rng.standard_normal(s).astype(np.float32) * 0.1 for s in zip(widths[:-1], widths[1:])]
+        parts = gcnsa.Parts(gcnsa.make_env(0), rowptr, col, x, (comm % 7).astype(np.int32), mask, widths[-1], 1, 0, 17)
+        model = gcnsa.Model(gcnsa.make_env(0), parts, widths, w0, epoch_graph=0)
+        before = gcnsa.launch_count()
+        for _ in range(2):
+            model.epoch()
+        out["planned"].append([gcnsa.launch_count() - before,
+                               _digest([model.get(what, l) for what in (gcnsa.GET_W, gcnsa.GET_B) for l in range(2)])])
+        model.close(); parts.close()
     out["debug_status"] = list(gcnsa.debug_status())
     out["tc_status"] = gcnsa.tc_status()
     return out
@@ -84,7 +99,8 @@ def test_checking_build_gives_identical_results_and_records_nothing():
     want = scenario()
     assert got["debug_status"] == [True, 0, 0], "the checking build recorded a violation (code, value)"
     assert want["debug_status"] == [False, 0, 0]
-    for key in ("plain", "measured", "builds", "tc_status"):
+    assert want["planned"][0][0] > want["planned"][2][0], "a planned product takes more launches"
+    for key in ("plain", "measured", "builds", "planned", "tc_status"):
         assert got[key] == want[key], key
 
 

@@ -33,9 +33,12 @@ if ROOT not in sys.path:
 METRIC = "GCN epochs/sec over all augmented partitions"
 # dram__bytes_read.sum + dram__bytes_write.sum per spmm_rows launch (mean over the four launches of one partition in
 # an ncu capture of this command on the kernel in use), keyed by (workload, factored_norm); None = not captured for
-# that kernel variant.  l1tex__data_pipe_lsu_wavefronts (% of peak) from the same captures.
-SPMM_TRAFFIC_BYTES = {("paper_scale", False): 177.0e6, ("paper_scale", True): 97.2e6}
-SPMM_L1_PIPE_PCT = {("paper_scale", False): 86.7, ("paper_scale", True): 86.1}
+# that kernel variant.  l1tex__data_pipe_lsu_wavefronts (% of peak) from the same captures.  (With factored_norm the
+# products of paper_scale run through the partitions' plans: profiles/spmm_planned_51k_rows.md.)
+SPMM_TRAFFIC_BYTES = {("paper_scale", False): 177.0e6}
+SPMM_L1_PIPE_PCT = {("paper_scale", False): 86.7}
+# sm__pipe_tensor_cycles_active (% of peak) of spmm_dense at F' = 128 in that profile
+PLANNED_TENSOR_PIPE_PCT = 72.5
 # the same for sage_concat_mean (mean over the hidden-layer and the output-layer launch of a batch)
 SAGE_TRAFFIC_BYTES = {"paper_scale": 38.3e6}
 UNIT = "epochs/s"
@@ -324,16 +327,21 @@ def run_ours(args):
         hbm_gbs_val = sp["alg_bytes_val"] / sp_s / 1e9
         l1_gbs = sp["l1_bytes"] / sp_s / 1e9
         key = (w.name, bool(args.factored_norm))
+        # gathers alone pull 4 F' bytes per stored entry (flops = 2 F' per entry); products through a plan far fewer
+        planned = sp["l1_bytes"] < 2.0 * sp["flops"]
         # the unit that binds is the one closest to its roof: HBM when the gathers miss L2 (no locality and a gathered
         # matrix beyond L2), the L1 data path of the SMs otherwise
         hbm_bound = hbm_gbs / peak_hbm >= l1_gbs / peak_l1
         roofline = {
-            "kernel": "spmm_rows", "bound": "hbm" if hbm_bound else "l1",
+            "kernel": "split_rows + spmm_dense + spmm_rest" if planned else "spmm_rows",
+            "bound": "hbm" if hbm_bound else "l1",
             "achieved": hbm_gbs if hbm_bound else l1_gbs, "peak": peak_hbm if hbm_bound else peak_l1, "unit": "GB/s",
             "frac": (hbm_gbs / peak_hbm) if hbm_bound else (l1_gbs / peak_l1),
             "peak_kind": (peak_kind + " HBM copy") if hbm_bound else
                          f"derived: {props.multi_processor_count} SMs x 128 B/clk x {sm_mhz:.0f} MHz (SM clock sampled under load)",
-            "why": ("the gathers miss L2: HBM is the unit closest to its roof" if hbm_bound else
+            "why": ("most entries run on the tensor cores, whose pipe is the busiest unit of spmm_dense; the entries that are "
+                    "left are gathers of a few hundred bytes per row, a chain of dependent loads" if planned else
+                    "the gathers miss L2: HBM is the unit closest to its roof" if hbm_bound else
                     "the gathers hit L2 (" + ("ids are community-ordered although the gathered matrix exceeds L2"
                                               if exceeds_l2 else "the gathered matrix is L2-resident") +
                     "): HBM carries little more than the compulsory bytes, the L1 data path is the unit closest to its roof"),
@@ -348,6 +356,7 @@ def run_ours(args):
             "frac_hbm": {"peak": peak_hbm, "peak_kind": peak_kind, "achieved": hbm_gbs, "frac": hbm_gbs / peak_hbm,
                          "achieved_8B_per_nnz": hbm_gbs_val, "frac_8B_per_nnz": hbm_gbs_val / peak_hbm},
             "l1_data_pipe_pct_of_peak_ncu": SPMM_L1_PIPE_PCT.get(key),
+            "spmm_dense_tensor_pipe_pct_of_peak_ncu": PLANNED_TENSOR_PIPE_PCT if planned else None,
             "launches": sp["launches"], "avg_launch_ms": sp["ms"] / max(sp["launches"], 1),
             "share_of_step": sp["ms"] / ms_profiled}
         # what the SMs can gather when the indices cost nothing: the library's probe (512-byte rows at indices the
@@ -374,8 +383,8 @@ def run_ours(args):
             "matrix_bytes": n_probe * 512, "no_l1_reuse": ceil_l2, "one_l1_hit_in_four": ceil_quarter,
             "all_l1_hits": ceil_l1,
             "note": "24 warps per SM, 16 independent 512-byte gathers in flight each, no index loads; spmm_rows has "
-                    "an L1 hit rate of 26 % on paper_scale (ncu), so one hit in four is the comparable line"}
-        roofline["frac_of_gather_ceiling"] = l1_gbs / ceil_quarter
+                    "an L1 hit rate of 26 % on paper_scale (ncu), so one hit in four is its comparable line"}
+        roofline["frac_of_gather_ceiling"] = None if planned else l1_gbs / ceil_quarter
         del xp, outp
         ge_s = max(ge["ms"] * 1e-3, 1e-12)
         useful = ge["flops"] / ge_s / 1e12

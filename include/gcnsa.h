@@ -312,7 +312,10 @@ int gcnsa_epoch_host(gcnsa_model* model, gcnsa_parts* parts, const float* const*
  * indices, values, one read of the source rows, one write of the result);
  * l1_bytes is what the SMs must pull through their L1 data path (SpMM: the same
  * with one gather of a source row per stored entry, 4 f nnz, in place of the one
- * read of the source rows; equal to alg_bytes for the other classes);
+ * read of the source rows; where the tensor cores take the product: the source
+ * rows and their bf16 terms, one read of these per tile of rows, the tiles' bits
+ * and partial sums, gathers for the entries that are left; equal to alg_bytes
+ * for the other classes);
  * alg_bytes_val is alg_bytes with 8 bytes per stored entry (index and value)
  * whether or not the kernel in use reads values; flops counts multiply-adds
  * as 2. */

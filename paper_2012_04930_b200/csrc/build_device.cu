@@ -970,7 +970,7 @@ struct Builder {
 };
 
 // A plan pays where a chunk of 64 columns takes enough entries off the gathers: per 64 features a chunk costs one SM
-// about 1 300 clocks, an entry 3.4 of a gathering SM (see spmm_dense), and the split of X and the second pass over the
+// 983 clocks, an entry 3.4 of a gathering SM (see kDenseMin), and the split of X and the second pass over the
 // rows come on top.  Measured at 1 640 and 1 230 entries per chunk: F' = 41 365 -> 178 us (58 241 rows, 28 M entries) and
 // F' = 128 435 -> 285 us (51 249 rows, 20.8 M entries: split 8, chunks 205 to 225, remainder 54); at 630 (245 000 rows,
 // 12.6 M entries) the planned product is as slow as the gathers.  A partition of fewer than kPlanMinNnz entries is a few microseconds of gathers, less than the

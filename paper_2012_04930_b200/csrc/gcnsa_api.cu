@@ -665,7 +665,9 @@ static int sparse_product(gcnsa_model* M, Lane& W, void* s, const DevPart& d, De
                                       aux, ldaux, y, ldy, W.dw, SpmmBounds{n, n, use == DenseUse::lossCols ? d.tm_nnz : d.info.nnz});
     if (r > 0) return cuda_fail((cudaError_t)r, "launch_spmm_planned");
     if (r == 0) {
-      M->prof_end(0, cost.bytes, cost.flops, cost.l1, cost.bytes_val);
+      const int64_t rest = d.info.nnz ? (int64_t)((double)d.plan.r_nnz * (double)nnz / (double)d.info.nnz) : 0;
+      const double mask_bytes = epi == GCNSA_EPI_MASK ? 4.0 * (double)f * (double)rows : 0.0;
+      M->prof_end(0, cost.bytes, cost.flops, spmm_planned_l1_bytes(d.plan, use, rows, rest, f) + mask_bytes, cost.bytes_val);
       return GCNSA_OK;
     }
   }

@@ -123,8 +123,11 @@ struct RowSplit {
 // in the leading chunks.  The entries in all other columns form the remainder CSR.  A + I is symmetric, so the plan
 // serves the transposed products as well; on the last layer these use the leading chunks only (its gradient has zero
 // rows elsewhere), and the forward product of the loss rows uses the leading tiles only.
-// kDenseMin: a column costs the tensor pipe 12 clocks of one SM per 64 features however few of its 256 bits are set,
-// an entry in the remainder a gather of 256 bytes, 3.4 clocks of one SM at the 21 TB/s the gathers reach.
+// kDenseMin: a column costs 15 clocks of one SM per 64 features however few of its 256 bits are set (983 clocks a chunk, 768
+// of them the tensor pipe's), an entry in the remainder a gather of 256 bytes, 3.4 clocks of one SM at the 21 TB/s that
+// long gathers reach and more in the short rows of the remainder.  Measured at 4 / 6 / 8 / 12, F' = 128: 51 249 rows of 20.8 M
+// entries 244 / 247 / 264 / 308 us, 46 593 of 12 M 193 / 198 / 211 / 237, 58 241 of 28 M 282 / 284 / 290 / 298; F' = 41 alike
+// (133 / 137 / 148 / 177, 108 / 111 / 120 / 138, 161 / 163 / 168 / 173).
 constexpr int kDenseRows = 256, kDenseCols = 64, kDenseMin = 4;
 struct DensePlan {
   int64_t n_rows = 0;  // rows = columns of the matrix
@@ -174,6 +177,7 @@ int launch_spmm_planned(void* stream, const DensePlan& d, DenseUse use, int64_t 
                         const float* src_scale, const float* x, int64_t ldx, int32_t f, int32_t epi, const float* aux,
                         int64_t ldaux, float* y, int64_t ldy, void* workspace, const SpmmBounds& bounds);
 size_t spmm_planned_workspace(const DensePlan& d, int32_t f);
+double spmm_planned_l1_bytes(const DensePlan& d, DenseUse use, int64_t n_rows, int64_t rest_nnz, int32_t f);
 // the remainder: row i adds its entries [rowptr[i], rowend[i]) and its partial sums
 int launch_spmm_rest(void* stream, int64_t n_rows, const int32_t* rowptr, const int32_t* rowend, const int32_t* col,
                      const float* row_scale, const float* src_scale, const int32_t* order, int64_t n_long, const float* x,
@@ -261,7 +265,6 @@ int launch_inv_sqrt_degree(void* stream, int64_t n, const int32_t* deg, float* d
 // dst[i, 0 .. f) = scale[i] * src[i, 0 .. f) (whole float4 chunks; leading dimensions multiples of 4; dst may be src)
 int launch_scale_rows(void* stream, int64_t n, int32_t f, const float* scale, const float* src, int64_t lds, float* dst,
                       int64_t ldd);
-// dst[i * ld + j] = src[i * f + j]: dense rows into padded rows
 int launch_mean(void* stream, const float* src, int count, float* dst);  // dst[0] = mean(src[0..count))
 
 }  // namespace gcnsa

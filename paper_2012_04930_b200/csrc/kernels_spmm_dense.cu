@@ -517,6 +517,17 @@ size_t spmm_planned_workspace(const DensePlan& d, int32_t f) {
   return kPlannedHead + pieces_bytes(d, sl) + (size_t)(d.n_rows + 1) * sl.n * sl.lines * 128;
 }
 
+// What the three kernels of a product pull through the SMs: X once and its terms (split_rows), a unit's lines, slots and bits
+// (spmm_dense), partial sums written and read, `rest_nnz` gathers, the result.
+double spmm_planned_l1_bytes(const DensePlan& d, DenseUse use, int64_t n_rows, int64_t rest_nnz, int32_t f) {
+  const Slabs sl = slabs_of(f);
+  const Use us = use_of(d, use);
+  const double units = (double)us.chunks * sl.n, line_bytes = (double)sl.lines * 128.0;
+  const double pieces = ((double)us.tiles * sl.n + sm_count()) * kDenseRows * sl.width * 4.0;
+  return (double)d.n_rows * (4.0 * f + sl.n * line_bytes) + units * (kDenseCols * (line_bytes + 4.0) + kBitBytes) + 2.0 * pieces +
+         (double)rest_nnz * (4.0 * f + 4.0) + (double)n_rows * (4.0 * f + 16.0);
+}
+
 // -1: too many units to count in an int (the caller then gathers)
 int launch_spmm_planned(void* stream, const DensePlan& d, DenseUse use, int64_t n_rows, const int32_t* rowptr,
                         const int32_t* col, const float* row_scale,

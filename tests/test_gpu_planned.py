@@ -175,3 +175,25 @@ def test_rows_by_length_match_fp64(n, width):
         _close(m.get(gcnsa.GET_GRAD_W, 0), torch.from_numpy(x).double().cuda().T @ product(g), ("dW", fact))
         m.close()
     parts.close()
+
+
+def test_profile_charges_a_planned_product_with_its_own_bytes():
+    """l1_bytes of a product through a plan: three launches, more than the compulsory bytes and far less than one gather of a
+    source row per stored entry, which is what the product without the plan is charged with."""
+    n, f = 3001, 41
+    rowptr, col, comm = graphs.chung_lu_communities(n, 640_000, 2.1, 3, 0.93, 5)
+    x = np.random.default_rng(3).standard_normal((n, f), dtype=np.float32)
+    env = gcnsa.make_env(0)
+    parts = gcnsa.Parts(env, rowptr, col, x, (comm % 3).astype(np.int32), np.ones(n, np.uint8), f, 1, 0, 3)
+    got = {}
+    for fact in (0, 1):
+        m = gcnsa.Model(env, parts, [f, f], [np.eye(f, dtype=np.float32)], factored_norm=fact, epoch_graph=0)
+        m.profile(True)
+        m.forward(0)
+        got[fact] = m.profile_read()["spmm"]
+        m.close()
+    gathers = 4.0 * f * parts.info(0).nnz
+    assert got[0]["launches"] == 1 and got[0]["l1_bytes"] > gathers
+    assert got[1]["launches"] == 3 and got[1]["alg_bytes"] < got[1]["l1_bytes"] < 0.5 * gathers
+    assert got[0]["flops"] == got[1]["flops"]
+    parts.close()

@@ -856,15 +856,6 @@ int gcnsa_forward(gcnsa_model* M, const gcnsa_parts* P, int32_t p, float* loss_d
   return GCNSA_OK;
 }
 
-// this partition's own optimizer step from the aggregated parameters (Section 3.2), folded into the mean
-static int local_step(gcnsa_model* M, int32_t p, bool first) {
-  PROF(M, 2, 32.0 * M->count, 0.0,
-       launch_adam_local_dev(M->env.e.stream, M->count, M->theta, M->gsum, M->am_parts + (size_t)p * M->count,
-                             M->av_parts + (size_t)p * M->count, M->theta_acc, first, 1.0f / (float)M->m, M->o.lr, M->o.beta1,
-                             M->o.beta2, M->o.eps, M->adam_state));
-  return GCNSA_OK;
-}
-
 int gcnsa_backward(gcnsa_model* M, const gcnsa_parts* P, int32_t p) {
   if (!M || !P || p < 0 || p >= P->m) return fail(GCNSA_ERR_ARG, "bad partition index or NULL");
   if (M->last_forward != p) return fail(GCNSA_ERR_ORDER, "gcnsa_backward needs gcnsa_forward on the same partition first");
@@ -873,25 +864,16 @@ int gcnsa_backward(gcnsa_model* M, const gcnsa_parts* P, int32_t p) {
   const int rc = backward_lane(M, P, p, M->lanes[0], s, M->gsum, 1);
   if (rc) return rc;
   if (M->o.agg_mode == GCNSA_AGG_PARAM_AVG) {
+    // this partition's own optimizer step from the aggregated parameters (Section 3.2), folded into the mean
     if (M->accumulated == 0)  // t -> t + 1 once per epoch
       PROF(M, 2, 0.0, 0.0, launch_adam_advance(s, M->adam_state, M->o.beta1, M->o.beta2));
-    const int rs = local_step(M, p, M->accumulated == 0);
-    if (rs) return rs;
+    PROF(M, 2, 32.0 * M->count, 0.0,
+         launch_adam_local_dev(s, M->count, M->theta, M->gsum, M->am_parts + (size_t)p * M->count,
+                               M->av_parts + (size_t)p * M->count, M->theta_acc, M->accumulated == 0,
+                               1.0f / (float)M->m, M->o.lr, M->o.beta1, M->o.beta2, M->o.eps, M->adam_state));
   }
   M->last_forward = -1;
   M->accumulated += 1;
-  return GCNSA_OK;
-}
-
-// the step from the gradient sum, or the mean of the partitions' own steps as the new parameters
-static int sum_step(gcnsa_model* M) {
-  if (M->o.agg_mode == GCNSA_AGG_PARAM_AVG) {
-    CK(cudaMemcpyAsync(M->theta, M->theta_acc, (size_t)M->count * sizeof(float), cudaMemcpyDeviceToDevice, M->env.stream()));
-    return GCNSA_OK;
-  }
-  PROF(M, 2, 28.0 * M->count, 0.0,
-       launch_adam_dev(M->env.e.stream, M->count, M->theta, M->gsum, M->am, M->av, 1.0f / (float)M->m, M->o.lr,
-                       M->o.beta1, M->o.beta2, M->o.eps, M->adam_state));
   return GCNSA_OK;
 }
 
@@ -899,10 +881,15 @@ int gcnsa_step(gcnsa_model* M) {
   if (!M) return fail(GCNSA_ERR_ARG, "model is NULL");
   if (M->accumulated != M->m) return fail(GCNSA_ERR_ORDER, "gcnsa_step needs one backward pass per partition");
   M->t += 1;
-  if (M->o.agg_mode != GCNSA_AGG_PARAM_AVG)
-    PROF(M, 2, 0.0, 0.0, launch_adam_advance(M->env.e.stream, M->adam_state, M->o.beta1, M->o.beta2));  // t -> t + 1
-  const int rc = sum_step(M);
-  if (rc) return rc;
+  if (M->o.agg_mode == GCNSA_AGG_PARAM_AVG) {
+    CK(cudaMemcpyAsync(M->theta, M->theta_acc, (size_t)M->count * sizeof(float), cudaMemcpyDeviceToDevice, M->env.stream()));
+    M->accumulated = 0;
+    return GCNSA_OK;
+  }
+  PROF(M, 2, 0.0, 0.0, launch_adam_advance(M->env.e.stream, M->adam_state, M->o.beta1, M->o.beta2));  // t -> t + 1
+  PROF(M, 2, 28.0 * M->count, 0.0,
+       launch_adam_dev(M->env.e.stream, M->count, M->theta, M->gsum, M->am, M->av, 1.0f / (float)M->m, M->o.lr,
+                       M->o.beta1, M->o.beta2, M->o.eps, M->adam_state));
   M->accumulated = 0;
   return GCNSA_OK;
 }
@@ -938,18 +925,22 @@ struct Fork {
   }
 };
 
-// forward and backward pass of partition p of an epoch in lane W
+// forward and backward pass of partition p of an epoch in lane W (without buffers of their own, as the calls step by step)
 static int epoch_partition(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& W, cudaStream_t s) {
-  int rc = forward_lane(M, P, p, W, s);
-  if (rc) return rc;
-  if (M->gparts) return backward_lane(M, P, p, W, s, M->gparts + (size_t)p * M->count, 0);
-  rc = backward_lane(M, P, p, W, s, M->gsum, 1);
-  return rc == GCNSA_OK && M->o.agg_mode == GCNSA_AGG_PARAM_AVG ? local_step(M, p, p == 0) : rc;
+  if (!M->gparts) {
+    const int rc = gcnsa_forward(M, P, p, nullptr);
+    return rc ? rc : gcnsa_backward(M, P, p);
+  }
+  const int rc = forward_lane(M, P, p, W, s);
+  return rc ? rc : backward_lane(M, P, p, W, s, M->gparts + (size_t)p * M->count, 0);
 }
 
-// the step from the gradients of all partitions in gparts, on top of what gcnsa_model_set has left in the gradient sum
-static int optimizer_step(gcnsa_model* M, cudaStream_t s) {
-  if (!M->gparts) return sum_step(M);
+// the step from the gradients of all partitions in gparts, on top of what gcnsa_model_set has left in the gradient sum;
+// advanced: the step count has been advanced already.  (Not before the passes of plain launches: where one fails, the count
+// on the device stays that of the host.)
+static int optimizer_step(gcnsa_model* M, cudaStream_t s, bool advanced) {
+  if (!M->gparts) return gcnsa_step(M);
+  if (!advanced) PROF(M, 2, 0.0, 0.0, launch_adam_advance(s, M->adam_state, M->o.beta1, M->o.beta2));  // t -> t + 1
   const float inv_m = 1.0f / (float)M->m;
   if (M->o.agg_mode == GCNSA_AGG_PARAM_AVG)
     PROF(M, 2, 32.0 * M->count * M->m, 0.0,
@@ -959,6 +950,7 @@ static int optimizer_step(gcnsa_model* M, cudaStream_t s) {
     PROF(M, 2, (24.0 + 4.0 * M->m) * M->count, 0.0,
          launch_adam_parts(s, M->count, M->m, M->theta, M->gsum, M->gparts, M->am, M->av, inv_m, M->o.lr, M->o.beta1, M->o.beta2,
                            M->o.eps, M->adam_state));
+  M->t += 1;
   return GCNSA_OK;
 }
 
@@ -976,8 +968,8 @@ static int epoch_body(gcnsa_model* M, const gcnsa_parts* P, float* loss_dev, For
   cudaStream_t aux = fork ? fork->side[lanes - 1] : s;
   if (fork)
     for (cudaStream_t st : fork->side) CK(fork->edge(s, st));
-  // t -> t + 1 (the steps of the partitions, where they come one by one, are on s)
-  PROF(M, 2, 0.0, 0.0, launch_adam_advance(M->gparts ? aux : s, M->adam_state, M->o.beta1, M->o.beta2));
+  const bool early = fork && M->gparts;  // (beside the passes)
+  if (early) PROF(M, 2, 0.0, 0.0, launch_adam_advance(aux, M->adam_state, M->o.beta1, M->o.beta2));  // t -> t + 1
   for (int32_t p = 0; p < P->m; ++p) {
     const int lane = (P->m - 1 - p) % lanes;
     rc = epoch_partition(M, P, p, M->lanes[lane], stream_of(lane));
@@ -989,12 +981,11 @@ static int epoch_body(gcnsa_model* M, const gcnsa_parts* P, float* loss_dev, For
     if (fork) CK(fork->edge(s, aux));
     CKL(launch_mean(aux, M->loss_parts, M->m, loss_dev));
   }
-  rc = optimizer_step(M, s);
+  rc = optimizer_step(M, s, early);
   if (rc) return rc;
   if (loss_dev && fork) CK(fork->edge(aux, s));
   M->last_forward = -1;
   M->last_n = P->parts[P->m - 1].info.n;
-  M->t += 1;
   return GCNSA_OK;
 }
 
@@ -1087,7 +1078,6 @@ int gcnsa_epoch_host(gcnsa_model* M, gcnsa_parts* P, const float* const* x_host,
   };
   auto epoch = [&]() -> int {
     for (int32_t p = 0; p < std::min(P->m, 2); ++p) CK(copy_in(p));
-    PROF(M, 2, 0.0, 0.0, launch_adam_advance(s, M->adam_state, M->o.beta1, M->o.beta2));  // t -> t + 1
     for (int32_t p = 0; p < P->m; ++p) {
       const DevPart& d = P->parts[p];
       CK(cudaStreamWaitEvent(s, P->ready[p], 0));
@@ -1098,7 +1088,7 @@ int gcnsa_epoch_host(gcnsa_model* M, gcnsa_parts* P, const float* const* x_host,
       const int r = epoch_partition(M, P, p, M->lanes[0], s);
       if (r) return r;
     }
-    return optimizer_step(M, s);
+    return optimizer_step(M, s, false);
   };
   rc = epoch();
   if (rc) {  // copies may be on their way: the caller's buffers are not read after the call
@@ -1107,7 +1097,6 @@ int gcnsa_epoch_host(gcnsa_model* M, gcnsa_parts* P, const float* const* x_host,
   }
   M->last_forward = -1;
   M->last_n = P->parts[P->m - 1].info.n;
-  M->t += 1;
   float* mean_dev = M->loss_parts + M->m;  // slot after the M partition losses
   CKL(launch_mean(M->env.e.stream, M->loss_parts, M->m, mean_dev));
   CK(cudaMemcpyAsync(loss_host, mean_dev, sizeof(float), cudaMemcpyDeviceToHost, M->env.stream()));

@@ -136,11 +136,15 @@ def _child(scenario):
             xs = [torch.from_numpy(w.x[parts.members(p)]).pin_memory() for p in range(w.m)]
             loss = np.zeros(1, np.float32)
             call = lambda: model.epoch_host([x.data_ptr() for x in xs], loss)  # noqa: E731
+            if scenario == "plain":
+                model.close()
+                model = gcnsa.Model(env, parts, w.dims, w.w0, w.b0, lr=w.lr, epoch_graph=0)
+                call = model.epoch
         call()
         L.shim_arm(0, stream.cuda_stream)
         call()
         total = L.shim_launches()
-        for at in (2, total // 3, total // 2, total - total // 20):
+        for at in (2, total // 3, total // 2, total - (total // 20 if scenario == "sage" else 6)):
             L.shim_arm(at, stream.cuda_stream)
             try:
                 call()
@@ -152,9 +156,17 @@ def _child(scenario):
         L.shim_arm(0, stream.cuda_stream)
         call()                       # and the object is usable
         stream.synchronize()
+        same = None
+        if scenario != "sage":       # as if the failed calls had not been made
+            other = gcnsa.Model(env, parts, w.dims, w.w0, w.b0, lr=w.lr, epoch_graph=0)
+            for _ in range(3):
+                other.epoch()
+            same = all(np.array_equal(model.get(what, l), other.get(what, l)) for l in range(2)
+                       for what in (gcnsa.GET_W, gcnsa.GET_B, gcnsa.GET_ADAM_M_W, gcnsa.GET_ADAM_V_W))
+            other.close()
         model.close()
         parts.close()
-    print(json.dumps({"m": w.m, "out": out, "err_cuda": gcnsa.ERR_CUDA}))
+    print(json.dumps({"m": w.m, "out": out, "same": same, "err_cuda": gcnsa.ERR_CUDA}))
 
 
 def test_a_failed_sage_epoch_joins_its_workers(tmp_path):
@@ -171,6 +183,13 @@ def test_a_failed_epoch_from_host_buffers_reads_them_no_longer(tmp_path):
     for code, _, syncs in got["out"]:
         assert code == got["err_cuda"]
         assert syncs == 1
+    assert got["same"]
+
+
+def test_an_epoch_that_failed_in_its_passes_can_be_made_again(tmp_path):
+    """A launch that fails in the passes of an epoch leaves the parameters, the moments and the step count as they were."""
+    got = _run("plain", tmp_path)
+    assert [o[0] for o in got["out"]] == [got["err_cuda"]] * 4 and got["same"]
 
 
 def test_no_host_memory_while_building_is_an_error_code(tmp_path):

@@ -1038,6 +1038,7 @@ int gcnsa_epoch(gcnsa_model* M, const gcnsa_parts* P, float* loss_dev) {
   }
   CK(cudaGraphLaunch(M->graph_exec, s));
   note_launch(M->graph_kernels);
+  M->last_forward = -1;  // its activations are gone
   M->t += 1;
   M->last_n = P->parts[P->m - 1].info.n;
   return GCNSA_OK;

@@ -604,3 +604,22 @@ def test_an_empty_partition_leaves_no_bias_gradient_of_other_partitions(tiny_wl)
             parts.close()
     for a, b in zip(*got):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("epoch_graph", [0, 1])
+def test_no_backward_pass_after_an_epoch_has_replaced_the_activations(tiny_wl, epoch_graph):
+    """forward, epoch, backward is refused whether the epoch is launched, recorded or replayed."""
+    w = tiny_wl
+    with torch.cuda.stream(torch.cuda.Stream()):
+        env = gcnsa.make_env(0)
+        parts = gcnsa.Parts(env, w.rowptr, w.col, w.x, w.y, w.train_mask, w.dims[-1], w.m, w.overlap_ppm, w.seed,
+                            w.part_mode, w.user_part, w.loss_on_halo)
+        model = gcnsa.Model(env, parts, w.dims, w.w0, w.b0, lr=w.lr, epoch_graph=epoch_graph)
+        for _ in range(3):
+            model.forward(0)
+            model.epoch()
+            with pytest.raises(gcnsa.GcnsaError) as ei:
+                model.backward(0)
+            assert ei.value.code == gcnsa.ERR_ORDER
+        model.close()
+        parts.close()

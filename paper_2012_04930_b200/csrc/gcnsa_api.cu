@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 #include <thread>
@@ -99,6 +100,7 @@ struct gcnsa_model {
   std::vector<int64_t> ax_version;  // x_version of the partition the product was computed from (0 = none yet)
   uint64_t ax_uid = 0;
   std::vector<Lane> lanes;        // at least one
+  mutable std::mutex pack;        // gcnsa_model_get packs rows in the work buffer of lane 0: one caller at a time
   float* gparts = nullptr;        // [m x count]: the gradient of every partition of an epoch; NULL: they go into gsum
   float* loss_parts = nullptr;
   // evaluation buffers (allocated on first gcnsa_evaluate)
@@ -1149,10 +1151,12 @@ int gcnsa_model_get(const gcnsa_model* M, int32_t what, int32_t layer, void* hos
     // are one piece, others are packed on the device first (tmp_b: no pass leaves anything there).  An evaluation that
     // fetches the logits: 116 483 x 41 1 595 -> 1 336 us, 20 000 x 20 201 -> 162, x 41 246 -> 209, x 5 165 -> 160.
     if (GCNSA_LD(cols) != cols) {
+      std::lock_guard<std::mutex> lock(M->pack);
       CKL(launch_copy_rows(M->env.e.stream, M->last_n, cols, src, GCNSA_LD(cols), M->lanes[0].tmp_b, cols));
-      src = M->lanes[0].tmp_b;
+      CK(cudaMemcpyAsync(host_dst, M->lanes[0].tmp_b, bytes, cudaMemcpyDeviceToHost, M->env.stream()));
+    } else {
+      CK(cudaMemcpyAsync(host_dst, src, bytes, cudaMemcpyDeviceToHost, M->env.stream()));
     }
-    CK(cudaMemcpyAsync(host_dst, src, bytes, cudaMemcpyDeviceToHost, M->env.stream()));
   }
   CK(cudaStreamSynchronize(M->env.stream()));
   return GCNSA_OK;

@@ -6,6 +6,7 @@ Bars: bit-exact partition assignment, sampled vertex sets, CSR and transposed
 CSR indices; fp32 tensors within 1e-4 * max|reference| after one step; epoch
 loss within 1e-3 relative at every epoch."""
 import copy
+import threading
 
 import numpy as np
 import pytest
@@ -623,3 +624,34 @@ def test_no_backward_pass_after_an_epoch_has_replaced_the_activations(tiny_wl, e
             assert ei.value.code == gcnsa.ERR_ORDER
         model.close()
         parts.close()
+
+
+def test_several_threads_may_read_a_models_tensors(small_wl):
+    """gcnsa_model_get leaves the model as it is: threads that read different layers at the same time get what one thread
+    gets (rows whose width is not that of the device's are packed on the way)."""
+    w = small_wl
+    env = gcnsa.make_env(0)
+    dims = [w.dims[0], 45, 37, w.dims[-1]]
+    rng = np.random.default_rng(4)
+    w0 = [rng.standard_normal(s).astype(np.float32) * 0.1 for s in zip(dims[:-1], dims[1:])]
+    parts = gcnsa.Parts(env, w.rowptr, w.col, w.x, w.y, w.train_mask, w.dims[-1], w.m, w.overlap_ppm, w.seed,
+                        w.part_mode, w.user_part, w.loss_on_halo)
+    model = gcnsa.Model(env, parts, dims, w0, loss_rows_only=0, epoch_graph=0)
+    model.forward(0)
+    n = parts.info(0).n
+    want = {l: model.get(gcnsa.GET_ACT, l, n) for l in (1, 2, 3)}
+    wrong = []
+
+    def read(l):
+        for _ in range(60):
+            if not np.array_equal(model.get(gcnsa.GET_ACT, l, n), want[l]):
+                wrong.append(l)
+
+    threads = [threading.Thread(target=read, args=(l,)) for l in (1, 2, 3)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
+    model.close()
+    parts.close()

@@ -541,10 +541,12 @@ int gcnsa_op_gather_probe_warps(int32_t* warps_out);
 
 /* The tensor-core kernels bound every wait (tens of milliseconds); a wait that
  * runs out stores a non-zero code in a device word instead of hanging.  The
- * word is sticky: while it is set, every tensor-core launch returns at once
- * without computing, so results after a non-zero status are undefined until
+ * word (one for the dense products, one for the planned sparse ones) is sticky:
+ * while it is set, every launch of its kind returns at once without computing,
+ * so results after a non-zero status are undefined until
  * gcnsa_tc_clear.  gcnsa_tc_status synchronizes the device and copies the word
- * to *status_host (0 = healthy); gcnsa_tc_clear synchronizes and resets it. */
+ * that is set to *status_host (0 = healthy); gcnsa_tc_clear synchronizes and
+ * resets both. */
 int gcnsa_tc_status(int32_t* status_host);
 int gcnsa_tc_clear(void);
 /* The checking build of the library (compiled with -DGCNSA_DEBUG into

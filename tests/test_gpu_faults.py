@@ -230,7 +230,7 @@ def test_a_model_without_memory_for_planned_products_gathers(agg_mode, cache_ax)
     rng = np.random.default_rng(1)
     w0 = [rng.standard_normal(s).astype(np.float32) / np.float32(np.sqrt(s[0])) for s in ((20, 12), (12, 7))]
     losses = {}
-    for fail_at in (0, -1):      # -1: the last allocation of the first round
+    for fail_at in (0, -1):      # -1: the last allocation of the first model
         alloc.arm(0 if fail_at == 0 else calls)
         m = gcnsa.Model(env, parts, [20, 12, 7], w0, agg_mode=agg_mode, cache_ax=cache_ax, epoch_graph=0)
         calls = alloc.calls
@@ -318,7 +318,7 @@ def test_many_partitions_of_a_large_model_share_one_gradient_sum():
 def test_buffers_a_model_needs_come_before_those_that_save_time(agg_mode, cache_ax):
     """An allocator with just the memory of a model that records nothing: the same model that records is created too."""
 
-    class Budget(FailingAllocator):
+    class Limited(FailingAllocator):
         room = 1 << 62
 
         def _alloc(self, nbytes, user):
@@ -331,7 +331,7 @@ def test_buffers_a_model_needs_come_before_those_that_save_time(agg_mode, cache_
     w0 = [rng.standard_normal(s).astype(np.float32) * 0.05 for s in zip(dims[:-1], dims[1:])]
     with torch.cuda.stream(torch.cuda.Stream()):
         parts = _sparse_parts(gcnsa.make_env(0), 8, 3000, dims[0], dims[-1])
-        alloc = Budget()
+        alloc = Limited()
         env = alloc.env()
         losses = []
         for graph in (0, 1):

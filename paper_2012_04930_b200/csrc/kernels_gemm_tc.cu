@@ -97,6 +97,21 @@ __device__ __forceinline__ void umma_tf32_ta(uint32_t tmem_d, uint32_t tmem_a, u
       "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(acc)
       : "memory");
 }
+constexpr int kMaxCluster = 8;  // k-slices that one cluster adds up
+// All threads of the cluster's blocks; what they wrote to shared memory before is there for the others after it.  (Blocks of a
+// cluster run at the same time, and one that has given up comes here too.)
+__device__ __forceinline__ void cluster_sync() {
+  __syncthreads();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// 16 bytes at this block's shared-memory address `addr` in block `rank` of the cluster
+__device__ __forceinline__ float4 cluster_load(uint32_t addr, int rank) {
+  uint32_t there;
+  float4 v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"(addr), "r"(rank));
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(there) : "memory");
+  return v;
+}
 __device__ __forceinline__ float epi_apply(float v, int epi, const float* __restrict__ aux, int64_t ldaux, int64_t i,
                                            int64_t j) {
   if (epi == GCNSA_EPI_BIAS || epi == GCNSA_EPI_BIAS_RELU) {
@@ -173,12 +188,15 @@ struct Work {
   int64_t m0, n0;
   int kb0, n_kb, z;
 };
-__device__ __forceinline__ Work decode_work(int w, int tiles_m, int tiles_n, int k_blocks, int kb_per_split, int bn) {
+// csplit > 1: the k-slices of a tile are the blocks of a cluster
+__device__ __forceinline__ Work decode_work(int w, int tiles_m, int tiles_n, int k_blocks, int kb_per_split, int bn, int csplit) {
   Work k;
+  const int slice = csplit > 1 ? w % csplit : 0;
+  if (csplit > 1) w /= csplit;
   const int nt = w % tiles_n, r = w / tiles_n;
   k.n0 = (int64_t)nt * bn;
   k.m0 = (int64_t)(r % tiles_m) * BM;
-  k.z = r / tiles_m;
+  k.z = csplit > 1 ? slice : r / tiles_m;
   k.kb0 = k.z * kb_per_split;
   k.n_kb = max(min(k_blocks, k.kb0 + kb_per_split) - k.kb0, 0);
   return k;
@@ -336,7 +354,7 @@ gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             int k_blocks, int k_blocks_per_split, int tiles_m, int tiles_n, int total_work, float* __restrict__ c,
             int64_t ldc, int accumulate, int epi, const float* __restrict__ aux, int64_t ldaux,
             int64_t slice_stride, int vec_ok, int terms, float* __restrict__ colsum_partial,
-            const float* __restrict__ post_scale) {
+            const float* __restrict__ post_scale, int csplit) {
   constexpr int BN = S::BN, NS = S::NS, NA = S::NA, B_BYTES = S::B_BYTES;
   constexpr int ACC_COLS = S::ACC_COLS, NBUF = S::NBUF;
   constexpr bool A_MN = S::A_MN, B_MN = S::B_MN;
@@ -361,6 +379,10 @@ gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
   __syncthreads();
   if (*abort_slot != 0) {
     wait_for_predecessors();
+    if (csplit > 1) {  // (the other blocks of the cluster read this one's shared memory between the two)
+      cluster_sync();
+      cluster_sync();
+    }
     return;
   }
   if (threadIdx.x == 0) {
@@ -403,7 +425,7 @@ gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
       uint32_t g = 0;  // k-blocks issued so far, over all items
       bool ok = true;
       for (int w = blockIdx.x; ok && w < total_work; w += gridDim.x) {
-        const Work wk = decode_work(w, tiles_m, tiles_n, k_blocks, k_blocks_per_split, BN);
+        const Work wk = decode_work(w, tiles_m, tiles_n, k_blocks, k_blocks_per_split, BN, csplit);
         for (int it = 0; it < wk.n_kb; ++it, ++g) {
           const uint32_t s = g % ring, ph = (g / ring) & 1;
           ok = mbar_wait(&freed[s], ph ^ 1, is_a ? 1 : 2);
@@ -450,7 +472,7 @@ gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
       uint32_t g = 0, item = 0;
       bool ok = true, issued = false;
       for (int w = blockIdx.x; ok && w < total_work; w += gridDim.x, ++item) {
-        const Work wk = decode_work(w, tiles_m, tiles_n, k_blocks, k_blocks_per_split, BN);
+        const Work wk = decode_work(w, tiles_m, tiles_n, k_blocks, k_blocks_per_split, BN, csplit);
         const uint32_t ab = item % NBUF, aph = (item / NBUF) & 1;
         ok = mbar_wait(&acc_empty[ab], aph ^ 1, 6);  // the epilogue has read this buffer's previous item back
         if (!ok) break;
@@ -505,7 +527,7 @@ gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     uint32_t g = 0;
     bool ok = true;
     for (int w = blockIdx.x; ok && w < total_work; w += gridDim.x) {
-      const Work wk = decode_work(w, tiles_m, tiles_n, k_blocks, k_blocks_per_split, BN);
+      const Work wk = decode_work(w, tiles_m, tiles_n, k_blocks, k_blocks_per_split, BN, csplit);
       for (int it = 0; it < wk.n_kb; ++it, ++g) {
         if ((int)(g % kSplitGroups) != group) continue;
         const uint32_t sa = g % NA, pa = (g / NA) & 1, s = g % NS, ps = (g / NS) & 1;
@@ -572,7 +594,7 @@ gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     const int64_t n_pad = min(ldc, (N + 3) / 4 * 4);  // C's pad columns [N, n_pad) are written as zeros
     uint32_t item = 0;
     for (int w = blockIdx.x; w < total_work; w += gridDim.x, ++item) {
-      const Work wk = decode_work(w, tiles_m, tiles_n, k_blocks, k_blocks_per_split, BN);
+      const Work wk = decode_work(w, tiles_m, tiles_n, k_blocks, k_blocks_per_split, BN, csplit);
       const uint32_t ab = item % NBUF, aph = (item / NBUF) & 1;
       const int64_t row_base = wk.m0 + quad * 32;
       float* const cz = c + (int64_t)wk.z * slice_stride;  // k-slices write slices of a partial buffer shaped like C
@@ -611,6 +633,27 @@ gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
       const uint32_t acc = tmem_base + ((uint32_t)(quad * 32) << 16) + ab * ACC_COLS;
       // steps of 32 columns; a step wholly outside C is not taken (C's zeroed pad columns end with N's step)
       const int last_c0 = (((int)min((int64_t)BN, N - wk.n0) + 31) / 32 - 1) * 32;
+      if (!S::DB && csplit > 1) {  // this slice's sums for the cluster, where A landed (all its boxes have been split)
+        const int r = quad * 32 + lane;
+        float* const stash = reinterpret_cast<float*>(smem) + r * BN;
+#pragma unroll 1
+        for (int c0 = 0; c0 <= last_c0; c0 += 32) {
+          uint32_t v[32];
+          tmem_ld32(acc + (uint32_t)c0, v);
+          if constexpr (S::MERGED) {
+            if (terms == 3) {
+              uint32_t u[32];
+              tmem_ld32(acc + (uint32_t)(BN + c0), u);
+#pragma unroll
+              for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + __uint_as_float(u[j]));
+            }
+          }
+#pragma unroll
+          for (int j = 0; j < 32; j += 4)  // 16-byte chunk c of row r at c ^ (r % 8)
+            *reinterpret_cast<uint4*>(stash + ((c0 + j) ^ ((r & 7) << 2))) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+        }
+        break;  // (a single item)
+      }
 #pragma unroll 1
       for (int c0 = 0; c0 <= last_c0; c0 += 32) {
         uint32_t v[32];
@@ -747,6 +790,48 @@ gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(S::TMEM_COLS) : "memory");
   }
+  if constexpr (!S::DB) {
+    if (csplit > 1) {
+      // ---------------- k-slices of a tile: every block adds up its share of the rows ----------------
+      cluster_sync();
+      const Work wk = decode_work(blockIdx.x, tiles_m, tiles_n, k_blocks, k_blocks_per_split, BN, csplit);
+      const int rows = (BM + csplit - 1) / csplit, r_end = min(BM, (wk.z + 1) * rows);
+      const int64_t n_pad = min(ldc, (N + 3) / 4 * 4);
+      const uint32_t base = smem_u32(smem);
+      for (int i = threadIdx.x; i < rows * (BN / 4); i += S::THREADS) {
+        const int r = wk.z * rows + i / (BN / 4), j = i % (BN / 4) * 4;
+        const int64_t row = wk.m0 + r, col = wk.n0 + j;
+        if (r >= r_end || row >= M || col >= n_pad) continue;
+        const uint32_t at = base + (uint32_t)((r * BN + (j ^ ((r & 7) << 2))) * 4);
+        float4 part[kMaxCluster];
+#pragma unroll
+        for (int z = 0; z < kMaxCluster; ++z)
+          part[z] = z < csplit ? cluster_load(at, z) : make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 a = part[0];
+#pragma unroll
+        for (int z = 1; z < kMaxCluster; ++z) {  // in slice order
+          if (z >= csplit) break;
+          a.x += part[z].x; a.y += part[z].y; a.z += part[z].z; a.w += part[z].w;
+        }
+        float v[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = col + e < N ? epi_apply(v[e], epi, aux, ldaux, row, col + e) : 0.f;
+        float* const dst = c + row * ldc + col;
+        if (vec_ok) {
+          if (accumulate) {
+            const float4 o = *reinterpret_cast<const float4*>(dst);
+            v[0] += o.x; v[1] += o.y; v[2] += o.z; v[3] += o.w;
+          }
+          *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (col + e < (accumulate ? N : n_pad)) dst[e] = accumulate ? dst[e] + v[e] : v[e];
+        }
+      }
+      cluster_sync();  // nobody leaves while its sums are being read
+    }
+  }
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -786,9 +871,13 @@ bool make_map(CUtensorMap* map, const float* base, int64_t outer, int64_t inner,
 }
 
 struct TcPlan {
-  int bn, splits, k_blocks, kb_per_split;
+  int bn, splits, cluster, k_blocks, kb_per_split;
   size_t partial_bytes;
 };
+
+constexpr int kClusterBlocks = 128;
+// a cluster lives in one of the chip's eight parts, of which at least 16 SMs each are counted on
+constexpr int kClusterParts = 8, kClusterSms = 16;
 
 int sm_count() {
   static int n = 0;
@@ -812,12 +901,20 @@ TcPlan tc_plan(int64_t m, int64_t n, int64_t k) {
   const int sms = sm_count();
   if (tiles < sms / 2 && p.k_blocks >= 16) splits = std::min<int64_t>(sms / tiles, p.k_blocks / 8);
   splits = std::max<int64_t>(splits, 1);
+  // Up to eight slices are a cluster: they meet in shared memory, and the pass over partial results in memory (5 to 8 us alone
+  // on the chip, a launch in the chain) is gone.  GraphSAGE epochs of 20 000 / 116 483 vertices 2 630 -> 2 330 us and 20.8 ->
+  // 19.7 ms, ten epochs on 2 000 / 20 000 vertices 727 -> 705 and 1 634 -> 1 545 us.  More slices only where eight of them
+  // would be long.
+  int64_t in_cluster = splits <= kMaxCluster || p.k_blocks <= kClusterBlocks ? std::min<int64_t>(splits, kMaxCluster) : 1;
+  while (in_cluster > 1 && tiles > kClusterParts * (kClusterSms / in_cluster)) --in_cluster;
+  if (in_cluster > 1) splits = in_cluster;
   p.kb_per_split = (int)((p.k_blocks + splits - 1) / splits);
   p.splits = (p.k_blocks + p.kb_per_split - 1) / p.kb_per_split;
   if (p.splits < 1) p.splits = 1;
+  p.cluster = in_cluster > 1 ? p.splits : 1;
   auto up = [](size_t b) { return (b + 255) / 256 * 256; };
   // the k-slices' partial results: [splits][m][n rounded up to 4] (rows that take 16-byte stores)
-  p.partial_bytes = up(p.splits > 1 ? (size_t)p.splits * m * ((n + 3) / 4 * 4) * sizeof(float) : 0);
+  p.partial_bytes = up(p.splits > 1 && p.cluster == 1 ? (size_t)p.splits * m * ((n + 3) / 4 * 4) * sizeof(float) : 0);
   return p;
 }
 
@@ -827,8 +924,13 @@ cudaError_t run_tc_shape(cudaStream_t s, const TcPlan& p, const CUtensorMap& ma,
                          int epi, const float* aux, int64_t ldaux, int64_t slice_stride, int vec_ok, int terms, float* colsum_partial, const float* post_scale) {
   cudaError_t e0 = cudaFuncSetAttribute(gemm_tf32x3<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_BYTES);
   if (e0 != cudaSuccess) return e0;
-  launch(gemm_tf32x3<S>, grid, S::THREADS, S::SMEM_BYTES, s, ma, mb, m, n, p.k_blocks, p.kb_per_split, tiles_m, tiles_n, total,
-                                                       c, ldc, accumulate, epi, aux, ldaux, slice_stride, vec_ok, terms, colsum_partial, post_scale);
+  if (p.cluster > 1)
+    launch_cluster(p.cluster, gemm_tf32x3<S>, grid, S::THREADS, S::SMEM_BYTES, s, ma, mb, m, n, p.k_blocks, p.kb_per_split, tiles_m,
+                   tiles_n, total, c, ldc, accumulate, epi, aux, ldaux, slice_stride, vec_ok, terms, colsum_partial, post_scale,
+                   p.cluster);
+  else
+    launch(gemm_tf32x3<S>, grid, S::THREADS, S::SMEM_BYTES, s, ma, mb, m, n, p.k_blocks, p.kb_per_split, tiles_m, tiles_n, total,
+           c, ldc, accumulate, epi, aux, ldaux, slice_stride, vec_ok, terms, colsum_partial, post_scale, 1);
   note_launch();
   return cudaGetLastError();
 }
@@ -901,7 +1003,7 @@ int launch_gemm_tc(void* stream, int32_t ta, int32_t tb, int64_t m, int64_t n, i
   if (((uintptr_t)a & 15) || (lda % 4) || ((uintptr_t)b & 15) || (ldb % 4)) return -1;
   if (!encode_fn()) return -1;
   uint8_t* ws = (uint8_t*)workspace;
-  float* partial = p.splits > 1 ? (float*)ws : nullptr;
+  float* partial = p.splits > 1 && p.cluster == 1 ? (float*)ws : nullptr;
   const bool a_mn = ta != 0;   // stored K x M: the M index is contiguous
   const bool b_mn = tb == 0;   // stored K x N: the N index is contiguous
   CUtensorMap ma, mb;

@@ -33,6 +33,26 @@ inline cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t sh
   c.numAttrs = (long long)grid.x * grid.y * grid.z <= kOverlapBlocks ? 1 : 0;
   return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
 }
+
+// the same in clusters of `cluster` consecutive blocks
+template <class... P, class... A>
+inline cudaError_t launch_cluster(int cluster, void (*kernel)(P...), dim3 grid, dim3 block, size_t shared, cudaStream_t stream,
+                                  A... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = shared;
+  c.stream = stream;
+  cudaLaunchAttribute a[2];
+  a[0].id = cudaLaunchAttributeClusterDimension;
+  a[0].val.clusterDim.x = cluster;
+  a[0].val.clusterDim.y = a[0].val.clusterDim.z = 1;
+  a[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a[1].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = a;
+  c.numAttrs = (long long)grid.x * grid.y * grid.z <= kOverlapBlocks ? 2 : 1;
+  return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
 #endif
 
 }  // namespace gcnsa

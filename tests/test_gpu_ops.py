@@ -342,6 +342,46 @@ def test_tensor_core_gemm_matches_fp64(m, n, k, ta, tb):
     assert torch.all(cd[:, n:_ld(n)] == 0)
 
 
+# two to eight k-slices of a tile (one cluster), the most of them with a short last one, tiles ragged both ways; more tiles than
+# clusters of that many fit at once; more slices than a cluster has (a pass over partial results)
+CLUSTER_SHAPES = [(130, 41, 520), (257, 130, 777), (100, 20, 1300), (640, 64, 1601), (64, 200, 1800), (1, 1, 2048), (128, 128, 2111),
+                  (2300, 128, 2100), (9000, 64, 520), (70, 33, 4500)]
+
+
+@pytest.mark.parametrize("m,n,k", CLUSTER_SHAPES)
+@pytest.mark.parametrize("ta,tb", [(0, 0), (1, 0), (0, 1)])
+def test_tensor_core_gemm_slices_meet_in_a_cluster(m, n, k, ta, tb):
+    """Every epilogue, results added to C and rows of C that take no 16-byte stores; the same bits again.  Bound: 2e-5 of the
+    largest entry as in the other tests of three TF32 products (the slices only group the fp32 sums differently)."""
+    rng = np.random.default_rng(m + 3 * n + k)
+    a = rng.standard_normal((k, m) if ta else (m, k)).astype(np.float32)
+    b = rng.standard_normal((n, k) if tb else (k, n)).astype(np.float32)
+    base = (a.T if ta else a).astype(np.float64) @ (b.T if tb else b).astype(np.float64)
+    ad, bd = _padded(a, _ld(a.shape[1])), _padded(b, _ld(b.shape[1]))
+    bias, scale = rng.standard_normal(n).astype(np.float32), rng.uniform(0.1, 2.0, m).astype(np.float32)
+    mask, c0 = rng.standard_normal((m, n)).astype(np.float32), rng.standard_normal((m, n)).astype(np.float32)
+    ws = torch.empty(gcnsa.op_gemm_workspace(ta, tb, m, n, k, gcnsa.GEMM_TF32X3) // 4 + 64, device="cuda")
+    tc0, fb0 = gcnsa.gemm_path_counts()
+    calls = 0
+    for epi, aux, want in ((gcnsa.EPI_NONE, None, base), (gcnsa.EPI_BIAS_RELU, _dev(bias), np.maximum(base + bias, 0)),
+                           (gcnsa.EPI_MASK, _padded(mask, _ld(n)), base * (mask > 0)),
+                           (gcnsa.EPI_ROWSCALE, _dev(scale), base * scale[:, None])):
+        for ldc in (_ld(n), n | 1):
+            for acc in (0, 1):
+                outs = []
+                for _ in range(2):
+                    cd = torch.full((m, ldc), 7.0, device="cuda")
+                    cd[:, :n] = _dev(c0)
+                    gcnsa.op_gemm(ad, bd, cd, m, n, k, ta=ta, tb=tb, accumulate=acc, epi=epi, aux=aux, workspace=ws,
+                                  mode=gcnsa.GEMM_TF32X3)
+                    calls += 1
+                    outs.append(cd)
+                assert torch.equal(outs[0], outs[1])
+                _close(outs[0][:, :n].cpu().numpy(), want + acc * c0, tol=2e-5, what=f"epi {epi} ldc {ldc} accumulate {acc}")
+                assert torch.all(outs[0][:, n:] == (7.0 if acc else 0.0))
+    assert gcnsa.tc_status() == 0 and gcnsa.gemm_path_counts() == (tc0 + calls, fb0)
+
+
 def test_tensor_core_gemm_split_k_epilogues_and_fallback():
     rng = np.random.default_rng(5)
     kk, m, n = 20_011, 130, 41                       # H^T dT: inner dimension = rows of a partition

@@ -273,6 +273,208 @@ __global__ void sage_hidden_grad(const float* __restrict__ dcat, const float* __
   dz1[idx] = h1[idx] > 0.f ? g : 0.f;
 }
 
+// The output layer of a batch and everything that a batch vertex's slots need from it, in one kernel: [h_v | mean h_u] W2 + b2,
+// softmax cross-entropy, the gradient dcat = g W2^T of the [self | mean] row and, sample by sample, the gradient of the hidden
+// layer's pre-activation.  A slot has one reader, so a block that holds kHeadRows vertices needs nothing of the others: what
+// was a chain of launches (gather, labels, product, softmax, product, gradient, column sums) is one, in fp32 FMAs.
+// What bounds it is latency: a few thousand FMAs a thread's worth of work, W2 (at most kHeadWeights floats) from L2 by every
+// block, so the loads of a phase are independent of one another and spread over all 256 threads.
+// Partial sums for the loss and both bias gradients leave one row per block, added up in block order by a later launch.
+// 20 000 vertices in batches of 256 (hidden 128, 20 classes): 2 330 -> 2 120 us per epoch; 116 483 (41 classes): 19.7 -> 19.1 ms.
+// Wider output layers and larger batches stay on the tensor cores: their products are work, not latency.
+constexpr int kHeadRows = 2, kHeadThreads = 256;
+constexpr int64_t kHeadWeights = 32768, kHeadBatch = 4096;
+struct Head {
+  const float* h1;
+  int ldh;
+  const int32_t* cnt2;
+  int r2, nb;
+  const float* w2;
+  int ldc, c, qp;  // qp: lanes per k in the forward product, a power of two and at least the quads of c
+  const float* b2;
+  const int32_t *y, *vertices;  // the label of row i is y[vertices[i]]
+  float inv_nb;
+  float *cat2, *logits, *g, *dz1;
+  float *loss_part, *g_sums, *dz_sums;  // [blocks], [blocks x 4 quads], [blocks x ldh]
+};
+__global__ void __launch_bounds__(kHeadThreads) sage_head(const Head p) {
+  wait_for_predecessors();
+  constexpr int V = kHeadRows, T = kHeadThreads;
+  extern __shared__ float4 head_smem[];
+  __shared__ float sh_loss[V];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int K = 2 * p.ldh, lv = p.ldh / 4, quads = (p.c + 3) / 4, cp = 4 * p.qp, v0 = blockIdx.x * V;
+  float* cat = reinterpret_cast<float*>(head_smem);  // [V][K]
+  float* dcat = cat + V * K;                         // [V][K]
+  float* part = dcat + V * K;                        // [slices][V][cp]; later [row lanes][ldh]
+  float* gs = part + 4 * T * V;                      // [V][cp]
+  for (int i = t; i < V * lv; i += T) {
+    const int v = i / lv, q = i - v * lv, row = v0 + v;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), m = a;
+    if (row < p.nb) {
+      const int n = __ldg(p.cnt2 + row);
+      const float4* col = reinterpret_cast<const float4*>(p.h1) + q;
+      a = __ldg(col + (int64_t)row * lv);
+      const float4* samp = col + ((int64_t)p.nb + (int64_t)row * p.r2) * lv;
+#pragma unroll 8
+      for (int s = 0; s < n; ++s) {
+        const float4 x = __ldg(samp + (int64_t)s * lv);
+        m.x += x.x; m.y += x.y; m.z += x.z; m.w += x.w;
+      }
+      const float inv = n > 0 ? 1.0f / (float)n : 0.f;
+      m.x *= inv; m.y *= inv; m.z *= inv; m.w *= inv;
+      float4* out = reinterpret_cast<float4*>(p.cat2 + (int64_t)row * K);  // the weight gradient's product reads it
+      out[q] = a;
+      out[lv + q] = m;
+    }
+    reinterpret_cast<float4*>(cat + v * K)[q] = a;
+    reinterpret_cast<float4*>(cat + v * K)[lv + q] = m;
+  }
+  __syncthreads();
+  {  // logits: thread = four classes of a slice of k
+    const int q = t & (p.qp - 1), slice = t / p.qp, slices = T / p.qp, per = (K + slices - 1) / slices;
+    const int k0 = slice * per, k1 = min(K, k0 + per);
+    float4 acc[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (q < quads) {
+#pragma unroll 8
+      for (int k = k0; k < k1; ++k) {
+        const float4 w = __ldg(reinterpret_cast<const float4*>(p.w2 + (int64_t)k * p.ldc) + q);
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+          const float x = cat[v * K + k];
+          acc[v].x = fmaf(x, w.x, acc[v].x); acc[v].y = fmaf(x, w.y, acc[v].y);
+          acc[v].z = fmaf(x, w.z, acc[v].z); acc[v].w = fmaf(x, w.w, acc[v].w);
+        }
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v) reinterpret_cast<float4*>(part + (slice * V + v) * cp)[q] = acc[v];
+  }
+  __syncthreads();
+  if (warp < V) {  // softmax: a warp per vertex, up to 256 classes
+    const int v = warp, row = v0 + v, slices = T / p.qp;
+    const bool in = row < p.nb;
+    const int yi = in ? __ldg(p.y + __ldg(p.vertices + row)) : 0;
+    float z[8], mx = -INFINITY, zy = -INFINITY;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int j = lane + 32 * i;
+      z[i] = -INFINITY;
+      if (j < p.c) {
+        float sum = 0.f;
+        for (int k = 0; k < slices; ++k) sum += part[(k * V + v) * cp + j];
+        z[i] = sum + __ldg(p.b2 + j);
+        if (in) p.logits[(int64_t)row * p.ldc + j] = z[i];
+        if (j == yi) zy = z[i];
+      }
+      mx = fmaxf(mx, z[i]);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, o));
+    zy = __shfl_sync(kFull, zy, yi & 31);
+    float se = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      z[i] = expf(z[i] - mx);
+      if (lane + 32 * i < p.c) se += z[i];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(kFull, se, o);
+    const float inv_se = 1.f / se;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int j = lane + 32 * i;
+      if (j >= 4 * quads) continue;
+      const float d = in && j < p.c ? (z[i] * inv_se - (j == yi ? 1.f : 0.f)) * p.inv_nb : 0.f;
+      gs[v * cp + j] = d;
+      if (in) p.g[(int64_t)row * p.ldc + j] = d;
+    }
+    if (lane == 0) sh_loss[v] = in ? (mx + logf(se)) - zy : 0.f;
+  }
+  __syncthreads();
+  if (t == 0) {
+    float sum = 0.f;
+#pragma unroll
+    for (int v = 0; v < V; ++v) sum += sh_loss[v];
+    p.loss_part[blockIdx.x] = sum;
+  }
+  for (int j = t; j < 4 * quads; j += T) {
+    float sum = 0.f;
+#pragma unroll
+    for (int v = 0; v < V; ++v) sum += gs[v * cp + j];
+    p.g_sums[(int64_t)blockIdx.x * 4 * quads + j] = sum;
+  }
+  for (int k = t; k < K; k += T) {  // dcat = g W2^T (W2's lines are in L1 by now)
+    const float4* w = reinterpret_cast<const float4*>(p.w2 + (int64_t)k * p.ldc);
+    float sum[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) sum[v] = 0.f;
+#pragma unroll 4
+    for (int q = 0; q < quads; ++q) {
+      const float4 x = __ldg(w + q);
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        const float4 d = reinterpret_cast<const float4*>(gs + v * cp)[q];
+        sum[v] = fmaf(d.x, x.x, fmaf(d.y, x.y, fmaf(d.z, x.z, fmaf(d.w, x.w, sum[v]))));
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v) dcat[v * K + k] = sum[v];
+  }
+  __syncthreads();
+  // hidden gradient, ReLU'(z) = [h > 0]: the vertex's own slot takes the first half of dcat, each of its samples 1 / count of the
+  // second; thread = four features of every ny-th slot
+  const int q = t % lv, ry = t / lv, ny = T / lv, slots = 1 + p.r2;
+  float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (ry < ny) {
+#pragma unroll 4
+    for (int i = ry; i < V * slots; i += ny) {
+      const int v = i / slots, s = i - v * slots - 1, row = v0 + v;  // s = -1: the vertex itself
+      if (row >= p.nb) break;
+      const int64_t slot = s < 0 ? row : p.nb + (int64_t)row * p.r2 + s;
+      const float4 h = __ldg(reinterpret_cast<const float4*>(p.h1) + slot * lv + q);
+      float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (s < 0) {
+        d = reinterpret_cast<const float4*>(dcat + v * K)[q];
+      } else {
+        const int n = __ldg(p.cnt2 + row);
+        if (s < n) {
+          d = reinterpret_cast<const float4*>(dcat + v * K)[lv + q];
+          const float den = (float)n;
+          d.x /= den; d.y /= den; d.z /= den; d.w /= den;
+        }
+      }
+      d.x = h.x > 0.f ? d.x : 0.f; d.y = h.y > 0.f ? d.y : 0.f; d.z = h.z > 0.f ? d.z : 0.f; d.w = h.w > 0.f ? d.w : 0.f;
+      reinterpret_cast<float4*>(p.dz1)[slot * lv + q] = d;
+      sum.x += d.x; sum.y += d.y; sum.z += d.z; sum.w += d.w;
+    }
+    reinterpret_cast<float4*>(part)[ry * lv + q] = sum;
+  }
+  __syncthreads();
+  for (int i = t; i < lv; i += T) {
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k = 0; k < ny; ++k) {
+      const float4 b = reinterpret_cast<const float4*>(part)[k * lv + i];
+      a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
+    }
+    reinterpret_cast<float4*>(p.dz_sums)[(int64_t)blockIdx.x * lv + i] = a;
+  }
+}
+// loss[0] = mean of the batch's losses from the blocks' partial sums (in block order by lane), loss[1] += their sum
+__global__ void sage_head_loss(const float* __restrict__ part, int count, float inv_nb, float weight, float* loss) {
+  wait_for_predecessors();
+  float s = 0.f;
+  for (int i = threadIdx.x; i < count; i += 32) s += part[i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+  if (threadIdx.x == 0) {
+    loss[0] = s * inv_nb;
+    loss[1] += loss[0] * weight;
+  }
+}
+
 // out[0] += number of source rows the [self | mean] kernel reads for these rows: 1 + cnt per row that has a vertex
 __global__ void sage_count_reads(const int32_t* __restrict__ self_idx, const int32_t* __restrict__ cnt, int64_t n_rows,
                                  u64* out) {
@@ -352,6 +554,7 @@ struct SageLane {
   // the batch
   int32_t *b1 = nullptr, *cnt2 = nullptr, *s1 = nullptr, *cnt1 = nullptr, *yb = nullptr;
   float *cat1 = nullptr, *h1 = nullptr, *cat2 = nullptr, *logits = nullptr, *g = nullptr, *dcat2 = nullptr, *dz1 = nullptr, *ce_sums = nullptr;
+  float *loss_part = nullptr, *g_sums = nullptr, *dz_sums = nullptr;  // of sage_head's blocks
   float* loss = nullptr;  // [0] batch loss, [1] sum over the worker's batches
   int64_t* batch_state = nullptr;
   void *ws = nullptr, *sc = nullptr;
@@ -366,6 +569,8 @@ struct gcnsa_sage {
   int64_t max_rows1 = 0;  // batch (1 + r2): rows of the hidden layer per batch
   int64_t nt_max = 1;     // training vertices of the partition that has most
   int64_t epoch = 0;
+  int head_qp = 0;        // 0: the output layer runs launch by launch; otherwise sage_head takes it (Head::qp)
+  size_t head_smem = 0;
   // parameters: aggregated; per worker its copy and its moments ([m x count] each)
   float *theta = nullptr, *copies = nullptr, *am = nullptr, *av = nullptr;
   double* adam_state = nullptr;  // [m x 4]
@@ -522,50 +727,74 @@ int run_batch(gcnsa_sage* S, const gcnsa_parts* P, int32_t p, int64_t epoch, int
   SCKL(launch_gemm(sv, mode, 0, 0, rows1, S->h, 2 * S->ldf, W.cat1, 2 * S->ldf, w + S->w1_off, S->ldh, W.h1, S->ldh, 0,
                    GCNSA_EPI_BIAS_RELU, w + S->b1_off, 0, W.ws, S->ws_bytes));
   S->prof_end(1, 0.0, fl1);
-  // ---- output layer: logits = [h_v | mean h_u] [W_self ; W_neigh] + b, the samples of vertex i in slots nb + i r2 + s
-  S->prof_begin();
-  launch(sage_concat_mean, blocks_for(nb * (S->ldh / 4), 256), 256, 0, s, W.h1, S->ldh, (int)S->h, nullptr, nullptr, W.cnt2, r2, nb, nb,
-                                                           W.cat2, S->ldh);
-  SLAUNCHED("sage_concat_mean");
-  S->prof_end(0, 8.0 * (double)nb * (double)S->ldh, 0.0);
-  S->prof_begin();
-  SCKL(launch_gemm(sv, mode, 0, 0, nb, S->c, 2 * S->ldh, W.cat2, 2 * S->ldh, w + S->w2_off, S->ldc, W.logits, S->ldc, 0,
-                   GCNSA_EPI_BIAS, w + S->b2_off, 0, W.ws, S->ws_bytes));
-  S->prof_end(1, 0.0, fl2);
-  // ---- loss over the batch and its gradient
-  S->prof_begin();
-  launch(sage_gather_labels, blocks_for(nb, 256), 256, 0, s, d.y, W.b1, nb, W.yb);
-  SLAUNCHED("sage_gather_labels");
-  CeSide side;  // the partial column sums of the logit gradient come with it
-  if (ce_by_groups((int32_t)S->c)) side.sums = W.ce_sums;
-  SCKL(launch_softmax_ce(sv, nb, (int32_t)S->c, W.logits, S->ldc, W.yb, S->ones, nb, W.loss, W.g, S->ldc, W.sc, side));
-  launch(sage_loss_add, 1, 32, 0, s, W.loss + 1, W.loss, (float)nb);
-  SLAUNCHED("sage_loss_add");
-  S->prof_end(2, 0.0, 0.0);
-  // ---- backward
   float* gr = W.grad;
-  S->prof_begin();
-  SCKL(launch_gemm(sv, mode, 1, 0, 2 * S->ldh, S->c, nb, W.cat2, 2 * S->ldh, W.g, S->ldc, gr + S->w2_off, S->ldc, 0,
-                   GCNSA_EPI_NONE, nullptr, 0, W.ws, S->ws_bytes));
-  SCKL(launch_gemm(sv, mode, 0, 1, nb, 2 * S->ldh, S->c, W.g, S->ldc, w + S->w2_off, S->ldc, W.dcat2, 2 * S->ldh, 0,
-                   GCNSA_EPI_NONE, nullptr, 0, W.ws, S->ws_bytes));
-  S->prof_end(1, 0.0, 2.0 * fl2);
-  S->prof_begin();
-  if (side.sums) {
-    SCKL(launch_ce_sums(sv, nb, (int32_t)S->c, W.ce_sums, gr + S->b2_off, 0));
+  if (S->head_qp > 0) {  // ---- output layer, loss and the gradient down to the hidden layer's pre-activation
+    Head hd;
+    hd.h1 = W.h1; hd.ldh = (int)S->ldh;
+    hd.cnt2 = W.cnt2; hd.r2 = r2; hd.nb = (int)nb;
+    hd.w2 = w + S->w2_off; hd.ldc = (int)S->ldc; hd.c = (int)S->c; hd.qp = S->head_qp;
+    hd.b2 = w + S->b2_off; hd.y = d.y; hd.vertices = W.b1;
+    hd.inv_nb = 1.0f / (float)nb;
+    hd.cat2 = W.cat2; hd.logits = W.logits; hd.g = W.g; hd.dz1 = W.dz1;
+    hd.loss_part = W.loss_part; hd.g_sums = W.g_sums; hd.dz_sums = W.dz_sums;
+    const unsigned blocks = blocks_for(nb, kHeadRows);
+    S->prof_begin();
+    launch(sage_head, blocks, kHeadThreads, S->head_smem, s, hd);
+    SLAUNCHED("sage_head");
+    launch(sage_head_loss, 1, 32, 0, s, W.loss_part, (int)blocks, hd.inv_nb, (float)nb, W.loss);
+    SLAUNCHED("sage_head_loss");
+    SCKL(launch_sum_rows(sv, blocks, (int32_t)S->c, W.g_sums, (S->c + 3) / 4 * 4, gr + S->b2_off, 0, W.sc));
+    SCKL(launch_sum_rows(sv, blocks, (int32_t)S->h, W.dz_sums, S->ldh, gr + S->b1_off, 0, W.sc));
+    S->prof_end(2, 0.0, 2.0 * fl2);
+    S->prof_begin();
+    SCKL(launch_gemm(sv, mode, 1, 0, 2 * S->ldh, S->c, nb, W.cat2, 2 * S->ldh, W.g, S->ldc, gr + S->w2_off, S->ldc, 0,
+                     GCNSA_EPI_NONE, nullptr, 0, W.ws, S->ws_bytes));
+    S->prof_end(1, 0.0, fl2);
   } else {
-    SCKL(launch_colsum(sv, nb, (int32_t)S->c, W.g, S->ldc, gr + S->b2_off, 0, W.sc));
+    // ---- output layer: logits = [h_v | mean h_u] [W_self ; W_neigh] + b, the samples of vertex i in slots nb + i r2 + s
+    S->prof_begin();
+    launch(sage_concat_mean, blocks_for(nb * (S->ldh / 4), 256), 256, 0, s, W.h1, S->ldh, (int)S->h, nullptr, nullptr, W.cnt2, r2, nb, nb,
+                                                             W.cat2, S->ldh);
+    SLAUNCHED("sage_concat_mean");
+    S->prof_end(0, 8.0 * (double)nb * (double)S->ldh, 0.0);
+    S->prof_begin();
+    SCKL(launch_gemm(sv, mode, 0, 0, nb, S->c, 2 * S->ldh, W.cat2, 2 * S->ldh, w + S->w2_off, S->ldc, W.logits, S->ldc, 0,
+                     GCNSA_EPI_BIAS, w + S->b2_off, 0, W.ws, S->ws_bytes));
+    S->prof_end(1, 0.0, fl2);
+    // ---- loss over the batch and its gradient
+    S->prof_begin();
+    launch(sage_gather_labels, blocks_for(nb, 256), 256, 0, s, d.y, W.b1, nb, W.yb);
+    SLAUNCHED("sage_gather_labels");
+    CeSide side;  // the partial column sums of the logit gradient come with it
+    if (ce_by_groups((int32_t)S->c)) side.sums = W.ce_sums;
+    SCKL(launch_softmax_ce(sv, nb, (int32_t)S->c, W.logits, S->ldc, W.yb, S->ones, nb, W.loss, W.g, S->ldc, W.sc, side));
+    launch(sage_loss_add, 1, 32, 0, s, W.loss + 1, W.loss, (float)nb);
+    SLAUNCHED("sage_loss_add");
+    S->prof_end(2, 0.0, 0.0);
+    // ---- backward
+    S->prof_begin();
+    SCKL(launch_gemm(sv, mode, 1, 0, 2 * S->ldh, S->c, nb, W.cat2, 2 * S->ldh, W.g, S->ldc, gr + S->w2_off, S->ldc, 0,
+                     GCNSA_EPI_NONE, nullptr, 0, W.ws, S->ws_bytes));
+    SCKL(launch_gemm(sv, mode, 0, 1, nb, 2 * S->ldh, S->c, W.g, S->ldc, w + S->w2_off, S->ldc, W.dcat2, 2 * S->ldh, 0,
+                     GCNSA_EPI_NONE, nullptr, 0, W.ws, S->ws_bytes));
+    S->prof_end(1, 0.0, 2.0 * fl2);
+    S->prof_begin();
+    if (side.sums) {
+      SCKL(launch_ce_sums(sv, nb, (int32_t)S->c, W.ce_sums, gr + S->b2_off, 0));
+    } else {
+      SCKL(launch_colsum(sv, nb, (int32_t)S->c, W.g, S->ldc, gr + S->b2_off, 0, W.sc));
+    }
+    launch(sage_hidden_grad, blocks_for(rows1 * S->ldh, 256), 256, 0, s, W.dcat2, W.h1, W.cnt2, nb, std::max(r2, 1), S->ldh, rows1,
+                                                                    W.dz1);
+    SLAUNCHED("sage_hidden_grad");
+    S->prof_end(2, 0.0, 0.0);
   }
-  launch(sage_hidden_grad, blocks_for(rows1 * S->ldh, 256), 256, 0, s, W.dcat2, W.h1, W.cnt2, nb, std::max(r2, 1), S->ldh, rows1,
-                                                                  W.dz1);
-  SLAUNCHED("sage_hidden_grad");
-  S->prof_end(2, 0.0, 0.0);
   S->prof_begin();
   SCKL(launch_gemm(sv, mode, 1, 0, 2 * S->ldf, S->h, rows1, W.cat1, 2 * S->ldf, W.dz1, S->ldh, gr + S->w1_off, S->ldh, 0,
                    GCNSA_EPI_NONE, nullptr, 0, W.ws, S->ws_bytes));
   S->prof_end(1, 0.0, fl1);
   S->prof_begin();
-  SCKL(launch_colsum(sv, rows1, (int32_t)S->h, W.dz1, S->ldh, gr + S->b1_off, 0, W.sc));
+  if (S->head_qp == 0) SCKL(launch_colsum(sv, rows1, (int32_t)S->h, W.dz1, S->ldh, gr + S->b1_off, 0, W.sc));
   // ---- the worker's Adam step (its own moments and step count)
   if (apply) {
     double* st = S->adam_state + 4 * (size_t)p;
@@ -674,6 +903,14 @@ int gcnsa_sage_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcns
   S->ws_bytes = ws;
   const size_t sc = std::max(std::max(softmax_ce_scratch(B), colsum_scratch(S->max_rows1, (int32_t)S->h)),
                              colsum_scratch(B, (int32_t)S->c));
+  // Small output layers (the 41 classes of a 128-wide hidden layer: 12 288 floats of W2) are one kernel; plain TF32 keeps its
+  // products on the tensor cores, which is what that mode is there to measure.
+  if (mode != GCNSA_GEMM_TF32 && B <= kHeadBatch && S->c <= 256 && 2 * S->ldh * S->ldc <= kHeadWeights && S->ldh <= 1024) {
+    S->head_qp = 1;
+    while (4 * S->head_qp < S->c) S->head_qp *= 2;
+    S->head_smem = sizeof(float) * (size_t)(kHeadRows * (4 * S->ldh + 4 * kHeadThreads + 4 * S->head_qp));
+  }
+  const size_t head_blocks = S->head_qp ? blocks_for(B, kHeadRows) : 0;
   const size_t f4 = sizeof(float), i4 = sizeof(int32_t);
   std::vector<Want> wants = {{(void**)&S->theta, pb}, {(void**)&S->copies, pb * (size_t)S->m},
                              {(void**)&S->am, pb * (size_t)S->m}, {(void**)&S->av, pb * (size_t)S->m},
@@ -690,6 +927,8 @@ int gcnsa_sage_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcns
         {(void**)&W.cat2, f4 * (size_t)(B * 2 * S->ldh)}, {(void**)&W.logits, f4 * (size_t)(B * S->ldc)},
         {(void**)&W.g, f4 * (size_t)(B * S->ldc)}, {(void**)&W.dcat2, f4 * (size_t)(B * 2 * S->ldh)},
         {(void**)&W.dz1, f4 * (size_t)(S->max_rows1 * S->ldh)}, {(void**)&W.ce_sums, ce_sums_scratch((int32_t)S->c)}, {(void**)&W.loss, f4 * 2},
+        {(void**)&W.loss_part, f4 * head_blocks}, {(void**)&W.g_sums, f4 * head_blocks * (size_t)((S->c + 3) / 4 * 4)},
+        {(void**)&W.dz_sums, f4 * head_blocks * (size_t)S->ldh},
         {(void**)&W.batch_state, sizeof(int64_t) * 2}, {&W.ws, ws}, {&W.sc, std::max<size_t>(sc, 256)}};
   };
   cudaStream_t s = S->env.stream();

@@ -5,6 +5,8 @@ against the fp64 checker on the same seeded inputs.
 Bars: batch membership and sampled neighbour sets identical (compared as sets:
 every draw is a set of unique keys); embeddings, logits, gradients within
 1e-4 * max|reference|; epoch loss within 1e-3 relative at every epoch."""
+import copy
+
 import numpy as np
 import pytest
 import torch
@@ -91,6 +93,23 @@ def _check_batch(model, pt, x, y, params, tg, seed, epoch, fanout, p, b):
     for got, want, nm in zip(_gpu_params(model, gcnsa.SAGE_GRAD_W_SELF), grads,
                              ("dWs1", "dWn1", "db1", "dWs2", "dWn2", "db2")):
         close(got, want, what=f"p{p} b{b} {nm}")
+
+
+@pytest.mark.parametrize("hidden,c,fanout,batch", [(1, 3, (2, 1), 7), (17, 33, (3, 4), 63), (100, 129, (4, 3), 64),
+                                                   (16, 256, (3, 2), 65), (16, 257, (3, 2), 64), (256, 41, (2, 5), 33),
+                                                   (512, 5, (2, 3), 40), (600, 41, (2, 3), 40), (24, 5, (3, 0), 32)])
+def test_output_layer_of_every_width(hidden, c, fanout, batch, tiny_wl):
+    """The output layer runs in one kernel up to 256 classes and 32 768 weights, two vertices to a block (odd batches), and
+    launch by launch beyond: a full and the ragged last batch against the checker."""
+    w = copy.copy(tiny_wl)
+    w.dims = [w.dims[0], hidden, c]
+    w.y = np.random.default_rng(c).integers(0, c, len(w.y)).astype(np.int32)
+    env, parts, model, rparts, params, xs, ys, trs = _setup(w, hidden, fanout, batch, 0.01, gcnsa.GEMM_TF32X3)
+    want = sage.batches(rparts[0], trs[0], w.seed, 0, batch)
+    for b in (0, len(want) - 1):
+        _check_batch(model, rparts[0], xs[0], ys[0], params, want[b], w.seed, 0, fanout, 0, b)
+    assert gcnsa.tc_status() == 0
+    model.close(); parts.close()
 
 
 @pytest.mark.parametrize("gemm_mode", [gcnsa.GEMM_FP32, gcnsa.GEMM_TF32X3])

@@ -197,10 +197,14 @@ int launch_gemm_tc(void* stream, int32_t ta, int32_t tb, int64_t m, int64_t n, i
 // gradient of a hidden layer, its bias gradient and the scaled copy the next sparse product reads, in one pass
 // over C when the tensor-core kernel takes the product (otherwise the product and the column-sum kernel).
 // scratch: gemm_colsum_scratch(m, n) bytes.
+// left_rows (nullable): where the column sums come as partial sums, these stay in scratch and *left_rows says how many rows of
+// them launch_mask_colsum_rest has to add up; 0: the sums are done
 int launch_gemm_mask_colsum(void* stream, int32_t mode, int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k,
                             const float* a, int64_t lda, const float* b, int64_t ldb, float* c, int64_t ldc,
                             const float* mask, int64_t ldmask, const float* row_scale, float* out, int32_t accumulate,
-                            void* scratch, void* workspace, size_t workspace_bytes);
+                            void* scratch, void* workspace, size_t workspace_bytes,
+                            int64_t* left_rows = nullptr);
+int launch_mask_colsum_rest(void* stream, int64_t left_rows, int64_t m, int64_t n, float* out, int32_t accumulate, void* scratch);
 size_t gemm_colsum_scratch(int64_t m, int32_t n);
 int64_t gemm_tc_colsum_rows(int32_t ta, int32_t tb, int64_t m, int64_t n);
 size_t gemm_tc_workspace(int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k);
@@ -225,6 +229,9 @@ struct CeSide {
 int launch_softmax_ce(void* stream, int64_t n, int32_t c, const float* logits, int64_t ld, const int32_t* y,
                       const uint8_t* mask, int64_t n_train, float* loss_dev, float* grad, int64_t ldg, void* scratch,
                       const CeSide& side = CeSide{});
+// loss_dev[0] = the loss whose partial sums launch_softmax_ce(loss_dev = NULL) has left in scratch (same n, c, n_train; rows on
+// 16-byte boundaries): for callers that have no use for it before other work
+int launch_ce_loss(void* stream, int64_t n, int32_t c, int64_t n_train, const void* scratch, float* loss_dev);
 size_t softmax_ce_scratch(int64_t n);
 // out[j] (+)= column sums of the gradient whose partial sums launch_softmax_ce(side.sums) left (same n, c)
 int launch_ce_sums(void* stream, int64_t n, int32_t c, const float* sums, float* out, int32_t accumulate);

@@ -388,10 +388,16 @@ size_t gemm_colsum_scratch(int64_t m, int32_t n) {
   return std::max(fused_partial_bytes(m, n) + colsum_scratch(gemm_tc_colsum_rows(1, 0, m, n), n), colsum_scratch(m, n));
 }
 
+int launch_mask_colsum_rest(void* stream, int64_t left_rows, int64_t m, int64_t n, float* out, int32_t accumulate, void* scratch) {
+  return launch_sum_rows(stream, left_rows, (int32_t)n, (const float*)scratch, (n + 3) / 4 * 4, out, accumulate,
+                         (uint8_t*)scratch + fused_partial_bytes(m, (int32_t)n));
+}
+
 int launch_gemm_mask_colsum(void* stream, int32_t mode, int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k,
                             const float* a, int64_t lda, const float* b, int64_t ldb, float* c, int64_t ldc,
                             const float* mask, int64_t ldmask, const float* row_scale, float* out, int32_t accumulate,
-                            void* scratch, void* workspace, size_t workspace_bytes) {
+                            void* scratch, void* workspace, size_t workspace_bytes, int64_t* left_rows) {
+  if (left_rows) *left_rows = 0;
   if (n == 0) return 0;
   if (m == 0)  // no rows: sums of nothing
     return accumulate ? 0 : (int)cudaMemsetAsync(out, 0, (size_t)n * sizeof(float), (cudaStream_t)stream);
@@ -400,8 +406,10 @@ int launch_gemm_mask_colsum(void* stream, int32_t mode, int32_t ta, int32_t tb, 
                                  workspace_bytes, mode == GCNSA_GEMM_TF32 ? 1 : 3, (float*)scratch, row_scale);
     if (r == 0) {
       note_gemm_path(true);
-      return launch_sum_rows(stream, gemm_tc_colsum_rows(ta, tb, m, n), n, (const float*)scratch, (n + 3) / 4 * 4, out,
-                             accumulate, (uint8_t*)scratch + fused_partial_bytes(m, n));
+      const int64_t rows = gemm_tc_colsum_rows(ta, tb, m, n);
+      if (!left_rows) return launch_mask_colsum_rest(stream, rows, m, n, out, accumulate, scratch);
+      *left_rows = rows;
+      return 0;
     }
     if (r > 0) return r;
   }

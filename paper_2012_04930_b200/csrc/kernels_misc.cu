@@ -535,6 +535,14 @@ int launch_softmax_ce(void* stream, int64_t n, int32_t c, const float* logits, i
   return (int)cudaGetLastError();
 }
 
+int launch_ce_loss(void* stream, int64_t n, int32_t c, int64_t n_train, const void* scratch, float* loss_dev) {
+  const int blocks = n <= 0 ? 0 : ce_by_groups(c) ? ce_group_blocks(n, c) : ce_blocks(n);
+  launch(loss_finalize, 1, 256, 0, (cudaStream_t)stream, (const float*)scratch, blocks, n_train > 0 ? 1.0f / (float)n_train : 0.f,
+         loss_dev);
+  note_launch();
+  return (int)cudaGetLastError();
+}
+
 size_t colsum_scratch(int64_t n, int32_t f) { return (size_t)colsum_blocks(n) * (size_t)f * sizeof(float); }
 
 int launch_colsum(void* stream, int64_t n, int32_t f, const float* g, int64_t ldg, float* out, int32_t accumulate,

@@ -875,7 +875,9 @@ struct TcPlan {
   size_t partial_bytes;
 };
 
-constexpr int kClusterBlocks = 128;
+// Eight slices where a product is at most this many k-blocks long, though more SMs are idle: ten epochs on 20 000 vertices in four
+// partitions (172 k-blocks) 1 486 -> 1 413 us; with a limit of 64 GraphSAGE batches (88) go 2 120 -> 2 285.
+constexpr int kClusterBlocks = 256;
 // a cluster lives in one of the chip's eight parts, of which at least 16 SMs each are counted on
 constexpr int kClusterParts = 8, kClusterSms = 16;
 

@@ -108,6 +108,7 @@ struct gcnsa_model {
   int32_t *ev_pred = nullptr, *ev_hits = nullptr;
   uint8_t* ev_mask = nullptr;
   size_t ws_bytes = 0, sc_bytes = 0, dw_bytes = 0;
+  int beside = 1;  // partitions a recorded epoch may work on at once (whether it does or not: results do not depend on it)
   int64_t ld_max = 0;
   int32_t last_forward = -1, accumulated = 0;
   int64_t last_n = 0;
@@ -484,6 +485,16 @@ static int epoch_lanes(const gcnsa_model* M, const gcnsa_parts* parts, size_t la
   return (int)std::min<int64_t>(std::min<int64_t>(parts->m, kMaxLanes), 1 + (int64_t)(kLaneBytes / lane_bytes));
 }
 
+// Whether the passes of a recorded epoch have branches: where partitions are small enough for lanes, kernels leave room beside
+// them and the chain of launches is the time.  A pass of two layers goes from 16 launches in a row to 11: ten epochs on
+// 2 000 vertices 702 -> 640 us, on 20 000 vertices 1 548 -> 1 486 us, partitions of 19 414 rows and 2 M entries alike
+// (3 085 -> 3 069 us).
+static bool beside(const gcnsa_parts* P) {
+  int64_t nnz_max = 0;
+  for (const DevPart& d : P->parts) nnz_max = std::max<int64_t>(nnz_max, d.info.nnz);
+  return nnz_max <= kLaneNnz && ce_by_groups(P->c);
+}
+
 // one lane's buffers; *bytes (nullable) grows by what was asked for
 static bool alloc_lane(gcnsa_model* M, Lane& W, size_t act, size_t* bytes_out = nullptr) {
   auto get = [&](size_t bytes) {
@@ -606,6 +617,7 @@ int gcnsa_model_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcn
   // and the lanes after the first, which only make a recorded epoch faster
   if (M->dw_bytes && !(M->lanes[0].dw = M->dalloc(M->dw_bytes))) M->dw_bytes = 0;
   M->lanes.resize((size_t)epoch_lanes(M, parts, lane_bytes));
+  if (M->gparts && beside(parts)) M->beside = std::min(parts->m, 3);
   for (size_t i = 1; i < M->lanes.size(); ++i) {
     const size_t mark = M->owned.size();
     Lane& W = M->lanes[i];
@@ -763,7 +775,7 @@ static int forward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& W
       // the product reads no values
       PROF(M, 1, gemm_bytes(n, dout, din), 2.0 * n * dout * din,
            launch_gemm(s, M->o.gemm_mode, 0, 0, n, dout, din, h, ldh, w, M->w_ld[l], W.tmp_a, ldo, 0,
-                       fact ? GCNSA_EPI_ROWSCALE : GCNSA_EPI_NONE, fact ? d.dinv : nullptr, 0, W.ws, M->ws_bytes));
+                       fact ? GCNSA_EPI_ROWSCALE : GCNSA_EPI_NONE, fact ? d.dinv : nullptr, 0, W.ws, M->ws_bytes, M->beside));
       // training reads the logits of the rows that carry loss only: the other rows are not computed
       const DenseUse use = last && M->o.loss_rows_only && !M->all_rows_once ? DenseUse::lossRows : DenseUse::all;
       const int rc = sparse_product(M, W, s, d, use, false, fact, W.tmp_a, ldo, dout, epi, bias, 0, W.H[l + 1], ldo);
@@ -782,7 +794,7 @@ static int forward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& W
       if (l == 0) W.s0_used = agg;
       PROF(M, 1, gemm_bytes(n, dout, din), 2.0 * n * dout * din,
            launch_gemm(s, M->o.gemm_mode, 0, 0, n, dout, din, agg, ldh, w, M->w_ld[l], W.H[l + 1], ldo, 0, epi, bias,
-                       0, W.ws, M->ws_bytes));
+                       0, W.ws, M->ws_bytes, M->beside));
     }
     h = W.H[l + 1];
     ldh = ldo;
@@ -868,7 +880,7 @@ static int backward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& 
       if (aside) CK(br.fork->edge((cudaStream_t)s, br.t));
       PROF(M, 1, gemm_bytes(din, dout, n), 2.0 * n * dout * din,
            launch_gemm(aside ? t : s, M->o.gemm_mode, 1, 0, din, dout, n, hprev, ldi, W.tmp_b, ldo, gw, M->w_ld[l], acc,
-                       GCNSA_EPI_NONE, nullptr, 0, W.ws, M->ws_bytes));
+                       GCNSA_EPI_NONE, nullptr, 0, W.ws, M->ws_bytes, M->beside));
       if (aside) CK(br.fork->mark(br.t, &q_read));
       bias_done = g_scaled = false;
       if (l > 0 && M->o.use_bias) {
@@ -892,7 +904,7 @@ static int backward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& 
       } else if (l > 0) {
         PROF(M, 1, gemm_bytes(n, din, dout) + 4.0 * n * din, 2.0 * n * dout * din,
              launch_gemm(s, M->o.gemm_mode, 0, 1, n, din, dout, W.tmp_b, ldo, w, M->w_ld[l], W.tmp_a, ldi, 0, GCNSA_EPI_MASK,
-                         hprev, ldi, W.ws, M->ws_bytes));
+                         hprev, ldi, W.ws, M->ws_bytes, M->beside));
         g = W.tmp_a;
       }
     } else {
@@ -900,11 +912,11 @@ static int backward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& 
       // dW += S^T G;  R = G W^T;  G^{l-1} = (A_hat^T R) .* [H^{l-1} > 0]
       PROF(M, 1, gemm_bytes(din, dout, n), 2.0 * n * dout * din,
            launch_gemm(s, M->o.gemm_mode, 1, 0, din, dout, n, l == 0 ? W.s0_used : W.S[l], ldi, g, ldo, gw, M->w_ld[l], acc,
-                       GCNSA_EPI_NONE, nullptr, 0, W.ws, M->ws_bytes));
+                       GCNSA_EPI_NONE, nullptr, 0, W.ws, M->ws_bytes, M->beside));
       if (l > 0) {
         PROF(M, 1, gemm_bytes(n, din, dout), 2.0 * n * dout * din,
              launch_gemm(s, M->o.gemm_mode, 0, 1, n, din, dout, g, ldo, w, M->w_ld[l], W.tmp_b, ldi, 0,
-                         fact ? GCNSA_EPI_ROWSCALE : GCNSA_EPI_NONE, fact ? d.dinv : nullptr, 0, W.ws, M->ws_bytes));
+                         fact ? GCNSA_EPI_ROWSCALE : GCNSA_EPI_NONE, fact ? d.dinv : nullptr, 0, W.ws, M->ws_bytes, M->beside));
         // (on the last layer R = G W^T has the zero rows of G)
         const int rc = sparse_product(M, W, s, d, l == M->L - 1 ? DenseUse::lossCols : DenseUse::all, true, fact, W.tmp_b, ldi,
                                       din, GCNSA_EPI_MASK, hprev, ldi, W.tmp_a, ldi);
@@ -995,16 +1007,6 @@ static int optimizer_step(gcnsa_model* M, cudaStream_t s, bool advanced) {
                            M->o.eps, M->adam_state));
   M->t += 1;
   return GCNSA_OK;
-}
-
-// Whether the passes of a recorded epoch have branches: where partitions are small enough for lanes, kernels leave room beside
-// them and the chain of launches is the time.  A pass of two layers goes from 16 launches in a row to 11: ten epochs on
-// 2 000 vertices 702 -> 640 us, on 20 000 vertices 1 548 -> 1 486 us, partitions of 19 414 rows and 2 M entries alike
-// (3 085 -> 3 069 us).
-static bool beside(const gcnsa_parts* P) {
-  int64_t nnz_max = 0;
-  for (const DevPart& d : P->parts) nnz_max = std::max<int64_t>(nnz_max, d.info.nnz);
-  return nnz_max <= kLaneNnz && ce_by_groups(P->c);
 }
 
 // One epoch: forward and backward of every partition, each with a gradient buffer of its own (see kGradBytes), then the

@@ -183,16 +183,17 @@ int launch_spmm_rest(void* stream, int64_t n_rows, const int32_t* rowptr, const 
                      const float* row_scale, const float* src_scale, const int32_t* order, int64_t n_long, const float* x,
                      int64_t ldx, int32_t f, int32_t epi, const float* aux, int64_t ldaux, float* y, int64_t ldy,
                      const SpmmBase& base, const SpmmBounds& bounds);
+// beside: how many such products the caller keeps in flight at a time (at most 3 count); they share the chip
 int launch_gemm(void* stream, int32_t mode, int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k, const float* a,
                 int64_t lda, const float* b, int64_t ldb, float* c, int64_t ldc, int32_t accumulate, int32_t epi,
-                const float* aux, int64_t ldaux, void* workspace, size_t workspace_bytes);
+                const float* aux, int64_t ldaux, void* workspace, size_t workspace_bytes, int beside = 1);
 size_t gemm_workspace(int32_t mode, int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k);
 // tensor-core path (3xTF32); returns -1 when the call has to fall back to the fp32 FMA kernel
 // terms: 3 = hi/lo split of both operands (fp32-level accuracy), 1 = the leading TF32 parts only
 int launch_gemm_tc(void* stream, int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k, const float* a, int64_t lda,
                    const float* b, int64_t ldb, float* c, int64_t ldc, int32_t accumulate, int32_t epi, const float* aux,
                    int64_t ldaux, void* workspace, size_t workspace_bytes, int terms = 3, float* colsum_partial = nullptr,
-                   const float* post_scale = nullptr);
+                   const float* post_scale = nullptr, int beside = 1);
 // C = (A B^T) .* [mask > 0], out (+)= column sums of C, then (row_scale given) row i of C times row_scale[i]: the
 // gradient of a hidden layer, its bias gradient and the scaled copy the next sparse product reads, in one pass
 // over C when the tensor-core kernel takes the product (otherwise the product and the column-sum kernel).

@@ -339,11 +339,11 @@ int launch_splitk_reduce(void* stream, int64_t m, int64_t n, int splits, const f
 
 int launch_gemm(void* stream, int32_t mode, int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k, const float* a,
                 int64_t lda, const float* b, int64_t ldb, float* c, int64_t ldc, int32_t accumulate, int32_t epi,
-                const float* aux, int64_t ldaux, void* workspace, size_t workspace_bytes) {
+                const float* aux, int64_t ldaux, void* workspace, size_t workspace_bytes, int beside) {
   if (m == 0 || n == 0) return 0;
   if (mode != GCNSA_GEMM_FP32 && k > 0) {
     const int r = launch_gemm_tc(stream, ta, tb, m, n, k, a, lda, b, ldb, c, ldc, accumulate, epi, aux, ldaux, workspace,
-                                 workspace_bytes, mode == GCNSA_GEMM_TF32 ? 1 : 3);
+                                 workspace_bytes, mode == GCNSA_GEMM_TF32 ? 1 : 3, nullptr, nullptr, beside);
     if (r >= 0) {  // done, or a CUDA error
       if (r == 0) note_gemm_path(true);
       return r;

@@ -892,7 +892,7 @@ int sm_count() {
   return n;
 }
 
-TcPlan tc_plan(int64_t m, int64_t n, int64_t k) {
+TcPlan tc_plan(int64_t m, int64_t n, int64_t k, int beside = 1) {
   TcPlan p;
   p.k_blocks = (int)((k + BK - 1) / BK);
   p.bn = n <= 64 ? 64 : 128;
@@ -902,6 +902,11 @@ TcPlan tc_plan(int64_t m, int64_t n, int64_t k) {
   // 30 slices would leave two work items for a second pass that takes as long as the first)
   const int sms = sm_count();
   if (tiles < sms / 2 && p.k_blocks >= 16) splits = std::min<int64_t>(sms / tiles, p.k_blocks / 8);
+  // Products that run side by side share the chip: a third of it each.  More slices end a product sooner alone, but each costs
+  // an SM the microseconds in which a block comes up, drains and meets its cluster.  Ten epochs on 20 000 vertices in four
+  // partitions 1 410 -> 1 289 us; GraphSAGE epochs (2 816 x 128 x 1 216, four and five at a time) 2 115 -> 1 998 us and 19.05 ->
+  // 17.0 ms.
+  if (beside > 1 && p.k_blocks <= kClusterBlocks) splits = std::min<int64_t>(splits, sms / std::min(beside, 3) / tiles);
   splits = std::max<int64_t>(splits, 1);
   // Up to eight slices are a cluster: they meet in shared memory, and the pass over partial results in memory (5 to 8 us alone
   // on the chip, a launch in the chain) is gone.  GraphSAGE epochs of 20 000 / 116 483 vertices 2 630 -> 2 330 us and 20.8 ->
@@ -994,10 +999,10 @@ size_t gemm_tc_workspace(int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k
 int launch_gemm_tc(void* stream, int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k, const float* a, int64_t lda,
                    const float* b, int64_t ldb, float* c, int64_t ldc, int32_t accumulate, int32_t epi, const float* aux,
                    int64_t ldaux, void* workspace, size_t workspace_bytes, int terms, float* colsum_partial,
-                   const float* post_scale) {
+                   const float* post_scale, int beside) {
   if (m <= 0 || n <= 0 || k <= 0 || m >= (1LL << 31) || n >= (1LL << 31) || k >= (1LL << 31)) return -1;
   cudaStream_t s = (cudaStream_t)stream;
-  const TcPlan p = tc_plan(m, n, k);
+  const TcPlan p = tc_plan(m, n, k, beside);
   const size_t need = p.partial_bytes;
   if (need > workspace_bytes) return -1;
   if (need && (!workspace || ((uintptr_t)workspace & 255))) return -1;

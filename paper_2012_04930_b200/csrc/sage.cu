@@ -578,6 +578,7 @@ struct gcnsa_sage {
   float* loss = nullptr;         // epoch loss
   uint8_t* ones = nullptr;
   size_t ws_bytes = 0;
+  int beside = 1;  // workers an epoch may run at once
   std::vector<SageLane> lanes;   // lane 0 also serves the calls that go batch by batch
   std::vector<cudaStream_t> side;  // streams of lanes 1, 2, ...
   cudaEvent_t fork_ev = nullptr;
@@ -725,7 +726,7 @@ int run_batch(gcnsa_sage* S, const gcnsa_parts* P, int32_t p, int64_t epoch, int
   const double fl1 = 2.0 * (double)rows1 * (double)S->h * 2.0 * (double)S->f, fl2 = 2.0 * (double)nb * (double)S->c * 2.0 * (double)S->h;
   S->prof_begin();
   SCKL(launch_gemm(sv, mode, 0, 0, rows1, S->h, 2 * S->ldf, W.cat1, 2 * S->ldf, w + S->w1_off, S->ldh, W.h1, S->ldh, 0,
-                   GCNSA_EPI_BIAS_RELU, w + S->b1_off, 0, W.ws, S->ws_bytes));
+                   GCNSA_EPI_BIAS_RELU, w + S->b1_off, 0, W.ws, S->ws_bytes, S->beside));
   S->prof_end(1, 0.0, fl1);
   float* gr = W.grad;
   if (S->head_qp > 0) {  // ---- output layer, loss and the gradient down to the hidden layer's pre-activation
@@ -748,7 +749,7 @@ int run_batch(gcnsa_sage* S, const gcnsa_parts* P, int32_t p, int64_t epoch, int
     S->prof_end(2, 0.0, 2.0 * fl2);
     S->prof_begin();
     SCKL(launch_gemm(sv, mode, 1, 0, 2 * S->ldh, S->c, nb, W.cat2, 2 * S->ldh, W.g, S->ldc, gr + S->w2_off, S->ldc, 0,
-                     GCNSA_EPI_NONE, nullptr, 0, W.ws, S->ws_bytes));
+                     GCNSA_EPI_NONE, nullptr, 0, W.ws, S->ws_bytes, S->beside));
     S->prof_end(1, 0.0, fl2);
   } else {
     // ---- output layer: logits = [h_v | mean h_u] [W_self ; W_neigh] + b, the samples of vertex i in slots nb + i r2 + s
@@ -759,7 +760,7 @@ int run_batch(gcnsa_sage* S, const gcnsa_parts* P, int32_t p, int64_t epoch, int
     S->prof_end(0, 8.0 * (double)nb * (double)S->ldh, 0.0);
     S->prof_begin();
     SCKL(launch_gemm(sv, mode, 0, 0, nb, S->c, 2 * S->ldh, W.cat2, 2 * S->ldh, w + S->w2_off, S->ldc, W.logits, S->ldc, 0,
-                     GCNSA_EPI_BIAS, w + S->b2_off, 0, W.ws, S->ws_bytes));
+                     GCNSA_EPI_BIAS, w + S->b2_off, 0, W.ws, S->ws_bytes, S->beside));
     S->prof_end(1, 0.0, fl2);
     // ---- loss over the batch and its gradient
     S->prof_begin();
@@ -774,9 +775,9 @@ int run_batch(gcnsa_sage* S, const gcnsa_parts* P, int32_t p, int64_t epoch, int
     // ---- backward
     S->prof_begin();
     SCKL(launch_gemm(sv, mode, 1, 0, 2 * S->ldh, S->c, nb, W.cat2, 2 * S->ldh, W.g, S->ldc, gr + S->w2_off, S->ldc, 0,
-                     GCNSA_EPI_NONE, nullptr, 0, W.ws, S->ws_bytes));
+                     GCNSA_EPI_NONE, nullptr, 0, W.ws, S->ws_bytes, S->beside));
     SCKL(launch_gemm(sv, mode, 0, 1, nb, 2 * S->ldh, S->c, W.g, S->ldc, w + S->w2_off, S->ldc, W.dcat2, 2 * S->ldh, 0,
-                     GCNSA_EPI_NONE, nullptr, 0, W.ws, S->ws_bytes));
+                     GCNSA_EPI_NONE, nullptr, 0, W.ws, S->ws_bytes, S->beside));
     S->prof_end(1, 0.0, 2.0 * fl2);
     S->prof_begin();
     if (side.sums) {
@@ -791,7 +792,7 @@ int run_batch(gcnsa_sage* S, const gcnsa_parts* P, int32_t p, int64_t epoch, int
   }
   S->prof_begin();
   SCKL(launch_gemm(sv, mode, 1, 0, 2 * S->ldf, S->h, rows1, W.cat1, 2 * S->ldf, W.dz1, S->ldh, gr + S->w1_off, S->ldh, 0,
-                   GCNSA_EPI_NONE, nullptr, 0, W.ws, S->ws_bytes));
+                   GCNSA_EPI_NONE, nullptr, 0, W.ws, S->ws_bytes, S->beside));
   S->prof_end(1, 0.0, fl1);
   S->prof_begin();
   if (S->head_qp == 0) SCKL(launch_colsum(sv, rows1, (int32_t)S->h, W.dz1, S->ldh, gr + S->b1_off, 0, W.sc));
@@ -833,8 +834,8 @@ int gcnsa_sage_destroy(gcnsa_sage* S) {
 // with five; 20 000 vertices, 4 workers: 7.7 -> 4.2 ms).  Larger batches fill the chip by themselves and their lanes
 // would cost gigabytes.  The lanes after the first take at most 1 GB (a batch of 2 816 rows of 602 features 17 MB each; with
 // fan-outs in the thousands the sample lists alone can be half a gigabyte).  The default stream runs one worker at a time.
+constexpr int64_t kLaneRows = 32768;
 static int sage_lanes(int32_t m, int64_t max_rows1, size_t lane_bytes, cudaStream_t s) {
-  constexpr int64_t kLaneRows = 32768;
   constexpr size_t kLaneBytes = (size_t)1 << 30;
   if (max_rows1 > kLaneRows || s == nullptr) return 1;
   return (int)std::min<int64_t>(std::min<int>(m, 8), 1 + (int64_t)(kLaneBytes / lane_bytes));
@@ -946,6 +947,7 @@ int gcnsa_sage_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcns
   size_t lane_bytes = 0;
   for (const Want& w : lane_wants(S->lanes[0])) lane_bytes += std::max<size_t>(w.bytes, 256);
   S->lanes.resize((size_t)sage_lanes(S->m, S->max_rows1, lane_bytes, s));
+  if (S->max_rows1 <= kLaneRows) S->beside = std::min(S->m, 3);
   for (size_t i = 0; i < S->lanes.size() && rc == GCNSA_OK; ++i) {
     const size_t mark = S->owned.size();
     rc = obtain(lane_wants(S->lanes[i]));

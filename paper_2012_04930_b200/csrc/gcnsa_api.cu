@@ -580,6 +580,7 @@ int gcnsa_model_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcn
     ws = std::max(ws, gemm_workspace(opts->gemm_mode, 0, 1, M->n_max, din, dout));
     sc = std::max(sc, colsum_scratch(M->n_max, (int32_t)dout));
     sc = std::max(sc, gemm_colsum_scratch(M->n_max, (int32_t)din));  // the fused bias gradient of the layer below
+    sc = std::max(sc, (size_t)4 * 148 * (size_t)((din + 3) / 4 * 4) * sizeof(float));  // ... as a narrow product leaves it
   }
   M->ws_bytes = ws; M->sc_bytes = sc;
   if (opts->factored_norm)
@@ -773,9 +774,20 @@ static int forward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& W
     if (M->transform_first[l]) {
       // factored_norm: A_hat T = diag(dinv) (A + I) (diag(dinv) T): the GEMM's epilogue scales the rows of T and
       // the product reads no values
-      PROF(M, 1, gemm_bytes(n, dout, din), 2.0 * n * dout * din,
-           launch_gemm(s, M->o.gemm_mode, 0, 0, n, dout, din, h, ldh, w, M->w_ld[l], W.tmp_a, ldo, 0,
-                       fact ? GCNSA_EPI_ROWSCALE : GCNSA_EPI_NONE, fact ? d.dinv : nullptr, 0, W.ws, M->ws_bytes, M->beside));
+      if (narrow_ok(M->o.gemm_mode, n, dout, din)) {
+        NarrowArgs na;
+        na.m = n; na.n = dout; na.k = din;
+        na.a = h; na.lda = ldh;
+        na.w = w; na.ldw = M->w_ld[l];
+        na.w_ready = l > 0;  // (the optimizer may be the kernel before the first)
+        na.c = W.tmp_a; na.ldc = ldo;
+        na.row_scale = fact ? d.dinv : nullptr;
+        PROF(M, 1, gemm_bytes(n, dout, din), 2.0 * n * dout * din, launch_narrow(s, na));
+      } else {
+        PROF(M, 1, gemm_bytes(n, dout, din), 2.0 * n * dout * din,
+             launch_gemm(s, M->o.gemm_mode, 0, 0, n, dout, din, h, ldh, w, M->w_ld[l], W.tmp_a, ldo, 0,
+                         fact ? GCNSA_EPI_ROWSCALE : GCNSA_EPI_NONE, fact ? d.dinv : nullptr, 0, W.ws, M->ws_bytes, M->beside));
+      }
       // training reads the logits of the rows that carry loss only: the other rows are not computed
       const DenseUse use = last && M->o.loss_rows_only && !M->all_rows_once ? DenseUse::lossRows : DenseUse::all;
       const int rc = sparse_product(M, W, s, d, use, false, fact, W.tmp_a, ldo, dout, epi, bias, 0, W.H[l + 1], ldo);
@@ -889,14 +901,30 @@ static int backward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& 
         const bool want_scaled = fact && M->transform_first[l - 1];
         int64_t left = 0;
         CK(wait(sums_read));
-        PROF(M, 1, gemm_bytes(n, din, dout) + 4.0 * n * din, 2.0 * n * dout * din,
-             launch_gemm_mask_colsum(s, M->o.gemm_mode, 0, 1, n, din, dout, W.tmp_b, ldo, w, M->w_ld[l], W.tmp_a, ldi, hprev,
-                                     ldi, want_scaled ? d.dinv : nullptr, grad + M->b_off[l - 1], acc, W.sc, W.ws,
-                                     M->ws_bytes, br.t ? &left : nullptr));
-        if (left) {
-          CK(br.fork->edge((cudaStream_t)s, br.t));
-          CKL(launch_mask_colsum_rest(t, left, n, din, grad + M->b_off[l - 1], acc, W.sc));
-          CK(br.fork->mark(br.t, &sums_read));
+        if (narrow_ok(M->o.gemm_mode, n, din, dout)) {
+          NarrowArgs na;
+          na.m = n; na.n = din; na.k = dout;
+          na.a = W.tmp_b; na.lda = ldo;
+          na.w = w; na.ldw = M->w_ld[l]; na.w_t = true; na.w_ready = true;
+          na.c = W.tmp_a; na.ldc = ldi;
+          na.row_scale = want_scaled ? d.dinv : nullptr;
+          na.mask = hprev; na.ldmask = ldi;
+          na.sums = (float*)W.sc;
+          PROF(M, 1, gemm_bytes(n, din, dout) + 4.0 * n * din, 2.0 * n * dout * din, launch_narrow(s, na));
+          if (br.t) CK(br.fork->edge((cudaStream_t)s, br.t));
+          PROF(M, 1, 0.0, 0.0, launch_sum_rows(t, narrow_blocks(n, din), din, na.sums, (din + 3) / 4 * 4, grad + M->b_off[l - 1], acc,
+                                               nullptr));
+          if (br.t) CK(br.fork->mark(br.t, &sums_read));
+        } else {
+          PROF(M, 1, gemm_bytes(n, din, dout) + 4.0 * n * din, 2.0 * n * dout * din,
+               launch_gemm_mask_colsum(s, M->o.gemm_mode, 0, 1, n, din, dout, W.tmp_b, ldo, w, M->w_ld[l], W.tmp_a, ldi, hprev,
+                                       ldi, want_scaled ? d.dinv : nullptr, grad + M->b_off[l - 1], acc, W.sc, W.ws,
+                                       M->ws_bytes, br.t ? &left : nullptr));
+          if (left) {
+            CK(br.fork->edge((cudaStream_t)s, br.t));
+            CKL(launch_mask_colsum_rest(t, left, n, din, grad + M->b_off[l - 1], acc, W.sc));
+            CK(br.fork->mark(br.t, &sums_read));
+          }
         }
         bias_done = true;
         g_scaled = want_scaled;

@@ -207,6 +207,27 @@ int launch_gemm_mask_colsum(void* stream, int32_t mode, int32_t ta, int32_t tb, 
                             int64_t* left_rows = nullptr);
 int launch_mask_colsum_rest(void* stream, int64_t left_rows, int64_t m, int64_t n, float* out, int32_t accumulate, void* scratch);
 size_t gemm_colsum_scratch(int64_t m, int32_t n);
+// Narrow products of small partitions (kernels_gemm.cu): C = A W [m x n], W [k x n] or (w_t) stored as W^T; then either
+// rows times row_scale (nullable), or .* [mask > 0] with sums (nullable; partial column sums, narrow_blocks rows of n rounded up
+// to 4) and rows times row_scale after them.  Rows of A, C and mask on 16-byte boundaries, pad columns of A zero.
+// w_ready: no kernel that is still to finish on the stream writes W.
+struct NarrowArgs {
+  int64_t m = 0;
+  int32_t n = 0, k = 0;
+  const float* a = nullptr;
+  int64_t lda = 0;
+  const float* w = nullptr;
+  int64_t ldw = 0;
+  bool w_t = false, w_ready = false;
+  float* c = nullptr;
+  int64_t ldc = 0;
+  const float *row_scale = nullptr, *mask = nullptr;
+  int64_t ldmask = 0;
+  float* sums = nullptr;
+};
+bool narrow_ok(int32_t mode, int64_t m, int32_t n, int32_t k);
+int64_t narrow_blocks(int64_t m, int32_t n);
+int launch_narrow(void* stream, const NarrowArgs& a);
 int64_t gemm_tc_colsum_rows(int32_t ta, int32_t tb, int64_t m, int64_t n);
 size_t gemm_tc_workspace(int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k);
 int launch_splitk_reduce(void* stream, int64_t m, int64_t n, int splits, const float* partial, int64_t ldp, float* c,

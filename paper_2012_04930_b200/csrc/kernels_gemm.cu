@@ -420,4 +420,95 @@ int launch_gemm_mask_colsum(void* stream, int32_t mode, int32_t ta, int32_t tb, 
   return launch_colsum_scaled(stream, m, n, c, ldc, out, accumulate, scratch, row_scale, row_scale ? c : nullptr, ldc);
 }
 
+namespace {
+
+// A product of a few thousand rows with an inner dimension and a width of at most 64 is over in a fraction of what the
+// tensor-core kernel needs to come up, split its operands and turn its accumulator around.  Here W lies in shared memory, a
+// thread computes four columns of a row from the row's float4s (threads of a row read the same ones), and nothing is staged.
+// What bounds it is the latency of one load of A and, with more rows, the FMA pipe and shared memory (fp32, one term): ten epochs on
+// 2 000 vertices (partitions of 1 100 rows) 630 -> 575 us, on 20 000 (5 500 rows) 1 289 -> 1 342, so 4 096 rows are the line.
+struct Narrow {
+  NarrowArgs a;
+  int q2, rows;  // quads of C's columns; rows per pass of a block
+};
+constexpr int kNarrowWidth = 64, kNarrowThreads = 256;
+constexpr int64_t kNarrowRows = 4096;
+__global__ void __launch_bounds__(kNarrowThreads) narrow_product(const __grid_constant__ Narrow p) {
+  const NarrowArgs& d = p.a;
+  if (!d.w_ready) wait_for_predecessors();
+  __shared__ float4 ws[kNarrowWidth * kNarrowWidth / 4];  // [k rounded up to 4][q2]
+  __shared__ float4 red[kNarrowThreads];
+  const int t = threadIdx.x, k4 = (d.k + 3) / 4, pitch = 4 * p.q2;
+  float* wf = reinterpret_cast<float*>(ws);
+  if (d.w_t) {
+    for (int i = t; i < 4 * k4 * pitch; i += kNarrowThreads) {
+      const int j = i / (4 * k4), k = i - j * 4 * k4;
+      wf[k * pitch + j] = j < d.n && k < d.k ? __ldg(d.w + (int64_t)j * d.ldw + k) : 0.f;
+    }
+  } else {
+    for (int i = t; i < 4 * k4 * pitch; i += kNarrowThreads) {
+      const int k = i / pitch, j = i - k * pitch;
+      wf[i] = j < d.n && k < d.k ? __ldg(d.w + (int64_t)k * d.ldw + j) : 0.f;
+    }
+  }
+  if (d.w_ready) wait_for_predecessors();
+  __syncthreads();
+  const int r = t / p.q2, q = t - r * p.q2;
+  float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (r < p.rows) {
+    for (int64_t row = (int64_t)blockIdx.x * p.rows + r; row < d.m; row += (int64_t)gridDim.x * p.rows) {
+      const float4* a = reinterpret_cast<const float4*>(d.a + row * d.lda);
+      float4 mk = make_float4(1.f, 1.f, 1.f, 1.f), acc = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (d.mask) mk = __ldg(reinterpret_cast<const float4*>(d.mask + row * d.ldmask) + q);
+      const float sc = d.row_scale ? __ldg(d.row_scale + row) : 1.f;
+#pragma unroll 8
+      for (int k = 0; k < k4; ++k) {
+        const float4 x = __ldg(a + k);
+        const float xs[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float4 w = ws[(4 * k + e) * p.q2 + q];
+          acc.x = fmaf(xs[e], w.x, acc.x); acc.y = fmaf(xs[e], w.y, acc.y);
+          acc.z = fmaf(xs[e], w.z, acc.z); acc.w = fmaf(xs[e], w.w, acc.w);
+        }
+      }
+      acc.x = mk.x > 0.f ? acc.x : 0.f; acc.y = mk.y > 0.f ? acc.y : 0.f;
+      acc.z = mk.z > 0.f ? acc.z : 0.f; acc.w = mk.w > 0.f ? acc.w : 0.f;
+      cs.x += acc.x; cs.y += acc.y; cs.z += acc.z; cs.w += acc.w;
+      acc.x *= sc; acc.y *= sc; acc.z *= sc; acc.w *= sc;
+      reinterpret_cast<float4*>(d.c + row * d.ldc)[q] = acc;
+    }
+    red[r * p.q2 + q] = cs;
+  }
+  if (!d.sums) return;
+  __syncthreads();
+  if (t < p.q2) {  // the block's rows in a fixed order
+    float4 sum = red[t];
+    for (int i = 1; i < p.rows; ++i) {
+      const float4 x = red[i * p.q2 + t];
+      sum.x += x.x; sum.y += x.y; sum.z += x.z; sum.w += x.w;
+    }
+    reinterpret_cast<float4*>(d.sums + (int64_t)blockIdx.x * pitch)[t] = sum;
+  }
+}
+
+}  // namespace
+
+bool narrow_ok(int32_t mode, int64_t m, int32_t n, int32_t k) {
+  return mode == GCNSA_GEMM_TF32X3 && m > 0 && m <= kNarrowRows && n > 0 && n <= kNarrowWidth && k > 0 && k <= kNarrowWidth;
+}
+int64_t narrow_blocks(int64_t m, int32_t n) {
+  const int64_t rows = kNarrowThreads / ((n + 3) / 4);
+  return std::min<int64_t>((m + rows - 1) / rows, 4 * 148);
+}
+int launch_narrow(void* stream, const NarrowArgs& a) {
+  Narrow p;
+  p.a = a;
+  p.q2 = (a.n + 3) / 4;
+  p.rows = kNarrowThreads / p.q2;
+  launch(narrow_product, (unsigned)narrow_blocks(a.m, a.n), kNarrowThreads, 0, (cudaStream_t)stream, p);
+  note_launch();
+  return (int)cudaGetLastError();
+}
+
 }  // namespace gcnsa

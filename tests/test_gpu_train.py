@@ -503,6 +503,43 @@ def test_cached_aggregated_features_give_the_same_training(epoch_graph, small_wl
         cached.close(); plain.close(); parts.close()
 
 
+@pytest.mark.parametrize("dims,factored_norm,use_bias", [
+    ([64, 1, 1], 1, 1), ([64, 64, 64], 1, 1), ([64, 65, 3], 1, 1), ([5, 3, 2], 1, 0), ([33, 33, 17, 5], 1, 1), ([61, 50, 29, 13], 0, 1),
+    ([30, 64, 33, 7], 1, 1)])
+def test_narrow_layers_of_small_partitions_match_checker(tiny_wl, dims, factored_norm, use_bias):
+    """Products of at most 64 inner columns and 64 wide run outside the tensor cores on partitions of up to 4 096 rows: widths at
+    and beside the quads and the limit, a widening layer, without bias, with stored values.  Bars of the other tests."""
+    w = copy.copy(tiny_wl)
+    rng = np.random.default_rng(len(dims) + dims[1])
+    w.dims, w.x = dims, np.ascontiguousarray(w.x[:, :dims[0]])
+    w.y = rng.integers(0, dims[-1], len(w.y)).astype(np.int32)
+    shapes = list(zip(dims[:-1], dims[1:]))
+    w.w0 = [(rng.standard_normal(s) / np.sqrt(s[0])).astype(np.float32) for s in shapes]
+    w.b0 = [(rng.standard_normal(s[1]) * (0.1 if use_bias else 0.0)).astype(np.float32) for s in shapes]
+    env, parts, model = _make(w, gemm_mode=gcnsa.GEMM_TF32X3, factored_norm=factored_norm, use_bias=use_bias)
+    _, rparts = oracle.build_partitions(w.rowptr, w.col, w.m, w.overlap_ppm, w.seed, w.part_mode, w.user_part)
+    ws, bs = [a.astype(np.float64) for a in w.w0], [b.astype(np.float64) for b in w.b0]
+    L = len(shapes)
+    gw, gb = [np.zeros_like(a) for a in ws], [np.zeros_like(b) for b in bs]
+    for p, pt in enumerate(rparts):
+        fw = oracle.forward(pt, w.x[pt.members], ws, bs if use_bias else None, w.y[pt.members], w.train_mask[pt.members],
+                            w.loss_on_halo)
+        model.forward(p)
+        h_gpu = [model.get(gcnsa.GET_ACT, l, rows=pt.n) for l in range(1, L + 1)]
+        for l in range(L):
+            _close(h_gpu[l], fw["H"][l + 1], what=f"p{p} H{l + 1}")
+        bw = oracle.backward(pt, fw, ws, w.y[pt.members], relu_on=_relu_decisions(fw, h_gpu[:-1]))
+        model.backward(p)
+        for l in range(L):
+            gw[l] += bw["dW"][l]; gb[l] += bw["db"][l]
+    for l in range(L):
+        _close(model.get(gcnsa.GET_GRAD_W, l), gw[l], what=f"dW{l}")
+        if use_bias:
+            _close(model.get(gcnsa.GET_GRAD_B, l), gb[l], what=f"db{l}")
+    assert gcnsa.tc_status() == 0
+    model.close(); parts.close()
+
+
 @pytest.mark.parametrize("c", [1, 32, 33, 64, 65, 128, 129, 256, 257])
 def test_last_layer_gradients_for_every_number_of_classes(tiny_wl, c):
     """The softmax kernel holds a row in 8, 16 or 32 lanes, one or two float4 each (up to 32, 64, 128, 256 columns), and

@@ -714,47 +714,91 @@ static int check_model(const gcnsa_model* M, const gcnsa_parts* P) {
   return GCNSA_OK;
 }
 
-// The streams a recorded epoch forks into (only while it is being recorded: a replay has the branches in its graph).
+// The branches of an epoch that is being recorded.  There is one stream; a branch is the set of recorded nodes that its next
+// launch depends on, and `use` makes that of another branch the stream's.  (A stream and events for each branch cost a first
+// epoch 0.1 to 0.2 ms a branch, and a replay has the branches in its graph anyway.)
 struct Fork {
-  std::vector<cudaStream_t> side;
-  std::vector<cudaEvent_t> ev;
-  size_t used = 0;
-  bool make(int n) {
-    for (int i = 0; i < n; ++i) {
-      cudaStream_t st;
-      if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) return false;
-      side.push_back(st);
+  struct Deps {
+    std::vector<cudaGraphNode_t> nodes;
+    std::vector<cudaGraphEdgeData> edges;
+    void add(const Deps& d) {
+      for (size_t i = 0; i < d.nodes.size(); ++i)
+        if (std::find(nodes.begin(), nodes.end(), d.nodes[i]) == nodes.end()) {
+          nodes.push_back(d.nodes[i]);
+          edges.push_back(d.edges[i]);
+        }
     }
-    return true;
+  };
+  cudaStream_t s = nullptr;
+  std::vector<Deps> at;
+  int cur = 0;
+  cudaError_t now(Deps* d) const {
+    cudaStreamCaptureStatus status;
+    const cudaGraphNode_t* nodes = nullptr;
+    const cudaGraphEdgeData* edges = nullptr;
+    size_t n = 0;
+    const cudaError_t rc = cudaStreamGetCaptureInfo_v3(s, &status, nullptr, nullptr, &nodes, &edges, &n);
+    if (rc != cudaSuccess) return rc;
+    if (status != cudaStreamCaptureStatusActive) return cudaErrorStreamCaptureInvalidated;
+    d->nodes.assign(nodes, nodes + n);
+    if (edges) d->edges.assign(edges, edges + n);
+    else d->edges.assign(n, cudaGraphEdgeData{});
+    return cudaSuccess;
   }
-  // what `from` has been given so far, for cudaStreamWaitEvent
-  cudaError_t mark(cudaStream_t from, cudaEvent_t* out) {
-    if (used == ev.size()) {
-      cudaEvent_t e;
-      cudaError_t rc = cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
-      if (rc != cudaSuccess) return rc;
-      ev.push_back(e);
+  cudaError_t put(Deps& d) const {
+    return cudaStreamUpdateCaptureDependencies_v2(s, d.nodes.data(), d.edges.data(), d.nodes.size(), cudaStreamSetCaptureDependencies);
+  }
+  // branches 0 (what the stream has been given so far) to n - 1
+  void begin(cudaStream_t stream, int n) {
+    s = stream;
+    at.assign((size_t)n, Deps());
+    cur = 0;
+  }
+  // what follows on the stream is branch k's
+  cudaError_t use(int k) {
+    if (k == cur) return cudaSuccess;
+    cudaError_t rc = now(&at[cur]);
+    if (rc == cudaSuccess) rc = put(at[k]);
+    if (rc == cudaSuccess) cur = k;
+    return rc;
+  }
+  // what branch k has been given so far
+  cudaError_t mark(int k, Deps* d) const {
+    if (k == cur) return now(d);
+    *d = at[k];
+    return cudaSuccess;
+  }
+  // branch k waits for what is in d
+  cudaError_t wait(int k, const Deps& d) {
+    if (k != cur) {
+      at[k].add(d);
+      return cudaSuccess;
     }
-    *out = ev[used++];
-    return cudaEventRecord(*out, from);
+    Deps mine;
+    cudaError_t rc = now(&mine);
+    mine.add(d);
+    return rc == cudaSuccess ? put(mine) : rc;
   }
-  // `to` waits for what `from` has been given so far
-  cudaError_t edge(cudaStream_t from, cudaStream_t to) {
-    cudaEvent_t e;
-    cudaError_t rc = mark(from, &e);
-    return rc == cudaSuccess ? cudaStreamWaitEvent(to, e, 0) : rc;
-  }
-  ~Fork() {
-    for (cudaStream_t st : side) cudaStreamDestroy(st);
-    for (cudaEvent_t e : ev) cudaEventDestroy(e);
+  cudaError_t edge(int from, int to) {
+    Deps d;
+    const cudaError_t rc = mark(from, &d);
+    return rc == cudaSuccess ? wait(to, d) : rc;
   }
 };
 
 // Where a recorded epoch puts what the next kernel of a pass does not read (the loss, bias gradients, the weight gradients
-// of all layers but the first): a branch t beside the pass's stream.  t == NULL: everything on the stream.
+// of all layers but the first): a branch `side` beside the pass's branch `lane`.  fork == NULL: everything in a row.
 struct Branch {
   Fork* fork = nullptr;
-  cudaStream_t t = nullptr;
+  int lane = 0, side = 0;
+  // launches go to the branch, after what the pass has been given so far (also = false: after what it was given when it was
+  // last asked), until back()
+  cudaError_t aside(bool also = true) const {
+    if (!fork) return cudaSuccess;
+    const cudaError_t rc = also ? fork->edge(lane, side) : cudaSuccess;
+    return rc == cudaSuccess ? fork->use(side) : rc;
+  }
+  cudaError_t back() const { return fork ? fork->use(lane) : cudaSuccess; }
 };
 
 // forward pass of partition p in the buffers of lane W on stream s; the partition's loss goes to loss_parts[p]
@@ -824,11 +868,12 @@ static int forward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& W
     }
   }
   PROF(M, 2, (side.scaled ? 12.0 : 8.0) * n * P->c + 5.0 * n, 0.0,
-       launch_softmax_ce(s, n, P->c, h, ldc, d.y, d.mask, d.info.n_train, br.t ? nullptr : M->loss_parts + p, W.dlogits, ldc,
+       launch_softmax_ce(s, n, P->c, h, ldc, d.y, d.mask, d.info.n_train, br.fork ? nullptr : M->loss_parts + p, W.dlogits, ldc,
                          W.ce_part, side));
-  if (br.t) {
-    CK(br.fork->edge((cudaStream_t)s, br.t));
-    CKL(launch_ce_loss(br.t, n, P->c, d.info.n_train, W.ce_part, M->loss_parts + p));
+  if (br.fork) {
+    CK(br.aside());
+    CKL(launch_ce_loss(s, n, P->c, d.info.n_train, W.ce_part, M->loss_parts + p));
+    CK(br.back());
   }
   return GCNSA_OK;
 }
@@ -839,11 +884,10 @@ static int backward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& 
                          const Branch& br = Branch{}) {
   const DevPart& d = P->parts[p];
   const int64_t n = d.info.n;
-  void* t = br.t ? (void*)br.t : s;
-  cudaEvent_t q_read = nullptr, sums_read = nullptr;  // the branch's readers of tmp_b and of sc
-  auto wait = [&](cudaEvent_t& e) {
-    const cudaError_t rc = e ? cudaStreamWaitEvent((cudaStream_t)s, e, 0) : cudaSuccess;
-    e = nullptr;
+  Fork::Deps q_read, sums_read;  // the branch's readers of tmp_b and of sc
+  auto wait = [&](Fork::Deps& e) {
+    const cudaError_t rc = e.nodes.empty() ? cudaSuccess : br.fork->wait(br.lane, e);
+    e = Fork::Deps();
     return rc;
   };
   const float* g = W.dlogits;  // gradient w.r.t. Z^l, [n x LD(dims[l+1])]
@@ -862,8 +906,11 @@ static int backward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& 
       scaled = g_scaled;
     } else if (l == M->L - 1 && ce_by_groups(dout)) {  // the softmax kernel has made the partial sums and the scaled copy
       scaled = fact && M->transform_first[l];
-      if (M->o.use_bias)
-        PROF(M, 2, 0.0, 0.0, launch_ce_sums(t, n, dout, W.ce_sums, grad + M->b_off[l], acc));
+      if (M->o.use_bias) {
+        CK(br.aside(false));
+        PROF(M, 2, 0.0, 0.0, launch_ce_sums(s, n, dout, W.ce_sums, grad + M->b_off[l], acc));
+        CK(br.back());
+      }
     } else if (M->o.use_bias) {
       CK(wait(sums_read));
       if (fact && M->transform_first[l]) {
@@ -888,12 +935,15 @@ static int backward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& 
                                     GCNSA_EPI_NONE, nullptr, 0, W.tmp_b, ldo);
       if (rc) return rc;
       // (the workspace has room for one of the two products of Q)
-      const bool aside = br.t && l > 0 && gemm_workspace(M->o.gemm_mode, 0, 1, n, din, dout) == 0;
-      if (aside) CK(br.fork->edge((cudaStream_t)s, br.t));
+      const bool aside = br.fork && l > 0 && gemm_workspace(M->o.gemm_mode, 0, 1, n, din, dout) == 0;
+      if (aside) CK(br.aside());
       PROF(M, 1, gemm_bytes(din, dout, n), 2.0 * n * dout * din,
-           launch_gemm(aside ? t : s, M->o.gemm_mode, 1, 0, din, dout, n, hprev, ldi, W.tmp_b, ldo, gw, M->w_ld[l], acc,
+           launch_gemm(s, M->o.gemm_mode, 1, 0, din, dout, n, hprev, ldi, W.tmp_b, ldo, gw, M->w_ld[l], acc,
                        GCNSA_EPI_NONE, nullptr, 0, W.ws, M->ws_bytes, M->beside));
-      if (aside) CK(br.fork->mark(br.t, &q_read));
+      if (aside) {
+        CK(br.fork->mark(br.side, &q_read));
+        CK(br.back());
+      }
       bias_done = g_scaled = false;
       if (l > 0 && M->o.use_bias) {
         // G^{l-1}, its column sums (the bias gradient of layer l - 1) and, where the next transposed product wants
@@ -911,19 +961,21 @@ static int backward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& 
           na.mask = hprev; na.ldmask = ldi;
           na.sums = (float*)W.sc;
           PROF(M, 1, gemm_bytes(n, din, dout) + 4.0 * n * din, 2.0 * n * dout * din, launch_narrow(s, na));
-          if (br.t) CK(br.fork->edge((cudaStream_t)s, br.t));
-          PROF(M, 1, 0.0, 0.0, launch_sum_rows(t, narrow_blocks(n, din), din, na.sums, (din + 3) / 4 * 4, grad + M->b_off[l - 1], acc,
+          CK(br.aside());
+          PROF(M, 1, 0.0, 0.0, launch_sum_rows(s, narrow_blocks(n, din), din, na.sums, (din + 3) / 4 * 4, grad + M->b_off[l - 1], acc,
                                                nullptr));
-          if (br.t) CK(br.fork->mark(br.t, &sums_read));
+          if (br.fork) CK(br.fork->mark(br.side, &sums_read));
+          CK(br.back());
         } else {
           PROF(M, 1, gemm_bytes(n, din, dout) + 4.0 * n * din, 2.0 * n * dout * din,
                launch_gemm_mask_colsum(s, M->o.gemm_mode, 0, 1, n, din, dout, W.tmp_b, ldo, w, M->w_ld[l], W.tmp_a, ldi, hprev,
                                        ldi, want_scaled ? d.dinv : nullptr, grad + M->b_off[l - 1], acc, W.sc, W.ws,
-                                       M->ws_bytes, br.t ? &left : nullptr));
+                                       M->ws_bytes, br.fork ? &left : nullptr));
           if (left) {
-            CK(br.fork->edge((cudaStream_t)s, br.t));
-            CKL(launch_mask_colsum_rest(t, left, n, din, grad + M->b_off[l - 1], acc, W.sc));
-            CK(br.fork->mark(br.t, &sums_read));
+            CK(br.aside());
+            CKL(launch_mask_colsum_rest(s, left, n, din, grad + M->b_off[l - 1], acc, W.sc));
+            CK(br.fork->mark(br.side, &sums_read));
+            CK(br.back());
           }
         }
         bias_done = true;
@@ -953,7 +1005,7 @@ static int backward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& 
       }
     }
   }
-  if (br.t) CK(br.fork->edge(br.t, (cudaStream_t)s));
+  if (br.fork) CK(br.fork->edge(br.side, br.lane));
   return GCNSA_OK;
 }
 
@@ -1046,29 +1098,40 @@ static int epoch_body(gcnsa_model* M, const gcnsa_parts* P, float* loss_dev, For
   int rc = check_model(M, P);
   if (rc) return rc;
   cudaStream_t s = M->env.stream();
-  const int lanes = fork ? (int)M->lanes.size() : 1;
-  auto stream_of = [&](int lane) { return lane == 0 || !fork ? s : fork->side[lane - 1]; };
-  cudaStream_t aux = fork ? fork->side[lanes - 1] : s;
-  if (fork)
-    for (int i = 0; i < lanes; ++i) CK(fork->edge(s, fork->side[i]));
+  // branches: the lanes, one for the step count and the loss, one beside every lane
+  const int lanes = fork ? (int)M->lanes.size() : 1, aux = lanes;
+  if (fork) {
+    fork->begin(s, 2 * lanes + 1);
+    for (int i = 1; i <= lanes; ++i) CK(fork->edge(0, i));
+  }
   const bool early = fork && M->gparts;  // (beside the passes)
-  if (early) PROF(M, 2, 0.0, 0.0, launch_adam_advance(aux, M->adam_state, M->o.beta1, M->o.beta2));  // t -> t + 1
+  if (early) {
+    CK(fork->use(aux));
+    PROF(M, 2, 0.0, 0.0, launch_adam_advance(s, M->adam_state, M->o.beta1, M->o.beta2));  // t -> t + 1
+  }
   for (int32_t p = 0; p < P->m; ++p) {
     const int lane = (P->m - 1 - p) % lanes;
     Branch br;
-    if (early && beside(P)) br = Branch{fork, fork->side[lanes + lane]};
-    rc = epoch_partition(M, P, p, M->lanes[lane], stream_of(lane), br);
+    if (early && beside(P)) br = Branch{fork, lane, lanes + 1 + lane};
+    if (fork) CK(fork->use(lane));
+    rc = epoch_partition(M, P, p, M->lanes[lane], s, br);
     if (rc) return rc;
   }
-  if (fork)
-    for (int i = 0; i < lanes; ++i) CK(fork->edge(fork->side[i], s));
+  if (fork) {
+    CK(fork->use(0));
+    for (int i = 1; i <= lanes; ++i) CK(fork->edge(i, 0));
+  }
   if (loss_dev) {
-    if (fork) CK(fork->edge(s, aux));
-    CKL(launch_mean(aux, M->loss_parts, M->m, loss_dev));
+    if (fork) {
+      CK(fork->edge(0, aux));
+      CK(fork->use(aux));
+    }
+    CKL(launch_mean(s, M->loss_parts, M->m, loss_dev));
+    if (fork) CK(fork->use(0));
   }
   rc = optimizer_step(M, s, early);
   if (rc) return rc;
-  if (loss_dev && fork) CK(fork->edge(aux, s));
+  if (loss_dev && fork) CK(fork->edge(aux, 0));
   M->last_forward = -1;
   M->last_n = P->parts[P->m - 1].info.n;
   return GCNSA_OK;
@@ -1096,7 +1159,7 @@ int gcnsa_epoch(gcnsa_model* M, const gcnsa_parts* P, float* loss_dev) {
     cudaGraph_t graph = nullptr;
     int rc = GCNSA_OK;
     Fork fork;
-    if (!fork.make(2 * (int)M->lanes.size()) || cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+    if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
       cudaGetLastError();
       M->graph_off = true;
       return epoch_body(M, P, loss_dev, nullptr);

@@ -485,15 +485,17 @@ static int epoch_lanes(const gcnsa_model* M, const gcnsa_parts* parts, size_t la
   return (int)std::min<int64_t>(std::min<int64_t>(parts->m, kMaxLanes), 1 + (int64_t)(kLaneBytes / lane_bytes));
 }
 
-// Whether the passes of a recorded epoch have branches: where partitions are small enough for lanes, kernels leave room beside
-// them and the chain of launches is the time.  A pass of two layers goes from 16 launches in a row to 11: ten epochs on
-// 2 000 vertices 702 -> 640 us, on 20 000 vertices 1 548 -> 1 486 us, partitions of 19 414 rows and 2 M entries alike
-// (3 085 -> 3 069 us).
+// Whether partitions are small enough that several are worked on at once (epoch_lanes: where kernels leave room beside them).
 static bool beside(const gcnsa_parts* P) {
   int64_t nnz_max = 0;
   for (const DevPart& d : P->parts) nnz_max = std::max<int64_t>(nnz_max, d.info.nnz);
-  return nnz_max <= kLaneNnz && ce_by_groups(P->c);
+  return nnz_max <= kLaneNnz;
 }
+// Whether the passes of a recorded epoch have branches: while the chain of launches is the time.  A pass of two layers goes from
+// 16 launches in a row to 11: ten epochs on 2 000 vertices 702 -> 640 us, on 20 000 vertices (partitions of 5 500 rows) 1 548 ->
+// 1 486 us, partitions of 21 400 rows alike (3 085 -> 3 069 us), 51 400 rows (a hidden layer of 222) 1 000 -> 1 013.
+constexpr int64_t kBranchRows = 16384;
+static bool branches(const gcnsa_parts* P) { return beside(P) && P->n_max <= kBranchRows && ce_by_groups(P->c); }
 
 // one lane's buffers; *bytes (nullable) grows by what was asked for
 static bool alloc_lane(gcnsa_model* M, Lane& W, size_t act, size_t* bytes_out = nullptr) {
@@ -1112,7 +1114,7 @@ static int epoch_body(gcnsa_model* M, const gcnsa_parts* P, float* loss_dev, For
   for (int32_t p = 0; p < P->m; ++p) {
     const int lane = (P->m - 1 - p) % lanes;
     Branch br;
-    if (early && beside(P)) br = Branch{fork, lane, lanes + 1 + lane};
+    if (early && branches(P)) br = Branch{fork, lane, lanes + 1 + lane};
     if (fork) CK(fork->use(lane));
     rc = epoch_partition(M, P, p, M->lanes[lane], s, br);
     if (rc) return rc;

@@ -1191,7 +1191,8 @@ int gcnsa_sage_profile_read(gcnsa_sage* S, gcnsa_profile* out) {
   }
   u64 rows[2] = {0, 0};
   SCK(cudaMemcpy(rows, S->read_rows, sizeof(rows), cudaMemcpyDeviceToHost));
-  out->alg_bytes[0] += 4.0 * ((double)rows[0] * (double)S->f + (double)rows[1] * (double)S->h);
+  out->alg_bytes[0] += 4.0 * (double)rows[0] * (double)S->f;
+  out->alg_bytes[S->head_qp > 0 ? 2 : 0] += 4.0 * (double)rows[1] * (double)S->h;  // (sage_head gathers them itself)
   for (int c = 0; c < 3; ++c) { out->l1_bytes[c] = out->alg_bytes[c]; out->alg_bytes_val[c] = out->alg_bytes[c]; }
   S->recs.clear();
   SCK(cudaMemsetAsync(S->read_rows, 0, 2 * sizeof(u64), S->env.stream()));

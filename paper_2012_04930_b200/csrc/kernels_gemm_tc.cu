@@ -21,7 +21,9 @@
 // A_lo B_hi - into a TMEM accumulator, and warps 12-15 read the accumulator
 // back, turn it through shared memory so that global accesses are
 // row-contiguous, and apply the epilogue - while the other roles already work on
-// the CTA's next item in a second accumulator buffer.  All
+// the CTA's next item in a second accumulator buffer.  Where the k-slices of a
+// tile form a cluster, each CTA leaves its sums in shared memory instead and all
+// of them add up their share of the rows (cluster_sync, cluster_load).  All
 // waits are bounded (tens of milliseconds; a healthy phase takes microseconds):
 // a wait that runs out sets an error word that the host reads
 // (gcnsa_tc_status) and the CTA winds down.  The word is sticky: waiting threads

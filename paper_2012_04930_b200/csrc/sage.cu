@@ -829,7 +829,7 @@ int gcnsa_sage_destroy(gcnsa_sage* S) {
 }
 
 // How many workers an epoch runs at once: up to eight while a batch has at most kLaneRows rows in the hidden layer.  The
-// two dozen kernels of a batch are a chain of microseconds on a fraction of the SMs, so workers side by side overlap
+// kernels of a batch (13, or two dozen) are a chain of microseconds on a fraction of the SMs, so workers side by side overlap
 // (116 K vertices, 5 workers, batches of 256: 63.2 ms per epoch with one lane, 47.7 with two, 38.4 with four, 29.9
 // with five; 20 000 vertices, 4 workers: 7.7 -> 4.2 ms).  Larger batches fill the chip by themselves and their lanes
 // would cost gigabytes.  The lanes after the first take at most 1 GB (a batch of 2 816 rows of 602 features 17 MB each; with

@@ -356,7 +356,8 @@ gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             int k_blocks, int k_blocks_per_split, int tiles_m, int tiles_n, int total_work, float* __restrict__ c,
             int64_t ldc, int accumulate, int epi, const float* __restrict__ aux, int64_t ldaux,
             int64_t slice_stride, int vec_ok, int terms, float* __restrict__ colsum_partial,
-            const float* __restrict__ post_scale, int csplit) {
+            const float* __restrict__ post_scale, int cluster) {
+  const int csplit = S::DB ? 1 : cluster;  // (blocks with several items are never in a cluster)
   constexpr int BN = S::BN, NS = S::NS, NA = S::NA, B_BYTES = S::B_BYTES;
   constexpr int ACC_COLS = S::ACC_COLS, NBUF = S::NBUF;
   constexpr bool A_MN = S::A_MN, B_MN = S::B_MN;

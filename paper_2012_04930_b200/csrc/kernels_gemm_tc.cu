@@ -878,9 +878,8 @@ struct TcPlan {
   size_t partial_bytes;
 };
 
-// Eight slices where a product is at most this many k-blocks long, though more SMs are idle: ten epochs on 20 000 vertices in four
-// partitions (172 k-blocks) 1 486 -> 1 413 us; with a limit of 64 GraphSAGE batches (88) go 2 120 -> 2 285.
-constexpr int kClusterBlocks = 256;
+// products that run side by side are cut by the rule below up to this many k-blocks
+constexpr int kBesideBlocks = 256;
 // a cluster lives in one of the chip's eight parts, of which at least 16 SMs each are counted on
 constexpr int kClusterParts = 8, kClusterSms = 16;
 
@@ -909,15 +908,14 @@ TcPlan tc_plan(int64_t m, int64_t n, int64_t k, int beside = 1) {
   // an SM the microseconds in which a block comes up, drains and meets its cluster.  Ten epochs on 20 000 vertices in four
   // partitions 1 410 -> 1 289 us; GraphSAGE epochs (2 816 x 128 x 1 216, four and five at a time) 2 115 -> 1 998 us and 19.05 ->
   // 17.0 ms.
-  if (beside > 1 && p.k_blocks <= kClusterBlocks) splits = std::min<int64_t>(splits, sms / std::min(beside, 3) / tiles);
+  if (beside > 1 && p.k_blocks <= kBesideBlocks) splits = std::min<int64_t>(splits, sms / std::min(beside, 3) / tiles);
   splits = std::max<int64_t>(splits, 1);
-  // Up to eight slices are a cluster: they meet in shared memory, and the pass over partial results in memory (5 to 8 us alone
-  // on the chip, a launch in the chain) is gone.  GraphSAGE epochs of 20 000 / 116 483 vertices 2 630 -> 2 330 us and 20.8 ->
-  // 19.7 ms, ten epochs on 2 000 / 20 000 vertices 727 -> 705 and 1 634 -> 1 545 us.  More slices only where eight of them
-  // would be long.
-  int64_t in_cluster = splits <= kMaxCluster || p.k_blocks <= kClusterBlocks ? std::min<int64_t>(splits, kMaxCluster) : 1;
-  while (in_cluster > 1 && tiles > kClusterParts * (kClusterSms / in_cluster)) --in_cluster;
-  if (in_cluster > 1) splits = in_cluster;
+  // Up to eight slices are a cluster: they meet in shared memory, and the pass over partial results in memory (a launch in the
+  // chain) is gone.  Alone on the chip 64 x 16 x 2 112: 9.7 -> 8.0 us, 256 x 256 x 2 112: 12.4 -> 12.1, 2 816 x 128 x 1 204: 16.0 -> 12.9.
+  // Eight slices where there would be more lose: each adds its 0.25 to 0.4 us per k-block (500 x 64 x 5 504, 21 slices: 10.5 us, eight:
+  // 14.0; 256 x 256 x 8 192: 13.9 and 22.8), and the tensor core cuts its sums off at 24 bits instead of rounding them, so that
+  // the error grows with the length of a slice (1.6e-6 with 8 k-blocks, 3.6e-6 with 22, 5.2e-6 with 32, of the 2-norm).
+  const int64_t in_cluster = splits <= kMaxCluster && tiles <= kClusterParts * (kClusterSms / splits) ? splits : 1;
   p.kb_per_split = (int)((p.k_blocks + splits - 1) / splits);
   p.splits = (p.k_blocks + p.kb_per_split - 1) / p.kb_per_split;
   if (p.splits < 1) p.splits = 1;

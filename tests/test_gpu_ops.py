@@ -383,6 +383,26 @@ def test_tensor_core_gemm_slices_meet_in_a_cluster(m, n, k, ta, tb):
     assert gcnsa.tc_status() == 0 and gcnsa.gemm_path_counts() == (tc0 + calls, fb0)
 
 
+# inner dimensions of 67 to 257 k-blocks: the rows of small partitions, where the weight gradients are cut into slices
+@pytest.mark.parametrize("k", [2144, 2752, 4096, 5504, 6400, 8192, 8224])
+@pytest.mark.parametrize("m,n", [(64, 16), (500, 64), (64, 128), (602, 128), (256, 256)])
+def test_tensor_core_gemm_slices_keep_fp32_accuracy(m, n, k):
+    """Activations behind a ReLU times a gradient, in the 2-norm.  The tensor core cuts every sum of 8 products off at 24 bits:
+    two cuts of at most 2^-23 per 8 k, half of that on average, on a sum that is half its end on average, make 2^-24 per 8 k
+    and 2.4e-7 per k-block of a slice; slices here have at most 9 k-blocks, and the dropped terms are 2^-22: 2.5e-6."""
+    rng = np.random.default_rng(m + 3 * n + k)
+    a = np.maximum(rng.standard_normal((k, m)), 0).astype(np.float32)
+    b = (1e-3 * rng.standard_normal((k, n))).astype(np.float32)
+    want = a.T.astype(np.float64) @ b.astype(np.float64)
+    cd = torch.empty((m, _ld(n)), device="cuda")
+    ws = torch.empty(gcnsa.op_gemm_workspace(1, 0, m, n, k, gcnsa.GEMM_TF32X3) // 4 + 64, device="cuda")
+    tc0, fb0 = gcnsa.gemm_path_counts()
+    gcnsa.op_gemm(_padded(a, _ld(m)), _padded(b, _ld(n)), cd, m, n, k, ta=1, workspace=ws, mode=gcnsa.GEMM_TF32X3)
+    assert gcnsa.tc_status() == 0 and gcnsa.gemm_path_counts() == (tc0 + 1, fb0)
+    err = np.linalg.norm(cd[:, :n].cpu().numpy() - want) / np.linalg.norm(want)
+    assert err <= 2.5e-6, err
+
+
 def test_tensor_core_gemm_split_k_epilogues_and_fallback():
     rng = np.random.default_rng(5)
     kk, m, n = 20_011, 130, 41                       # H^T dT: inner dimension = rows of a partition

@@ -157,8 +157,11 @@ __device__ __forceinline__ void split_buffer(const uint8_t* hi_buf, uint8_t* lo_
 // Tensor memory has 512 columns: four A stages take 256, the accumulators the rest.  Where 2 BN columns per
 // accumulator buffer fit (64-column tiles; 128-column tiles when every CTA has a single item, so one buffer),
 // A_hi [B_hi | B_lo] is ONE instruction of 2 BN columns into two accumulators that the epilogue adds, and with
-// A_lo B_hi that makes two instructions per 8 k; otherwise the three products are three instructions into one
-// accumulator.  With the issuing thread behind elect.sync the tensor pipe sets the pace (see elect_one); behind
+// A_lo B_hi, into the second of them, that makes two instructions per 8 k; otherwise the three products are three
+// instructions into one accumulator.  The tensor core cuts a sum off at 24 bits where an fp32 addition rounds, always toward
+// zero, so the error of a sum grows with the instructions that add to it.  Small terms that have an accumulator of their own
+// (2^-11 of the other) leave one cut per 8 k in the large one instead of two: 1.65e-6 -> 0.93e-6 of the 2-norm with slices of
+// 8 or 9 k-blocks, 5.2e-6 -> 2.7e-6 with 33, at the same speed.  With the issuing thread behind elect.sync the tensor pipe sets the pace (see elect_one); behind
 // `lane == 0` an instruction cost it 97 clocks whether 128 or 256 columns wide.  51 249 x 128 x 602: 57 -> 47 us,
 // 269 498 x 256 x 256: 201 -> 151 us, 256 x 256 x 269 498: 169 -> 151 us (L2 flushed).
 template <int BN_, bool A_MN_, bool B_MN_, bool DB_, bool MASKED_ = false>
@@ -283,7 +286,7 @@ __device__ __forceinline__ void masked_epilogue(int w_epi, int lane, uint32_t tm
       uint32_t v[32];
       tmem_ld32(acc + (uint32_t)c0, v);
       if constexpr (S::MERGED) {
-        if (terms == 3) {  // the second accumulator: A_hi B_lo
+        if (terms == 3) {  // the second accumulator: A_hi B_lo + A_lo B_hi
           uint32_t u[32];
           tmem_ld32(acc + (uint32_t)(BN + c0), u);
 #pragma unroll
@@ -499,8 +502,8 @@ gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             if (terms != 3) {
               umma_tf32_ta(d, ta, b_hi + adv_b, idesc, first);       // plain TF32: the leading parts only
             } else if constexpr (S::MERGED) {
-              umma_tf32_ta(d, ta, b_hi + adv_b, idesc2, first);      // A_hi [B_hi | B_lo]
-              umma_tf32_ta(d, ta + 32, b_hi + adv_b, idesc, 1);      // + A_lo B_hi on the first half
+              umma_tf32_ta(d, ta, b_hi + adv_b, idesc2, first);       // A_hi [B_hi | B_lo]
+              umma_tf32_ta(d + BN, ta + 32, b_hi + adv_b, idesc, 1);  // + A_lo B_hi on the second half
             } else {
               umma_tf32_ta(d, ta, b_hi + adv_b, idesc, first);
               umma_tf32_ta(d, ta, b_lo + adv_b, idesc, 1);
@@ -662,7 +665,7 @@ gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         uint32_t v[32];
         tmem_ld32(acc + (uint32_t)c0, v);
         if constexpr (S::MERGED) {
-          if (terms == 3) {  // the second accumulator: A_hi B_lo
+          if (terms == 3) {  // the second accumulator: A_hi B_lo + A_lo B_hi
             uint32_t u[32];
             tmem_ld32(acc + (uint32_t)(BN + c0), u);
 #pragma unroll
@@ -906,15 +909,19 @@ TcPlan tc_plan(int64_t m, int64_t n, int64_t k, int beside = 1) {
   if (tiles < sms / 2 && p.k_blocks >= 16) splits = std::min<int64_t>(sms / tiles, p.k_blocks / 8);
   // Products that run side by side share the chip: a third of it each.  More slices end a product sooner alone, but each costs
   // an SM the microseconds in which a block comes up, drains and meets its cluster.  Ten epochs on 20 000 vertices in four
-  // partitions 1 410 -> 1 289 us; GraphSAGE epochs (2 816 x 128 x 1 216, four and five at a time) 2 115 -> 1 998 us and 19.05 ->
-  // 17.0 ms.
-  if (beside > 1 && p.k_blocks <= kBesideBlocks) splits = std::min<int64_t>(splits, sms / std::min(beside, 3) / tiles);
+  // partitions 1 476 -> 1 314 us; GraphSAGE epochs (2 816 x 128 x 1 216, four and five at a time) 2 292 -> 2 004 us and 19.9 -> 17.6 ms.
   splits = std::max<int64_t>(splits, 1);
+  if (beside > 1 && splits > 1 && p.k_blocks <= kBesideBlocks) {
+    const int64_t third = sms / std::min(beside, 3) / tiles, length = (p.k_blocks + splits - 1) / splits;
+    // Slices of up to twice the length have the error that slices alone would have with all terms in one accumulator (above
+    // Shape); unbounded, GraphSAGE's hidden weights ended an epoch 1.2e-5 from fp64 instead of 5e-7.
+    splits = std::min(splits, std::max(third, (p.k_blocks + 2 * length - 1) / (2 * length)));
+  }
   // Up to eight slices are a cluster: they meet in shared memory, and the pass over partial results in memory (a launch in the
   // chain) is gone.  Alone on the chip 64 x 16 x 2 112: 9.7 -> 8.0 us, 256 x 256 x 2 112: 12.4 -> 12.1, 2 816 x 128 x 1 204: 16.0 -> 12.9.
   // Eight slices where there would be more lose: each adds its 0.25 to 0.4 us per k-block (500 x 64 x 5 504, 21 slices: 10.5 us, eight:
   // 14.0; 256 x 256 x 8 192: 13.9 and 22.8), and the tensor core cuts its sums off at 24 bits instead of rounding them, so that
-  // the error grows with the length of a slice (1.6e-6 with 8 k-blocks, 3.6e-6 with 22, 5.2e-6 with 32, of the 2-norm).
+  // the error grows with the length of a slice (0.9e-6 of the 2-norm with 8 k-blocks, 2.7e-6 with 33).
   const int64_t in_cluster = splits <= kMaxCluster && tiles <= kClusterParts * (kClusterSms / splits) ? splits : 1;
   p.kb_per_split = (int)((p.k_blocks + splits - 1) / splits);
   p.splits = (p.k_blocks + p.kb_per_split - 1) / p.kb_per_split;

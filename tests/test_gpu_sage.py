@@ -149,6 +149,28 @@ def test_one_batch_matches_checker(name, hidden, fanout, batch, gemm_mode, tiny_
     model.close(); parts.close()
 
 
+@pytest.mark.parametrize("hidden", [64, 128])
+def test_products_of_workers_side_by_side_keep_fp32_accuracy(hidden, small_wl):
+    """Four workers' products are cut for several that run at once: hidden layer and its weight gradients of three batches
+    against the checker in the 2-norm.  A slice has at most 16 k-blocks with one cut of at most 2^-23 per 8 k, half of that on
+    average, on a sum that is half its end on average: 2^-23 per k-block, 1.9e-6, with the dropped terms 2.1e-6; 0.4e-6 for
+    the rest of the batch."""
+    w = small_wl
+    env, parts, model, rparts, params, xs, ys, trs = _setup(w, hidden, (25, 10), 256, 0.01, gcnsa.GEMM_TF32X3)
+    errs = []
+    for b, tg in enumerate(sage.batches(rparts[0], trs[0], w.seed, 0, 256)[:3]):
+        fw = sage.batch_forward(rparts[0], xs[0], params, tg, ys[0], w.seed, 0, (25, 10))
+        model.run_batch(0, 0, b, apply=False)
+        e = model.batch_export()
+        grads, _ = sage.batch_backward(fw, xs[0], params, relu_on=_relu_decisions(fw, e))
+        valid = e["vertices"] >= 0
+        rows = np.array([fw["where"][int(v)] for v in e["vertices"][valid]])
+        pairs = [(e["hidden"][valid], fw["h1"][rows])] + list(zip(_gpu_params(model, gcnsa.SAGE_GRAD_W_SELF)[:2], grads[:2]))
+        errs.append([np.linalg.norm(got - want) / np.linalg.norm(want) for got, want in pairs])
+    assert gcnsa.tc_status() == 0 and np.max(errs) <= 2.5e-6, errs
+    model.close(); parts.close()
+
+
 @pytest.mark.parametrize("name,hidden,fanout,batch,epochs,lr", [("tiny", 16, (25, 10), 256, 10, 0.003),
                                                                ("small", 64, (25, 10), 256, 5, 0.0005)])
 def test_loss_curve_and_averaged_parameters_match_checker(name, hidden, fanout, batch, epochs, lr, tiny_wl, small_wl):

@@ -540,6 +540,28 @@ def test_narrow_layers_of_small_partitions_match_checker(tiny_wl, dims, factored
     model.close(); parts.close()
 
 
+def test_weight_gradients_of_partitions_side_by_side_keep_fp32_accuracy(small_wl):
+    """Partitions of 5 500 rows (172 k-blocks) whose products are cut for several that run at once: the first layer's weight
+    gradient against the checker in the 2-norm.  A slice has at most 18 k-blocks with one cut of at most 2^-23 per 8 k, half of
+    that on average, on a sum that is half its end on average: 2^-23 per k-block, 2.1e-6, with the dropped terms 2.3e-6;
+    0.4e-6 for the sparse products and the softmax in front of it."""
+    w = small_wl
+    env, parts, model = _make(w, gemm_mode=gcnsa.GEMM_TF32X3, factored_norm=1)
+    _, rparts = oracle.build_partitions(w.rowptr, w.col, w.m, w.overlap_ppm, w.seed, w.part_mode, w.user_part)
+    ws, bs = [a.astype(np.float64) for a in w.w0], [b.astype(np.float64) for b in w.b0]
+    gw = np.zeros_like(ws[0])
+    for p, pt in enumerate(rparts):
+        assert pt.n > 5000
+        fw = oracle.forward(pt, w.x[pt.members], ws, bs, w.y[pt.members], w.train_mask[pt.members], w.loss_on_halo)
+        model.forward(p)
+        h_gpu = [model.get(gcnsa.GET_ACT, l, rows=pt.n) for l in (1, 2)]
+        gw += oracle.backward(pt, fw, ws, w.y[pt.members], relu_on=_relu_decisions(fw, h_gpu[:-1]))["dW"][0]
+        model.backward(p)
+    err = np.linalg.norm(model.get(gcnsa.GET_GRAD_W, 0) - gw) / np.linalg.norm(gw)
+    assert gcnsa.tc_status() == 0 and err <= 2.7e-6, err
+    model.close(); parts.close()
+
+
 @pytest.mark.parametrize("c", [1, 32, 33, 64, 65, 128, 129, 256, 257])
 def test_last_layer_gradients_for_every_number_of_classes(tiny_wl, c):
     """The softmax kernel holds a row in 8, 16 or 32 lanes, one or two float4 each (up to 32, 64, 128, 256 columns), and

@@ -577,9 +577,10 @@ int gcnsa_model_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcn
   size_t ws = 0, sc = 0;
   for (int l = 0; l < M->L; ++l) {
     const int64_t din = opts->dims[l], dout = opts->dims[l + 1];
-    ws = std::max(ws, gemm_workspace(opts->gemm_mode, 1, 0, din, dout, M->n_max));
-    ws = std::max(ws, gemm_workspace(opts->gemm_mode, 0, 0, M->n_max, dout, din));
-    ws = std::max(ws, gemm_workspace(opts->gemm_mode, 0, 1, M->n_max, din, dout));
+    // (partitions have at most n_max rows, and one with fewer may be cut into more slices)
+    ws = std::max(ws, gemm_workspace_upto(opts->gemm_mode, 1, 0, din, dout, M->n_max, true));
+    ws = std::max(ws, gemm_workspace_upto(opts->gemm_mode, 0, 0, M->n_max, dout, din, false));
+    ws = std::max(ws, gemm_workspace_upto(opts->gemm_mode, 0, 1, M->n_max, din, dout, false));
     sc = std::max(sc, colsum_scratch(M->n_max, (int32_t)dout));
     sc = std::max(sc, gemm_colsum_scratch(M->n_max, (int32_t)din));  // the fused bias gradient of the layer below
     sc = std::max(sc, (size_t)4 * 148 * (size_t)((din + 3) / 4 * 4) * sizeof(float));  // ... as a narrow product leaves it

@@ -187,7 +187,10 @@ int launch_spmm_rest(void* stream, int64_t n_rows, const int32_t* rowptr, const 
 int launch_gemm(void* stream, int32_t mode, int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k, const float* a,
                 int64_t lda, const float* b, int64_t ldb, float* c, int64_t ldc, int32_t accumulate, int32_t epi,
                 const float* aux, int64_t ldaux, void* workspace, size_t workspace_bytes, int beside = 1);
+// (also enough where the product runs beside others: it has no more slices then)
 size_t gemm_workspace(int32_t mode, int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k);
+// ... for this product and those with a smaller k (inner) or a smaller m (otherwise)
+size_t gemm_workspace_upto(int32_t mode, int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k, bool inner);
 // tensor-core path (3xTF32); returns -1 when the call has to fall back to the fp32 FMA kernel
 // terms: 3 = hi/lo split of both operands (fp32-level accuracy), 1 = the leading TF32 parts only
 int launch_gemm_tc(void* stream, int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k, const float* a, int64_t lda,
@@ -230,6 +233,7 @@ int64_t narrow_blocks(int64_t m, int32_t n);
 int launch_narrow(void* stream, const NarrowArgs& a);
 int64_t gemm_tc_colsum_rows(int32_t ta, int32_t tb, int64_t m, int64_t n);
 size_t gemm_tc_workspace(int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k);
+size_t gemm_tc_workspace_upto(int64_t m, int64_t n, int64_t k);  // ... and for every smaller k
 int launch_splitk_reduce(void* stream, int64_t m, int64_t n, int splits, const float* partial, int64_t ldp, float* c,
                          int64_t ldc,
                          int accumulate, int epi, const float* aux, int64_t ldaux);

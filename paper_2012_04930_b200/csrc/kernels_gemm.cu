@@ -262,8 +262,10 @@ splitk_reduce_v4(int64_t total4, int64_t N, int n_pad4, int splits, const float4
 
 struct Plan {
   int bm, bn, splits;
-  int64_t k_per_split;
+  int64_t wanted, k_per_split;  // wanted: slices before their length is rounded up, at least as many as after
 };
+
+constexpr int64_t kTarget = 2 * 148;  // two resident CTAs on each of the 148 SMs
 
 Plan make_plan(int64_t m, int64_t n, int64_t k) {
   Plan p;
@@ -271,12 +273,12 @@ Plan make_plan(int64_t m, int64_t n, int64_t k) {
   p.bn = n <= 64 ? 64 : 128;
   if (m <= 64) p.bm = 64;
   const int64_t tiles = ((m + p.bm - 1) / p.bm) * ((n + p.bn - 1) / p.bn);
-  const int64_t target = 2 * 148;  // two resident CTAs on each of the 148 SMs
   int64_t splits = 1;
-  if (tiles < target / 2 && k >= 2048) {
-    splits = std::min<int64_t>((target + tiles - 1) / tiles, k / 512);
+  if (tiles < kTarget / 2 && k >= 2048) {
+    splits = std::min<int64_t>((kTarget + tiles - 1) / tiles, k / 512);
     splits = std::max<int64_t>(splits, 1);
   }
+  p.wanted = splits;
   int64_t kps = (k + splits - 1) / splits;
   kps = (kps + BK - 1) / BK * BK;  // keeps every split's first k a multiple of 16 (vector alignment)
   if (kps < BK) kps = BK;          // k = 0 (an empty partition as the inner dimension): one split, no k steps
@@ -316,6 +318,23 @@ size_t gemm_workspace(int32_t mode, int32_t ta, int32_t tb, int64_t m, int64_t n
   const Plan p = make_plan(m, n, k);
   size_t need = p.splits > 1 ? (size_t)p.splits * (size_t)m * (size_t)n * sizeof(float) : 0;
   if (mode != GCNSA_GEMM_FP32) need = std::max(need, gemm_tc_workspace(ta, tb, m, n, k));
+  return need;
+}
+
+// Slices of whole steps make the room that a product needs a sawtooth of its sizes: 500 x 64 takes 33 slices of 9 500 rows
+// and 36 of 9 215.
+size_t gemm_workspace_upto(int32_t mode, int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k, bool inner) {
+  size_t need = 0;
+  if (inner) {
+    const Plan p = make_plan(m, n, k);
+    if (p.wanted > 1) need = (size_t)p.wanted * (size_t)m * (size_t)n * sizeof(float);
+    return mode == GCNSA_GEMM_FP32 ? need : std::max(need, gemm_tc_workspace_upto(m, n, k));
+  }
+  // products of kTarget / 2 tiles or more have one slice; within a tile more rows need more
+  for (int64_t rows = 64; rows <= kTarget / 2 * 128; rows = rows < 128 ? 128 : rows + 128) {
+    need = std::max(need, gemm_workspace(mode, ta, tb, std::min(rows, m), n, k));
+    if (rows >= m) break;
+  }
   return need;
 }
 

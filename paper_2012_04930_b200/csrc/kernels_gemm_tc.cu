@@ -878,7 +878,7 @@ bool make_map(CUtensorMap* map, const float* base, int64_t outer, int64_t inner,
 
 struct TcPlan {
   int bn, splits, cluster, k_blocks, kb_per_split;
-  size_t partial_bytes;
+  size_t partial_bytes, partial_bytes_upto;  // upto: of every smaller k, too
 };
 
 // products that run side by side are cut by the rule below up to this many k-blocks
@@ -911,6 +911,7 @@ TcPlan tc_plan(int64_t m, int64_t n, int64_t k, int beside = 1) {
   // an SM the microseconds in which a block comes up, drains and meets its cluster.  Ten epochs on 20 000 vertices in four
   // partitions 1 476 -> 1 314 us; GraphSAGE epochs (2 816 x 128 x 1 216, four and five at a time) 2 292 -> 2 004 us and 19.9 -> 17.6 ms.
   splits = std::max<int64_t>(splits, 1);
+  const int64_t alone = splits;
   if (beside > 1 && splits > 1 && p.k_blocks <= kBesideBlocks) {
     const int64_t third = sms / std::min(beside, 3) / tiles, length = (p.k_blocks + splits - 1) / splits;
     // Slices of up to twice the length have the error that slices alone would have with all terms in one accumulator (above
@@ -922,14 +923,18 @@ TcPlan tc_plan(int64_t m, int64_t n, int64_t k, int beside = 1) {
   // Eight slices where there would be more lose: each adds its 0.25 to 0.4 us per k-block (500 x 64 x 5 504, 21 slices: 10.5 us, eight:
   // 14.0; 256 x 256 x 8 192: 13.9 and 22.8), and the tensor core cuts its sums off at 24 bits instead of rounding them, so that
   // the error grows with the length of a slice (0.9e-6 of the 2-norm with 8 k-blocks, 2.7e-6 with 33).
-  const int64_t in_cluster = splits <= kMaxCluster && tiles <= kClusterParts * (kClusterSms / splits) ? splits : 1;
+  auto fits = [&](int64_t s) { return s <= kMaxCluster && tiles <= kClusterParts * (kClusterSms / s); };
+  const int64_t in_cluster = fits(splits) ? splits : 1;
   p.kb_per_split = (int)((p.k_blocks + splits - 1) / splits);
   p.splits = (p.k_blocks + p.kb_per_split - 1) / p.kb_per_split;
   if (p.splits < 1) p.splits = 1;
   p.cluster = in_cluster > 1 ? p.splits : 1;
   auto up = [](size_t b) { return (b + 255) / 256 * 256; };
   // the k-slices' partial results: [splits][m][n rounded up to 4] (rows that take 16-byte stores)
-  p.partial_bytes = up(p.splits > 1 && p.cluster == 1 ? (size_t)p.splits * m * ((n + 3) / 4 * 4) * sizeof(float) : 0);
+  const size_t slice = (size_t)m * ((n + 3) / 4 * 4) * sizeof(float);
+  p.partial_bytes = up(p.splits > 1 && p.cluster == 1 ? (size_t)p.splits * slice : 0);
+  // a smaller k makes no more slices than these before they are rounded, and where these fit a cluster fewer do
+  p.partial_bytes_upto = up(alone > 1 && !fits(alone) ? (size_t)alone * slice : 0);
   return p;
 }
 
@@ -1001,6 +1006,8 @@ size_t gemm_tc_workspace(int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k
   (void)ta; (void)tb;  // operands are read in the layout they have: no transposed copies to make room for
   return tc_plan(m, n, k).partial_bytes;
 }
+
+size_t gemm_tc_workspace_upto(int64_t m, int64_t n, int64_t k) { return tc_plan(m, n, k).partial_bytes_upto; }
 
 // Returns 0 on success, a cudaError_t on a CUDA failure, -1 when this shape / alignment / workspace cannot take
 // the tensor-core path (the caller then uses the fp32 FMA kernel).

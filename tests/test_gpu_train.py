@@ -12,7 +12,7 @@ import numpy as np
 import pytest
 import torch
 
-from gen import configs
+from gen import configs, graphs
 from oracle import oracle
 from paper_2012_04930_b200 import gcnsa
 
@@ -560,6 +560,30 @@ def test_weight_gradients_of_partitions_side_by_side_keep_fp32_accuracy(small_wl
     err = np.linalg.norm(model.get(gcnsa.GET_GRAD_W, 0) - gw) / np.linalg.norm(gw)
     assert gcnsa.tc_status() == 0 and err <= 2.7e-6, err
     model.close(); parts.close()
+
+
+@pytest.mark.parametrize("rows,dims", [((9500, 9215, 8200), [500, 64, 5]), ((8500, 8245, 4500), [602, 128, 7])])
+@pytest.mark.parametrize("epoch_graph", [0, 1])
+def test_products_of_partitions_of_any_size_have_their_workspace(rows, dims, epoch_graph):
+    """Partitions with fewer rows than the largest may be cut into more k-slices (500 x 64: 33 of 9 500 rows, 36 of 9 215): no
+    product falls back to the fp32 FMA kernel."""
+    n = sum(rows)
+    rowptr, col = graphs.permutation_graph(n, 3, 5)
+    rng = np.random.default_rng(n)
+    x = rng.standard_normal((n, dims[0]), dtype=np.float32)
+    w0 = [(rng.standard_normal(s) / np.sqrt(s[0])).astype(np.float32) for s in zip(dims[:-1], dims[1:])]
+    with torch.cuda.stream(torch.cuda.Stream()):
+        env = gcnsa.make_env(0)
+        parts = gcnsa.Parts(env, rowptr, col, x, rng.integers(0, dims[-1], n), np.ones(n, np.uint8), dims[-1], len(rows), 0, 3,
+                            gcnsa.PART_USER, np.repeat(np.arange(len(rows)), rows).astype(np.int32))
+        assert tuple(parts.info(p).n for p in range(len(rows))) == rows
+        model = gcnsa.Model(env, parts, dims, w0, gemm_mode=gcnsa.GEMM_TF32X3, epoch_graph=epoch_graph)
+        tc0, fb0 = gcnsa.gemm_path_counts()
+        for _ in range(2):
+            model.epoch()
+        tc1, fb1 = gcnsa.gemm_path_counts()
+        assert tc1 > tc0 and fb1 == fb0 and gcnsa.tc_status() == 0
+        model.close(); parts.close()
 
 
 @pytest.mark.parametrize("c", [1, 32, 33, 64, 65, 128, 129, 256, 257])

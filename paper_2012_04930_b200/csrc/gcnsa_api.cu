@@ -821,7 +821,7 @@ static int forward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& W
     if (M->transform_first[l]) {
       // factored_norm: A_hat T = diag(dinv) (A + I) (diag(dinv) T): the GEMM's epilogue scales the rows of T and
       // the product reads no values
-      if (narrow_ok(M->o.gemm_mode, n, dout, din)) {
+      if (narrow_ok(M->o.gemm_mode, n, dout, din, l == 0)) {
         NarrowArgs na;
         na.m = n; na.n = dout; na.k = din;
         na.a = h; na.lda = ldh;
@@ -954,7 +954,7 @@ static int backward_lane(gcnsa_model* M, const gcnsa_parts* P, int32_t p, Lane& 
         const bool want_scaled = fact && M->transform_first[l - 1];
         int64_t left = 0;
         CK(wait(sums_read));
-        if (narrow_ok(M->o.gemm_mode, n, din, dout)) {
+        if (narrow_ok(M->o.gemm_mode, n, din, dout, false)) {
           NarrowArgs na;
           na.m = n; na.n = din; na.k = dout;
           na.a = W.tmp_b; na.lda = ldo;

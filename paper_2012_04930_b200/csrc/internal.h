@@ -228,7 +228,7 @@ struct NarrowArgs {
   int64_t ldmask = 0;
   float* sums = nullptr;
 };
-bool narrow_ok(int32_t mode, int64_t m, int32_t n, int32_t k);
+bool narrow_ok(int32_t mode, int64_t m, int32_t n, int32_t k, bool first);  // first: of a forward pass
 int64_t narrow_blocks(int64_t m, int32_t n);
 int launch_narrow(void* stream, const NarrowArgs& a);
 int64_t gemm_tc_colsum_rows(int32_t ta, int32_t tb, int64_t m, int64_t n);

@@ -444,14 +444,18 @@ namespace {
 // A product of a few thousand rows with an inner dimension and a width of at most 64 is over in a fraction of what the
 // tensor-core kernel needs to come up, split its operands and turn its accumulator around.  Here W lies in shared memory, a
 // thread computes four columns of a row from the row's float4s (threads of a row read the same ones), and nothing is staged.
-// What bounds it is the latency of one load of A and, with more rows, the FMA pipe and shared memory (fp32, one term): ten epochs on
-// 2 000 vertices (partitions of 1 100 rows) 630 -> 575 us, on 20 000 (5 500 rows) 1 289 -> 1 342, so 4 096 rows are the line.
+// What bounds it is the latency of one load of A and, with more rows or weights, the FMA pipe and shared memory (fp32, one term).
+// Ten epochs on 2 000 vertices (partitions of 1 100 rows) 630 -> 575 us, on 20 000 (5 500 rows) 1 289 -> 1 342, so 4 096 rows are
+// the line.  Weights: recorded epochs of 800 to 4 000 rows and one to eight partitions gain 2 to 20 % with products of up to
+// 64 x 24, are level at 48 x 40 and lose up to 8 % at 64 x 32, 11 % at 64 x 40, 18 % at 64 x 64.  The first product of a pass, which
+// has no kernel before it to come up behind, gains up to 64 x 48 (0 to 12 %) and is level at 64 x 64 (0.96 to 1.07).
 struct Narrow {
   NarrowArgs a;
   int q2, rows;  // quads of C's columns; rows per pass of a block
 };
 constexpr int kNarrowWidth = 64, kNarrowThreads = 256;
 constexpr int64_t kNarrowRows = 4096;
+constexpr int kNarrowWeights = 48 * 40, kNarrowFirstWeights = 64 * 48;
 __global__ void __launch_bounds__(kNarrowThreads) narrow_product(const __grid_constant__ Narrow p) {
   const NarrowArgs& d = p.a;
   if (!d.w_ready) wait_for_predecessors();
@@ -513,8 +517,9 @@ __global__ void __launch_bounds__(kNarrowThreads) narrow_product(const __grid_co
 
 }  // namespace
 
-bool narrow_ok(int32_t mode, int64_t m, int32_t n, int32_t k) {
-  return mode == GCNSA_GEMM_TF32X3 && m > 0 && m <= kNarrowRows && n > 0 && n <= kNarrowWidth && k > 0 && k <= kNarrowWidth;
+bool narrow_ok(int32_t mode, int64_t m, int32_t n, int32_t k, bool first) {
+  return mode == GCNSA_GEMM_TF32X3 && m > 0 && m <= kNarrowRows && n > 0 && n <= kNarrowWidth && k > 0 && k <= kNarrowWidth &&
+         n * k <= (first ? kNarrowFirstWeights : kNarrowWeights);
 }
 int64_t narrow_blocks(int64_t m, int32_t n) {
   const int64_t rows = kNarrowThreads / ((n + 3) / 4);

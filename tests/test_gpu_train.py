@@ -540,6 +540,25 @@ def test_narrow_layers_of_small_partitions_match_checker(tiny_wl, dims, factored
     model.close(); parts.close()
 
 
+@pytest.mark.parametrize("dims,on_tensor_cores", [([64, 16, 5], 2), ([64, 48, 10], 2), ([64, 48, 40], 2), ([64, 48, 41], 4),
+                                                  ([64, 64, 5], 3), ([64, 64, 30], 3), ([64, 64, 31], 5), ([64, 64, 64], 5)])
+def test_wide_products_of_small_partitions_stay_on_the_tensor_cores(tiny_wl, dims, on_tensor_cores):
+    """Of a partition's five products the two weight gradients always run there, the others where they have more than 48 x 40
+    weights (the first of the forward pass: 64 x 48)."""
+    w = copy.copy(tiny_wl)
+    rng = np.random.default_rng(1)
+    w.dims, w.y = dims, rng.integers(0, dims[-1], len(w.y)).astype(np.int32)
+    w.w0 = [(rng.standard_normal(s) / np.sqrt(s[0])).astype(np.float32) for s in zip(dims[:-1], dims[1:])]
+    w.b0 = [np.zeros(d, np.float32) for d in dims[1:]]
+    env, parts, model = _make(w, gemm_mode=gcnsa.GEMM_TF32X3, factored_norm=1)
+    tc0, fb0 = gcnsa.gemm_path_counts()
+    model.forward(0)
+    model.backward(0)
+    tc1, fb1 = gcnsa.gemm_path_counts()
+    assert (tc1 - tc0, fb1 - fb0) == (on_tensor_cores, 0)
+    model.close(); parts.close()
+
+
 def test_weight_gradients_of_partitions_side_by_side_keep_fp32_accuracy(small_wl):
     """Partitions of 5 500 rows (172 k-blocks) whose products are cut for several that run at once: the first layer's weight
     gradient against the checker in the 2-norm.  A slice has at most 18 k-blocks with one cut of at most 2^-23 per 8 k, half of

@@ -281,9 +281,16 @@ __global__ void sage_hidden_grad(const float* __restrict__ dcat, const float* __
 // block, so the loads of a phase are independent of one another and spread over all 256 threads.
 // Partial sums for the loss and both bias gradients leave one row per block, added up in block order by a later launch.
 // 20 000 vertices in batches of 256 (hidden 128, 20 classes): 2 330 -> 2 120 us per epoch; 116 483 (41 classes): 19.7 -> 19.1 ms.
-// Wider output layers and larger batches stay on the tensor cores: their products are work, not latency.
+// Wider output layers and larger batches stay on the tensor cores: their products are work, not latency.  Epochs of workers side by
+// side, one kernel against the launches: 64 to 256 x 20 to 64 in batches of 64 take 0.73 to 0.79 of the time, of 256 0.79 to 0.99; with
+// batches of 1 024 128 x 20 0.92, 128 x 47 0.97, 128 x 64 1.09, 64 x 256 1.36; with 4 096 128 x 20 1.03, 64 x 256 1.57.  Up to 16 classes take
+// 0.82 to 1.02 in batches of 4 096.  So the lines are batch x classes (logits, softmax) and batch x weights (both products).
 constexpr int kHeadRows = 2, kHeadThreads = 256;
-constexpr int64_t kHeadWeights = 32768, kHeadBatch = 4096;
+constexpr int64_t kHeadWeights = 32768, kHeadBatch = 4096, kHeadFewClasses = 16, kHeadBatchClasses = 45000, kHeadBatchWeights = 12 << 20;
+bool head_pays(int64_t batch, int64_t ldh, int64_t ldc, int64_t c) {
+  if (batch > kHeadBatch || c > 256 || ldh > 1024 || 2 * ldh * ldc > kHeadWeights) return false;
+  return c <= kHeadFewClasses || (batch * c <= kHeadBatchClasses && batch * 2 * ldh * ldc <= kHeadBatchWeights);
+}
 struct Head {
   const float* h1;
   int ldh;
@@ -906,7 +913,7 @@ int gcnsa_sage_create(const gcnsa_env* env, const gcnsa_parts* parts, const gcns
                              colsum_scratch(B, (int32_t)S->c));
   // Small output layers (the 41 classes of a 128-wide hidden layer: 12 288 floats of W2) are one kernel; plain TF32 keeps its
   // products on the tensor cores, which is what that mode is there to measure.
-  if (mode != GCNSA_GEMM_TF32 && B <= kHeadBatch && S->c <= 256 && 2 * S->ldh * S->ldc <= kHeadWeights && S->ldh <= 1024) {
+  if (mode != GCNSA_GEMM_TF32 && head_pays(B, S->ldh, S->ldc, S->c)) {
     S->head_qp = 1;
     while (4 * S->head_qp < S->c) S->head_qp *= 2;
     S->head_smem = sizeof(float) * (size_t)(kHeadRows * (4 * S->ldh + 4 * kHeadThreads + 4 * S->head_qp));

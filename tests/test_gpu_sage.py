@@ -99,8 +99,8 @@ def _check_batch(model, pt, x, y, params, tg, seed, epoch, fanout, p, b):
                                                    (16, 256, (3, 2), 65), (16, 257, (3, 2), 64), (256, 41, (2, 5), 33),
                                                    (512, 5, (2, 3), 40), (600, 41, (2, 3), 40), (24, 5, (3, 0), 32)])
 def test_output_layer_of_every_width(hidden, c, fanout, batch, tiny_wl):
-    """The output layer runs in one kernel up to 256 classes and 32 768 weights, two vertices to a block (odd batches), and
-    launch by launch beyond: a full and the ragged last batch against the checker."""
+    """The output layer of small batches runs in one kernel up to 256 classes and 32 768 weights, two vertices to a block (odd
+    batches), and launch by launch beyond: a full and the ragged last batch against the checker."""
     w = copy.copy(tiny_wl)
     w.dims = [w.dims[0], hidden, c]
     w.y = np.random.default_rng(c).integers(0, c, len(w.y)).astype(np.int32)
@@ -109,6 +109,22 @@ def test_output_layer_of_every_width(hidden, c, fanout, batch, tiny_wl):
     for b in (0, len(want) - 1):
         _check_batch(model, rparts[0], xs[0], ys[0], params, want[b], w.seed, 0, fanout, 0, b)
     assert gcnsa.tc_status() == 0
+    model.close(); parts.close()
+
+
+@pytest.mark.parametrize("hidden,c,batch,one_kernel", [
+    (128, 41, 256, 1), (128, 41, 1023, 1), (128, 47, 1024, 0), (256, 256, 64, 0), (64, 256, 175, 1), (64, 256, 176, 0), (256, 64, 384, 1),
+    (256, 64, 385, 0), (512, 16, 4096, 1), (32, 17, 2647, 1), (32, 17, 2648, 0)])
+def test_output_layers_that_are_work_stay_on_the_tensor_cores(hidden, c, batch, one_kernel, tiny_wl):
+    """A batch has three products on the tensor cores where the output layer runs in one kernel, and five otherwise."""
+    w = copy.copy(tiny_wl)
+    w.dims = [w.dims[0], hidden, c]
+    w.y = np.random.default_rng(c).integers(0, c, len(w.y)).astype(np.int32)
+    env, parts, model, *_ = _setup(w, hidden, (2, 2), batch, 0.01, gcnsa.GEMM_TF32X3)
+    tc0, fb0 = gcnsa.gemm_path_counts()
+    model.run_batch(0, 0, 0)
+    tc1, fb1 = gcnsa.gemm_path_counts()
+    assert (tc1 - tc0, fb1 - fb0) == (3 if one_kernel else 5, 0) and gcnsa.tc_status() == 0
     model.close(); parts.close()
 
 

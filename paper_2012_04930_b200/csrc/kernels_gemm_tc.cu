@@ -164,11 +164,15 @@ __device__ __forceinline__ void split_buffer(const uint8_t* hi_buf, uint8_t* lo_
 // 8 or 9 k-blocks, 5.2e-6 -> 2.7e-6 with 33, at the same speed.  With the issuing thread behind elect.sync the tensor pipe sets the pace (see elect_one); behind
 // `lane == 0` an instruction cost it 97 clocks whether 128 or 256 columns wide.  51 249 x 128 x 602: 57 -> 47 us,
 // 269 498 x 256 x 256: 201 -> 151 us, 256 x 256 x 269 498: 169 -> 151 us (L2 flushed).
-template <int BN_, bool A_MN_, bool B_MN_, bool DB_, bool MASKED_ = false>
+template <int BN_, bool A_MN_, bool B_MN_, bool DB_, bool MASKED_ = false, bool CLUSTER_ = false>
 struct Shape {
   static constexpr int BN = BN_;
   static constexpr bool A_MN = A_MN_, B_MN = B_MN_, DB = DB_;
   static constexpr int B_BYTES = BN * BK * 4;
+  // Blocks with one item whose tile's k-slices are a cluster, a kernel of its own: with the cluster's code in it a product that
+  // has none takes 0.1 to 0.4 us longer (2 304 x 128 x 2 080 15.7 us instead of 15.3), and without the other epilogue it has 84
+  // registers a thread instead of 128, which leaves room for other kernels' blocks (GraphSAGE epochs 17.6 -> 16.7 ms).
+  static constexpr bool CLUSTER = CLUSTER_;
   static constexpr bool MASKED = MASKED_;                 // the epilogue of masked_epilogue
   static constexpr int EPI_WARPS = MASKED ? 8 : 4, THREADS = 32 * (kEpiWarp0 + EPI_WARPS);
   static constexpr int EPI_BYTES = EPI_WARPS * 32 * (MASKED ? 32 : EPI_PITCH) * 4;
@@ -360,7 +364,8 @@ gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             int64_t ldc, int accumulate, int epi, const float* __restrict__ aux, int64_t ldaux,
             int64_t slice_stride, int vec_ok, int terms, float* __restrict__ colsum_partial,
             const float* __restrict__ post_scale, int cluster) {
-  const int csplit = S::DB ? 1 : cluster;  // (blocks with several items are never in a cluster)
+  const int csplit = S::CLUSTER ? cluster : 1;
+  if constexpr (S::CLUSTER) __builtin_assume(csplit > 1);  // (so that the other blocks' epilogue is not in this kernel)
   constexpr int BN = S::BN, NS = S::NS, NA = S::NA, B_BYTES = S::B_BYTES;
   constexpr int ACC_COLS = S::ACC_COLS, NBUF = S::NBUF;
   constexpr bool A_MN = S::A_MN, B_MN = S::B_MN;
@@ -639,7 +644,7 @@ gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
       const uint32_t acc = tmem_base + ((uint32_t)(quad * 32) << 16) + ab * ACC_COLS;
       // steps of 32 columns; a step wholly outside C is not taken (C's zeroed pad columns end with N's step)
       const int last_c0 = (((int)min((int64_t)BN, N - wk.n0) + 31) / 32 - 1) * 32;
-      if (!S::DB && csplit > 1) {  // this slice's sums for the cluster, where A landed (all its boxes have been split)
+      if (csplit > 1) {  // this slice's sums for the cluster, where A landed (all its boxes have been split)
         const int r = quad * 32 + lane;
         float* const stash = reinterpret_cast<float*>(smem) + r * BN;
 #pragma unroll 1
@@ -796,7 +801,7 @@ gemm_tf32x3(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(S::TMEM_COLS) : "memory");
   }
-  if constexpr (!S::DB) {
+  if constexpr (S::CLUSTER) {
     if (csplit > 1) {
       // ---------------- k-slices of a tile: every block adds up its share of the rows ----------------
       cluster_sync();
@@ -978,6 +983,9 @@ cudaError_t run_tc(cudaStream_t s, const TcPlan& p, const CUtensorMap& ma, const
   if (total > grid)
     return run_tc_shape<Shape<BN, A_MN, B_MN, true>>(s, p, ma, mb, m, n, (int)tiles_m, (int)tiles_n, (int)total, grid, c,
                                                      ldc, accumulate, epi, aux, ldaux, slice_stride, vec_ok, terms, colsum_partial, post_scale);
+  if (p.cluster > 1)
+    return run_tc_shape<Shape<BN, A_MN, B_MN, false, false, true>>(s, p, ma, mb, m, n, (int)tiles_m, (int)tiles_n, (int)total, grid, c,
+                                                                   ldc, accumulate, epi, aux, ldaux, slice_stride, vec_ok, terms, colsum_partial, post_scale);
   return run_tc_shape<Shape<BN, A_MN, B_MN, false>>(s, p, ma, mb, m, n, (int)tiles_m, (int)tiles_n, (int)total, grid, c,
                                                     ldc, accumulate, epi, aux, ldaux, slice_stride, vec_ok, terms, colsum_partial, post_scale);
 }

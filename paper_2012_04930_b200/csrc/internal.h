@@ -187,7 +187,7 @@ int launch_spmm_rest(void* stream, int64_t n_rows, const int32_t* rowptr, const 
 int launch_gemm(void* stream, int32_t mode, int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k, const float* a,
                 int64_t lda, const float* b, int64_t ldb, float* c, int64_t ldc, int32_t accumulate, int32_t epi,
                 const float* aux, int64_t ldaux, void* workspace, size_t workspace_bytes, int beside = 1);
-// (also enough where the product runs beside others: it has no more slices then)
+// (also where the product runs beside others)
 size_t gemm_workspace(int32_t mode, int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k);
 // ... for this product and those with a smaller k (inner) or a smaller m (otherwise)
 size_t gemm_workspace_upto(int32_t mode, int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k, bool inner);

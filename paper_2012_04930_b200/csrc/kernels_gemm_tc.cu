@@ -888,8 +888,6 @@ struct TcPlan {
 
 // products that run side by side are cut by the rule below up to this many k-blocks
 constexpr int kBesideBlocks = 256;
-// a cluster lives in one of the chip's eight parts, of which at least 16 SMs each are counted on
-constexpr int kClusterParts = 8, kClusterSms = 16;
 
 int sm_count() {
   static int n = 0;
@@ -900,6 +898,35 @@ int sm_count() {
       n = 148;
   });
   return n;
+}
+
+// How many clusters of that many blocks (an SM each) run at the same time.  A cluster lives in one of the chip's parts, whose
+// numbers of SMs differ: 16 tiles of eight slices (2 048 x 128 x 2 080) are two rounds and take 24.6 us, 15.1 as single blocks.
+int cluster_room(int64_t blocks) {
+  static int room[kMaxCluster + 1];
+  static std::once_flag once;
+  std::call_once(once, [] {
+    constexpr int kB200[kMaxCluster + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15};  // where there is no device to ask
+    typedef Shape<128, true, true, false, false, true> S;
+    const bool there = cudaFuncSetAttribute(gemm_tf32x3<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM_BYTES) == cudaSuccess;
+    for (int c = kMaxCluster; c > 0; --c) {
+      cudaLaunchConfig_t config = {};
+      config.gridDim = 840;  // a multiple of all sizes
+      config.blockDim = S::THREADS;
+      config.dynamicSmemBytes = S::SMEM_BYTES;
+      cudaLaunchAttribute size;
+      size.id = cudaLaunchAttributeClusterDimension;
+      size.val.clusterDim.x = c;
+      size.val.clusterDim.y = size.val.clusterDim.z = 1;
+      config.attrs = &size;
+      config.numAttrs = 1;
+      int n = 0;
+      if (!there || cudaOccupancyMaxActiveClusters(&n, gemm_tf32x3<S>, &config) != cudaSuccess || n <= 0) n = kB200[c];
+      room[c] = std::max(n, c < kMaxCluster ? room[c + 1] : 0);
+    }
+    cudaGetLastError();
+  });
+  return room[blocks];
 }
 
 TcPlan tc_plan(int64_t m, int64_t n, int64_t k, int beside = 1) {
@@ -916,20 +943,23 @@ TcPlan tc_plan(int64_t m, int64_t n, int64_t k, int beside = 1) {
   // an SM the microseconds in which a block comes up, drains and meets its cluster.  Ten epochs on 20 000 vertices in four
   // partitions 1 476 -> 1 314 us; GraphSAGE epochs (2 816 x 128 x 1 216, four and five at a time) 2 292 -> 2 004 us and 19.9 -> 17.6 ms.
   splits = std::max<int64_t>(splits, 1);
-  const int64_t alone = splits;
-  if (beside > 1 && splits > 1 && p.k_blocks <= kBesideBlocks) {
-    const int64_t third = sms / std::min(beside, 3) / tiles, length = (p.k_blocks + splits - 1) / splits;
-    // Slices of up to twice the length have the error that slices alone would have with all terms in one accumulator (above
-    // Shape); unbounded, GraphSAGE's hidden weights ended an epoch 1.2e-5 from fp64 instead of 5e-7.
-    splits = std::min(splits, std::max(third, (p.k_blocks + 2 * length - 1) / (2 * length)));
-  }
+  // Slices of up to twice the length have the error that slices alone would have with all terms in one accumulator (above
+  // Shape); unbounded, GraphSAGE's hidden weights ended an epoch 1.2e-5 from fp64 instead of 5e-7.
+  const int64_t alone = splits, longest = 2 * ((p.k_blocks + alone - 1) / alone);
+  if (beside > 1 && splits > 1 && p.k_blocks <= kBesideBlocks)
+    splits = std::min(splits, std::max<int64_t>(sms / std::min(beside, 3) / tiles, (p.k_blocks + longest - 1) / longest));
   // Up to eight slices are a cluster: they meet in shared memory, and the pass over partial results in memory (a launch in the
   // chain) is gone.  Alone on the chip 64 x 16 x 2 112: 9.7 -> 8.0 us, 256 x 256 x 2 112: 12.4 -> 12.1, 2 816 x 128 x 1 204: 16.0 -> 12.9.
-  // Eight slices where there would be more lose: each adds its 0.25 to 0.4 us per k-block (500 x 64 x 5 504, 21 slices: 10.5 us, eight:
-  // 14.0; 256 x 256 x 8 192: 13.9 and 22.8), and the tensor core cuts its sums off at 24 bits instead of rounding them, so that
-  // the error grows with the length of a slice (0.9e-6 of the 2-norm with 8 k-blocks, 2.7e-6 with 33).
-  auto fits = [&](int64_t s) { return s <= kMaxCluster && tiles <= kClusterParts * (kClusterSms / s); };
-  const int64_t in_cluster = fits(splits) ? splits : 1;
+  // Fewer slices than there would be, for a cluster's sake, while they are little longer, at 0.25 to 0.4 us per k-block: eight for ten
+  // of 64 x 16 x 2 752 9.6 -> 8.5 us (602 x 128 x 2 752 13.0 -> 13.2, three at a time 20.1 -> 14.9), five for seven of 2 560 x 128 x 2 080 16.2
+  // -> 14.6, three for four of 4 608 x 128 x 2 080 21.4 -> 18.5; but eight for 21 of 500 x 64 x 5 504 10.5 -> 14.0, for 37 of 256 x 256 x 8 192
+  // 13.9 -> 22.8.
+  auto fits = [&](int64_t s) { return s <= kMaxCluster && tiles <= cluster_room(s); };
+  int64_t in_cluster = std::min<int64_t>(splits, kMaxCluster);
+  while (in_cluster > 1 && !fits(in_cluster)) --in_cluster;
+  const int64_t now = (p.k_blocks + splits - 1) / splits;
+  if ((p.k_blocks + in_cluster - 1) / in_cluster > std::min(longest, now + std::max<int64_t>(4, now / 3))) in_cluster = 1;
+  if (in_cluster > 1) splits = in_cluster;
   p.kb_per_split = (int)((p.k_blocks + splits - 1) / splits);
   p.splits = (p.k_blocks + p.kb_per_split - 1) / p.kb_per_split;
   if (p.splits < 1) p.splits = 1;
@@ -938,7 +968,7 @@ TcPlan tc_plan(int64_t m, int64_t n, int64_t k, int beside = 1) {
   // the k-slices' partial results: [splits][m][n rounded up to 4] (rows that take 16-byte stores)
   const size_t slice = (size_t)m * ((n + 3) / 4 * 4) * sizeof(float);
   p.partial_bytes = up(p.splits > 1 && p.cluster == 1 ? (size_t)p.splits * slice : 0);
-  // a smaller k makes no more slices than these before they are rounded, and where these fit a cluster fewer do
+  // a smaller k makes no more slices than these before they are rounded, and where these fit a cluster fewer do, too
   p.partial_bytes_upto = up(alone > 1 && !fits(alone) ? (size_t)alone * slice : 0);
   return p;
 }
@@ -1012,7 +1042,7 @@ int64_t gemm_tc_colsum_rows(int32_t ta, int32_t tb, int64_t m, int64_t n) {
 
 size_t gemm_tc_workspace(int32_t ta, int32_t tb, int64_t m, int64_t n, int64_t k) {
   (void)ta; (void)tb;  // operands are read in the layout they have: no transposed copies to make room for
-  return tc_plan(m, n, k).partial_bytes;
+  return std::max({tc_plan(m, n, k).partial_bytes, tc_plan(m, n, k, 2).partial_bytes, tc_plan(m, n, k, 3).partial_bytes});
 }
 
 size_t gemm_tc_workspace_upto(int64_t m, int64_t n, int64_t k) { return tc_plan(m, n, k).partial_bytes_upto; }

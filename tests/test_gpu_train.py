@@ -430,6 +430,40 @@ def test_partitions_of_a_recorded_epoch_run_side_by_side(tiny_wl, m):
         parts.close()
 
 
+@pytest.mark.parametrize("name,dims,m,factored_norm,use_bias,loss_rows_only", [
+    ("tiny", [64, 32, 24, 16, 5], 11, 1, 1, 1), ("tiny", [64, 50, 33, 7], 3, 0, 1, 0), ("tiny", [64, 100, 96, 80, 5], 11, 1, 1, 1),
+    ("tiny", [64, 96, 32, 90, 24, 9], 3, 1, 1, 0), ("tiny", [30, 64, 96, 41], 4, 1, 1, 1), ("tiny", [40, 48, 20, 33, 5], 9, 0, 1, 1),
+    ("tiny", [64, 70, 24, 16, 5], 5, 1, 0, 1), ("small", [500, 96, 80, 20], 4, 1, 1, 1), ("small", [500, 64, 40, 24, 20], 4, 0, 1, 0)])
+def test_recorded_epochs_of_deep_models_equal_plain_launches(name, dims, m, factored_norm, use_bias, loss_rows_only, tiny_wl, small_wl):
+    """In a recorded epoch loss, bias gradients and the weight gradients of all layers but the first run beside the pass, whose
+    next layer writes the buffers that they read: three to five layers, narrow products and tensor-core ones alone and in turn,
+    a widening layer, without bias, more partitions than are worked on at once.  Bit for bit the plain launches."""
+    w = tiny_wl if name == "tiny" else small_wl
+    rng = np.random.default_rng(len(dims) + dims[1] + m)
+    x = np.ascontiguousarray(w.x[:, :dims[0]])
+    y = rng.integers(0, dims[-1], len(w.y)).astype(np.int32)
+    shapes = list(zip(dims[:-1], dims[1:]))
+    w0 = [(rng.standard_normal(s) / np.sqrt(s[0])).astype(np.float32) for s in shapes]
+    b0 = [(0.1 * rng.standard_normal(s[1])).astype(np.float32) for s in shapes] if use_bias else None
+    with torch.cuda.stream(torch.cuda.Stream()):
+        env = gcnsa.make_env(0)
+        parts = gcnsa.Parts(env, w.rowptr, w.col, x, y, w.train_mask, dims[-1], m, w.overlap_ppm, w.seed)
+        models = [gcnsa.Model(env, parts, dims, w0, b0, use_bias=use_bias, lr=w.lr, gemm_mode=gcnsa.GEMM_TF32X3,
+                              factored_norm=factored_norm, loss_rows_only=loss_rows_only, epoch_graph=k) for k in (0, 1)]
+        loss = torch.zeros(2, device="cuda")
+        for e in range(4):
+            for k, m_ in enumerate(models):
+                m_.epoch(loss[k:].data_ptr())
+            assert loss[0].item() == loss[1].item(), e
+        for l in range(len(shapes)):
+            for what in (gcnsa.GET_W, gcnsa.GET_ADAM_M_W, gcnsa.GET_ADAM_V_W) + ((gcnsa.GET_B, gcnsa.GET_ADAM_M_B) if use_bias else ()):
+                assert np.array_equal(models[0].get(what, l), models[1].get(what, l)), (what, l)
+        assert gcnsa.tc_status() == 0
+        for m_ in models:
+            m_.close()
+        parts.close()
+
+
 def test_recorded_epoch_on_the_default_stream_falls_back(tiny_wl):
     """The legacy default stream cannot be recorded: epoch_graph then runs
     plain launches with the same results."""

@@ -941,7 +941,7 @@ TcPlan tc_plan(int64_t m, int64_t n, int64_t k, int beside = 1) {
   if (tiles < sms / 2 && p.k_blocks >= 16) splits = std::min<int64_t>(sms / tiles, p.k_blocks / 8);
   // Products that run side by side share the chip: a third of it each.  More slices end a product sooner alone, but each costs
   // an SM the microseconds in which a block comes up, drains and meets its cluster.  Ten epochs on 20 000 vertices in four
-  // partitions 1 476 -> 1 314 us; GraphSAGE epochs (2 816 x 128 x 1 216, four and five at a time) 2 292 -> 2 004 us and 19.9 -> 17.6 ms.
+  // partitions 1 476 -> 1 300 us; GraphSAGE epochs (2 816 x 128 x 1 216, four and five at a time) 2 292 -> 1 970 us and 19.9 -> 16.7 ms.
   splits = std::max<int64_t>(splits, 1);
   // Slices of up to twice the length have the error that slices alone would have with all terms in one accumulator (above
   // Shape); unbounded, GraphSAGE's hidden weights ended an epoch 1.2e-5 from fp64 instead of 5e-7.
